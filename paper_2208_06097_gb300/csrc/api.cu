@@ -842,6 +842,7 @@ sea_status sea_poisson_batch(const double h[3], int n_box, const int* ext, const
     return SEA_ERR_OOM;
   }
   long long tot = 0;
+  int pad_max = 0;
   sea_status rs = SEA_OK;
   for (int b = 0; b < n_box && rs == SEA_OK; ++b) {
     PairInfo P;
@@ -851,6 +852,7 @@ sea_status sea_poisson_batch(const double h[3], int n_box, const int* ext, const
       if (P.ext[a] < 1 || P.ext[a] > 1024) rs = SEA_ERR_ARG;
     }
     P.n = P.ext[0] * P.ext[1] * P.ext[2];
+    pad_max = std::max(pad_max, sea::cg_pad_volume(P.ext[0], P.ext[1], P.ext[2]));
     hb[b] = P;
     ho[b] = tot;
     tot += P.n;
@@ -894,7 +896,7 @@ sea_status sea_poisson_batch(const double h[3], int n_box, const int* ext, const
   if (e == cudaSuccess) e = cudaMemsetAsync(dst, 0, sizeof(unsigned), st);
   if (e == cudaSuccess)
     e = sea::launch_cg_boxes(st, device, h, n_box, dbox, dvoff, dord, rhs, x, r, pp, qq, dit, dst,
-                             dq, tol, tol_mode, max_iter);
+                             dq, tol, tol_mode, max_iter, pad_max);
   unsigned hst = 0;
   if (e == cudaSuccess && iters)
     e = cudaMemcpyAsync(iters, dit, n_box * sizeof(int), cudaMemcpyDeviceToHost, st);

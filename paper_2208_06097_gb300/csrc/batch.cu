@@ -166,9 +166,10 @@ extern "C" sea_status sea_apply_vxx_batch(sea_ctx* const* ctxs, int n, double* c
   // descriptors and items (longest-first ranks dealt round-robin)
   const size_t db = sea::batch_desc_bytes();
   std::vector<unsigned char> hdesc((size_t)n * db);
-  int pad_cap = 0;
+  int pad_cap = 0, pad_cap_f = 0;  // of the mixed-form and FP64 configurations
   for (int k = 0; k < n; ++k) {
-    pad_cap = std::max(pad_cap, sea::cg_pad_cap(ctxs[k]));
+    int& cap = ctxs[k]->prm.precision == 1 ? pad_cap : pad_cap_f;
+    cap = std::max(cap, sea::cg_pad_cap(ctxs[k]));
     ctxs[k]->cg_warm = false;  // the batched form solves from zero
     sea::make_batch_desc(ctxs[k], &hdesc[(size_t)k * db]);
   }
@@ -272,7 +273,7 @@ extern "C" sea_status sea_apply_vxx_batch(sea_ctx* const* ctxs, int n, double* c
     if (e != cudaSuccess) return e;
     e = sea::launch_cg_batch(st, c0->device, c0->bdesc.p,
                              (const int2*)c0->bitems.p + total_mixed, (int)(total - total_mixed),
-                             (int*)c0->queue.p, 0, false, tuned.per_sm_fp64);
+                             (int*)c0->queue.p, pad_cap_f, false, tuned.per_sm_fp64);
     if (e != cudaSuccess) return e;
     c0->launches += (total_mixed > 0) + (total > total_mixed);
     for (int k = 0; k < n; ++k) {
@@ -296,7 +297,7 @@ extern "C" sea_status sea_apply_vxx_batch(sea_ctx* const* ctxs, int n, double* c
     SEA_BCK(cudaEventRecord(ev[2], st), "event");
     for (int k = 0; k < n; ++k) SEA_BCK(sea::launch_pair_setup(ctxs[k]), "pair setup (tuning)");
     const int occ_m = sea::cg_batch_max_ctas_per_sm(c0->device, pad_cap, true);
-    const int occ_f = sea::cg_batch_max_ctas_per_sm(c0->device, 0, false);
+    const int occ_f = sea::cg_batch_max_ctas_per_sm(c0->device, pad_cap_f, false);
     double best = 1e300;
     std::vector<int2> items;
     for (int o = 0; o < N_ORDERS; ++o) {
@@ -315,7 +316,7 @@ extern "C" sea_status sea_apply_vxx_batch(sea_ctx* const* ctxs, int n, double* c
         for (int j = (o == 0 ? 0 : 1); j <= occ; ++j) {  // j = 0: the warm-up launch
           SEA_BCK(cudaEventRecord(ev[0], st), "event");
           SEA_BCK(sea::launch_cg_batch(st, c0->device, c0->bdesc.p, it0, (int)cnt,
-                                       (int*)c0->queue.p, mixed ? pad_cap : 0, mixed, j < 1 ? 1 : j),
+                                       (int*)c0->queue.p, mixed ? pad_cap : pad_cap_f, mixed, j < 1 ? 1 : j),
                   "batched CG (tuning)");
           SEA_BCK(cudaEventRecord(ev[1], st), "event");
           SEA_BCK(cudaEventSynchronize(ev[1]), "tuning");

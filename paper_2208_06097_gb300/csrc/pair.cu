@@ -14,6 +14,7 @@
 //   integral sum rho v dV of Eq. exxGen_mlwf.
 #include <cstring>
 
+#include "cg_fixed.cuh"
 #include "sea_internal.cuh"
 
 namespace sea {
@@ -450,7 +451,32 @@ struct CgArgs {
   int* queue;
   int warm;  // x holds an initial guess (else the solve starts from 0)
   unsigned long long budget_ns;  // time budget of the launch (0: none)
+  FixArgs fix;
 };
+
+// After a pair's solve (the whole CTA): the pair integral of Eq. exxGen_mlwf
+// over Omega_ij (skipped for a bare batch of boxes, phi == nullptr), the
+// iteration count (negative: capped) and the cap flag.
+__device__ __forceinline__ void cg_finish(const CgArgs& A, const PairInfo& P, int pidx,
+                                          const double* __restrict__ x, int iters, double* slots) {
+  const size_t ng = (size_t)A.nx * A.ny * A.nz;
+  const int ex = P.ext[0], ey = P.ext[1];
+  const double* fi = A.phi ? A.phi + (size_t)P.i * ng : nullptr;
+  const double* fj = A.phi ? A.phi + (size_t)P.j * ng : nullptr;
+  double e = 0.0;
+  for (int t = threadIdx.x; fi && t < P.n; t += blockDim.x) {
+    const int xx = t % ex, yy = (t / ex) % ey, zz = t / (ex * ey);
+    const size_t g = ((size_t)wrapi(P.lo[2] + zz, A.nz) * A.ny + wrapi(P.lo[1] + yy, A.ny)) * A.nx +
+                     wrapi(P.lo[0] + xx, A.nx);
+    e = fma(fi[g] * fj[g], x[t], e);
+  }
+  e = block_sum(e, slots);
+  if (threadIdx.x == 0) {
+    if (A.epair) A.epair[pidx] = e * A.dV;
+    A.iters[pidx] = iters;
+    if (iters < 0) atomicOr(A.status, SEA_FLAG_CG_CAP);
+  }
+}
 
 // One pair's FP64 CG (the whole CTA), results into A's per-pair arrays.
 __device__ __forceinline__ void cg_pair_fp64(const CgArgs& A, const StencilW& W, int pidx,
@@ -528,23 +554,157 @@ __device__ __forceinline__ void cg_pair_fp64(const CgArgs& A, const StencilW& W,
     for (int t = threadIdx.x; t < n; t += blockDim.x) pv[t] = fma(beta, pv[t], r[t]);
     __syncthreads();
   }
-  // pair integral of Eq. exxGen_mlwf over Omega_ij (skipped for a bare
-  // batch of boxes, phi == nullptr)
-  const double* fi = A.phi ? A.phi + (size_t)P.i * ng : nullptr;
-  const double* fj = A.phi ? A.phi + (size_t)P.j * ng : nullptr;
-  double e = 0.0;
-  for (int t = threadIdx.x; fi && t < n; t += blockDim.x) {
-    const int xx = t % ex, yy = (t / ex) % ey, zz = t / (ex * ey);
-    const size_t g = ((size_t)wrapi(P.lo[2] + zz, A.nz) * A.ny + wrapi(P.lo[1] + yy, A.ny)) * A.nx +
-                     wrapi(P.lo[0] + xx, A.nx);
-    e = fma(fi[g] * fj[g], x[t], e);
+  cg_finish(A, P, pidx, x, done ? it : -it, red[1]);
+}
+
+// The same CG with the stencil in fixed point (cg_fixed.cuh): the search
+// direction's integers live in shared memory in the mixed CG's padded layout
+// (8 bytes a point), the vectors x and p in global memory, r and q in
+// registers for boxes of at most KPT points per thread (KPT = 0: in global
+// memory, any size).  Same iteration, stopping rule and counts as
+// cg_pair_fp64; q is kept without the factor s_x, which goes into the step.
+// `slots`: 2 x 32 int4.  Returns the iterations (negative: capped).
+template <bool ISO, int KPT>
+__device__ __forceinline__ int cg_fix_loop(const CgArgs& A, int n, int ex, int ey, int ez,
+                                           double* __restrict__ x, double* __restrict__ rg,
+                                           double* __restrict__ pg, double* __restrict__ qg,
+                                           double rr, double target2, int2* __restrict__ Ps,
+                                           int4* slots) {
+  const int S = blockDim.x;
+  constexpr int K = KPT > 0 ? KPT : 1;
+  const int PXY = ex * (ey + SEA_FDP), gap = SEA_FDP * ex, org = SEA_FDP * PXY;
+  const int Vp = PXY * (ez + 2 * SEA_FDP);
+  const double s0 = A.fix.s[0];
+  const double ry = A.fix.s[1] / s0, rz = A.fix.s[2] / s0;
+  double r[K], q[K];
+  int at[K];  // padded index | x coordinate << 20
+  unsigned rmax = 0;
+  for (int t = threadIdx.x; t < Vp; t += S) Ps[t] = make_int2(0, 0);
+  if (KPT > 0) {
+    BoxWalk w(threadIdx.x, S, ex, ey);
+#pragma unroll
+    for (int u = 0; u < K; ++u, w.next(S)) {
+      r[u] = w.t < n ? rg[w.t] : 0.0;
+      q[u] = 0.0;
+      at[u] = (org + w.t + w.z * gap) | (w.x << 20);
+      rmax = max(rmax, (unsigned)__double2hiint(r[u]) & 0x7FFFFFFFu);
+    }
+  } else {
+    for (int t = threadIdx.x; t < n; t += S)
+      rmax = max(rmax, (unsigned)__double2hiint(rg[t]) & 0x7FFFFFFFu);
   }
-  e = block_sum(e, red[1]);
-  if (threadIdx.x == 0) {
-    if (A.epair) A.epair[pidx] = e * A.dV;
-    A.iters[pidx] = done ? it : -it;
-    if (!done) atomicOr(A.status, SEA_FLAG_CG_CAP);
+  // every point of this thread: f(t, padded index, x coordinate, r, q)
+  auto each = [&](auto&& f) {
+    if (KPT > 0) {
+#pragma unroll
+      for (int u = 0; u < K; ++u) {
+        const int t = threadIdx.x + u * S;
+        if (t < n) f(t, at[u] & 0xFFFFF, at[u] >> 20, r[u], q[u]);
+      }
+    } else {
+      BoxWalk w(threadIdx.x, S, ex, ey);
+      for (; w.t < n; w.next(S)) f(w.t, org + w.t + w.z * gap, w.x, rg[w.t], qg[w.t]);
+    }
+  };
+  // bound of |p|, just above the largest |r| (its high word plus one)
+  fix_block_sum(0.0, rmax, slots, &rmax);
+  double M = __hiloint2double((int)(rmax + 1u), 0);
+  int E = (int)(rmax + 1u >> 20) - 1022;
+  each([&](int t, int tp, int, double& rt, double&) { Ps[tp] = fix_quant(rt, E); });
+  __syncthreads();
+  int it = 0;
+  for (;;) {
+    double pq = 0.0;
+    each([&](int t, int tp, int xx, double&, double& qt) {
+      const double pt = pg[t];
+      const double qv = fix_stencil<ISO>(Ps, tp, xx, ex, PXY, ry, rz, E - FIX_BITS);
+      qt = qv;
+      pq = fma(pt, qv, pq);
+    });
+    unsigned none;
+    pq = fix_block_sum(pq, 0u, slots + 32, &none);
+    const double as = rr / pq, alpha = as / s0;
+    double rn = 0.0;
+    rmax = 0;
+    each([&](int t, int, int, double& rt, double& qt) {
+      const double v = fma(-as, qt, rt);
+      rt = v;
+      rn = fma(v, v, rn);
+      rmax = max(rmax, (unsigned)__double2hiint(v) & 0x7FFFFFFFu);
+    });
+    rn = fix_block_sum(rn, rmax, slots, &rmax);
+    ++it;
+    const bool done = rn <= target2;
+    if (done || it >= A.max_iter) {
+      each([&](int t, int, int, double&, double&) { x[t] = fma(alpha, pg[t], x[t]); });
+      __syncthreads();  // Ps is free for the next pair
+      return done ? it : -it;
+    }
+    const double beta = rn / rr;
+    rr = rn;
+    M = fma(beta, M, __hiloint2double((int)(rmax + 1u), 0));
+    E = (int)(((unsigned)__double2hiint(M) & 0x7FFFFFFFu) >> 20) - 1022;
+    each([&](int t, int tp, int, double& rt, double&) {
+      const double po = pg[t];
+      x[t] = fma(alpha, po, x[t]);
+      const double pn = fma(beta, po, rt);
+      pg[t] = pn;
+      Ps[tp] = fix_quant(pn, E);
+    });
+    __syncthreads();
   }
+}
+
+// One pair's FP64-form solve (the whole CTA): the fixed-point stencil where
+// the padded box fits the launch's shared memory and the values stay far
+// from the ends of the FP64 range (also where they are finite), else
+// cg_pair_fp64.
+#define SEA_FIX_KPT 4
+template <bool ISO>
+__device__ __forceinline__ bool cg_pair_fix(const CgArgs& A, const StencilW& W, int pidx,
+                                            double (*red)[32], int4* slots, int2* Ps) {
+  const PairInfo P = A.pinfo[pidx];
+  const int ex = P.ext[0], ey = P.ext[1], ez = P.ext[2], n = P.n;
+  const long long off = A.voff[pidx];
+  double *x = A.x + off, *r = A.r + off, *pv = A.p + off, *q = A.q + off;
+  const double* b = A.b + off;
+  double rr = 0.0, bb = 0.0;
+  for (int t = threadIdx.x; t < n; t += blockDim.x) {
+    const double bt = b[t];
+    double rt = bt;
+    if (A.warm)  // r = b - A x0
+      rt = bt - neg_lap(x, t, t % ex, (t / ex) % ey, t / (ex * ey), ex, ey, ez, W);
+    r[t] = rt;
+    pv[t] = rt;
+    rr = fma(rt, rt, rr);
+    bb = fma(bt, bt, bb);
+  }
+  rr = block_sum(rr, red[0]);
+  bb = block_sum(bb, red[1]);
+  __syncthreads();  // both slot arrays are read before their next use
+  const double target = A.tol_mode == 0 ? A.tol * sqrt(bb)
+                                        : A.tol * 4.0 * 3.14159265358979323846 * sqrt((double)n);
+  const double target2 = target * target;
+  if (!(target2 >= 1e-260 && rr <= 1e200 && bb <= 1e200)) return false;
+  if (!A.warm)
+    for (int t = threadIdx.x; t < n; t += blockDim.x) x[t] = 0.0;
+  int it = 0;
+  if (sqrt(rr) > target)
+    it = n <= SEA_FIX_KPT * (int)blockDim.x
+             ? cg_fix_loop<ISO, SEA_FIX_KPT>(A, n, ex, ey, ez, x, r, pv, q, rr, target2, Ps, slots)
+             : cg_fix_loop<ISO, 0>(A, n, ex, ey, ez, x, r, pv, q, rr, target2, Ps, slots);
+  cg_finish(A, P, pidx, x, it, red[1]);
+  return true;
+}
+
+__device__ __forceinline__ void cg_pair_plain(const CgArgs& A, const StencilW& W, int pidx,
+                                              double (*red)[32], int4* slots, int2* Ps) {
+  const int* e = A.pinfo[pidx].ext;
+  bool solved = false;
+  if (A.fix.mode && cg_pad_volume(e[0], e[1], e[2]) <= A.fix.cap)
+    solved = A.fix.mode == 2 ? cg_pair_fix<true>(A, W, pidx, red, slots, Ps)
+                             : cg_pair_fix<false>(A, W, pidx, red, slots, Ps);
+  if (!solved) cg_pair_fp64(A, W, pidx, red);
 }
 
 // The device's nanosecond clock (the same on every SM).
@@ -567,11 +727,16 @@ __device__ __forceinline__ int claim_item(int* queue, int P, unsigned long long 
   return atomicAdd(queue, 1);
 }
 
-// 3 CTAs per SM: fewer pairs start at once and the longest-first queue
-// balances the tail (measured faster than the 4 CTAs/SM the compiler picks).
-__global__ void __launch_bounds__(256, 3) k_cg(CgArgs A, StencilW W) {
+// CTA size of the plain CG.
+#define SEA_FIX_THREADS 512
+// Padded points of a pair box that two CTAs per SM can hold (8 bytes each).
+#define SEA_FIX_PAD_LIMIT 13824
+
+__global__ void __launch_bounds__(SEA_FIX_THREADS, 2) k_cg(CgArgs A, StencilW W) {
   __shared__ double red[2][32];
+  __shared__ int4 slots[64];
   __shared__ int s_item;
+  extern __shared__ int2 Ps[];  // A.fix.cap points
   const unsigned long long t0 = A.budget_ns ? global_ns() : 0ull;
   for (;;) {
     if (threadIdx.x == 0) s_item = claim_item(A.queue, A.P, A.budget_ns, t0, A.status);
@@ -579,7 +744,7 @@ __global__ void __launch_bounds__(256, 3) k_cg(CgArgs A, StencilW W) {
     const int item = s_item;
     if (item >= A.P) break;
     const int pidx = A.order[item];
-    cg_pair_fp64(A, W, pidx, red);
+    cg_pair_plain(A, W, pidx, red, slots, Ps);
     __syncthreads();
   }
 }
@@ -685,17 +850,6 @@ __device__ __forceinline__ float neg_lap_f(const float* __restrict__ pv, int t, 
   const float ay = lap_axis_f(pv, t, y, ey, ex, W.ax[1]);
   const float az = fmaf(W.center, pv[t], lap_axis_f(pv, t, z, ez, ex * ey, W.ax[2]));
   return (ax + ay) + az;
-}
-
-// Shared-memory layout of the mixed CG's residual: the pair box's planes of
-// ex x ey points stored row after row (so consecutive points of a warp sit
-// in consecutive banks), each plane followed by F = SEA_FDP zero rows, which
-// serve as the y halo on both sides, and F zero planes before and after the
-// box for the z halo.  Box point t = (z ey + y) ex + x sits at
-// org + t + z F ex.  Neighbours along y and z outside the box read zeros;
-// along x they are masked.
-__host__ __device__ __forceinline__ int cg_pad_volume(int ex, int ey, int ez) {
-  return ex * (ey + SEA_FDP) * (ez + 2 * SEA_FDP);
 }
 
 // -Lap_h r at padded index tp (box x coordinate x, row length ex, plane
@@ -1113,17 +1267,20 @@ struct BatchCg {
 };
 
 // MIXED: the items are all mixed-form (CTA of SEA_CG_THREADS, as k_cg_mixed)
-// or all FP64 (CTA of 256, as k_cg), so every pair is solved with the same
-// CTA size, hence the same bits, as in its own configuration's launch.
+// or all FP64 (CTA of SEA_FIX_THREADS, as k_cg), so every pair is solved with
+// the same CTA size, hence the same bits, as in its own configuration's launch.
 template <bool MIXED>
-__global__ void __launch_bounds__(MIXED ? SEA_CG_THREADS : 256, MIXED ? 1024 / SEA_CG_THREADS : 2)
+__global__ void __launch_bounds__(MIXED ? SEA_CG_THREADS : SEA_FIX_THREADS,
+                                  MIXED ? 1024 / SEA_CG_THREADS : 2)
     k_cg_batch(const BatchCg* __restrict__ descs, const int2* __restrict__ items, int total,
                int* __restrict__ queue) {
   __shared__ double red[2][32];
   __shared__ int s_item;
   __shared__ BatchCg d;
   __shared__ double bc;
-  extern __shared__ float pS[];  // the largest pad_cap of the descriptors
+  __shared__ int4 slots[64];
+  extern __shared__ int2 Ps[];  // the largest capacity of the descriptors
+  float* pS = reinterpret_cast<float*>(Ps);
   for (;;) {
     if (threadIdx.x == 0) s_item = atomicAdd(queue, 1);
     __syncthreads();
@@ -1140,7 +1297,7 @@ __global__ void __launch_bounds__(MIXED ? SEA_CG_THREADS : 256, MIXED ? 1024 / S
     if (MIXED)
       cg_pair_mixed(d.m, d.W, d.Wf, d.m.order[it.y], red, &bc, pS);
     else
-      cg_pair_fp64(d.a, d.W, d.a.order[it.y], red);
+      cg_pair_plain(d.a, d.W, d.a.order[it.y], red, slots, Ps);
     __syncthreads();
   }
 }
@@ -1232,6 +1389,19 @@ static CgMixedArgs mixed_args(sea_ctx* c) {
   return A;
 }
 
+// The fixed-point stencil's arguments for spacings h and boxes of at most
+// pad_max padded points; not used for spacings whose weights leave 1e+-30.
+static FixArgs make_fix(const double h[3], int pad_max) {
+  FixArgs F;
+  F.mode = h[0] == h[1] && h[1] == h[2] ? 2 : 1;
+  for (int a = 0; a < 3; ++a) {
+    F.s[a] = 1.0 / (SEA_FIX_DEN * h[a] * h[a]);
+    if (!(F.s[a] > 1e-30 && F.s[a] < 1e30)) F.mode = 0;
+  }
+  F.cap = F.mode ? std::min(pad_max, SEA_FIX_PAD_LIMIT) : 0;
+  return F;
+}
+
 static CgArgs fp64_args(sea_ctx* c) {
   CgArgs A;
   memset(&A, 0, sizeof(A));
@@ -1258,39 +1428,50 @@ static CgArgs fp64_args(sea_ctx* c) {
   A.queue = (int*)c->queue.p;
   A.warm = c->cg_warm ? 1 : 0;
   A.budget_ns = (unsigned long long)(c->prm.timeout_ms * 1e6);
+  A.fix = make_fix(c->h, c->cg_pad_max);
   return A;
 }
 
-// Shared memory of the mixed CG's padded search direction: the largest
-// padded pair box, at most SEA_CG_PAD_LIMIT floats (four CTAs per SM);
-// pairs above the limit solve on global vectors.
+// Shared memory of the CG's padded vector: the largest padded pair box, at
+// most the form's limit (two CTAs per SM); pairs above it solve on global
+// vectors.  Mixed form: floats of the residual; FP64 form: 8-byte fixed-point
+// values of the search direction.
 #define SEA_CG_PAD_LIMIT 13824
 int cg_pad_cap(const sea_ctx* c) {
-  return c->prm.precision == 1 ? std::min(c->cg_pad_max, SEA_CG_PAD_LIMIT) : 0;
+  return c->prm.precision == 1 ? std::min(c->cg_pad_max, SEA_CG_PAD_LIMIT)
+                               : make_fix(c->h, c->cg_pad_max).cap;
+}
+static size_t cg_smem_bytes(int pad_cap, bool mixed) {
+  return (size_t)pad_cap * (mixed ? sizeof(float) : sizeof(int2));
+}
+static cudaError_t cg_allow_smem(const void* kernel, bool mixed) {
+  return cudaFuncSetAttribute(
+      kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+      (int)(mixed ? SEA_CG_PAD_LIMIT * sizeof(float) : SEA_FIX_PAD_LIMIT * sizeof(int2)));
 }
 
 cudaError_t launch_cg(sea_ctx* c) {
   if (c->P == 0) return cudaSuccess;
   int nsm = 0, occ = 0;
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device);
-  const int pad_cap = cg_pad_cap(c);
-  const size_t smem = (size_t)pad_cap * sizeof(float);
-  if (c->prm.precision == 1) {
-    cudaError_t e = cudaFuncSetAttribute(k_cg_mixed, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)(SEA_CG_PAD_LIMIT * sizeof(float)));
+  const bool mixed = c->prm.precision == 1;
+  const size_t smem = cg_smem_bytes(cg_pad_cap(c), mixed);
+  {
+    const cudaError_t e = cg_allow_smem(mixed ? (const void*)k_cg_mixed : (const void*)k_cg, mixed);
     if (e != cudaSuccess) return e;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_cg_mixed, SEA_CG_THREADS, smem);
-  } else {
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_cg, 256, 0);
   }
+  if (mixed)
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_cg_mixed, SEA_CG_THREADS, smem);
+  else
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_cg, SEA_FIX_THREADS, smem);
   if (occ < 1) occ = 1;
   const int grid = min(c->P, nsm * occ);
   cudaMemsetAsync(c->queue.p, 0, sizeof(int), c->stream);
   const StencilW W = make_weights(c);
-  if (c->prm.precision == 1)
+  if (mixed)
     k_cg_mixed<<<grid, SEA_CG_THREADS, smem, c->stream>>>(mixed_args(c), W, make_weights_f(W));
   else
-    k_cg<<<grid, 256, 0, c->stream>>>(fp64_args(c), W);
+    k_cg<<<grid, SEA_FIX_THREADS, smem, c->stream>>>(fp64_args(c), W);
   c->launches += 1;
   return cudaGetLastError();
 }
@@ -1342,12 +1523,10 @@ void make_batch_desc(sea_ctx* c, void* out) {
 size_t batch_desc_bytes() { return sizeof(BatchCg); }
 
 int cg_batch_max_ctas_per_sm(int device, int pad_cap, bool mixed) {
-  const size_t smem = (size_t)pad_cap * sizeof(float);
-  const int threads = mixed ? SEA_CG_THREADS : 256;
+  const size_t smem = cg_smem_bytes(pad_cap, mixed);
+  const int threads = mixed ? SEA_CG_THREADS : SEA_FIX_THREADS;
   auto kern = mixed ? k_cg_batch<true> : k_cg_batch<false>;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)(SEA_CG_PAD_LIMIT * sizeof(float))) != cudaSuccess)
-    return 1;
+  if (cg_allow_smem((const void*)kern, mixed) != cudaSuccess) return 1;
   int occ = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, threads, smem);
   (void)device;
@@ -1359,8 +1538,8 @@ cudaError_t launch_cg_batch(cudaStream_t st, int device, const void* descs, cons
   if (total == 0) return cudaSuccess;
   int nsm = 0;
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, device);
-  const size_t smem = (size_t)pad_cap * sizeof(float);
-  const int threads = mixed ? SEA_CG_THREADS : 256;
+  const size_t smem = cg_smem_bytes(pad_cap, mixed);
+  const int threads = mixed ? SEA_CG_THREADS : SEA_FIX_THREADS;
   auto kern = mixed ? k_cg_batch<true> : k_cg_batch<false>;
   const int occ = cg_batch_max_ctas_per_sm(device, pad_cap, mixed);
   const int per_sm = ctas_per_sm >= 1 ? min(ctas_per_sm, occ) : occ;
@@ -1372,12 +1551,13 @@ cudaError_t launch_cg_batch(cudaStream_t st, int device, const void* descs, cons
 
 // Batched solve of -Lap_h x = rhs on independent boxes (no pair energies):
 // boxes[] and voff[] on the device, order[] the processing order; r, p, q
-// scratch of the same total length as x.
+// scratch of the same total length as x; pad_max the boxes' largest
+// cg_pad_volume.
 cudaError_t launch_cg_boxes(cudaStream_t stream, int device, const double h[3], int nbox,
                             const PairInfo* boxes, const long long* voff, const int* order,
                             const double* rhs, double* x, double* r, double* p, double* q,
                             int* iters, unsigned* status, int* queue, double tol, int tol_mode,
-                            int max_iter) {
+                            int max_iter, int pad_max) {
   if (nbox == 0) return cudaSuccess;
   double w[SEA_FDP + 1];
   fornberg_weights(w);
@@ -1393,12 +1573,16 @@ cudaError_t launch_cg_boxes(cudaStream_t stream, int device, const double h[3], 
   }
   int nsm = 0, occ = 0;
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, device);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_cg, 256, 0);
-  if (occ < 1) occ = 1;
-  cudaError_t e = cudaMemsetAsync(queue, 0, sizeof(int), stream);
-  if (e != cudaSuccess) return e;
   CgArgs A;
   memset(&A, 0, sizeof(A));
+  A.fix = make_fix(h, pad_max);
+  const size_t smem = cg_smem_bytes(A.fix.cap, false);
+  cudaError_t e = cg_allow_smem((const void*)k_cg, false);
+  if (e != cudaSuccess) return e;
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_cg, SEA_FIX_THREADS, smem);
+  if (occ < 1) occ = 1;
+  e = cudaMemsetAsync(queue, 0, sizeof(int), stream);
+  if (e != cudaSuccess) return e;
   A.phi = nullptr;
   A.nx = A.ny = A.nz = 1;
   A.pinfo = boxes;
@@ -1418,7 +1602,7 @@ cudaError_t launch_cg_boxes(cudaStream_t stream, int device, const double h[3], 
   A.iters = iters;
   A.status = status;
   A.queue = queue;
-  k_cg<<<min(nbox, nsm * occ), 256, 0, stream>>>(A, W);
+  k_cg<<<min(nbox, nsm * occ), SEA_FIX_THREADS, smem, stream>>>(A, W);
   return cudaGetLastError();
 }
 

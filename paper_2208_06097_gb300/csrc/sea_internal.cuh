@@ -939,6 +939,18 @@ __device__ __forceinline__ void contrib_range(int part, bool compact, const WinS
 }
 
 
+// Shared-memory layout of a CG vector on a pair box: the planes of ex x ey
+// points stored row after row (so consecutive points of a warp sit in
+// consecutive banks), each plane followed by F = SEA_FDP zero rows, which
+// serve as the y halo on both sides, and F zero planes before and after the
+// box for the z halo.  Box point t = (z ey + y) ex + x sits at
+// F ex (ey + F) + t + z F ex.  Neighbours along y and z outside the box read
+// zeros; along x they are masked.  Points of the layout (INT_MAX above that):
+__host__ __device__ __forceinline__ int cg_pad_volume(int ex, int ey, int ez) {
+  const long long v = (long long)ex * (ey + SEA_FDP) * (ez + 2 * SEA_FDP);
+  return v > 2147483647LL ? 2147483647 : (int)v;
+}
+
 // Launch wrappers (each file implements its own).
 cudaError_t launch_plan_boxes(sea_ctx* c);
 cudaError_t launch_plan_pairs(sea_ctx* c);
@@ -1004,6 +1016,6 @@ cudaError_t launch_cg_boxes(cudaStream_t stream, int device, const double h[3], 
                             const PairInfo* boxes, const long long* voff, const int* order,
                             const double* rhs, double* x, double* r, double* p, double* q,
                             int* iters, unsigned* status, int* queue, double tol, int tol_mode,
-                            int max_iter);
+                            int max_iter, int pad_max);
 cudaError_t upload_harmonics_accum();
 }  // namespace sea
