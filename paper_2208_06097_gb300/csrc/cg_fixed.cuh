@@ -98,25 +98,66 @@ __device__ __forceinline__ FixSum fix_warp_sum(double v) {
   return FixSum{fix_warp_add(X), (int)em};
 }
 
-// Block sum and block maximum in one barrier; `slots` holds one int4 per warp
-// (at most 32), reused only after the next __syncthreads.
-__device__ __forceinline__ double fix_block_sum(double v, unsigned vmax, int4* slots,
-                                                unsigned* bmax) {
+// The warp's part of a block sum and a block maximum: lane 0 posts them.
+__device__ __forceinline__ void fix_post(double v, unsigned vmax, int4* slots) {
   const FixSum w = fix_warp_sum(v);
   const unsigned wm = __reduce_max_sync(0xffffffffu, vmax);
+  if ((threadIdx.x & 31) == 0)
+    slots[threadIdx.x >> 5] = make_int4((int)(unsigned)w.X, (int)(w.X >> 32), w.e, (int)wm);
+}
+
+// The block's sum (and maximum) from the warps' posts, by one whole warp.
+__device__ __forceinline__ FixSum fix_combine(const int4* slots, unsigned* bmax) {
   const int lane = threadIdx.x & 31, nw = (blockDim.x + 31) >> 5;
-  if (lane == 0)
-    slots[threadIdx.x >> 5] =
-        make_int4((int)(unsigned)w.X, (int)(w.X >> 32), w.e, (int)wm);
-  __syncthreads();
   int4 s = make_int4(0, 0, 0, 0);
   if (lane < nw) s = slots[lane];
   const int E = (int)__reduce_max_sync(0xffffffffu, (unsigned)s.z);
   *bmax = __reduce_max_sync(0xffffffffu, (unsigned)s.w);
   const long long X = ((long long)s.y << 32) | (long long)(unsigned)s.x;
-  const long long S = fix_warp_add(X >> min(E - s.z + 5, 63));  // 5 bits of room for 32 warps
-  return scaled_i64(S, E - 1080 + 5);
+  // 5 bits of room for 32 warps
+  return FixSum{fix_warp_add(X >> min(E - s.z + 5, 63)), E + 5};
 }
+
+// 1 / b as Y 2^e for a positive sum b (Y = 0 if it is not), good to 2^-59:
+// two Newton steps in integer arithmetic from the FP32 reciprocal of b's
+// leading 24 bits.
+struct FixRecip {
+  unsigned long long Y;
+  int e;
+};
+__device__ __forceinline__ FixRecip fix_recip(FixSum b) {
+  const int lb = __clzll(b.X);
+  const unsigned long long B = (unsigned long long)b.X << lb;
+  const float f = __frcp_rn((float)(unsigned)(B >> 40));  // in (2^-24, 2^-23]
+  // Y ~ 2^126 / B, kept below 2^63
+  unsigned long long Y = ((unsigned long long)(unsigned)(f * 140737488355328.0f) << 39) - 1ULL;
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const long long d = (1LL << 62) - (long long)__umul64hi(B, Y);
+    Y += (unsigned long long)(__mul64hi((long long)Y, d) << 2);
+  }
+  return FixRecip{b.X > 0 ? Y : 0ULL, lb - b.e - 126};
+}
+// a / b from b's reciprocal, for a positive a (else 0), one rounding to FP64.
+__device__ __forceinline__ double fix_ratio(FixSum a, FixRecip r) {
+  if (a.X <= 0) return 0.0;
+  const int la = __clzll(a.X);
+  const long long Q = (long long)__umul64hi((unsigned long long)a.X << la, r.Y);
+  return scaled_i64(Q, 64 - la + a.e + r.e);
+}
+
+// An FP32 value just above the non-negative FP64 value with high word h,
+// divided by 2^k (at least 2^-120).
+__device__ __forceinline__ float fix_upper(unsigned h, int k) {
+  const int ef = (int)(h >> 20) - 1023 - k + 127;
+  return __uint_as_float(((unsigned)max(ef, 7) << 23 | (h & 0xFFFFFu) << 3) + 8u);
+}
+
+// Scalars of a step that one warp forms for the block.
+struct FixScal {
+  double as, beta;
+  int E, done;
+};
 
 // What the fixed-point solve needs beside the CG's own arguments.
 struct FixArgs {

@@ -558,99 +558,125 @@ __device__ __forceinline__ void cg_pair_fp64(const CgArgs& A, const StencilW& W,
 }
 
 // The same CG with the stencil in fixed point (cg_fixed.cuh): the search
-// direction's integers live in shared memory in the mixed CG's padded layout
-// (8 bytes a point), the vectors x and p in global memory, r and q in
-// registers for boxes of at most KPT points per thread (KPT = 0: in global
-// memory, any size).  Same iteration, stopping rule and counts as
-// cg_pair_fp64; q is kept without the factor s_x, which goes into the step.
-// `slots`: 2 x 32 int4.  Returns the iterations (negative: capped).
-template <bool ISO, int KPT>
+// direction's integers live in shared memory in the padded layout (8 bytes a
+// point), the FP64 vectors x, r, p and q in global memory (L1 and L2; holding
+// r and q in registers measured the same).  Same iteration, stopping rule and
+// counts as cg_pair_fp64; q is kept without the factor s_x, which goes into
+// the step.  The step's scalars are formed by the last warp, whose share of
+// the points is the smallest, in integer arithmetic: one warp's FP64
+// instruction takes as long as a full one's, and every warp dividing took
+// more of the FP64 unit than the vector updates.  `slots`: 2 x 32 int4.
+// Returns the iterations (negative: capped).
+template <bool ISO>
 __device__ __forceinline__ int cg_fix_loop(const CgArgs& A, int n, int ex, int ey, int ez,
-                                           double* __restrict__ x, double* __restrict__ rg,
-                                           double* __restrict__ pg, double* __restrict__ qg,
-                                           double rr, double target2, int2* __restrict__ Ps,
-                                           int4* slots) {
+                                           double* __restrict__ x, double* __restrict__ r,
+                                           double* __restrict__ p, double* __restrict__ q,
+                                           double target2, int2* __restrict__ Ps, int4* slots) {
+  __shared__ FixScal sc;
   const int S = blockDim.x;
-  constexpr int K = KPT > 0 ? KPT : 1;
   const int PXY = ex * (ey + SEA_FDP), gap = SEA_FDP * ex, org = SEA_FDP * PXY;
   const int Vp = PXY * (ez + 2 * SEA_FDP);
-  const double s0 = A.fix.s[0];
+  const double s0 = A.fix.s[0], inv_s0 = 1.0 / s0;
   const double ry = A.fix.s[1] / s0, rz = A.fix.s[2] / s0;
-  double r[K], q[K];
-  int at[K];  // padded index | x coordinate << 20
-  unsigned rmax = 0;
+  const bool lead = (threadIdx.x >> 5) == (blockDim.x >> 5) - 1;
+  const bool post = (threadIdx.x & 31) == 0;
   for (int t = threadIdx.x; t < Vp; t += S) Ps[t] = make_int2(0, 0);
-  if (KPT > 0) {
-    BoxWalk w(threadIdx.x, S, ex, ey);
-#pragma unroll
-    for (int u = 0; u < K; ++u, w.next(S)) {
-      r[u] = w.t < n ? rg[w.t] : 0.0;
-      q[u] = 0.0;
-      at[u] = (org + w.t + w.z * gap) | (w.x << 20);
-      rmax = max(rmax, (unsigned)__double2hiint(r[u]) & 0x7FFFFFFFu);
-    }
-  } else {
-    for (int t = threadIdx.x; t < n; t += S)
-      rmax = max(rmax, (unsigned)__double2hiint(rg[t]) & 0x7FFFFFFFu);
-  }
-  // every point of this thread: f(t, padded index, x coordinate, r, q)
-  auto each = [&](auto&& f) {
-    if (KPT > 0) {
-#pragma unroll
-      for (int u = 0; u < K; ++u) {
-        const int t = threadIdx.x + u * S;
-        if (t < n) f(t, at[u] & 0xFFFFF, at[u] >> 20, r[u], q[u]);
-      }
-    } else {
-      BoxWalk w(threadIdx.x, S, ex, ey);
-      for (; w.t < n; w.next(S)) f(w.t, org + w.t + w.z * gap, w.x, rg[w.t], qg[w.t]);
-    }
+  // r to v and rmax: the sum of squares and the largest high word
+  auto square = [&](double rt, double& v, unsigned& rmax) {
+    v = fma(rt, rt, v);
+    rmax = max(rmax, (unsigned)__double2hiint(rt) & 0x7FFFFFFFu);
   };
-  // bound of |p|, just above the largest |r| (its high word plus one)
-  fix_block_sum(0.0, rmax, slots, &rmax);
-  double M = __hiloint2double((int)(rmax + 1u), 0);
-  int E = (int)(rmax + 1u >> 20) - 1022;
-  each([&](int t, int tp, int, double& rt, double&) { Ps[tp] = fix_quant(rt, E); });
+  // lead warp: rr, its reciprocal, and the bound M 2^k0 of |p| (M FP32, kept
+  // from below by rounding up): the next |p| <= |r| + beta |p|
+  FixSum rr{0, 0};
+  FixRecip irr{0, 0};
+  float M = 0.f;
+  int k0 = 0;
+  {
+    double v = 0.0;
+    unsigned rmax = 0;
+    for (int t = threadIdx.x; t < n; t += S) square(r[t], v, rmax);
+    fix_post(v, rmax, slots);
+    __syncthreads();
+    if (lead) {
+      rr = fix_combine(slots, &rmax);
+      irr = fix_recip(rr);
+      k0 = (int)(rmax >> 20) - 1023;
+      M = fix_upper(rmax, k0);
+      if (post) sc.E = k0 + (int)(__float_as_uint(M) >> 23) - 126;
+    }
+    __syncthreads();
+  }
+  int E = sc.E;
+  for (BoxWalk w(threadIdx.x, S, ex, ey); w.t < n; w.next(S))
+    Ps[org + w.t + w.z * gap] = fix_quant(r[w.t], E);
   __syncthreads();
   int it = 0;
   for (;;) {
-    double pq = 0.0;
-    each([&](int t, int tp, int xx, double&, double& qt) {
-      const double pt = pg[t];
-      const double qv = fix_stencil<ISO>(Ps, tp, xx, ex, PXY, ry, rz, E - FIX_BITS);
-      qt = qv;
-      pq = fma(pt, qv, pq);
-    });
-    unsigned none;
-    pq = fix_block_sum(pq, 0u, slots + 32, &none);
-    const double as = rr / pq, alpha = as / s0;
-    double rn = 0.0;
-    rmax = 0;
-    each([&](int t, int, int, double& rt, double& qt) {
-      const double v = fma(-as, qt, rt);
-      rt = v;
-      rn = fma(v, v, rn);
-      rmax = max(rmax, (unsigned)__double2hiint(v) & 0x7FFFFFFFu);
-    });
-    rn = fix_block_sum(rn, rmax, slots, &rmax);
+    double v = 0.0;
+    for (BoxWalk w(threadIdx.x, S, ex, ey); w.t < n; w.next(S)) {
+      const double pt = p[w.t];
+      const double qt = fix_stencil<ISO>(Ps, org + w.t + w.z * gap, w.x, ex, PXY, ry, rz,
+                                         E - FIX_BITS);
+      q[w.t] = qt;
+      v = fma(pt, qt, v);
+    }
+    fix_post(v, 0u, slots);
+    __syncthreads();
+    if (lead) {
+      unsigned none;
+      const double as = fix_ratio(rr, fix_recip(fix_combine(slots, &none)));
+      if (post) sc.as = as;
+    }
+    __syncthreads();
+    const double as = sc.as;
+    v = 0.0;
+    unsigned rmax = 0;
+    for (int t = threadIdx.x; t < n; t += 2 * S) {  // two points' loads in flight
+      const bool two = t + S < n;
+      const double q0 = q[t], r0 = r[t];
+      const double q1 = two ? q[t + S] : 0.0, r1 = two ? r[t + S] : 0.0;
+      const double y0 = fma(-as, q0, r0);
+      r[t] = y0;
+      square(y0, v, rmax);
+      if (two) {
+        const double y1 = fma(-as, q1, r1);
+        r[t + S] = y1;
+        square(y1, v, rmax);
+      }
+    }
+    fix_post(v, rmax, slots + 32);
+    __syncthreads();
     ++it;
-    const bool done = rn <= target2;
+    if (lead) {
+      rr = fix_combine(slots + 32, &rmax);
+      const double beta = fix_ratio(rr, irr);
+      M = __fmaf_ru(fix_upper((unsigned)__double2hiint(beta), 0), M, fix_upper(rmax, k0));
+      if (post) {
+        sc.beta = beta;
+        sc.E = k0 + (int)(__float_as_uint(M) >> 23) - 126;
+        // non-negative FP64 values compare as their bit patterns
+        sc.done = __double_as_longlong(scaled_i64(rr.X, rr.e - 1080)) <=
+                  __double_as_longlong(target2);
+      }
+    }
+    __syncthreads();
+    const double alpha = as * inv_s0, beta = sc.beta;
+    E = sc.E;
+    const bool done = sc.done;
     if (done || it >= A.max_iter) {
-      each([&](int t, int, int, double&, double&) { x[t] = fma(alpha, pg[t], x[t]); });
-      __syncthreads();  // Ps is free for the next pair
+      for (int t = threadIdx.x; t < n; t += S) x[t] = fma(alpha, p[t], x[t]);
+      __syncthreads();  // Ps and sc are free for the next pair
       return done ? it : -it;
     }
-    const double beta = rn / rr;
-    rr = rn;
-    M = fma(beta, M, __hiloint2double((int)(rmax + 1u), 0));
-    E = (int)(((unsigned)__double2hiint(M) & 0x7FFFFFFFu) >> 20) - 1022;
-    each([&](int t, int tp, int, double& rt, double&) {
-      const double po = pg[t];
-      x[t] = fma(alpha, po, x[t]);
+    for (BoxWalk w(threadIdx.x, S, ex, ey); w.t < n; w.next(S)) {
+      const double po = p[w.t], rt = r[w.t];
+      x[w.t] = fma(alpha, po, x[w.t]);
       const double pn = fma(beta, po, rt);
-      pg[t] = pn;
-      Ps[tp] = fix_quant(pn, E);
-    });
+      p[w.t] = pn;
+      Ps[org + w.t + w.z * gap] = fix_quant(pn, E);
+    }
+    if (lead) irr = fix_recip(rr);
     __syncthreads();
   }
 }
@@ -659,7 +685,6 @@ __device__ __forceinline__ int cg_fix_loop(const CgArgs& A, int n, int ex, int e
 // the padded box fits the launch's shared memory and the values stay far
 // from the ends of the FP64 range (also where they are finite), else
 // cg_pair_fp64.
-#define SEA_FIX_KPT 4
 template <bool ISO>
 __device__ __forceinline__ bool cg_pair_fix(const CgArgs& A, const StencilW& W, int pidx,
                                             double (*red)[32], int4* slots, int2* Ps) {
@@ -685,14 +710,12 @@ __device__ __forceinline__ bool cg_pair_fix(const CgArgs& A, const StencilW& W, 
   const double target = A.tol_mode == 0 ? A.tol * sqrt(bb)
                                         : A.tol * 4.0 * 3.14159265358979323846 * sqrt((double)n);
   const double target2 = target * target;
-  if (!(target2 >= 1e-260 && rr <= 1e200 && bb <= 1e200)) return false;
+  if (!(target2 >= 1e-260 && target2 >= 1e-60 * rr && rr <= 1e200 && bb <= 1e200)) return false;
   if (!A.warm)
     for (int t = threadIdx.x; t < n; t += blockDim.x) x[t] = 0.0;
   int it = 0;
   if (sqrt(rr) > target)
-    it = n <= SEA_FIX_KPT * (int)blockDim.x
-             ? cg_fix_loop<ISO, SEA_FIX_KPT>(A, n, ex, ey, ez, x, r, pv, q, rr, target2, Ps, slots)
-             : cg_fix_loop<ISO, 0>(A, n, ex, ey, ez, x, r, pv, q, rr, target2, Ps, slots);
+    it = cg_fix_loop<ISO>(A, n, ex, ey, ez, x, r, pv, q, target2, Ps, slots);
   cg_finish(A, P, pidx, x, it, red[1]);
   return true;
 }
