@@ -330,8 +330,10 @@ sea_status sea_create(const double cell[3], const int grid[3], const sea_params*
   return SEA_OK;
 }
 
-sea_status sea_set_orbitals(sea_ctx* c, const double* phi, int n_orb, int on_device) {
-  if (!c) return SEA_ERR_ARG;
+// The orbitals into one of the context's arrays (phi, or vxx_dev as the input
+// of the localization), with their checks and the buffers their count needs.
+static sea_status load_orbitals(sea_ctx* c, const double* phi, int n_orb, int on_device,
+                                SeaBuf sea_ctx::*into) {
   if (c->poisoned) return sea_fail(c, SEA_ERR_STATE, "context poisoned by an earlier CUDA error");
   if (!phi || n_orb < 1 || n_orb > 4096) return sea_fail(c, SEA_ERR_ARG, "bad orbitals");
   c->have_phi = c->have_vxx = c->have_ace = false;
@@ -362,7 +364,7 @@ sea_status sea_set_orbitals(sea_ctx* c, const double* phi, int n_orb, int on_dev
   SEA_ALLOC(onorm, (size_t)n_orb * SEA_NORM_CHUNKS * sizeof(double));
   double* npart = (double*)c->onorm.p;
   SEA_CK(cudaMemsetAsync(c->status.p, 0, sizeof(unsigned), c->stream), "memset");
-  double* pd = (double*)c->phi.p;
+  double* pd = (double*)(c->*into).p;
   if (on_device) {
     sea::k_check_orbitals<true><<<dim3(SEA_NORM_CHUNKS, n_orb), 256, 0, c->stream>>>(
         phi, pd, c->ng, (unsigned*)c->status.p, npart);
@@ -405,16 +407,21 @@ sea_status sea_set_orbitals(sea_ctx* c, const double* phi, int n_orb, int on_dev
   if (st & SEA_FLAG_NONFINITE) return sea_fail(c, SEA_ERR_INPUT, "orbitals hold non-finite values");
   if (st & SEA_FLAG_NORM)
     return sea_fail(c, SEA_ERR_INPUT, "an orbital's norm <phi|phi> differs from 1 by more than orth_tol");
-  c->have_phi = true;
   c->stats.n_orb = n_orb;
   return SEA_OK;
 }
 
+sea_status sea_set_orbitals(sea_ctx* c, const double* phi, int n_orb, int on_device) {
+  if (!c) return SEA_ERR_ARG;
+  const sea_status s = load_orbitals(c, phi, n_orb, on_device, &sea_ctx::phi);
+  if (s == SEA_OK) c->have_phi = true;
+  return s;
+}
+
 sea_status sea_scdm(sea_ctx* c, const double* phi, int n_orb, int on_device, double* U, int* cols) {
   if (!c) return SEA_ERR_ARG;
-  const sea_status st0 = sea_set_orbitals(c, phi, n_orb, on_device);
+  const sea_status st0 = load_orbitals(c, phi, n_orb, on_device, &sea_ctx::vxx_dev);
   if (st0 != SEA_OK) return st0;
-  c->have_phi = false;
   const size_t nn = (size_t)n_orb * n_orb;
   SEA_ALLOC(scdm_u, nn * sizeof(double));
   SEA_ALLOC(scdm_c, (size_t)n_orb * sizeof(long long));
@@ -972,7 +979,7 @@ void sea_destroy(sea_ctx* c) {
                    &c->qbuf, &c->eptr, &c->eent, &c->ewin, &c->coff, &c->cbuf, &c->status,
                    &c->exx_dev, &c->queue, &c->tmask, &c->tptr_o, &c->tlist_o, &c->tslot_o,
                    &c->tptr_t, &c->tlist_t, &c->partial, &c->Mbuf, &c->Abuf, &c->Lbuf, &c->wdig, &c->wx, &c->xevb, &c->gbuf, &c->flowbuf,
-                   &c->scdm_u, &c->scdm_c,
+                   &c->scdm_u, &c->scdm_c, &c->scdm_s, &c->scdm_a,
                    &c->Linv, &c->Gbuf, &c->Hbuf, &c->Hbuf2, &c->bdesc, &c->bitems,
                    &c->onorm};
   for (SeaBuf* b : all) release(*b);
