@@ -437,6 +437,8 @@ sea_status sea_scdm(sea_ctx* c, const double* phi, int n_orb, int on_device, dou
          "copy pivots");
   SEA_CK(cudaMemcpyAsync(&st, c->status.p, sizeof(unsigned), cudaMemcpyDeviceToHost, c->stream), "status");
   SEA_CK(cudaStreamSynchronize(c->stream), "scdm");
+  if (st & SEA_FLAG_WAIT)
+    return sea_fail(c, SEA_ERR_CUDA, "a tensor-core completion wait timed out (SCDM rotation)");
   if (st & SEA_FLAG_NOT_PD) return sea_fail(c, SEA_ERR_INPUT, "orbitals are rank deficient (SCDM pivot of zero norm)");
   if (cols)
     for (int k = 0; k < n_orb; ++k) cols[k] = (int)hc[k];
@@ -979,7 +981,7 @@ void sea_destroy(sea_ctx* c) {
                    &c->qbuf, &c->eptr, &c->eent, &c->ewin, &c->coff, &c->cbuf, &c->status,
                    &c->exx_dev, &c->queue, &c->tmask, &c->tptr_o, &c->tlist_o, &c->tslot_o,
                    &c->tptr_t, &c->tlist_t, &c->partial, &c->Mbuf, &c->Abuf, &c->Lbuf, &c->wdig, &c->wx, &c->xevb, &c->gbuf, &c->flowbuf,
-                   &c->scdm_u, &c->scdm_c, &c->scdm_s, &c->scdm_a,
+                   &c->scdm_u, &c->scdm_c, &c->scdm_s, &c->scdm_a, &c->rot,
                    &c->Linv, &c->Gbuf, &c->Hbuf, &c->Hbuf2, &c->bdesc, &c->bitems,
                    &c->onorm};
   for (SeaBuf* b : all) release(*b);

@@ -104,11 +104,6 @@ __device__ __forceinline__ void digit_floats(long long X, float* f) {
   f[0] = __int_as_float(0x4B400000 + (int)(Y >> 40)) - 12582912.0f;
 }
 
-// BF16 bit patterns of two small integer-valued floats, packed low/high.
-__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
-  return __byte_perm(__float_as_uint(lo), __float_as_uint(hi), 0x7632);
-}
-
 // FP16 bit patterns of two small integer-valued floats (|v| <= 2048, exact),
 // packed low/high.
 __device__ __forceinline__ uint32_t pack_f16(float lo, float hi) {
@@ -496,11 +491,6 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map
 // L2 prefetch of bytes (a multiple of 16) at p (16-byte aligned).
 __device__ __forceinline__ void bulk_prefetch_l2(const void* p, uint32_t bytes) {
   asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
-}
-
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes)
-               : "memory");
 }
 
 // A's digits in the TMA kernel: unsigned bytes of |x| on the segment's
@@ -1089,16 +1079,6 @@ __global__ void __launch_bounds__(MBLK)
                                 (p & 7) * 16) = make_uint4(pk[k][0], pk[k][1], pk[k][2], pk[k][3]);
   }
 }
-
-__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes,
-                                          uint32_t bar) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::
-          "r"(dst),
-      "l"(src), "r"(bytes), "r"(bar)
-      : "memory");
-}
-
 
 // E_v of the expansion for every (tile, vector): the largest biased
 // exponent of H(j, v) 2^(E_j) over the tile's list (0 where all are zero);

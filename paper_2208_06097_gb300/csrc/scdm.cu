@@ -478,38 +478,6 @@ __global__ void __launch_bounds__(128)
   }
 }
 
-// out[i][r] = sum_j U[j][i] phi[j][r]: thread per point r, U in shared memory
-// in chunks of 32 columns i.
-__global__ void __launch_bounds__(256)
-    k_rotate(const double* __restrict__ phi, int n, size_t N, const double* __restrict__ U,
-             double* __restrict__ out) {
-  __shared__ double su[64][33];
-  const size_t r = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  for (int i0 = 0; i0 < n; i0 += 32) {
-    double acc[32];
-#pragma unroll
-    for (int u = 0; u < 32; ++u) acc[u] = 0.0;
-    for (int j0 = 0; j0 < n; j0 += 64) {
-      __syncthreads();
-      for (int q = threadIdx.x; q < 64 * 32; q += blockDim.x) {
-        const int jj = q / 32, ii = q % 32;
-        su[jj][ii] = (j0 + jj < n && i0 + ii < n) ? U[(size_t)(j0 + jj) * n + i0 + ii] : 0.0;
-      }
-      __syncthreads();
-      if (r < N)
-        for (int jj = 0; jj < 64 && j0 + jj < n; ++jj) {
-          const double v = phi[(size_t)(j0 + jj) * N + r];
-#pragma unroll
-          for (int u = 0; u < 32; ++u) acc[u] = fma(su[jj][u], v, acc[u]);
-        }
-    }
-    if (r < N)
-#pragma unroll
-      for (int u = 0; u < 32; ++u)
-        if (i0 + u < n) out[(size_t)(i0 + u) * N + r] = acc[u];
-  }
-}
-
 }  // namespace
 
 // The pivots among the candidates; *done = false if they do not decide all
@@ -646,9 +614,7 @@ cudaError_t launch_scdm(sea_ctx* c, double* U_dev, long long* C_dev) {
     last = d;
   }
   if (X != U_dev) cudaMemcpyAsync(U_dev, X, nn, cudaMemcpyDeviceToDevice, st);
-  k_rotate<<<gN, 256, 0, st>>>(phi, n, N, U_dev, (double*)c->phi.p);
-  c->launches += 1;
-  return cudaGetLastError();
+  return launch_rotate(c, phi, n, N, U_dev, (double*)c->phi.p);
 }
 
 }  // namespace sea

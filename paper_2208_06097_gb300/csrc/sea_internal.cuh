@@ -625,6 +625,7 @@ struct sea_ctx {
   SeaBuf flowbuf;  // the mixed form's one-launch Cholesky chain: DF blocks and task flags
   SeaBuf scdm_u, scdm_c;  // SCDM rotation and pivots
   SeaBuf scdm_s, scdm_a;  // SCDM step state; candidates' rows and coefficients
+  SeaBuf rot;             // digit images of the SCDM rotation
   SeaBuf tmask, tptr_o, tlist_o, tslot_o, tptr_t, tlist_t, partial, Mbuf, Abuf, Lbuf, Linv,
       Gbuf, Hbuf, Hbuf2;
   int n_tiles = 0, tile_inc = 0, max_tile_list = 0;
@@ -984,6 +985,9 @@ cudaError_t launch_warm_start(sea_ctx* c);
 // SCDM localization of the orbitals in c->vxx_dev (scdm.cu): U and the pivots
 // on the device; the localized orbitals go to c->phi.
 cudaError_t launch_scdm(sea_ctx* c, double* U_dev, long long* C_dev);
+// out[i][r] = sum_j U[j][i] phi[j][r] on the tensor cores (rotate_tc.cu).
+cudaError_t launch_rotate(sea_ctx* c, const double* phi, int n, size_t N, const double* U,
+                          double* out);
 // Damped Jacobi sweeps on every pair's starting vector (pair.cu).
 cudaError_t launch_smooth(sea_ctx* c, int sweeps, double omega);
 // Mixed form's contraction with W on the tensor cores.  launch_w_digits
