@@ -38,12 +38,12 @@ namespace {
 
 constexpr int RD = 8;     // digits per value
 constexpr int RT = 128;   // points per tile (M)
-constexpr int RK = 32;    // orbitals per stage
+constexpr int RK = 16;    // orbitals per stage
 constexpr int RN = 32;    // outputs per block
 constexpr int RSEG = 512 / RK;  // stages per exact accumulation
 constexpr uint32_t RA_PLANE = RT * RK * 2, RA_STAGE = RD * RA_PLANE, RA_LBO = RT * 16;
 constexpr uint32_t RB_STAGE = RD * RN * RK * 2, RB_LBO = RD * RN * 16;
-constexpr int R_STAGES = 2;
+constexpr int R_STAGES = 5;
 constexpr int RE_WARPS = 8;                     // epilogue warps
 constexpr int R_THREADS = 32 * (RE_WARPS + 2);  // and a loading and an issuing warp
 constexpr size_t R_SMEM = R_STAGES * (RA_STAGE + RB_STAGE) + 128;
@@ -106,36 +106,38 @@ __global__ void __launch_bounds__(256)
     for (int q = 0; q < 8; ++q) v[q] = (i < n && 8 * kg + q < n) ? U[(size_t)(8 * kg + q) * n + i] : 0.0;
     uint4 d[RD];
     digits8_b7(v, em[li], d);
-    unsigned char* dst = ub + ((size_t)blockIdx.x * nst + kg / 4) * RB_STAGE + (kg % 4) * RB_LBO;
+    unsigned char* dst = ub + ((size_t)blockIdx.x * nst + kg / (RK / 8)) * RB_STAGE + (kg % (RK / 8)) * RB_LBO;
 #pragma unroll
     for (int l = 0; l < RD; ++l) *reinterpret_cast<uint4*>(dst + (l * RN + li) * 16) = d[l];
   }
 }
 
-// phi's digit image of the slab's tiles (points r0 + 128 blockIdx.x ..):
-// ab[tile][stage][plane 8 KB][k group 2 KB][point 16 B], eexp[tile][point].
-__global__ void __launch_bounds__(256)
+// phi's digit image of the slab's tiles (points r0 + 128 blockIdx.x ..), four
+// threads a point:
+// ab[tile][stage][plane 4 KB][k group 2 KB][point 16 B], eexp[tile][point].
+constexpr int RQ = 4;
+__global__ void __launch_bounds__(RT* RQ)
     k_rot_digits(const double* __restrict__ phi, int n, size_t N, size_t r0, int nst,
                  unsigned char* __restrict__ ab, int* __restrict__ eexp) {
-  __shared__ int em[2][RT];
-  const int p = threadIdx.x % RT, half = threadIdx.x / RT;
+  __shared__ int em[RQ][RT];
+  const int p = threadIdx.x % RT, part = threadIdx.x / RT;
   const size_t r = r0 + (size_t)blockIdx.x * RT + p;
   const double* src = phi + r;
   int e = 0;
   if (r < N)
-    for (int j = half; j < n; j += 2) e = max(e, biased_exp(src[(size_t)j * N]));
-  em[half][p] = e;
+    for (int j = part; j < n; j += RQ) e = max(e, biased_exp(src[(size_t)j * N]));
+  em[part][p] = e;
   __syncthreads();
-  e = max(em[0][p], em[1][p]);
-  if (half == 0) eexp[blockIdx.x * RT + p] = e;
-  for (int kg = half; kg < nst * (RK / 8); kg += 2) {
+  for (int q = 0; q < RQ; ++q) e = max(e, em[q][p]);
+  if (part == 0) eexp[blockIdx.x * RT + p] = e;
+  for (int kg = part; kg < nst * (RK / 8); kg += RQ) {
     double v[8];
 #pragma unroll
     for (int q = 0; q < 8; ++q) v[q] = (r < N && 8 * kg + q < n) ? src[(size_t)(8 * kg + q) * N] : 0.0;
     uint4 d[RD];
     digits8_b7(v, e, d);
     unsigned char* dst =
-        ab + ((size_t)blockIdx.x * nst + kg / 4) * RA_STAGE + (kg % 4) * RA_LBO + p * 16;
+        ab + ((size_t)blockIdx.x * nst + kg / (RK / 8)) * RA_STAGE + (kg % (RK / 8)) * RA_LBO + p * 16;
 #pragma unroll
     for (int k = 0; k < RD; ++k) *reinterpret_cast<uint4*>(dst + k * RA_PLANE) = d[k];
   }
@@ -319,7 +321,7 @@ cudaError_t launch_rotate(sea_ctx* c, const double* phi, int n, size_t N, const 
   c->launches += 1;
   for (size_t t0 = 0; t0 < tiles; t0 += slab) {
     const unsigned g = (unsigned)std::min(slab, tiles - t0);
-    k_rot_digits<<<g, 256, 0, c->stream>>>(phi, n, N, t0 * RT, nst, ab, eexp);
+    k_rot_digits<<<g, RT * RQ, 0, c->stream>>>(phi, n, N, t0 * RT, nst, ab, eexp);
     k_rot_gemm<<<g, R_THREADS, R_SMEM, c->stream>>>(ab, ub, eexp, fexp, n, N, t0 * RT, nst, out,
                                                    (unsigned*)c->status.p);
     c->launches += 2;

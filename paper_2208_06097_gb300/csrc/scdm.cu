@@ -174,8 +174,10 @@ constexpr int SC_THREADS = 512;  // of k_scdm_step
 // The class of density c against the largest cmax: floor(4 log2(cmax / c)),
 // decided on cmax 2^(-m/4) (edge m: the lower edge of class m - 1).
 __device__ __forceinline__ double sc_edge(double cmax, int m) {
-  const double f[4] = {1.0, 0.84089641525371454, 0.70710678118654752, 0.59460355750136054};
-  return ldexp(cmax * f[m & 3], -(m >> 2));
+  const double f = (m & 3) == 0 ? 1.0
+                   : (m & 3) == 1 ? 0.84089641525371454
+                   : (m & 3) == 2 ? 0.70710678118654752 : 0.59460355750136054;
+  return cmax * f * (1.0 / (double)(1 << (m >> 2)));
 }
 
 // cmax over the block maxima of k_argmax1; one CTA.  cnt[0..SC_CLASSES] = 0.
@@ -202,7 +204,8 @@ __global__ void __launch_bounds__(256)
     k_scdm_classes(const double* __restrict__ c, size_t N, const double* __restrict__ cmax_p,
                    int mode, int cap, int* __restrict__ cnt, int* __restrict__ list) {
   __shared__ int n_of[SC_CLASSES], at[SC_CLASSES];
-  const double cmax = *cmax_p, low = sc_edge(cmax, SC_CLASSES);
+  __shared__ double edge[SC_CLASSES + 1];
+  if (threadIdx.x <= SC_CLASSES) edge[threadIdx.x] = sc_edge(*cmax_p, threadIdx.x);
   const size_t per = (N + gridDim.x - 1) / gridDim.x;
   const size_t b0 = min(N, per * blockIdx.x), b1 = min(N, b0 + per);
   if (threadIdx.x < SC_CLASSES) n_of[threadIdx.x] = 0;
@@ -210,9 +213,9 @@ __global__ void __launch_bounds__(256)
   for (int pass = 0; pass <= mode; ++pass) {
     for (size_t r = b0 + threadIdx.x; r < b1; r += blockDim.x) {
       const double v = c[r];
-      if (!(v >= low)) continue;
+      if (!(v >= edge[SC_CLASSES])) continue;
       int m = 0;
-      while (m < SC_CLASSES - 1 && v < sc_edge(cmax, m + 1)) ++m;
+      while (m < SC_CLASSES - 1 && v < edge[m + 1]) ++m;
       const int k = atomicAdd(pass == 0 ? &n_of[m] : &at[m], 1);
       if (pass == 1 && k < cap) list[k] = (int)r;
     }
@@ -273,7 +276,7 @@ __global__ void __launch_bounds__(SC_THREADS)
                 const int* __restrict__ start, const int* __restrict__ n_kept,
                 const double* __restrict__ cmax_p, double* __restrict__ cA, double* __restrict__ L,
                 const ScMax* __restrict__ mx_in, ScMax* __restrict__ mx_out,
-                const ScState* __restrict__ st_in, ScState* __restrict__ st_out,
+                const ScState* __restrict__ st_in, ScState* __restrict__ st_out, int first_open,
                 int* __restrict__ piv_a, long long* __restrict__ C) {
   extern __shared__ double sp[];  // pivot's a_p [n], -L[p] [n], 1 / sqrt(c_p)
   __shared__ ScMax wb[SC_THREADS / 32];
@@ -353,11 +356,13 @@ __global__ void __launch_bounds__(SC_THREADS)
     }
     ++st.k;
   } else {
-    // open the next class, if it was kept whole
-    if (st.open >= SC_CLASSES || start[st.open + 1] > kept) {
+    // open the next class (at the start the first first_open ones), if it was
+    // kept whole
+    const int open = st.open == 0 ? first_open : st.open + 1;
+    if (open > SC_CLASSES || start[open] > kept) {
       st.stop = 1;
     } else {
-      const int b0 = start[st.open], end = start[st.open + 1];
+      const int b0 = start[st.open], end = start[open];
       for (int a = gw; a < end; a += nw) {
         if (a < b0) {  // already open: its c stands
           keep(cA[a], a);
@@ -376,16 +381,17 @@ __global__ void __launch_bounds__(SC_THREADS)
         if (lane == 0) cA[a] = c;
         keep(c, a);
       }
-      ++st.open;
+      st.open = open;
     }
   }
   if (lane == 0) wb[warp] = mine;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < SC_THREADS / 32; ++w)
-      if (sc_better(wb[w], mine)) mine = wb[w];
-    mx_out[blockIdx.x] = mine;
-    if (blockIdx.x == 0) *st_out = st;
+  if (warp == 0) {
+    mine = warp_best(lane < SC_THREADS / 32 ? wb[lane] : ScMax{-2.0, 0x7fffffff, -1});
+    if (lane == 0) {
+      mx_out[blockIdx.x] = mine;
+      if (blockIdx.x == 0) *st_out = st;
+    }
   }
 }
 
@@ -531,11 +537,16 @@ static cudaError_t pivots_lazy(sea_ctx* c, const double* cn, const double* bv, i
   cudaMemcpyAsync(kept, &na, sizeof(int), cudaMemcpyHostToDevice, st);
   cudaMemsetAsync(state, 0, sizeof(ScState), st);
   cudaMemsetAsync(mx, 0xff, (size_t)nsm * sizeof(ScMax), st);  // NaN: no class is open
-  const int launches = n + m;  // every pivot and every class
+  // at the start as many classes as two candidates a warp make: their c is
+  // kept up to date at every step, which costs less than making up for their
+  // coefficients later (0.14 to 0.42 ms a class at n = 128)
+  int first = 1;
+  while (first < m && hs[first + 1] <= 2 * nsm * (SC_THREADS / 32)) ++first;
+  const int launches = n + m - first + 1;  // every pivot, every opening
   for (int l = 0; l < launches; ++l)
     k_scdm_step<<<nsm, SC_THREADS, smem, st>>>(A, n, list, start, kept, cmax, cA, L,
                                                mx + (l & 1) * nsm, mx + ((l + 1) & 1) * nsm,
-                                               state + (l & 1), state + ((l + 1) & 1), piv_a, C_dev);
+                                               state + (l & 1), state + ((l + 1) & 1), first, piv_a, C_dev);
   ScState hst;
   cudaMemcpyAsync(&hst, state + (launches & 1), sizeof(hst), cudaMemcpyDeviceToHost, st);
   e = cudaStreamSynchronize(st);
