@@ -181,77 +181,6 @@ __global__ void k_max_int(const int* __restrict__ in, int n, int* __restrict__ o
 }
 
 
-// partial[(tptr[T] + s) * m + a] = sum_{r in T} A[a][r] W[list[s]][r].
-// CTA per (tile, chunk of 64 rows of A).  The tile's 128 points of the 64
-// A rows and of up to 32 W rows sit in shared memory; a work unit is
-// (W row, half of the A rows), units are dealt to warps in a warp-uniform
-// loop (no predicated FMAs: on this part a predicated-off FP64 FMA still
-// costs FP64 pipe time), each lane one A row; the dot product runs over the
-// W row's sub-box of the tile only (W is exactly zero outside it), with
-// four independent FMA chains along x.
-#define GA 64
-#define GJB 32
-#define GROW (TP + 1)
-#define GRAM_SMEM ((size_t)(GA + GJB) * GROW * sizeof(double))
-__global__ void __launch_bounds__(256, 2)
-    k_gram_partial(const double* __restrict__ A, int m, const double* __restrict__ W,
-                   TileGeom G, size_t ng, const int* __restrict__ tptr,
-                   const int* __restrict__ tlist, const int* __restrict__ tsub,
-                   double* __restrict__ partial) {
-  const int T = blockIdx.x;
-  const int a0 = blockIdx.y * GA;
-  const int j0 = tptr[T], nJ = tptr[T + 1] - j0;
-  if (nJ == 0) return;
-  extern __shared__ double gsm[];
-  double* As = gsm;               // [GA][GROW]
-  double* Ws = gsm + GA * GROW;   // [GJB][GROW]
-  __shared__ long long addr[TP];
-  __shared__ int wrow[GJB];
-  for (int r = threadIdx.x; r < TP; r += blockDim.x) addr[r] = tile_point(G, T, r);
-  __syncthreads();
-  for (int idx = threadIdx.x; idx < GA * TP; idx += blockDim.x) {
-    const int a = idx / TP, pt = idx % TP;
-    const long long g = addr[pt];
-    As[a * GROW + pt] = (a0 + a < m && g >= 0) ? A[(size_t)(a0 + a) * ng + g] : 0.0;
-  }
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
-  for (int jb = 0; jb < nJ; jb += GJB) {
-    const int nj = min(GJB, nJ - jb);
-    __syncthreads();
-    if (threadIdx.x < nj) wrow[threadIdx.x] = tlist[j0 + jb + threadIdx.x];
-    __syncthreads();
-    for (int idx = threadIdx.x; idx < nj * TP; idx += blockDim.x) {
-      const int jl = idx / TP, pt = idx % TP;
-      const long long g = addr[pt];
-      Ws[jl * GROW + pt] = g >= 0 ? W[(size_t)wrow[jl] * ng + g] : 0.0;
-    }
-    __syncthreads();
-    for (int u = warp; u < 2 * nj; u += nwarp) {
-      const int jl = u >> 1, ah = u & 1;
-      const double* ar = As + (ah * 32 + lane) * GROW;
-      const double* wr = Ws + jl * GROW;
-      const int sb = tsub[j0 + jb + jl];
-      const int x0 = sb & 15, x1 = (sb >> 4) & 15, y0 = (sb >> 8) & 15, y1 = (sb >> 12) & 15,
-                z0 = (sb >> 16) & 15, z1 = (sb >> 20) & 15;
-      double c0 = 0.0, c1 = 0.0, c2 = 0.0, c3 = 0.0;
-      for (int z = z0; z < z1; ++z)
-        for (int y = y0; y < y1; ++y) {
-          const int base = (z * TY + y) * TX;
-          int x = x0;
-          for (; x + 4 <= x1; x += 4) {
-            c0 = fma(ar[base + x], wr[base + x], c0);
-            c1 = fma(ar[base + x + 1], wr[base + x + 1], c1);
-            c2 = fma(ar[base + x + 2], wr[base + x + 2], c2);
-            c3 = fma(ar[base + x + 3], wr[base + x + 3], c3);
-          }
-          for (; x < x1; ++x) c0 = fma(ar[base + x], wr[base + x], c0);
-        }
-      const int a = a0 + ah * 32 + lane;
-      if (a < m) partial[(size_t)(j0 + jb + jl) * m + a] = (c0 + c1) + (c2 + c3);
-    }
-  }
-}
-
 // ---------------------------------------------------------------------------
 // Mixed form of the expansion W H (k_tile_expand_x): FP64 operands split into
 // FP32 pairs (v = hi + lo, hi = fl32(v), lo = fl32(v - hi)), each product
@@ -780,10 +709,11 @@ __global__ void __launch_bounds__(256)
     k_tile_expand(const double* __restrict__ W, TileGeom G, size_t ng,
                   const int* __restrict__ tptr, const int* __restrict__ tlist,
                   const int* __restrict__ tsub, const double* __restrict__ H, long long hj,
-                  long long hv, int m, double sign, double* __restrict__ out) {
+                  long long hv, int m, double sign, int skip_upto, double* __restrict__ out) {
   const int T = blockIdx.x;
   const int v0 = blockIdx.y * EV;
   const int j0 = tptr[T], nJ = tptr[T + 1] - j0;
+  if (nJ <= skip_upto) return;  // done by the tensor-core expansion
   extern __shared__ double Hs[];  // [nJ][EV]
   for (int idx = threadIdx.x; idx < nJ * EV; idx += blockDim.x) {
     const int jl = idx / EV, vl = idx % EV;
@@ -878,44 +808,36 @@ static cudaError_t launch_exx_ace(sea_ctx* c, int transA, const double* d) {
   return cudaGetLastError();
 }
 
-// The contractions with W: FP64 kernels for the plain form, the
-// tensor-core kernel (exact BF16 digit splitting) for the mixed form.
+// Digits per operand of the tensor-core contractions with W: 47-bit integers
+// in the mixed form, 55- and 56-bit ones in the plain form.
+static int ace_digits(const sea_ctx* c) { return c->prm.precision == 1 ? 6 : 7; }
+
+// The contraction with W on the tensor cores (exact digit splitting).
 static cudaError_t launch_gram(sea_ctx* c, const double* A, int m, const TileGeom& G,
-                               const int* tptr, const int* tlist, const int* tsub) {
-  const double* W = (const double*)c->vxx_dev.p;
-  if (c->prm.precision == 1)
-    return launch_gram_tc(c->stream, c->device, A, m, G, c->ng, c->n_tiles, tptr, c->tile_inc,
-                          c->wdig.p, (double*)c->partial.p, (int*)c->counts.p + 20,
-                          (unsigned*)c->status.p);
-  k_gram_partial<<<dim3(c->n_tiles, (m + GA - 1) / GA), 256, GRAM_SMEM, c->stream>>>(
-      A, m, W, G, c->ng, tptr, tlist, tsub, (double*)c->partial.p);
-  return cudaGetLastError();
+                               const int* tptr) {
+  return launch_gram_tc(c->stream, c->device, A, m, G, c->ng, c->n_tiles, tptr, c->tile_inc,
+                        c->wdig.p, (double*)c->partial.p, (int*)c->counts.p + 20,
+                        (unsigned*)c->status.p, ace_digits(c));
 }
 
+// The expansion W H: tiles with at most expand_tc_max_list() W rows on the
+// tensor cores, longer lists (if any) in FP64, or FP32 pairs (mixed form).
 static cudaError_t launch_expand(sea_ctx* c, const TileGeom& G, const int* tptr,
                                  const int* tlist, const int* tsub, const double* H, long long hj,
                                  long long hv, int m, double sign, double* out) {
-  if (c->prm.precision == 1) {
-    // tiles with at most expand_tc_max_list() W rows on the tensor cores,
-    // longer lists (if any) by the FP32 kernel
-    if (!sea_ensure(c, c->xevb, (size_t)max(c->n_tiles, 1) * m * sizeof(int)))
-      return cudaErrorMemoryAllocation;
-    const cudaError_t e = launch_expand_tc(c->stream, c->device, c->wx.p, G, c->ng, c->n_tiles,
-                                           tptr, tlist, H, hj, hv, m, sign < 0.0, out,
-                                           (int*)c->xevb.p, (int*)c->counts.p + 24,
-                                           (unsigned*)c->status.p);
-    if (e != cudaSuccess) return e;
-    if (c->max_tile_list > expand_tc_max_list()) {
-      const size_t smem = (size_t)c->max_tile_list * 32 * sizeof(float2);
-      k_tile_expand_x<<<dim3(c->n_tiles, (m + 31) / 32), 256, smem, c->stream>>>(
-          (const double*)c->vxx_dev.p, G, c->ng, tptr, tlist, tsub, H, hj, hv, m, sign,
-          expand_tc_max_list(), out);
-      c->launches += 1;
-    }
-  } else {
+  if (!sea_ensure(c, c->xevb, (size_t)max(c->n_tiles, 1) * m * sizeof(int)))
+    return cudaErrorMemoryAllocation;
+  const cudaError_t e = launch_expand_tc(
+      c->stream, c->device, c->wx.p, G, c->ng, c->n_tiles, tptr, tlist, H, hj, hv, m, sign < 0.0, out,
+      (int*)c->xevb.p, (int*)c->counts.p + 24, (unsigned*)c->status.p, ace_digits(c));
+  if (e != cudaSuccess) return e;
+  if (c->max_tile_list > expand_tc_max_list()) {
     const size_t smem = (size_t)c->max_tile_list * EV * sizeof(double);
-    k_tile_expand<<<dim3(c->n_tiles, (m + EV - 1) / EV), 256, smem, c->stream>>>(
-        (const double*)c->vxx_dev.p, G, c->ng, tptr, tlist, tsub, H, hj, hv, m, sign, out);
+    (c->prm.precision == 1 ? k_tile_expand_x : k_tile_expand)<<<
+        dim3(c->n_tiles, (m + EV - 1) / EV), 256, smem, c->stream>>>(
+        (const double*)c->vxx_dev.p, G, c->ng, tptr, tlist, tsub, H, hj, hv, m, sign,
+        expand_tc_max_list(), out);
+    c->launches += 1;
   }
   return cudaGetLastError();
 }
@@ -1077,38 +999,34 @@ cudaError_t launch_ace_build(sea_ctx* c) {
   const int* tsub = tlist + c->list_cap;
   const int* oslot = (const int*)c->tlist_o.p + c->list_cap;
   // M = Phi^T W dV
-  err = cudaFuncSetAttribute(k_gram_partial, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)GRAM_SMEM);
+  // from W's digits
+  const int digits = ace_digits(c);
+  if (!sea_ensure(c, c->wdig, w_digits_bytes(hinc, digits)) ||
+      !sea_ensure(c, c->wx, wx_digits_bytes(nt, hinc, digits)))
+    return cudaErrorMemoryAllocation;
+  err = launch_w_digits(c->stream, (const double*)c->vxx_dev.p, G, c->ng, nt, c->max_tile_list, tptr,
+                        tlist, hinc, c->wdig.p, digits);
   if (err != cudaSuccess) return err;
-  if (c->prm.precision == 1) {  // W's digits for the tensor-core contractions
-    if (!sea_ensure(c, c->wdig, w_digits_bytes(hinc))) return cudaErrorMemoryAllocation;
-    err = launch_w_digits(c->stream, (const double*)c->vxx_dev.p, G, c->ng, nt, c->max_tile_list,
-                          tptr, tlist, hinc, c->wdig.p);
-    if (err != cudaSuccess) return err;
-    if (!sea_ensure(c, c->wx, wx_digits_bytes(nt, hinc))) return cudaErrorMemoryAllocation;
-    c->launches += 2;
-  }
+  c->launches += 2;
   cudaEventRecord(c->ev[10], c->stream);
-  err = launch_gram(c, (const double*)c->phi.p, n, G, tptr, tlist, tsub);
+  err = launch_gram(c, (const double*)c->phi.p, n, G, tptr);
   if (err != cudaSuccess) return err;
   cudaEventRecord(c->ev[11], c->stream);
-  if (c->prm.precision == 1) {
-    // W's per-tile images for the expansion (used by sea_apply_ace only) on
-    // a second stream, beside the latency-bound Cholesky chain below; the
-    // context stream waits for them before the build ends
-    err = cudaStreamWaitEvent(c->xfer[0], c->ev[11], 0);
-    if (err == cudaSuccess)
-      err = launch_wx_digits(c->xfer[0], (const double*)c->vxx_dev.p, G, c->ng, nt, tptr, tlist,
-                             tsub, c->wx.p);
-    if (err == cudaSuccess) err = cudaEventRecord(c->xev[0], c->xfer[0]);
-    if (err != cudaSuccess) return err;
-  }
+  // W's per-tile images for the expansion (used by sea_apply_ace only) on
+  // a second stream, beside the latency-bound Cholesky chain below; the
+  // context stream waits for them before the build ends
+  err = cudaStreamWaitEvent(c->xfer[0], c->ev[11], 0);
+  if (err == cudaSuccess)
+    err = launch_wx_digits(c->xfer[0], (const double*)c->vxx_dev.p, G, c->ng, nt, tptr, tlist, tsub,
+                           c->wx.p, digits);
+  if (err == cudaSuccess) err = cudaEventRecord(c->xev[0], c->xfer[0]);
+  if (err != cudaSuccess) return err;
   (c->prm.precision == 1 ? k_gram_reduce_df : k_gram_reduce)<<<dim3((n + GR_A - 1) / GR_A, n), GR_A * GR_Z, 0, c->stream>>>(
       (const double*)c->partial.p, n, n, optr, oslot, c->dV, (double*)c->Mbuf.p,
       n, 1);
   c->launches += 2;
   err = launch_chol_chain(c);
-  if (err == cudaSuccess && c->prm.precision == 1) err = cudaStreamWaitEvent(c->stream, c->xev[0], 0);
+  if (err == cudaSuccess) err = cudaStreamWaitEvent(c->stream, c->xev[0], 0);
   return err;
 }
 
@@ -1180,7 +1098,7 @@ cudaError_t launch_ace_apply(sea_ctx* c, const double* psi, int nv, double* out)
   // G[o][v] = <W_o|psi_v> dV
   cudaEventRecord(c->ev[12], c->stream);
   {
-    const cudaError_t e = launch_gram(c, psi, nv, G, tptr, tlist, tsub);
+    const cudaError_t e = launch_gram(c, psi, nv, G, tptr);
     if (e != cudaSuccess) return e;
   }
   cudaEventRecord(c->ev[13], c->stream);

@@ -1,4 +1,4 @@
-// gram_tc.cu -- the mixed form's contraction with W on the tensor cores.
+// gram_tc.cu -- the contractions with W on the tensor cores.
 //
 //   partial[s m + a] = sum over the points r of tile T of A[a][r] W[list(T)[s]][r]
 //
@@ -24,6 +24,16 @@
 // (2^-47 of the segment maximum) and the dropped diagonals d >= S (below
 // 2^-45.7 of max|x| max|w| times the segment length).
 //
+// The plain form (DIG = 7) has seven digits per operand: 55-bit integers for W,
+// 56-bit ones for A's bytes, seven diagonals (each still below 2^24), each
+// half tile rounded to nearest and the two added in FP64.  Values within a
+// factor of 8 (A) or 4 (W) of their segment's largest are kept whole, the
+// others to 2^-56 and 2^-55 of it, and the dropped diagonals stay below 2^-54
+// of max|x| max|w| per product: the error of a partial is below the rounding
+// of an FP64 chain of its 64 products.  The FP64 unit took 3.68 ms per
+// contraction (256 rows, 96^3) and 3.51 ms for the expansion.  Segments with
+// a non-finite value give NaN.
+//
 // Kernel shape: persistent CTAs (one per SM) take tiles from a queue and
 // walk units (W block of up to 32 slots, A block of 128 rows, half tile).
 // Per unit the A digits go to shared memory in the tensor core's K-major
@@ -47,26 +57,32 @@
 // tensor memory and ends.
 #include <cuda.h>
 
+#include "cg_fixed.cuh"
 #include "sea_internal.cuh"
 #include "tcgen05.cuh"
 
 namespace sea {
 namespace {
 
-constexpr int DIG = 6;                          // digits per operand
+// DIG digits per operand: 6 in the mixed form, 7 in the plain form
 constexpr int KH = 64;                          // points per half tile
-constexpr int NBLK = 32;                        // W rows per block
 constexpr int MBLK = 128;                       // A rows per block
 constexpr int GT_THREADS = 512;
 constexpr uint32_t A_PLANE = MBLK * KH * 2;     // bytes per digit plane of A
-constexpr uint32_t W_HALF = DIG * NBLK * KH * 2;  // bytes of W digits per half tile
 constexpr uint32_t A_LBO = (MBLK / 8) * 128;    // K-adjacent core matrices of A
 constexpr uint32_t CORE_SBO = 128;              // row-group-adjacent core matrices
-constexpr uint32_t SMEM_A = DIG * A_PLANE;      // 96 KB
-constexpr uint32_t SMEM_W = 2 * W_HALF;         // 48 KB (both halves)
-constexpr size_t GT_SMEM = SMEM_A + 2 * SMEM_W + 128;  // A digits, two W buffers
-constexpr uint32_t TMEM_HALF = DIG * NBLK;      // accumulator columns per half tile
-constexpr uint32_t TMEM_COLS = 512;             // 2 x 192 columns used
+constexpr uint32_t TMEM_COLS = 512;
+template <int DIG>
+struct GramSizes {
+  // W rows per block: seven digit planes of A beside the raw rows leave room
+  // for 16 (all but 92 of the 6912 tiles of 256 orbitals on 96^3 have no more)
+  static constexpr int NBLK = DIG == 6 ? 32 : 16;
+  static constexpr uint32_t W_HALF = DIG * NBLK * KH * 2;  // bytes of W digits per half tile
+  static constexpr uint32_t SMEM_A = DIG * A_PLANE;        // 96 KB with six digits
+  static constexpr uint32_t SMEM_W = 2 * W_HALF;           // 48 KB (both halves)
+  static constexpr size_t GT_SMEM = SMEM_A + 2 * SMEM_W + 128;  // A digits, two W buffers
+  static constexpr uint32_t TMEM_HALF = DIG * NBLK;        // accumulator columns per half tile
+};
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool valid) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst), "l"(src),
                "r"(valid ? 16 : 0));
@@ -75,33 +91,42 @@ __device__ __forceinline__ void cp_async_wait_all() {
   asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;\n" ::: "memory");
 }
 
-// x 2^-E on the 2^-47 grid (truncated toward zero), E = emax - 1022 for
-// the segment's largest biased exponent emax: a signed integer below 2^47.
-// Integer operations only.
-__device__ __forceinline__ long long fixed47(double v, int emax) {
+// x 2^-E on the 2^-(8 DIG - 1) grid (truncated toward zero), E = emax - 1022
+// for the segment's largest biased exponent emax: a signed integer below
+// 2^(8 DIG - 1).  Integer operations only.
+template <int DIG>
+__device__ __forceinline__ long long fixed_bal(double v, int emax) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(v);
   const int e = (int)((b >> 52) & 0x7FF);
-  const int sh = emax - e + 6;
-  if (e == 0 || sh > 60) return 0;
-  const long long X = (long long)(((b & 0xFFFFFFFFFFFFFULL) | (1ULL << 52)) >> sh);
-  return (b >> 63) ? -X : X;
+  unsigned long long X;
+  if (DIG == 6) {
+    const int sh = emax - e + 6;
+    if (e == 0 || sh > 60) return 0;
+    X = ((b & 0xFFFFFFFFFFFFFULL) | (1ULL << 52)) >> sh;
+  } else {
+    if (e == 0) return 0;
+    X = shr64c(((b & 0xFFFFFFFFFFFFFULL) | (1ULL << 52)) << 2, (unsigned)(emax - e));
+  }
+  return (b >> 63) ? -(long long)X : (long long)X;
 }
 
-// Balanced base-256 digits of X: with Y = X + 128 (256^0 + ... + 256^4),
-// digit 5 - i = byte i of Y minus 128 (i < 5) and digit 0 = Y >> 40, so
-// X = sum_k d_k 256^(5-k), d_1..d_5 in [-128, 127], |d_0| <= 128.  Each
-// digit as an FP32 value (exact), from the bit pattern 0x4B4000bb = 2^23 +
-// 2^22 + b.
+// Balanced base-256 digits of X: with Y = X + 128 (256^0 + ... +
+// 256^(DIG-2)), digit DIG - 1 - i = byte i of Y minus 128 (i < DIG - 1) and
+// digit 0 = Y >> 8 (DIG - 1), so X = sum_k d_k 256^(DIG-1-k), d_1.. in [-128,
+// 127], |d_0| <= 128.  Each digit as an FP32 value (exact), from the bit
+// pattern 0x4B4000bb = 2^23 + 2^22 + b.
+template <int DIG>
 __device__ __forceinline__ void digit_floats(long long X, float* f) {
-  const long long Y = X + 0x8080808080LL;
+  const long long Y = X + (DIG == 6 ? 0x8080808080LL : 0x808080808080LL);
   const unsigned lo = (unsigned)Y, hi = (unsigned)(Y >> 32);
   const float m = 12582912.0f + 128.0f;
-  f[5] = __uint_as_float(__byte_perm(lo, 0x4B400000u, 0x7650)) - m;
-  f[4] = __uint_as_float(__byte_perm(lo, 0x4B400000u, 0x7651)) - m;
-  f[3] = __uint_as_float(__byte_perm(lo, 0x4B400000u, 0x7652)) - m;
-  f[2] = __uint_as_float(__byte_perm(lo, 0x4B400000u, 0x7653)) - m;
-  f[1] = __uint_as_float(__byte_perm(hi, 0x4B400000u, 0x7650)) - m;
-  f[0] = __int_as_float(0x4B400000 + (int)(Y >> 40)) - 12582912.0f;
+  f[DIG - 1] = __uint_as_float(__byte_perm(lo, 0x4B400000u, 0x7650)) - m;
+  f[DIG - 2] = __uint_as_float(__byte_perm(lo, 0x4B400000u, 0x7651)) - m;
+  f[DIG - 3] = __uint_as_float(__byte_perm(lo, 0x4B400000u, 0x7652)) - m;
+  f[DIG - 4] = __uint_as_float(__byte_perm(lo, 0x4B400000u, 0x7653)) - m;
+  f[DIG - 5] = __uint_as_float(__byte_perm(hi, 0x4B400000u, 0x7650)) - m;
+  if (DIG == 7) f[1] = __uint_as_float(__byte_perm(hi, 0x4B400000u, 0x7651)) - m;
+  f[0] = __int_as_float(0x4B400000 + (int)(Y >> (8 * (DIG - 1)))) - 12582912.0f;
 }
 
 // FP16 bit patterns of two small integer-valued floats (|v| <= 2048, exact),
@@ -116,13 +141,15 @@ __device__ __forceinline__ uint32_t pack_f16(float lo, float hi) {
 // registers: the warp's lane l takes row l % 8 and the x-runs u = l / 8 and
 // l / 8 + 4 (run u: y = u % 4, z = 2h + u / 4, 8 points along x).  Row
 // pointer rp (nullptr: zero row).
+template <int DIG>
 struct GroupDigits {
   uint32_t w[2][DIG][4];  // [run][digit plane][pair of points]
   int emax;               // the row's largest biased exponent
 };
 
+template <int DIG>
 __device__ __forceinline__ void make_digits(const double* __restrict__ rp, const TileGeom& G,
-                                            int T, int h, GroupDigits& o) {
+                                            int T, int h, GroupDigits<DIG>& o) {
   const int lane = threadIdx.x & 31;
   const int txi = T % G.ntx, tyi = (T / G.ntx) % G.nty, tzi = T / (G.ntx * G.nty);
   const int gx0 = txi * TX;
@@ -157,8 +184,8 @@ __device__ __forceinline__ void make_digits(const double* __restrict__ rp, const
 #pragma unroll
     for (int p = 0; p < 4; ++p) {
       float f0[DIG], f1[DIG];
-      digit_floats(fixed47(v[q][2 * p], em), f0);
-      digit_floats(fixed47(v[q][2 * p + 1], em), f1);
+      digit_floats<DIG>(fixed_bal<DIG>(v[q][2 * p], em), f0);
+      digit_floats<DIG>(fixed_bal<DIG>(v[q][2 * p + 1], em), f1);
 #pragma unroll
       for (int k = 0; k < DIG; ++k) o.w[q][k][p] = pack_f16(f0[k], f1[k]);
     }
@@ -167,7 +194,8 @@ __device__ __forceinline__ void make_digits(const double* __restrict__ rp, const
 // Digit planes of the group to shared memory (core matrices: row group g
 // 128 B apart, run u one lbo apart, row l % 8 at 16 B), and the exponent
 // (lanes 0..7) to emax_row[l % 8].
-__device__ __forceinline__ void store_digits(const GroupDigits& o, unsigned char* plane0,
+template <int DIG>
+__device__ __forceinline__ void store_digits(const GroupDigits<DIG>& o, unsigned char* plane0,
                                              uint32_t plane_bytes, uint32_t lbo, int g,
                                              int* emax_row) {
   const int lane = threadIdx.x & 31;
@@ -208,13 +236,26 @@ __device__ __forceinline__ int float_int(float f) {
 }
 
 
+// Seven diagonal sums (integer-valued floats, |D_0|, |D_1| < 2^22, the others
+// below 2^24) as sum_d D_d 256^(6-d) 2^e0, rounded to nearest.
+__device__ __forceinline__ double combine7(const uint32_t* f, int e0) {
+  auto big = [](uint32_t x) { return (long long)__float2int_rz(__uint_as_float(x)); };
+  const long long hi = ((long long)small_float_int(f[0]) << 20) +
+                       ((long long)small_float_int(f[1]) << 12) + (big(f[2]) << 4);
+  const long long lo = (big(f[3]) << 24) + (big(f[4]) << 16) + (big(f[5]) << 8) + big(f[6]);
+  return fix_to_double(hi, lo, e0);
+}
+__device__ __forceinline__ double quiet_nan() { return __longlong_as_double(0x7FF8000000000000LL); }
+constexpr int EXP_NONFINITE = 0x7FF;
+
 // W digits, once per W: for every slot s of every tile list and half h,
 // wdig[((s * 2 + h) * DIG + k) * 8 + u] = the 8 BF16 digits (16 bytes) of
 // plane k, x-run u of W row list[s] on that half tile, and wexp[2 s + h]
 // the row segment's largest biased exponent.  Warp per (tile, half, group
 // of 8 slots).  Four CTAs per SM: the warps wait on their row loads, so
 // occupancy is what hides the latency.
-__global__ void __launch_bounds__(256, 4)
+template <int DIG>
+__global__ void __launch_bounds__(256, DIG == 6 ? 4 : 3)
     k_w_digits(const double* __restrict__ W, TileGeom G, size_t ng, int n_tiles, int ngroups,
                const int* __restrict__ tptr, const int* __restrict__ tlist, uint4* __restrict__ wdig,
                int* __restrict__ wexp) {
@@ -225,7 +266,7 @@ __global__ void __launch_bounds__(256, 4)
   if (8 * g >= nJ) return;  // warp-uniform
   const int lane = threadIdx.x & 31, r = lane & 7, s = 8 * g + r;
   const double* rp = s < nJ ? W + (size_t)tlist[j0 + s] * ng : nullptr;
-  GroupDigits d;
+  GroupDigits<DIG> d;
   make_digits(rp, G, T, h, d);
   if (s < nJ) {
     uint4* dst = wdig + ((size_t)(j0 + s) * 2 + h) * DIG * 8;
@@ -247,11 +288,16 @@ struct Unit {
 };
 
 
+template <int DIG>
 __global__ void __launch_bounds__(GT_THREADS, 1)
     k_gram_tc_ldg(const double* __restrict__ A, int m, TileGeom G, size_t ng, int n_tiles,
               const int* __restrict__ tptr, const uint4* __restrict__ wdig,
               const int* __restrict__ wexp, double* __restrict__ partial, int* __restrict__ queue,
               unsigned* __restrict__ status) {
+  using Z = GramSizes<DIG>;
+  constexpr int NBLK = Z::NBLK;
+  constexpr uint32_t W_HALF = Z::W_HALF, SMEM_A = Z::SMEM_A, SMEM_W = Z::SMEM_W,
+                     TMEM_HALF = Z::TMEM_HALF;
   extern __shared__ unsigned char gt_raw[];
   unsigned char* sA = gt_raw + ((128 - (smem_addr(gt_raw) & 127)) & 127);
   unsigned char* sW = sA + SMEM_A;  // two buffers of SMEM_W
@@ -364,11 +410,17 @@ __global__ void __launch_bounds__(GT_THREADS, 1)
       double sum = 0.0;
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        long long acc = 0;
+        const int ea = h ? ea1 : ea0, ew = Wexp[u.wb][h][c];
+        if constexpr (DIG == 7) {
+          const bool bad = ea + 1022 == EXP_NONFINITE || ew == EXP_NONFINITE;
+          sum += bad ? quiet_nan() : combine7(f + h * DIG, ea + ew - 1022 - 62);
+        } else {
+          long long acc = 0;
 #pragma unroll
-        for (int d = 0; d < DIG; ++d)
-          acc += (long long)float_int(__uint_as_float(f[h * DIG + d])) << (8 * (DIG - 1 - d));
-        sum += scaled_i64(acc, (h ? ea1 : ea0) + (Wexp[u.wb][h][c] - 1022) - 54);
+          for (int d = 0; d < DIG; ++d)
+            acc += (long long)float_int(__uint_as_float(f[h * DIG + d])) << (8 * (DIG - 1 - d));
+          sum += scaled_i64(acc, ea + (ew - 1022) - 54);
+        }
       }
       if (a < m) partial[(size_t)(u.j0 + u.jb + c) * m + a] = sum;
     }
@@ -398,7 +450,7 @@ __global__ void __launch_bounds__(GT_THREADS, 1)
   cur.wb = 1;
   if (claim(cur)) {
     load_w(cur);
-    GroupDigits dg;
+    GroupDigits<DIG> dg;
     make_digits(a_row(cur), G, cur.T, cur.h, dg);
     Unit prev = cur;
     bool have_prev = false;
@@ -475,9 +527,12 @@ constexpr int GT2_CONV = 512;                        // converting threads: 4 pe
 constexpr int GT2_THREADS = GT2_CONV + 32;           // and one MMA-issuing warp
 constexpr uint32_t A2_LBO = (MBLK / 8) * 128 + 32;   // 2080: x-runs 8 banks apart
 constexpr uint32_t A2_PLANE = 8 * A2_LBO;            // 8 runs of 8 points
-constexpr uint32_t SMEM_A2 = DIG * A2_PLANE;         // 99,840
 constexpr uint32_t RAW_KHALF = MBLK * (KH / 2) * 8;  // 32 KB: 128 rows x 32 points
-constexpr size_t GT2_SMEM = 1024 + 2 * RAW_KHALF + SMEM_A2 + SMEM_W;
+template <int DIG>
+struct GramTmaSizes {
+  static constexpr uint32_t SMEM_A2 = DIG * A2_PLANE;  // 99,840 with six digits
+  static constexpr size_t SMEM = 1024 + 2 * RAW_KHALF + SMEM_A2 + GramSizes<DIG>::SMEM_W;
+};
 
 __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map, int c0, int c1,
                                             int c2, int c3, uint32_t bar) {
@@ -509,54 +564,65 @@ __device__ __forceinline__ void bulk_prefetch_l2(const void* p, uint32_t bytes) 
 // shift count, the significand word, one 64-bit shift; per pair of values
 // nine byte permutations and the sign word.
 
-// 64-bit right shift, the count clamped at 64 (shr.b64 semantics).
-__device__ __forceinline__ unsigned long long shr64(unsigned long long a, uint32_t n) {
-  unsigned long long r;
-  asm("shr.b64 %0, %1, %2;" : "=l"(r) : "l"(a), "r"(n));
-  return r;
-}
-
 __device__ __forceinline__ uint32_t hfma2_u(uint32_t a, uint32_t b, uint32_t c) {
   uint32_t r;
   asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "r"(c));
   return r;
 }
 
+// With seven digits X = floor(|x| 2^(56 - E)) = 8 m >> (emax - e) < 2^56, the
+// bytes 6 - k; em_sh = emax << 20, nothing but zeros and subnormals (taken
+// as zero) when emax is 0.
+
 // X of one value: the significand of v (bits h, l) shifted onto the grid.
-__device__ __forceinline__ unsigned long long fixed48(uint32_t h, uint32_t l, uint32_t em_sh) {
+template <int DIG>
+__device__ __forceinline__ unsigned long long fixed_uns(uint32_t h, uint32_t l, uint32_t em_sh) {
   const uint32_t sh = (em_sh - (h & 0x7FF00000u)) >> 20;
   const unsigned long long m = ((unsigned long long)((h & 0xFFFFFu) | 0x100000u) << 32) | l;
-  return shr64(m, sh);
+  if (DIG == 6) return shr64c(m, sh);
+  return (h & 0x7FF00000u) ? shr64c(m << 3, sh) : 0ULL;
 }
 
-// The six FP16 digit planes of 8 consecutive points: d[k] = their 8 signed
-// digits of plane k (points 2i, 2i + 1 in word i, low half first).
-__device__ __forceinline__ void digits8_u(const double (&v)[8], uint32_t em_sh, uint4 (&d)[DIG]) {
+// The digit planes of a pair of values from their integers X0, X1 and high
+// words (signs): d(k) receives plane k's two signed FP16 digits.
+template <int DIG, class Put>
+__device__ __forceinline__ void digit_pair_u(unsigned long long X0, unsigned long long X1,
+                                             uint32_t h0, uint32_t h1, Put&& put) {
   constexpr uint32_t K64 = 0x64646464u;
+  const uint32_t x0h = (uint32_t)(X0 >> 32), x0l = (uint32_t)X0;
+  const uint32_t x1h = (uint32_t)(X1 >> 32), x1l = (uint32_t)X1;
+  // bytes of the two points interleaved: [p0 b, p1 b, p0 b', p1 b']
+  const uint32_t tH = __byte_perm(x0h, x1h, 0x5140);  // bytes 4, 5 of X
+  const uint32_t tB = __byte_perm(x0l, x1l, 0x7362);  // bytes 2, 3
+  const uint32_t tA = __byte_perm(x0l, x1l, 0x5140);  // bytes 0, 1
+  // sign word: FP16 pair (s0, s1) = +-1, and -1024 (s0, s1)
+  const uint32_t S = (__byte_perm(h0, h1, 0x7030) & 0x80008000u) | 0x3C003C00u;
+  const uint32_t C = S ^ 0xD800D800u;
+  // plane k = byte DIG - 1 - k: FP16 1024 + b from the pattern 0x64bb
+  if (DIG == 7) {
+    const uint32_t tT = __byte_perm(x0h, x1h, 0x7362);  // byte 6 (and 7, zero)
+    put(0, hfma2_u(__byte_perm(tT, K64, 0x4140), S, C));
+  }
+  put(DIG - 6, hfma2_u(__byte_perm(tH, K64, 0x4342), S, C));
+  put(DIG - 5, hfma2_u(__byte_perm(tH, K64, 0x4140), S, C));
+  put(DIG - 4, hfma2_u(__byte_perm(tB, K64, 0x4342), S, C));
+  put(DIG - 3, hfma2_u(__byte_perm(tB, K64, 0x4140), S, C));
+  put(DIG - 2, hfma2_u(__byte_perm(tA, K64, 0x4342), S, C));
+  put(DIG - 1, hfma2_u(__byte_perm(tA, K64, 0x4140), S, C));
+}
+
+// The FP16 digit planes of 8 consecutive points: d[k] = their 8 signed
+// digits of plane k (points 2i, 2i + 1 in word i, low half first).
+template <int DIG>
+__device__ __forceinline__ void digits8_u(const double (&v)[8], uint32_t em_sh, uint4 (&d)[DIG]) {
   uint32_t w[DIG][4];
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     const unsigned long long b0 = (unsigned long long)__double_as_longlong(v[2 * i]);
     const unsigned long long b1 = (unsigned long long)__double_as_longlong(v[2 * i + 1]);
     const uint32_t h0 = (uint32_t)(b0 >> 32), h1 = (uint32_t)(b1 >> 32);
-    const unsigned long long X0 = fixed48(h0, (uint32_t)b0, em_sh);
-    const unsigned long long X1 = fixed48(h1, (uint32_t)b1, em_sh);
-    const uint32_t x0h = (uint32_t)(X0 >> 32), x0l = (uint32_t)X0;
-    const uint32_t x1h = (uint32_t)(X1 >> 32), x1l = (uint32_t)X1;
-    // bytes of the two points interleaved: [p0 b, p1 b, p0 b', p1 b']
-    const uint32_t tH = __byte_perm(x0h, x1h, 0x5140);  // bytes 4, 5 of X
-    const uint32_t tB = __byte_perm(x0l, x1l, 0x7362);  // bytes 2, 3
-    const uint32_t tA = __byte_perm(x0l, x1l, 0x5140);  // bytes 0, 1
-    // sign word: FP16 pair (s0, s1) = +-1, and -1024 (s0, s1)
-    const uint32_t S = (__byte_perm(h0, h1, 0x7030) & 0x80008000u) | 0x3C003C00u;
-    const uint32_t C = S ^ 0xD800D800u;
-    // plane k = byte 5 - k: FP16 1024 + b from the pattern 0x64bb
-    w[0][i] = hfma2_u(__byte_perm(tH, K64, 0x4342), S, C);
-    w[1][i] = hfma2_u(__byte_perm(tH, K64, 0x4140), S, C);
-    w[2][i] = hfma2_u(__byte_perm(tB, K64, 0x4342), S, C);
-    w[3][i] = hfma2_u(__byte_perm(tB, K64, 0x4140), S, C);
-    w[4][i] = hfma2_u(__byte_perm(tA, K64, 0x4342), S, C);
-    w[5][i] = hfma2_u(__byte_perm(tA, K64, 0x4140), S, C);
+    digit_pair_u<DIG>(fixed_uns<DIG>(h0, (uint32_t)b0, em_sh), fixed_uns<DIG>(h1, (uint32_t)b1, em_sh),
+                      h0, h1, [&](int k, uint32_t x) { w[k][i] = x; });
   }
 #pragma unroll
   for (int k = 0; k < DIG; ++k) d[k] = make_uint4(w[k][0], w[k][1], w[k][2], w[k][3]);
@@ -564,31 +630,30 @@ __device__ __forceinline__ void digits8_u(const double (&v)[8], uint32_t em_sh, 
 
 // The same unsigned-byte FP16 digits for a pair of values with exponents of
 // their own (the expansion's H(j, v) 2^E_j against E_v): emax0, emax1 are
-// the largest biased exponents the two values are measured against (below 64:
-// the value counts as zero).  pk[k][e] = the pair's digits of plane k.
+// the largest biased exponents the two values are measured against (six
+// digits, below 64: the value counts as zero).  pk[k][e] = the pair's digits
+// of plane k.
+template <int DIG>
 __device__ __forceinline__ void digits2_u(double v0, double v1, int emax0, int emax1,
                                           uint32_t (&pk)[DIG][2], int e) {
-  constexpr uint32_t K64 = 0x64646464u;
-  const uint32_t em0 = emax0 >= 64 ? (uint32_t)(emax0 + 5) << 20 : 0xF0000000u;
-  const uint32_t em1 = emax1 >= 64 ? (uint32_t)(emax1 + 5) << 20 : 0xF0000000u;
   const unsigned long long b0 = (unsigned long long)__double_as_longlong(v0);
   const unsigned long long b1 = (unsigned long long)__double_as_longlong(v1);
   const uint32_t h0 = (uint32_t)(b0 >> 32), h1 = (uint32_t)(b1 >> 32);
-  const unsigned long long X0 = fixed48(h0, (uint32_t)b0, em0);
-  const unsigned long long X1 = fixed48(h1, (uint32_t)b1, em1);
-  const uint32_t x0h = (uint32_t)(X0 >> 32), x0l = (uint32_t)X0;
-  const uint32_t x1h = (uint32_t)(X1 >> 32), x1l = (uint32_t)X1;
-  const uint32_t tH = __byte_perm(x0h, x1h, 0x5140);
-  const uint32_t tB = __byte_perm(x0l, x1l, 0x7362);
-  const uint32_t tA = __byte_perm(x0l, x1l, 0x5140);
-  const uint32_t S = (__byte_perm(h0, h1, 0x7030) & 0x80008000u) | 0x3C003C00u;
-  const uint32_t C = S ^ 0xD800D800u;
-  pk[0][e] = hfma2_u(__byte_perm(tH, K64, 0x4342), S, C);
-  pk[1][e] = hfma2_u(__byte_perm(tH, K64, 0x4140), S, C);
-  pk[2][e] = hfma2_u(__byte_perm(tB, K64, 0x4342), S, C);
-  pk[3][e] = hfma2_u(__byte_perm(tB, K64, 0x4140), S, C);
-  pk[4][e] = hfma2_u(__byte_perm(tA, K64, 0x4342), S, C);
-  pk[5][e] = hfma2_u(__byte_perm(tA, K64, 0x4140), S, C);
+  unsigned long long X0, X1;
+  if (DIG == 6) {
+    X0 = fixed_uns<6>(h0, (uint32_t)b0, emax0 >= 64 ? (uint32_t)(emax0 + 5) << 20 : 0xF0000000u);
+    X1 = fixed_uns<6>(h1, (uint32_t)b1, emax1 >= 64 ? (uint32_t)(emax1 + 5) << 20 : 0xF0000000u);
+  } else {
+    // exponents may leave the FP64 range here: plain integer shift counts
+    auto fixed = [](uint32_t h, uint32_t l, int emax) -> unsigned long long {
+      const int ex = (int)((h >> 20) & 0x7FFu);
+      const unsigned long long m = ((unsigned long long)((h & 0xFFFFFu) | 0x100000u) << 32) | l;
+      return ex ? shr64c(m << 3, (unsigned)max(emax - ex, 0)) : 0ULL;
+    };
+    X0 = fixed(h0, (uint32_t)b0, emax0);
+    X1 = fixed(h1, (uint32_t)b1, emax1);
+  }
+  digit_pair_u<DIG>(X0, X1, h0, h1, [&](int k, uint32_t x) { pk[k][e] = x; });
 }
 
 // Converting warps 0..15 (named barrier 1) and the issuing warp 16.  Per
@@ -611,11 +676,16 @@ __device__ __forceinline__ bool conv_sync_or(bool v) {
   return r != 0;
 }
 
+template <int DIG>
 __global__ void __launch_bounds__(GT2_THREADS, 1)
     k_gram_tc(const __grid_constant__ CUtensorMap tmA, int m, TileGeom G, int n_tiles,
               const int* __restrict__ tptr, const uint4* __restrict__ wdig,
               const int* __restrict__ wexp, double* __restrict__ partial, int* __restrict__ queue,
               unsigned* __restrict__ status) {
+  using Z = GramSizes<DIG>;
+  constexpr int NBLK = Z::NBLK;
+  constexpr uint32_t W_HALF = Z::W_HALF, TMEM_HALF = Z::TMEM_HALF,
+                     SMEM_A2 = GramTmaSizes<DIG>::SMEM_A2;
   extern __shared__ unsigned char gt_raw[];
   unsigned char* sR = gt_raw + ((1024 - (smem_addr(gt_raw) & 1023)) & 1023);  // two K halves
   unsigned char* sA = sR + 2 * RAW_KHALF;
@@ -839,36 +909,62 @@ __global__ void __launch_bounds__(GT2_THREADS, 1)
         // magnitude, 64 points): D_0, D_1 (< 2^22) by the 2^22 conversion on
         // the FP32 pipe, the others by the conversion unit (exact: integer
         // values below 2^24); D_0 256 + D_1 and D_2 256 + D_3 stay below 2^31
-        long long acc[2][2];  // [half][column]
+        if constexpr (DIG == 7) {  // each half rounded to FP64, then added
+          double y[2] = {0.0, 0.0};
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          uint32_t f[DIG][2];
+          for (int h = 0; h < 2; ++h) {
+            uint32_t f[2][DIG];
 #pragma unroll
-          for (int d = 0; d < DIG; ++d)
-            tmem_ld2(lane_addr + (uint32_t)(h * TMEM_HALF + d * P + c0), f[d]);
-          tmem_wait_ld();
+            for (int d = 0; d < DIG; ++d) {
+              uint32_t t[2];
+              tmem_ld2(lane_addr + (uint32_t)(h * TMEM_HALF + d * P + c0), t);
+              f[0][d] = t[0];
+              f[1][d] = t[1];
+            }
+            tmem_wait_ld();
+            const int ea = h ? ea1 : ea0;
+#pragma unroll
+            for (int cc = 0; cc < 2; ++cc) {
+              const int ew = Wexp[u.wb][h][min(c0 + cc, NBLK - 1)];
+              const bool bad = ea + 1022 == EXP_NONFINITE || ew == EXP_NONFINITE;
+              y[cc] += bad ? quiet_nan() : combine7(f[cc], ea + ew - 1022 - 63);
+            }
+          }
+#pragma unroll
+          for (int cc = 0; cc < 2; ++cc)
+            if (c0 + cc < nj && a < m) partial[(size_t)(u.j0 + u.jb + c0 + cc) * m + a] = y[cc];
+        } else {
+          long long acc[2][2];  // [half][column]
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            uint32_t f[DIG][2];
+#pragma unroll
+            for (int d = 0; d < DIG; ++d)
+              tmem_ld2(lane_addr + (uint32_t)(h * TMEM_HALF + d * P + c0), f[d]);
+            tmem_wait_ld();
+#pragma unroll
+            for (int cc = 0; cc < 2; ++cc) {
+              const int t01 = small_float_int(f[0][cc]) * 256 + small_float_int(f[1][cc]);
+              const int t23 = __float2int_rz(__uint_as_float(f[2][cc])) * 256 +
+                              __float2int_rz(__uint_as_float(f[3][cc]));
+              acc[h][cc] = ((long long)t01 << 32) + ((long long)t23 << 16) +
+                           ((long long)__float2int_rz(__uint_as_float(f[4][cc])) << 8) +
+                           (long long)__float2int_rz(__uint_as_float(f[5][cc]));
+            }
+          }
+          // sum_r x w = 2^(E_x + E_w - 55) acc; the two halves on the larger
+          // scale (the other truncated at its unit, 2^-55 of that segment's
+          // scale), one truncation
 #pragma unroll
           for (int cc = 0; cc < 2; ++cc) {
-            const int t01 = small_float_int(f[0][cc]) * 256 + small_float_int(f[1][cc]);
-            const int t23 = __float2int_rz(__uint_as_float(f[2][cc])) * 256 +
-                            __float2int_rz(__uint_as_float(f[3][cc]));
-            acc[h][cc] = ((long long)t01 << 32) + ((long long)t23 << 16) +
-                         ((long long)__float2int_rz(__uint_as_float(f[4][cc])) << 8) +
-                         (long long)__float2int_rz(__uint_as_float(f[5][cc]));
-          }
-        }
-        // sum_r x w = 2^(E_x + E_w - 55) acc; the two halves on the larger
-        // scale (the other truncated at its unit, 2^-55 of that segment's
-        // scale), one truncation
-#pragma unroll
-        for (int cc = 0; cc < 2; ++cc) {
-          const int c = c0 + cc;
-          if (c < nj) {
-            const int e0 = ea0 + Wexp[u.wb][0][c] - 1022 - 55, e1 = ea1 + Wexp[u.wb][1][c] - 1022 - 55;
-            const bool b0 = e0 >= e1;
-            const int sh = min(b0 ? e0 - e1 : e1 - e0, 63);
-            const long long s2 = (b0 ? acc[0][cc] : acc[1][cc]) + ((b0 ? acc[1][cc] : acc[0][cc]) >> sh);
-            if (a < m) partial[(size_t)(u.j0 + u.jb + c) * m + a] = scaled_i64_rz_cvt(s2, b0 ? e0 : e1);
+            const int c = c0 + cc;
+            if (c < nj) {
+              const int e0 = ea0 + Wexp[u.wb][0][c] - 1022 - 55, e1 = ea1 + Wexp[u.wb][1][c] - 1022 - 55;
+              const bool b0 = e0 >= e1;
+              const int sh = min(b0 ? e0 - e1 : e1 - e0, 63);
+              const long long s2 = (b0 ? acc[0][cc] : acc[1][cc]) + ((b0 ? acc[1][cc] : acc[0][cc]) >> sh);
+              if (a < m) partial[(size_t)(u.j0 + u.jb + c) * m + a] = scaled_i64_rz_cvt(s2, b0 ? e0 : e1);
+            }
           }
         }
       }
@@ -922,7 +1018,7 @@ __global__ void __launch_bounds__(GT2_THREADS, 1)
         emf = max(emf, __shfl_xor_sync(0xffffffffu, emf, 1));
         emf = max(emf, __shfl_xor_sync(0xffffffffu, emf, 2));
         const int em = (int)(emf >> 20);
-        const uint32_t em_sh = em < 64 ? 0xF0000000u : emf + (5u << 20);
+        const uint32_t em_sh = DIG == 6 ? (em < 64 ? 0xF0000000u : emf + (5u << 20)) : emf;
         if (tid == 0) q_step();
         if (conv_sync_or(!ok)) {  // B1: both raw buffers consumed
           fail = true;
@@ -938,10 +1034,10 @@ __global__ void __launch_bounds__(GT2_THREADS, 1)
         // each K half's digits replace those prev's MMAs of that half read
         uint4 d[DIG];
         ok = wait_mma(0);
-        digits8_u(v[0], em_sh, d);
+        digits8_u<DIG>(v[0], em_sh, d);
         store_digits(d, 0);
         ok = wait_mma(1) && ok;
-        digits8_u(v[1], em_sh, d);
+        digits8_u<DIG>(v[1], em_sh, d);
         store_digits(d, 1);
         tc_fence_after();
         if (have_prev && prev.h == 1) epilogue(prev);  // all of prev's MMAs are done
@@ -1025,20 +1121,28 @@ __global__ void __launch_bounds__(GT2_THREADS, 1)
 constexpr int XJ = 32, XKS = 16, XN = 32;
 constexpr uint32_t XA_BLOCK = MBLK * XKS * 2;          // 4 KB: one plane, one K step
 constexpr uint32_t XA_LBO = (MBLK / 8) * 128;          // 2048
-constexpr uint32_t XA_STEP = DIG * XA_BLOCK;           // 24 KB
-constexpr uint32_t XA_TILE = 2 * XA_STEP;              // 48 KB
-constexpr uint32_t XB_LBO = (DIG * XN / 8) * 128;      // 3072
-constexpr uint32_t XB_CHUNK = 2 * XB_LBO;              // 6 KB: 192 rows x 16 K
-constexpr uint32_t XT_COLS = DIG * XN;                 // 192
+constexpr int XR = 4;                                  // ring slots (chunks of XN vectors)
+template <int DIG>
+struct ExpandSizes {  // with six digits
+  static constexpr uint32_t XA_STEP = DIG * XA_BLOCK;       // 24 KB
+  static constexpr uint32_t XA_TILE = 2 * XA_STEP;          // 48 KB
+  static constexpr uint32_t XB_LBO = (DIG * XN / 8) * 128;  // 3072
+  static constexpr uint32_t XB_CHUNK = 2 * XB_LBO;          // 6 KB: 192 rows x 16 K
+  static constexpr uint32_t XT_COLS = DIG * XN;             // 192
+  static constexpr uint32_t XS_SLOT = 2 * XB_CHUNK;         // 12 KB: both K steps of one chunk
+  static constexpr size_t XE_SMEM = 2 * XA_TILE + XR * XS_SLOT + 128;
+};
 
 // W's digit image: CTA per tile (thread = point p), for tiles whose list has
 // 1..XJ entries.  wx[T][(q 6 + k) 4096 + (p / 8) 128 + (jq / 8) 2048 +
 // (p % 8) 16 + (jq % 8) 2] = digit k of W[list(16 q + jq)] at point p (zero
 // outside the entry's sub-box and beyond the list), wxexp[slot] = E_j + 1022.
+template <int DIG>
 __global__ void __launch_bounds__(MBLK)
     k_wx_digits(const double* __restrict__ W, TileGeom G, size_t ng, int n_tiles,
                 const int* __restrict__ tptr, const int* __restrict__ tlist,
                 const int* __restrict__ tsub, uint4* __restrict__ wx, int* __restrict__ wxexp) {
+  constexpr uint32_t XA_STEP = ExpandSizes<DIG>::XA_STEP, XA_TILE = 2 * XA_STEP;
   const int T = blockIdx.x;
   const int j0 = tptr[T], nJ = tptr[T + 1] - j0;
   if (nJ == 0 || nJ > XJ) return;  // uniform
@@ -1067,8 +1171,8 @@ __global__ void __launch_bounds__(MBLK)
     for (int e = 0; e < 8; e += 2) {
       const int jl = 8 * grp + e;
       float f0[DIG], f1[DIG];
-      digit_floats(jl < nJ ? fixed47(wval(jl), emx[jl]) : 0, f0);
-      digit_floats(jl + 1 < nJ ? fixed47(wval(jl + 1), emx[jl + 1]) : 0, f1);
+      digit_floats<DIG>(jl < nJ ? fixed_bal<DIG>(wval(jl), emx[jl]) : 0, f0);
+      digit_floats<DIG>(jl + 1 < nJ ? fixed_bal<DIG>(wval(jl + 1), emx[jl + 1]) : 0, f1);
 #pragma unroll
       for (int k = 0; k < DIG; ++k) pk[k][e / 2] = pack_f16(f0[k], f1[k]);
     }
@@ -1083,7 +1187,10 @@ __global__ void __launch_bounds__(MBLK)
 // E_v of the expansion for every (tile, vector): the largest biased
 // exponent of H(j, v) 2^(E_j) over the tile's list (0 where all are zero);
 // thread = vector, grid y = tile.  Tiles with an empty list or more than XJ
-// entries are skipped (not read).
+// entries are skipped (not read).  STRICT: EV_NONFINITE where a factor is not
+// finite.
+constexpr int EV_NONFINITE = 1 << 20;
+template <bool STRICT>
 __global__ void __launch_bounds__(128)
     k_expand_ev(const int* __restrict__ tptr, const int* __restrict__ tlist,
                 const int* __restrict__ wxexp, const double* __restrict__ H, long long hj,
@@ -1097,6 +1204,7 @@ __global__ void __launch_bounds__(128)
         (int)((__double_as_longlong(H[(long long)tlist[j0 + jl] * hj + (long long)v * hv]) >> 52) &
               0x7FF);
     if (e) em = max(em, e + wxexp[j0 + jl] - 1022);
+    if (STRICT && (e == EXP_NONFINITE || wxexp[j0 + jl] == EXP_NONFINITE)) em = EV_NONFINITE;
   }
   ev[(size_t)T * m + v] = em;
 }
@@ -1105,9 +1213,6 @@ constexpr int XE_WARPS = 16;                 // epilogue warps (tensor-memory re
 constexpr int XP_WARPS = 8;                  // H-digit warps
 constexpr int XE_ISSUER = XE_WARPS + XP_WARPS;           // the MMA-issuing warp
 constexpr int XE_THREADS = 32 * (XE_ISSUER + 1);         // 800
-constexpr int XR = 4;                                    // ring slots (chunks of XN vectors)
-constexpr uint32_t XS_SLOT = 2 * XB_CHUNK;               // 12 KB: both K steps of one chunk
-constexpr size_t XE_SMEM = 2 * XA_TILE + XR * XS_SLOT + 128;
 constexpr int XF_FIRST = 1, XF_LAST = 2, XF_END = 4;    // slot flags
 
 // Persistent CTAs (one per SM) over the tiles whose list has at most XJ
@@ -1132,12 +1237,16 @@ constexpr int XF_FIRST = 1, XF_LAST = 2, XF_END = 4;    // slot flags
 // hv]; out[v ng + r].  Every wait is bounded; on expiry the role stops, the
 // others see s_fail (or expire themselves) and the kernel reports
 // SEA_FLAG_WAIT after the MMAs and copies in flight are done.
+template <int DIG>
 __global__ void __launch_bounds__(XE_THREADS, 1)
     k_expand_tc(const uint4* __restrict__ wx, const int* __restrict__ wxexp, TileGeom G, size_t ng,
                 int n_tiles, const int* __restrict__ tptr, const int* __restrict__ tlist,
                 const double* __restrict__ H, long long hj, long long hv, int m, int negate,
                 double* __restrict__ out, const int* __restrict__ evp, int* __restrict__ queue,
                 unsigned* __restrict__ status) {
+  using Z = ExpandSizes<DIG>;
+  constexpr uint32_t XA_STEP = Z::XA_STEP, XA_TILE = Z::XA_TILE, XB_LBO = Z::XB_LBO,
+                     XB_CHUNK = Z::XB_CHUNK, XT_COLS = Z::XT_COLS, XS_SLOT = Z::XS_SLOT;
   extern __shared__ unsigned char xe_raw[];
   unsigned char* sA = xe_raw + ((128 - (smem_addr(xe_raw) & 127)) & 127);  // two tile images
   unsigned char* sS = sA + 2 * XA_TILE;                                     // XR chunk slots
@@ -1274,8 +1383,8 @@ __global__ void __launch_bounds__(XE_THREADS, 1)
 #pragma unroll
           for (int e = 0; e < 2; ++e) {
             const int jl = jb + 2 * e;
-            digits2_u(h[2 * e], h[2 * e + 1], jl < nJ ? ev - p_shj[jl] : 0,
-                      jl + 1 < nJ ? ev - p_shj[jl + 1] : 0, pk, e);
+            digits2_u<DIG>(h[2 * e], h[2 * e + 1], jl < nJ ? ev - p_shj[jl] : 0,
+                           jl + 1 < nJ ? ev - p_shj[jl + 1] : 0, pk, e);
           }
           // entries jb.. of K step jb / 16: core matrix (jb / 8) % 2, bytes
           // (jb % 8) 2 of its 16-byte rows
@@ -1426,17 +1535,26 @@ __global__ void __launch_bounds__(XE_THREADS, 1)
           }
 #pragma unroll
           for (int u = 0; u < 4; ++u) {
-            // sum_d D_d 256^(5 - d) in three 32-bit pairs; |D_d| < 2^22 except
-            // D_4 and D_5 of lists longer than 16 (below 2^23): those by the
-            // conversion instruction
-            const int t01 = small_float_int(f[0][u]) * 256 + small_float_int(f[1][u]);
-            const int t23 = small_float_int(f[2][u]) * 256 + small_float_int(f[3][u]);
-            const int d4 = wide ? __float2int_rz(__uint_as_float(f[4][u])) : small_float_int(f[4][u]);
-            const int d5 = wide ? __float2int_rz(__uint_as_float(f[5][u])) : small_float_int(f[5][u]);
-            const int t45 = d4 * 256 + d5;
-            const long long base = ((long long)t01 << 32) + (long long)t45;
-            const long long acc = base + (long long)t23 * 65536LL;
-            const double val = scaled_i64_rz_cvt(acc, ev[4 * hh + u] - 1022 - 55);
+            double val;
+            if constexpr (DIG == 7) {
+              uint32_t fd[DIG];
+#pragma unroll
+              for (int d = 0; d < DIG; ++d) fd[d] = f[d][u];
+              const int e = ev[4 * hh + u];
+              val = e >= EV_NONFINITE ? quiet_nan() : combine7(fd, e - 1022 - 63);
+            } else {
+              // sum_d D_d 256^(5 - d) in three 32-bit pairs; |D_d| < 2^22 except
+              // D_4 and D_5 of lists longer than 16 (below 2^23): those by the
+              // conversion instruction
+              const int t01 = small_float_int(f[0][u]) * 256 + small_float_int(f[1][u]);
+              const int t23 = small_float_int(f[2][u]) * 256 + small_float_int(f[3][u]);
+              const int d4 = wide ? __float2int_rz(__uint_as_float(f[4][u])) : small_float_int(f[4][u]);
+              const int d5 = wide ? __float2int_rz(__uint_as_float(f[5][u])) : small_float_int(f[5][u]);
+              const int t45 = d4 * 256 + d5;
+              const long long base = ((long long)t01 << 32) + (long long)t45;
+              const long long acc = base + (long long)t23 * 65536LL;
+              val = scaled_i64_rz_cvt(acc, ev[4 * hh + u] - 1022 - 55);
+            }
             if (g >= 0 && (full || vbase + 4 * hh + u < m)) o[(size_t)(4 * hh + u) * ng] = val;
           }
         }
@@ -1461,21 +1579,22 @@ __global__ void __launch_bounds__(XE_THREADS, 1)
 }  // namespace
 
 
-size_t w_digits_bytes(long long slots) {
-  return (size_t)std::max(slots, 1LL) * 2 * DIG * 8 * sizeof(uint4) +
+size_t w_digits_bytes(long long slots, int digits) {
+  return (size_t)std::max(slots, 1LL) * 2 * digits * 8 * sizeof(uint4) +
          (size_t)std::max(slots, 1LL) * 2 * sizeof(int);
+}
+static int* w_digits_exp(const void* wbuf, long long slots, int digits) {
+  return (int*)((uint4*)wbuf + (size_t)std::max(slots, 1LL) * 2 * digits * 8);
 }
 
 cudaError_t launch_w_digits(cudaStream_t st, const double* W, const TileGeom& G, size_t ng,
                             int n_tiles, int max_list, const int* tptr, const int* tlist,
-                            long long slots, void* wbuf) {
+                            long long slots, void* wbuf, int digits) {
   if (n_tiles <= 0 || max_list <= 0) return cudaSuccess;
-  uint4* wdig = (uint4*)wbuf;
-  int* wexp = (int*)(wdig + (size_t)std::max(slots, 1LL) * 2 * DIG * 8);
   const int ngroups = (max_list + 7) / 8;
   const long long warps = (long long)n_tiles * 2 * ngroups;
-  k_w_digits<<<(unsigned)((warps + 7) / 8), 256, 0, st>>>(W, G, ng, n_tiles, ngroups, tptr, tlist,
-                                                          wdig, wexp);
+  (digits == 7 ? k_w_digits<7> : k_w_digits<6>)<<<(unsigned)((warps + 7) / 8), 256, 0, st>>>(
+      W, G, ng, n_tiles, ngroups, tptr, tlist, (uint4*)wbuf, w_digits_exp(wbuf, slots, digits));
   return cudaGetLastError();
 }
 
@@ -1517,77 +1636,94 @@ static bool make_a_map(const double* A, int m, const TileGeom& G, CUtensorMap* m
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-size_t wx_digits_bytes(int n_tiles, long long slots) {
-  return (size_t)std::max(n_tiles, 1) * XA_TILE + (size_t)std::max(slots, 1LL) * sizeof(int);
+static size_t xa_tile(int digits) {
+  return digits == 7 ? ExpandSizes<7>::XA_TILE : ExpandSizes<6>::XA_TILE;
+}
+size_t wx_digits_bytes(int n_tiles, long long slots, int digits) {
+  return (size_t)std::max(n_tiles, 1) * xa_tile(digits) +
+         (size_t)std::max(slots, 1LL) * sizeof(int);
 }
 
 cudaError_t launch_wx_digits(cudaStream_t st, const double* W, const TileGeom& G, size_t ng,
                              int n_tiles, const int* tptr, const int* tlist, const int* tsub,
-                             void* wxbuf) {
+                             void* wxbuf, int digits) {
   if (n_tiles <= 0) return cudaSuccess;
   uint4* wx = (uint4*)wxbuf;
-  int* wxexp = (int*)((unsigned char*)wxbuf + (size_t)n_tiles * XA_TILE);
-  k_wx_digits<<<n_tiles, MBLK, 0, st>>>(W, G, ng, n_tiles, tptr, tlist, tsub, wx, wxexp);
+  int* wxexp = (int*)((unsigned char*)wxbuf + (size_t)n_tiles * xa_tile(digits));
+  (digits == 7 ? k_wx_digits<7> : k_wx_digits<6>)<<<n_tiles, MBLK, 0, st>>>(W, G, ng, n_tiles, tptr,
+                                                                           tlist, tsub, wx, wxexp);
+  return cudaGetLastError();
+}
+
+template <int DIG>
+static cudaError_t expand_tc(cudaStream_t st, int device, const void* wxbuf, const TileGeom& G,
+                             size_t ng, int n_tiles, const int* tptr, const int* tlist,
+                             const double* H, long long hj, long long hv, int m, bool negate,
+                             double* out, int* evbuf, int* queue, unsigned* status) {
+  constexpr size_t smem = ExpandSizes<DIG>::XE_SMEM;
+  cudaError_t e =
+      cudaFuncSetAttribute(k_expand_tc<DIG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  if (n_tiles <= 0 || m <= 0) return cudaSuccess;
+  const uint4* wx = (const uint4*)wxbuf;
+  const int* wxexp = (const int*)((const unsigned char*)wxbuf + (size_t)n_tiles * xa_tile(DIG));
+  int nsm = 0;
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, device);
+  e = cudaMemsetAsync(queue, 0, sizeof(int), st);
+  if (e != cudaSuccess) return e;
+  k_expand_ev<DIG == 7><<<dim3((m + 127) / 128, n_tiles), 128, 0, st>>>(tptr, tlist, wxexp, H, hj,
+                                                                       hv, m, evbuf);
+  k_expand_tc<DIG><<<std::min(nsm, n_tiles), XE_THREADS, smem, st>>>(
+      wx, wxexp, G, ng, n_tiles, tptr, tlist, H, hj, hv, m, negate ? 1 : 0, out, evbuf, queue,
+      status);
   return cudaGetLastError();
 }
 
 cudaError_t launch_expand_tc(cudaStream_t st, int device, const void* wxbuf, const TileGeom& G,
                              size_t ng, int n_tiles, const int* tptr, const int* tlist,
                              const double* H, long long hj, long long hv, int m, bool negate,
-                             double* out, int* evbuf, int* queue, unsigned* status) {
-  static bool attr_set[64] = {};
-  if (device < 0 || device >= 64) return cudaErrorInvalidDevice;
-  if (!attr_set[device]) {
-    const cudaError_t e =
-        cudaFuncSetAttribute(k_expand_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)XE_SMEM);
-    if (e != cudaSuccess) return e;
-    attr_set[device] = true;
-  }
-  if (n_tiles <= 0 || m <= 0) return cudaSuccess;
-  const uint4* wx = (const uint4*)wxbuf;
-  const int* wxexp = (const int*)((const unsigned char*)wxbuf + (size_t)n_tiles * XA_TILE);
-  int nsm = 0;
-  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, device);
-  cudaError_t e = cudaMemsetAsync(queue, 0, sizeof(int), st);
-  if (e != cudaSuccess) return e;
-  k_expand_ev<<<dim3((m + 127) / 128, n_tiles), 128, 0, st>>>(tptr, tlist, wxexp, H, hj, hv, m,
-                                                             evbuf);
-  k_expand_tc<<<std::min(nsm, n_tiles), XE_THREADS, XE_SMEM, st>>>(
-      wx, wxexp, G, ng, n_tiles, tptr, tlist, H, hj, hv, m, negate ? 1 : 0, out, evbuf, queue,
-      status);
-  return cudaGetLastError();
+                             double* out, int* evbuf, int* queue, unsigned* status, int digits) {
+  return (digits == 7 ? expand_tc<7> : expand_tc<6>)(st, device, wxbuf, G, ng, n_tiles, tptr, tlist,
+                                                     H, hj, hv, m, negate, out, evbuf, queue, status);
 }
 
 int expand_tc_max_list() { return XJ; }
 
-cudaError_t launch_gram_tc(cudaStream_t st, int device, const double* A, int m, const TileGeom& G,
+template <int DIG>
+static cudaError_t gram_tc(cudaStream_t st, int device, const double* A, int m, const TileGeom& G,
                            size_t ng, int n_tiles, const int* tptr, long long slots,
                            const void* wbuf, double* partial, int* queue, unsigned* status) {
-  static bool attr_set[64] = {};
-  if (device < 0 || device >= 64) return cudaErrorInvalidDevice;
-  if (!attr_set[device]) {
-    cudaError_t e = cudaFuncSetAttribute(k_gram_tc_ldg, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)GT_SMEM);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_gram_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GT2_SMEM);
-    if (e != cudaSuccess) return e;
-    attr_set[device] = true;
-  }
+  constexpr size_t smem_ldg = GramSizes<DIG>::GT_SMEM, smem_tma = GramTmaSizes<DIG>::SMEM;
+  static_assert(smem_ldg <= 232448 - 4096 && smem_tma <= 232448 - 4096, "shared memory of an SM");
+  cudaError_t e = cudaFuncSetAttribute(k_gram_tc_ldg<DIG>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_ldg);
+  if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(k_gram_tc<DIG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)smem_tma);
+  if (e != cudaSuccess) return e;
   const uint4* wdig = (const uint4*)wbuf;
-  const int* wexp = (const int*)(wdig + (size_t)std::max(slots, 1LL) * 2 * DIG * 8);
+  const int* wexp = w_digits_exp(wbuf, slots, DIG);
   int nsm = 0;
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, device);
-  cudaError_t e = cudaMemsetAsync(queue, 0, sizeof(int), st);
+  e = cudaMemsetAsync(queue, 0, sizeof(int), st);
   if (e != cudaSuccess) return e;
   const int grid = std::min(nsm, std::max(n_tiles, 1));
   alignas(64) CUtensorMap map;
   if (make_a_map(A, m, G, &map))
-    k_gram_tc<<<grid, GT2_THREADS, GT2_SMEM, st>>>(map, m, G, n_tiles, tptr, wdig, wexp, partial,
-                                                  queue, status);
+    k_gram_tc<DIG><<<grid, GT2_THREADS, smem_tma, st>>>(map, m, G, n_tiles, tptr, wdig, wexp,
+                                                       partial, queue, status);
   else
-    k_gram_tc_ldg<<<grid, GT_THREADS, GT_SMEM, st>>>(A, m, G, ng, n_tiles, tptr, wdig, wexp,
-                                                     partial, queue, status);
+    k_gram_tc_ldg<DIG><<<grid, GT_THREADS, smem_ldg, st>>>(A, m, G, ng, n_tiles, tptr, wdig, wexp,
+                                                          partial, queue, status);
   return cudaGetLastError();
+}
+
+cudaError_t launch_gram_tc(cudaStream_t st, int device, const double* A, int m, const TileGeom& G,
+                           size_t ng, int n_tiles, const int* tptr, long long slots,
+                           const void* wbuf, double* partial, int* queue, unsigned* status,
+                           int digits) {
+  return (digits == 7 ? gram_tc<7> : gram_tc<6>)(st, device, A, m, G, ng, n_tiles, tptr, slots, wbuf,
+                                                 partial, queue, status);
 }
 
 }  // namespace sea

@@ -990,26 +990,28 @@ cudaError_t launch_rotate(sea_ctx* c, const double* phi, int n, size_t N, const 
                           double* out);
 // Damped Jacobi sweeps on every pair's starting vector (pair.cu).
 cudaError_t launch_smooth(sea_ctx* c, int sweeps, double omega);
-// Mixed form's contraction with W on the tensor cores.  launch_w_digits
+// The contraction with W on the tensor cores.  launch_w_digits
 // splits W's rows on every tile of every list once into wbuf
 // (w_digits_bytes(slots), slots = total list length); launch_gram_tc then
 // forms partial[slot m + a] for A's m rows.  *queue is reset on the stream.
-size_t w_digits_bytes(long long slots);
+// digits: 6 (mixed form) or 7 (plain form).
+size_t w_digits_bytes(long long slots, int digits);
 cudaError_t launch_w_digits(cudaStream_t st, const double* W, const TileGeom& G, size_t ng,
                             int n_tiles, int max_list, const int* tptr, const int* tlist,
-                            long long slots, void* wbuf);
-size_t wx_digits_bytes(int n_tiles, long long slots);
+                            long long slots, void* wbuf, int digits);
+size_t wx_digits_bytes(int n_tiles, long long slots, int digits);
 cudaError_t launch_wx_digits(cudaStream_t st, const double* W, const TileGeom& G, size_t ng,
                              int n_tiles, const int* tptr, const int* tlist, const int* tsub,
-                             void* wxbuf);
+                             void* wxbuf, int digits);
 cudaError_t launch_expand_tc(cudaStream_t st, int device, const void* wxbuf, const TileGeom& G,
                              size_t ng, int n_tiles, const int* tptr, const int* tlist,
                              const double* H, long long hj, long long hv, int m, bool negate,
-                             double* out, int* evbuf, int* queue, unsigned* status);
+                             double* out, int* evbuf, int* queue, unsigned* status, int digits);
 int expand_tc_max_list();
 cudaError_t launch_gram_tc(cudaStream_t st, int device, const double* A, int m, const TileGeom& G,
                            size_t ng, int n_tiles, const int* tptr, long long slots,
-                           const void* wbuf, double* partial, int* queue, unsigned* status);
+                           const void* wbuf, double* partial, int* queue, unsigned* status,
+                           int digits);
 cudaError_t launch_ace_lists(sea_ctx* c, cudaStream_t st);
 cudaError_t launch_ace_build(sea_ctx* c);
 cudaError_t launch_ace_eigen(sea_ctx* c);
