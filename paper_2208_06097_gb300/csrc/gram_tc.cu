@@ -237,13 +237,24 @@ __device__ __forceinline__ int float_int(float f) {
 
 
 // Seven diagonal sums (integer-valued floats, |D_0|, |D_1| < 2^22, the others
-// below 2^24) as sum_d D_d 256^(6-d) 2^e0, rounded to nearest.
+// below 2^24) as y = sum_d D_d 256^(6-d) 2^e0, |y| < 2^(e0 + 62 + DROP): the
+// sum's lowest DROP bits truncated so that 64 bits hold it, one rounding to
+// nearest (the conversion instruction, on the FP64 pipe that the integer
+// epilogues leave idle), the scaling added to the exponent field.
+template <int DROP>
 __device__ __forceinline__ double combine7(const uint32_t* f, int e0) {
-  auto big = [](uint32_t x) { return (long long)__float2int_rz(__uint_as_float(x)); };
-  const long long hi = ((long long)small_float_int(f[0]) << 20) +
-                       ((long long)small_float_int(f[1]) << 12) + (big(f[2]) << 4);
-  const long long lo = (big(f[3]) << 24) + (big(f[4]) << 16) + (big(f[5]) << 8) + big(f[6]);
-  return fix_to_double(hi, lo, e0);
+  auto big = [](uint32_t x) { return __float2int_rz(__uint_as_float(x)); };
+  const long long hi = (long long)(small_float_int(f[0]) * 256 + small_float_int(f[1])) * 4096 +
+                       (long long)big(f[2]) * 16;
+  const long long lo = (long long)big(f[3]) * 16777216 + (long long)big(f[4]) * 65536 +
+                       (long long)big(f[5]) * 256 + (long long)big(f[6]);
+  const long long v = (hi << (28 - DROP)) + (lo >> DROP);
+  const int e2 = e0 + DROP;
+  const long long b = __double_as_longlong(__ll2double_rn(v));
+  const int ex = (int)((b >> 52) & 0x7FF) + e2;  // biased exponent of the result
+  if (v == 0 || ex <= 0) return 0.0;
+  if (ex >= 0x7FF) return __longlong_as_double((b & (1LL << 63)) | 0x7FF0000000000000LL);
+  return __longlong_as_double(b + ((long long)e2 << 52));
 }
 __device__ __forceinline__ double quiet_nan() { return __longlong_as_double(0x7FF8000000000000LL); }
 constexpr int EXP_NONFINITE = 0x7FF;
@@ -413,7 +424,7 @@ __global__ void __launch_bounds__(GT_THREADS, 1)
         const int ea = h ? ea1 : ea0, ew = Wexp[u.wb][h][c];
         if constexpr (DIG == 7) {
           const bool bad = ea + 1022 == EXP_NONFINITE || ew == EXP_NONFINITE;
-          sum += bad ? quiet_nan() : combine7(f + h * DIG, ea + ew - 1022 - 62);
+          sum += bad ? quiet_nan() : combine7<6>(f + h * DIG, ea + ew - 1022 - 62);
         } else {
           long long acc = 0;
 #pragma unroll
@@ -927,7 +938,7 @@ __global__ void __launch_bounds__(GT2_THREADS, 1)
             for (int cc = 0; cc < 2; ++cc) {
               const int ew = Wexp[u.wb][h][min(c0 + cc, NBLK - 1)];
               const bool bad = ea + 1022 == EXP_NONFINITE || ew == EXP_NONFINITE;
-              y[cc] += bad ? quiet_nan() : combine7(f[cc], ea + ew - 1022 - 63);
+              y[cc] += bad ? quiet_nan() : combine7<7>(f[cc], ea + ew - 1022 - 63);
             }
           }
 #pragma unroll
@@ -1541,7 +1552,7 @@ __global__ void __launch_bounds__(XE_THREADS, 1)
 #pragma unroll
               for (int d = 0; d < DIG; ++d) fd[d] = f[d][u];
               const int e = ev[4 * hh + u];
-              val = e >= EV_NONFINITE ? quiet_nan() : combine7(fd, e - 1022 - 63);
+              val = e >= EV_NONFINITE ? quiet_nan() : combine7<6>(fd, e - 1022 - 63);
             } else {
               // sum_d D_d 256^(5 - d) in three 32-bit pairs; |D_d| < 2^22 except
               // D_4 and D_5 of lists longer than 16 (below 2^23): those by the
