@@ -7,8 +7,9 @@
 //   v_ij phi_i on Omega_ii (v_ji = v_ij).
 // v_ij is the CG solution inside Omega_ij and the multipole expansion
 // (Eq. me) outside it.
-//   k_contrib   (grid over entries x chunks): c = v * phi_partner on the
-//               entry's window, stored per entry; no accumulation here.
+//   k_far, k_near (grid over entries x chunks): c = v * phi_partner on the
+//               entry's window outside and inside the pair box, stored per
+//               entry; no accumulation here.
 //   k_accumulate (CTA per orbital x z-plane): the plane is built in
 //               shared memory from zero, each entry of the orbital
 //               subtracted in pair order (a fixed order: no floating-point
@@ -18,6 +19,8 @@
 //               touch).  Planes too large for shared memory take the same
 //               steps on a global slab, with full stores.
 #include <algorithm>
+#include <cmath>
+#include <type_traits>
 
 #include "sea_internal.cuh"
 
@@ -153,40 +156,196 @@ __global__ void k_entry_offsets(const Entry* __restrict__ ent, const int* __rest
   }
 }
 
-// Window contributions of the entries (grid y) in chunks of SEA_CHUNK window
-// points (grid x); `part` as in contrib_range (1: the far field on a side
-// stream beside the CG, 2: the points inside the pair boxes after it).  DFM: double-float arithmetic (mixed form),
-// four CTAs per SM there (64 registers, no spills): the nested Horner steps
-// of the potential are one dependent chain per point, so the warps resident
-// per SM set the rate (measured 0.81 -> 0.77 ms per step against two CTAs).
+// Window contributions c = v phi_partner (Eq. tDxx) of the entries (grid y),
+// window-compact output out[t], t = (tz wy + ty) wx + tx.  Two kernels: the
+// points outside the pair boxes need the moments alone (on a side stream
+// beside the CG), the points inside need the CG's solution.  DFM:
+// double-float arithmetic (mixed form), else FP64.
+
+// Outside: a thread per `seg` points of a line along x (me_line), whole lines
+// where there are enough of them.  Bound by the FP64 unit (plain form) or
+// FP32 issue (double-float), not by its 16 bytes a point in L2.  256 orbitals
+// on 96^3, 4.9 million points: FP64 1.39 -> 0.50 ms, double-float 0.315 ->
+// 0.16 ms against the full Horner form at every point.
+#define FAR_T 128
 template <bool DFM>
-__global__ void __launch_bounds__(256, DFM ? 4 : 1)
-    k_contrib(const double* __restrict__ phi, int nx, int ny, int nz, const Entry* __restrict__ ent,
-              const long long* __restrict__ coff, const PairInfo* __restrict__ pinfo,
-              const long long* __restrict__ voff, const double* __restrict__ vbuf,
-              const double* __restrict__ Qg, double hx, double hy, double hz,
-              double* __restrict__ cbuf, int part) {
+__global__ void __launch_bounds__(FAR_T, 4)
+    k_far(const double* __restrict__ phi, int nx, int ny, int nz, const Entry* __restrict__ ent,
+          const long long* __restrict__ coff, const PairInfo* __restrict__ pinfo,
+          const double* __restrict__ Qg, double hx, double hy, double hz, int seg,
+          double* __restrict__ cbuf) {
+  typedef typename std::conditional<DFM, MeDF, MeF64>::type R;
+  typedef typename R::T T;
   const Entry e = ent[blockIdx.y];
   const PairInfo P = pinfo[e.pair];
-  const int nw = e.wl[0] * e.wl[1] * e.wl[2];
   const WinSplit sp = window_split(e, P);
-  // parts 1 and 2 enumerate their own points (divisions exact below 2^24)
-  const bool compact = part != 0 && nw < (1 << 24);
-  const int cnt = !compact ? nw : part == 1 ? sp.n_out : sp.n_in;
-  const int t0 = blockIdx.x * SEA_CHUNK;
-  if (t0 >= cnt) return;
-  __shared__ double Ps[SEA_NMONO];
-  __shared__ DF Pd[SEA_NMONO];
-  if (part != 2 && threadIdx.x < SEA_NMONO) {
+  const WinLines nl = window_lines(sp, e.wl);
+  const int nseg = (e.wl[0] + seg - 1) / seg;
+  const int items = (nl.n_whole + nl.n_cut) * nseg;
+  if ((int)blockIdx.x * FAR_T >= items) return;
+  __shared__ T Ps[SEA_NMONO];
+  if (threadIdx.x < SEA_NMONO) {
     const double q = Qg[(size_t)e.pair * SEA_QSTRIDE + SEA_NQ + threadIdx.x];
-    if (DFM)
-      Pd[threadIdx.x] = df_from_double(q);
+    if constexpr (DFM)
+      Ps[threadIdx.x] = df_from_double(q);
     else
       Ps[threadIdx.x] = q;
   }
   __syncthreads();
-  contrib_range<DFM>(part, compact, sp, e, P, phi, nx, ny, nz, vbuf + voff[e.pair], Pd, Ps, hx, hy,
-                     hz, cbuf + coff[blockIdx.y], t0, min(cnt, t0 + SEA_CHUNK));
+  // (k - (ext - 1) / 2) h for a box coordinate k
+  auto coord = [](int k, int ext, double h) -> T {
+    if constexpr (DFM)
+      return df_mul_f(i2f_exact(k) - 0.5f * i2f_exact(ext - 1), df_from_double(h));
+    else
+      return (k - 0.5 * (ext - 1)) * h;
+  };
+  const double* fp = phi + (size_t)e.partner * ((size_t)nx * ny * nz);
+  double* out = cbuf + coff[blockIdx.y];
+  const int gx0 = wrapi(e.ws[0], nx), gy0 = wrapi(e.ws[1], ny), gz0 = wrapi(e.ws[2], nz);
+  const int lx0 = e.ws[0] - P.lo[0];
+  for (int it = blockIdx.x * FAR_T + threadIdx.x; it < items; it += gridDim.x * FAR_T) {
+    const int i = it / nseg, x0 = (it - i * nseg) * seg, x1 = min(e.wl[0], x0 + seg);
+    asm volatile("" ::: "memory");  // P is read anew for each line, not kept in 168 registers
+    int ty, tz;
+    window_outside_line(sp, e.wl, i, &ty, &tz);
+    const T y = coord(e.ws[1] + ty - P.lo[1], P.ext[1], hy);
+    const T z = coord(e.ws[2] + tz - P.lo[2], P.ext[2], hz);
+    T c[ME_LINE];
+    me_line<R, 0>(Ps, y, z, c);
+    const T q = R::fma_(z, z, R::mul(y, y));
+    int gy = gy0 + ty, gz = gz0 + tz;  // window lengths are at most n
+    gy -= gy >= ny ? ny : 0;
+    gz -= gz >= nz ? nz : 0;
+    const double* frow = fp + ((size_t)gz * ny + gy) * nx;
+    double* orow = out + (size_t)(tz * e.wl[1] + ty) * e.wl[0];
+    const bool cut = i >= nl.n_whole;
+    for (int tx = cut && x0 >= sp.b0[0] && x0 < sp.b1[0] ? sp.b1[0] : x0; tx < x1;) {
+      int gx = gx0 + tx;
+      gx -= gx >= nx ? nx : 0;
+      const double f = frow[gx];
+      const T v = me_line_at<R>(c, coord(lx0 + tx, P.ext[0], hx), q);
+      if constexpr (DFM) {
+        const float2 fs = split64(f);
+        orow[tx] = df_to_double(df_mul(v, DF{fs.x, fs.y}));
+      } else {
+        orow[tx] = __dmul_rn(v, f);
+      }
+      ++tx;
+      if (cut && tx == sp.b0[0]) tx = sp.b1[0];
+    }
+  }
+}
+
+// Inside: v is the pair's CG solution (box layout).  The loop is bound by the
+// latency of its two loads per point, so each thread takes NEAR_U points with
+// all their loads issued before the first product; chunks of NEAR_CHUNK box
+// points (grid x).
+#define NEAR_CHUNK 1024
+template <bool DFM>
+__global__ void __launch_bounds__(256)
+    k_near(const double* __restrict__ phi, int nx, int ny, int nz, const Entry* __restrict__ ent,
+           const long long* __restrict__ coff, const PairInfo* __restrict__ pinfo,
+           const long long* __restrict__ voff, const double* __restrict__ vbuf,
+           double* __restrict__ cbuf) {
+  constexpr int NEAR_U = 4;
+  const Entry e = ent[blockIdx.y];
+  const PairInfo P = pinfo[e.pair];
+  const WinSplit sp = window_split(e, P);
+  const int t0 = blockIdx.x * NEAR_CHUNK;
+  if (t0 >= sp.n_in) return;
+  const int t1 = min(sp.n_in, t0 + NEAR_CHUNK);
+  const double* v = vbuf + voff[e.pair];
+  const double* fp = phi + (size_t)e.partner * ((size_t)nx * ny * nz);
+  double* out = cbuf + coff[blockIdx.y];
+  const int wx = e.wl[0], wy = e.wl[1], S = blockDim.x;
+  const int gx0 = wrapi(e.ws[0], nx), gy0 = wrapi(e.ws[1], ny), gz0 = wrapi(e.ws[2], nz);
+  const int bx = sp.b1[0] - sp.b0[0], by = sp.b1[1] - sp.b0[1], bxy = bx * by;
+  // (kx, ky, kz) in the box within the window, advanced by the CTA stride
+  // without divisions
+  const int dz = S / bxy, dy = (S - dz * bxy) / bx, dx = S - dz * bxy - dy * bx;
+  int kz = (t0 + (int)threadIdx.x) / bxy;
+  int ky = (t0 + (int)threadIdx.x - kz * bxy) / bx;
+  int kx = t0 + (int)threadIdx.x - kz * bxy - ky * bx;
+  const int l0 = e.ws[0] - P.lo[0], l1 = e.ws[1] - P.lo[1], l2 = e.ws[2] - P.lo[2];
+  for (int t = t0 + threadIdx.x; t < t1; t += NEAR_U * S) {
+    int lq[NEAR_U], tq[NEAR_U];
+    size_t gq[NEAR_U];
+#pragma unroll
+    for (int u = 0; u < NEAR_U; ++u) {
+      const int tx = sp.b0[0] + kx, ty = sp.b0[1] + ky, tz = sp.b0[2] + kz;
+      kx += dx;
+      ky += dy;
+      kz += dz;
+      if (kx >= bx) {
+        kx -= bx;
+        ++ky;
+      }
+      if (ky >= by) {
+        ky -= by;
+        ++kz;
+      }
+      int gx = gx0 + tx, gy = gy0 + ty, gz = gz0 + tz;
+      gx -= gx >= nx ? nx : 0;
+      gy -= gy >= ny ? ny : 0;
+      gz -= gz >= nz ? nz : 0;
+      gq[u] = ((size_t)gz * ny + gy) * nx + gx;
+      tq[u] = (tz * wy + ty) * wx + tx;
+      lq[u] = ((l2 + tz) * P.ext[1] + (l1 + ty)) * P.ext[0] + (l0 + tx);
+    }
+    double vq[NEAR_U], fq[NEAR_U];
+#pragma unroll
+    for (int u = 0; u < NEAR_U; ++u)
+      if (t + u * S < t1) {
+        vq[u] = v[lq[u]];
+        fq[u] = fp[gq[u]];
+      }
+#pragma unroll
+    for (int u = 0; u < NEAR_U; ++u)
+      if (t + u * S < t1) {
+        if (DFM) {
+          const float2 s = split64(vq[u]), f = split64(fq[u]);
+          out[tq[u]] = df_to_double(df_mul(DF{s.x, s.y}, DF{f.x, f.y}));
+        } else {
+          out[tq[u]] = __dmul_rn(vq[u], fq[u]);
+        }
+      }
+  }
+}
+
+// The far field of entries [e_begin, e_end) on stream st, and the points
+// inside the boxes on the context stream.
+static cudaError_t launch_far(sea_ctx* c, int e_begin, int e_end, cudaStream_t st) {
+  // points per thread: a line's 112 operations are spread over as many
+  // points as leave every SM three times 256 threads, eight at least
+  int nsm = 0;
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device);
+  const int seg = (int)std::min<long long>(1024, std::max<long long>(8, c->WC / (768LL * nsm)));
+  // CTAs for the largest window taken as a cube; others loop
+  const int most = (int)std::min<long long>(c->max_window, 1LL << 20);
+  const int edge = std::max(1, (int)std::cbrt((double)most));
+  const unsigned gx =
+      (unsigned)std::max(1, (most / edge * ((edge + seg - 1) / seg) + FAR_T - 1) / FAR_T);
+  for (int e0 = e_begin; e0 < e_end; e0 += 65535) {
+    const int ne = std::min(65535, e_end - e0);
+    (c->prm.precision == 1 ? k_far<true> : k_far<false>)<<<dim3(gx, ne), FAR_T, 0, st>>>(
+        (const double*)c->phi.p, c->N[0], c->N[1], c->N[2], (const Entry*)c->ewin.p + e0,
+        (const long long*)c->coff.p + e0, (const PairInfo*)c->pinfo.p, (const double*)c->Q.p, c->h[0],
+        c->h[1], c->h[2], seg, (double*)c->cbuf.p);
+    c->launches += 1;
+  }
+  return cudaGetLastError();
+}
+static cudaError_t launch_near(sea_ctx* c, int e_begin, int e_end) {
+  const unsigned gx = (unsigned)((c->max_window + NEAR_CHUNK - 1) / NEAR_CHUNK);
+  for (int e0 = e_begin; e0 < e_end; e0 += 65535) {
+    const int ne = std::min(65535, e_end - e0);
+    (c->prm.precision == 1 ? k_near<true> : k_near<false>)<<<dim3(gx, ne), 256, 0, c->stream>>>(
+        (const double*)c->phi.p, c->N[0], c->N[1], c->N[2], (const Entry*)c->ewin.p + e0,
+        (const long long*)c->coff.p + e0, (const PairInfo*)c->pinfo.p,
+        (const long long*)c->voff.p, (const double*)c->vbuf.p, (double*)c->cbuf.p);
+    c->launches += 1;
+  }
+  return cudaGetLastError();
 }
 
 // Global-memory form: CTA per (orbital, slab of SLAB z-planes); out2, when
@@ -444,17 +603,9 @@ cudaError_t launch_entries(sea_ctx* c) {
 cudaError_t launch_accumulate_range(sea_ctx* c, double* out, int o_begin, int o_end, int e_begin,
                                     int e_end, double* out2) {
   if (e_end > e_begin) {
-    const int chunks = (int)((c->max_window + SEA_CHUNK - 1) / SEA_CHUNK);
-    for (int e0 = e_begin; e0 < e_end; e0 += 65535) {
-      const int ne = std::min(65535, e_end - e0);
-      auto kern = c->prm.precision == 1 ? k_contrib<true> : k_contrib<false>;
-      kern<<<dim3(chunks, ne), 256, 0, c->stream>>>(
-          (const double*)c->phi.p, c->N[0], c->N[1], c->N[2], (const Entry*)c->ewin.p + e0,
-          (const long long*)c->coff.p + e0, (const PairInfo*)c->pinfo.p,
-          (const long long*)c->voff.p, (const double*)c->vbuf.p, (const double*)c->Q.p, c->h[0],
-          c->h[1], c->h[2], (double*)c->cbuf.p, c->far_side ? 2 : 0);
-      c->launches += 1;
-    }
+    cudaError_t e = c->far_side ? cudaSuccess : launch_far(c, e_begin, e_end, c->stream);
+    if (e == cudaSuccess) e = launch_near(c, e_begin, e_end);
+    if (e != cudaSuccess) return e;
   }
   if (o_end > o_begin) {
     if (c->far_side) {  // the contributions outside the pair boxes are in
@@ -491,26 +642,16 @@ cudaError_t launch_accumulate_range(sea_ctx* c, double* out, int o_begin, int o_
 // the context's first copy stream, beside the CG: submitted after the CG's
 // launch, whose persistent CTAs fill the GPU, they take the SMs that the CG's
 // last pairs leave idle.  The accumulation later forms the points inside
-// the boxes and waits for this launch.  Mixed form only.
+// the boxes and waits for this launch.
 cudaError_t launch_contrib_far(sea_ctx* c, cudaEvent_t setup_done) {
   c->far_side = false;
-  if (c->prm.precision != 1 || c->E == 0) return cudaSuccess;
+  if (c->E == 0) return cudaSuccess;
   cudaError_t e = cudaStreamWaitEvent(c->xfer[0], setup_done, 0);
-  if (e != cudaSuccess) return e;
-  const int chunks = (int)((c->max_window + SEA_CHUNK - 1) / SEA_CHUNK);
-  for (int e0 = 0; e0 < c->E; e0 += 65535) {
-    const int ne = std::min(65535, c->E - e0);
-    k_contrib<true><<<dim3(chunks, ne), 256, 0, c->xfer[0]>>>(
-        (const double*)c->phi.p, c->N[0], c->N[1], c->N[2], (const Entry*)c->ewin.p + e0,
-        (const long long*)c->coff.p + e0, (const PairInfo*)c->pinfo.p,
-        (const long long*)c->voff.p, (const double*)c->vbuf.p, (const double*)c->Q.p, c->h[0],
-        c->h[1], c->h[2], (double*)c->cbuf.p, 1);
-    c->launches += 1;
-  }
-  e = cudaEventRecord(c->xev[1], c->xfer[0]);
+  if (e == cudaSuccess) e = launch_far(c, 0, c->E, c->xfer[0]);
+  if (e == cudaSuccess) e = cudaEventRecord(c->xev[1], c->xfer[0]);
   if (e != cudaSuccess) return e;
   c->far_side = true;
-  return cudaGetLastError();
+  return cudaSuccess;
 }
 
 // E_xx and the CG statistics (after every pair energy is final), on
@@ -527,7 +668,5 @@ cudaError_t launch_accumulate(sea_ctx* c, double* out, double* out2, bool with_e
   cudaError_t e = launch_accumulate_range(c, out, 0, c->n_orb, 0, c->E, out2);
   return e != cudaSuccess || !with_exx ? e : launch_exx(c, c->stream);
 }
-
-cudaError_t upload_harmonics_accum() { return upload_harmonics_here(); }
 
 }  // namespace sea

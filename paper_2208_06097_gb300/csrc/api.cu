@@ -54,12 +54,6 @@ HarmCoef make_harmonic_coefficients() {
                                  ((double)(l + m + 1) * (double)(l - m + 1)));
       h.gam[l][m + SEA_LMAX] = c * sig[l - 1][m + SEA_LMAX] / sig[l + 1][m + SEA_LMAX];
     }
-  for (int l = 0; l < SEA_LMAX; ++l)
-    for (int k = 0; k < 2 * SEA_LMAX + 1; ++k) {
-      const float hi = (float)h.gam[l][k];
-      h.gam_hi[l][k] = hi;
-      h.gam_lo[l][k] = (float)(h.gam[l][k] - (double)hi);
-    }
   // D_lm as polynomials: coefficient arrays P[a][b][c] of x^a y^b z^c, the
   // recurrence applied to them (multiplication by x, y, z, r^2 shifts them)
   constexpr int E = SEA_LMAX + 1;
@@ -302,7 +296,7 @@ sea_status sea_create(const double cell[3], const int grid[3], const sea_params*
     for (int k = 0; k <= SEA_FDP; ++k) c->w_ax[a][k] = -w[k] * ih2;
     c->w_center += -w[0] * ih2;
   }
-  if (sea::upload_harmonics_pair() != cudaSuccess || sea::upload_harmonics_accum() != cudaSuccess) {
+  if (sea::upload_harmonics_pair() != cudaSuccess) {
     delete c;
     return SEA_ERR_CUDA;
   }

@@ -12,7 +12,9 @@
 //   the 37-point O(h^12) operator written as 37 fused multiply-adds (on this
 //   part the FP64 FMA pipe issues faster than FP64 add); then the pair
 //   integral sum rho v dV of Eq. exxGen_mlwf.
+#include <cmath>
 #include <cstring>
+#include <type_traits>
 
 #include "cg_fixed.cuh"
 #include "sea_internal.cuh"
@@ -159,18 +161,29 @@ __global__ void __launch_bounds__(256)
 #pragma unroll
       for (int a = 0; a < MOM_E; ++a) s[a] = R::zero();
       int gx = gx0;
-      for (int x = 0; x < ex; ++x) {
-        const double av = fi[rowg + gx], cv = fj[rowg + gx];
-        brow[x] = fourpi * (av * cv);
-        T pk = R::prod(av, cv);
-        const int u = 2 * x - (ex - 1);
-        s[0] = R::add(s[0], pk);
+      for (int x0 = 0; x0 < ex; x0 += 4) {  // four points' loads in flight
+        double av[4], cv[4];
 #pragma unroll
-        for (int a = 1; a < MOM_E; ++a) {
-          pk = R::mul_i(pk, u);
-          s[a] = R::add(s[a], pk);
+        for (int q = 0; q < 4; ++q) {
+          const bool in = x0 + q < ex;
+          av[q] = in ? fi[rowg + gx] : 0.0;
+          cv[q] = in ? fj[rowg + gx] : 0.0;
+          if (++gx == nx) gx = 0;
         }
-        if (++gx == nx) gx = 0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int x = x0 + q;
+          if (x >= ex) break;
+          brow[x] = fourpi * (av[q] * cv[q]);
+          T pk = R::prod(av[q], cv[q]);
+          const int u = 2 * x - (ex - 1);
+          s[0] = R::add(s[0], pk);
+#pragma unroll
+          for (int a = 1; a < MOM_E; ++a) {
+            pk = R::mul_i(pk, u);
+            s[a] = R::add(s[a], pk);
+          }
+        }
       }
 #pragma unroll
       for (int a = 0; a < MOM_E; ++a) S[(size_t)r * MOM_E + a] = s[a];
@@ -231,9 +244,8 @@ __global__ void __launch_bounds__(256)
 // the ghost values of every line across the axis (one evaluation per
 // thread) into a global buffer, per pair at 36 voff (12 values per line;
 // the three faces, each at most the box's volume, fit in 36 times it).
-// k_boundary_apply (a CTA per pair): one thread per (line, boundary point)
-// adds the weighted ghost values into b, the axes one after the other, so
-// every b entry is updated in a fixed order.
+// k_boundary_apply adds the weighted ghost values into b, the axes one after
+// the other, so every b entry is updated in a fixed order.
 // The stencil's right-hand-side weights as double-float pairs (mixed form).
 struct StencilWd {
   float hi[3][SEA_FDP + 1], lo[3][SEA_FDP + 1];
@@ -250,105 +262,155 @@ __device__ __forceinline__ void ghost_face(int a, int ex, int ey, int ez, int* e
   *goff = 2 * SEA_FDP * (a == 0 ? 0 : (a == 1 ? ey * ez : ey * ez + ex * ez));
 }
 
-// DFM: the potentials in double-float arithmetic (mixed form; four CTAs per
-// SM, the nested Horner steps being one dependent chain per point).
+// A thread per line (me_line) and its NG ghost points in turn, or with halves =
+// 2 a thread per line and side (a third more arithmetic; for launches that
+// would leave SMs with less than eight warps).  DFM: double-float arithmetic
+// (mixed form), else FP64.
+#define GHOST_T 128
+template <bool DFM, int AX>
+__device__ __forceinline__ void ghost_lines(
+    const typename std::conditional<DFM, DF, double>::type* P, int ex, int ey, int ez,
+    double hx, double hy, double hz, int halves, double* __restrict__ G0) {
+  typedef typename std::conditional<DFM, MeDF, MeF64>::type R;
+  typedef typename R::T T;
+  constexpr int NG = 2 * SEA_FDP;  // ghost values per line: d = 1..FDP below, then above
+  int e1, e2, ea, sa, goff;
+  ghost_face(AX, ex, ey, ez, &e1, &e2, &ea, &sa, &goff);
+  const double h1 = AX == 0 ? hy : hx, h2 = AX == 2 ? hy : hz, ha = AX == 0 ? hx : AX == 1 ? hy : hz;
+  // (k - (ext - 1) / 2) h: half-integers, exact in FP32 and FP64
+  auto coord = [](int k, int ext, double h) -> T {
+    if constexpr (DFM)
+      return df_mul_f(i2f_exact(k) - 0.5f * i2f_exact(ext - 1), df_from_double(h));
+    else
+      return (k - 0.5 * (ext - 1)) * h;
+  };
+  T* G = reinterpret_cast<T*>(G0 + goff);
+  const int per = NG / halves;
+  for (int it = threadIdx.x; it < e1 * e2 * halves; it += blockDim.x) {
+    const int line = halves == 2 ? it >> 1 : it, k0 = halves == 2 ? (it & 1) * per : 0;
+    asm volatile("" ::: "memory");  // P is read anew for each line, not kept in 168 registers
+    int u1;
+    const int u2 = divmod_small(line, e1, &u1);
+    const T s = coord(u1, e1, h1), t = coord(u2, e2, h2);
+    T c[ME_LINE];
+    me_line<R, AX>(P, s, t, c);
+    const T q = R::fma_(s, s, R::mul(t, t));
+#pragma unroll 1
+    for (int k = k0; k < k0 + per; ++k)
+      G[(size_t)line * NG + k] =
+          me_line_at<R>(c, coord(k < SEA_FDP ? -(k + 1) : ea + k - SEA_FDP, ea, ha), q);
+  }
+}
+
 template <bool DFM>
-__global__ void __launch_bounds__(256, DFM ? 4 : 1)
+__global__ void __launch_bounds__(GHOST_T, 4)
     k_ghost_eval(const PairInfo* __restrict__ pinfo, const long long* __restrict__ voff,
-                 double hx, double hy, double hz, const double* __restrict__ Qg,
+                 double hx, double hy, double hz, const double* __restrict__ Qg, int halves,
                  double* __restrict__ gbuf, const int* __restrict__ order) {
-  const int a = blockIdx.x;
+  typedef typename std::conditional<DFM, DF, double>::type T;
   const int p = order[blockIdx.y];  // the largest pairs first: the small ones fill the tail
   const PairInfo P = pinfo[p];
-  const int ex = P.ext[0], ey = P.ext[1], ez = P.ext[2];
-  __shared__ double Ps[SEA_NMONO];
-  __shared__ DF Pd[SEA_NMONO];
+  __shared__ T Ps[SEA_NMONO];
   if (threadIdx.x < SEA_NMONO) {
     const double q = Qg[(size_t)p * SEA_QSTRIDE + SEA_NQ + threadIdx.x];
-    if (DFM)
-      Pd[threadIdx.x] = df_from_double(q);
+    if constexpr (DFM)
+      Ps[threadIdx.x] = df_from_double(q);
     else
       Ps[threadIdx.x] = q;
   }
   __syncthreads();
-  // the potential at grid offsets (ox, oy, oz) from the box centre, in
-  // units of h (half-integers, exact in FP32)
-  const DF Hx = df_from_double(hx), Hy = df_from_double(hy), Hz = df_from_double(hz);
-  const float cx = 0.5f * i2f_exact(ex - 1), cy = 0.5f * i2f_exact(ey - 1),
-              cz = 0.5f * i2f_exact(ez - 1);
-  constexpr int NG = 2 * SEA_FDP;  // ghost values per line: d = 1..FDP below, then above
-  int e1, e2, ea, sa, goff;
-  ghost_face(a, ex, ey, ez, &e1, &e2, &ea, &sa, &goff);
-  const float ca = a == 0 ? cx : (a == 1 ? cy : cz);
-  double* G = gbuf + 36 * voff[p] + goff;
-  const int nl = e1 * e2;
-  for (int e = threadIdx.x; e < nl * NG; e += blockDim.x) {
-    const int line = e / NG, k = e % NG;
-    const int u1 = line % e1, u2 = line / e1;
-    const float o1 = i2f_exact(u1) - (a == 0 ? cy : cx), o2 = i2f_exact(u2) - (a == 2 ? cy : cz);
-    const int d = k % SEA_FDP + 1;
-    const float t = i2f_exact(k < SEA_FDP ? -d : ea - 1 + d) - ca;
-    const float ox = a == 0 ? t : o1, oy = a == 0 ? o1 : (a == 1 ? t : o2);
-    const float oz = a == 2 ? t : o2;
-    if (DFM) {
-      const DF g = me_potential_cart_df(Pd, df_mul_f(ox, Hx), df_mul_f(oy, Hy), df_mul_f(oz, Hz));
-      reinterpret_cast<DF*>(G)[e] = g;
-    } else {
-      G[e] = me_potential_cart(Ps, (double)ox * hx, (double)oy * hy, (double)oz * hz);
-    }
-  }
+  double* G = gbuf + 36 * voff[p];
+  if (blockIdx.x == 0)
+    ghost_lines<DFM, 0>(Ps, P.ext[0], P.ext[1], P.ext[2], hx, hy, hz, halves, G);
+  else if (blockIdx.x == 1)
+    ghost_lines<DFM, 1>(Ps, P.ext[0], P.ext[1], P.ext[2], hx, hy, hz, halves, G);
+  else
+    ghost_lines<DFM, 2>(Ps, P.ext[0], P.ext[1], P.ext[2], hx, hy, hz, halves, G);
 }
 
+// Walks the points t = t0, t0 + S, t0 + 2S, ... of an ex x ey x ez box in
+// [z][y][x] order with their coordinates, without divisions in the loop.
+struct BoxWalk {
+  int t, x, y, z, dx, dy, dz, ex, ey;
+  __device__ BoxWalk(int t0, int S, int ex_, int ey_) : ex(ex_), ey(ey_) {
+    t = t0;
+    x = t0 % ex;
+    y = (t0 / ex) % ey;
+    z = t0 / (ex * ey);
+    dx = S % ex;
+    dy = (S / ex) % ey;
+    dz = S / (ex * ey);
+  }
+  __device__ __forceinline__ void next(int S) {
+    t += S;
+    x += dx;
+    int cy = 0;
+    if (x >= ex) {
+      x -= ex;
+      cy = 1;
+    }
+    y += dy + cy;
+    int cz = 0;
+    if (y >= ey) {
+      y -= ey;
+      cz = 1;
+    }
+    z += dz + cz;
+  }
+};
+
+// The weighted ghost values of axis a that the stencil reaches from
+// coordinate ta of a line (G: its NG ghost values), extent ea, in a fixed order.
+template <bool DFM>
+__device__ __forceinline__ double ghost_sum(const StencilW& W, const StencilWd& Wd, int a, int ta,
+                                            int ea, const double* __restrict__ Gl) {
+  if (DFM) {
+    const DF* G = reinterpret_cast<const DF*>(Gl);
+    DF add{0.f, 0.f};
+#pragma unroll
+    for (int k = 1; k <= SEA_FDP; ++k) {
+      const DF w{Wd.hi[a][k], Wd.lo[a][k]};
+      if (ta - k < 0) add = df_add(add, df_mul(w, G[k - ta - 1]));
+      if (ta + k > ea - 1) add = df_add(add, df_mul(w, G[SEA_FDP + ta + k - (ea - 1) - 1]));
+    }
+    return df_to_double(add);
+  }
+  double add = 0.0;
+#pragma unroll
+  for (int k = 1; k <= SEA_FDP; ++k) {
+    if (ta - k < 0) add += W.rhs[a][k] * Gl[k - ta - 1];
+    if (ta + k > ea - 1) add += W.rhs[a][k] * Gl[SEA_FDP + ta + k - (ea - 1) - 1];
+  }
+  return add;
+}
+
+// b += the three axes' weighted ghost values, a thread per box point (nearly
+// every point of a box lies within six of a face), the axes one after the
+// other; BND_CTAS CTAs share a pair, so that a few pairs still fill the GPU.
+#define BND_CTAS 4
 template <bool DFM>
 __global__ void __launch_bounds__(256)
     k_boundary_apply(const PairInfo* __restrict__ pinfo, const long long* __restrict__ voff,
                      StencilW W, StencilWd Wd, const double* __restrict__ gbuf,
                      double* __restrict__ bbuf, const int* __restrict__ order) {
-  const int p = order[blockIdx.x];
+  const int p = order[blockIdx.y];
   const PairInfo P = pinfo[p];
   const int ex = P.ext[0], ey = P.ext[1], ez = P.ext[2];
   double* b = bbuf + voff[p];
   constexpr int NG = 2 * SEA_FDP;
-  for (int a = 0; a < 3; ++a) {
-    int e1, e2, ea, sa, goff;
-    ghost_face(a, ex, ey, ez, &e1, &e2, &ea, &sa, &goff);
-    const double* Gp = gbuf + 36 * voff[p] + goff;
-    const int nl = e1 * e2;
-    const int nbp = min(ea, NG);  // points of a line within FDP of either end
-    // thread per (line, boundary point); the terms of each point in a fixed
-    // order, the axes one after the other
-    for (int e = threadIdx.x; e < nl * nbp; e += blockDim.x) {
-      const int line = e / nbp, idx = e % nbp;
-      const int ta = ea <= NG ? idx : (idx < SEA_FDP ? idx : ea - NG + idx);
-      const int u1 = line % e1, u2 = line / e1;
-      int bx = 0, by = 0, bz = 0;
-      if (a == 0) { by = u1; bz = u2; }
-      else if (a == 1) { bx = u1; bz = u2; }
-      else { bx = u1; by = u2; }
-      const int base = (bz * ey + by) * ex + bx;
-      // ghost value d below: entry d - 1; above: entry FDP + d - 1
-      if (DFM) {
-        const DF* G = reinterpret_cast<const DF*>(Gp) + (size_t)line * NG;
-        DF add{0.f, 0.f};
-#pragma unroll
-        for (int k = 1; k <= SEA_FDP; ++k) {
-          const DF w{Wd.hi[a][k], Wd.lo[a][k]};
-          if (ta - k < 0) add = df_add(add, df_mul(w, G[k - ta - 1]));
-          if (ta + k > ea - 1) add = df_add(add, df_mul(w, G[SEA_FDP + ta + k - (ea - 1) - 1]));
-        }
-        b[base + ta * sa] += df_to_double(add);
-      } else {
-        const double* G = Gp + (size_t)line * NG;
-        double add = 0.0;
-#pragma unroll
-        for (int k = 1; k <= SEA_FDP; ++k) {
-          if (ta - k < 0) add += W.rhs[a][k] * G[k - ta - 1];
-          if (ta + k > ea - 1) add += W.rhs[a][k] * G[SEA_FDP + ta + k - (ea - 1) - 1];
-        }
-        b[base + ta * sa] += add;
-      }
-    }
-    __syncthreads();
+  const double* G = gbuf + 36 * voff[p];
+  const double* Gy = G + NG * ey * ez;
+  const double* Gz = Gy + NG * ex * ez;
+  auto near = [](int u, int e) { return u < SEA_FDP || u >= e - SEA_FDP; };
+  const int S = BND_CTAS * 256;
+  for (BoxWalk w(blockIdx.x * 256 + threadIdx.x, S, ex, ey); w.t < P.n; w.next(S)) {
+    const bool nx = near(w.x, ex), ny = near(w.y, ey), nz = near(w.z, ez);
+    if (!(nx || ny || nz)) continue;
+    double v = b[w.t];
+    if (nx) v += ghost_sum<DFM>(W, Wd, 0, w.x, ex, G + (size_t)(w.z * ey + w.y) * NG);
+    if (ny) v += ghost_sum<DFM>(W, Wd, 1, w.y, ey, Gy + (size_t)(w.z * ex + w.x) * NG);
+    if (nz) v += ghost_sum<DFM>(W, Wd, 2, w.z, ez, Gz + (size_t)(w.y * ex + w.x) * NG);
+    b[w.t] = v;
   }
 }
 
@@ -404,37 +466,6 @@ __device__ __forceinline__ DF neg_lap_df(const float2* __restrict__ pv, int t, i
   return df_add(df_add(ax, ay), az);
 }
 
-// Walks the points t = t0, t0 + S, t0 + 2S, ... of an ex x ey x ez box in
-// [z][y][x] order with their coordinates, without divisions in the loop.
-struct BoxWalk {
-  int t, x, y, z, dx, dy, dz, ex, ey;
-  __device__ BoxWalk(int t0, int S, int ex_, int ey_) : ex(ex_), ey(ey_) {
-    t = t0;
-    x = t0 % ex;
-    y = (t0 / ex) % ey;
-    z = t0 / (ex * ey);
-    dx = S % ex;
-    dy = (S / ex) % ey;
-    dz = S / (ex * ey);
-  }
-  __device__ __forceinline__ void next(int S) {
-    t += S;
-    x += dx;
-    int cy = 0;
-    if (x >= ex) {
-      x -= ex;
-      cy = 1;
-    }
-    y += dy + cy;
-    int cz = 0;
-    if (y >= ey) {
-      y -= ey;
-      cz = 1;
-    }
-    z += dz + cz;
-  }
-};
-
 struct CgArgs {
   const double* phi;
   int nx, ny, nz;
@@ -481,7 +512,6 @@ __device__ __forceinline__ void cg_finish(const CgArgs& A, const PairInfo& P, in
 // One pair's FP64 CG (the whole CTA), results into A's per-pair arrays.
 __device__ __forceinline__ void cg_pair_fp64(const CgArgs& A, const StencilW& W, int pidx,
                                              double (*red)[32]) {
-  const size_t ng = (size_t)A.nx * A.ny * A.nz;
   const PairInfo P = A.pinfo[pidx];
   const int ex = P.ext[0], ey = P.ext[1], ez = P.ext[2], n = P.n;
   const long long off = A.voff[pidx];
@@ -1360,10 +1390,15 @@ cudaError_t launch_pair_setup(sea_ctx* c) {
       Wd.hi[a][k] = (float)W.rhs[a][k];
       Wd.lo[a][k] = (float)(W.rhs[a][k] - (double)Wd.hi[a][k]);
     }
-  geval<<<dim3(3, c->P), 256, 0, c->stream>>>(
+  int nsm = 0;
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device);
+  // lines: three faces of about (U / P)^(2/3) a pair
+  const double lines = 3.0 * c->P * std::cbrt((double)c->U / c->P) * std::cbrt((double)c->U / c->P);
+  const int halves = lines < 256.0 * nsm ? 2 : 1;
+  geval<<<dim3(3, c->P), GHOST_T, 0, c->stream>>>(
       (const PairInfo*)c->pinfo.p, (const long long*)c->voff.p, c->h[0], c->h[1], c->h[2],
-      (const double*)c->Q.p, (double*)c->gbuf.p, (const int*)c->order.p);
-  gapply<<<c->P, 256, 0, c->stream>>>((const PairInfo*)c->pinfo.p, (const long long*)c->voff.p, W,
+      (const double*)c->Q.p, halves, (double*)c->gbuf.p, (const int*)c->order.p);
+  gapply<<<dim3(BND_CTAS, c->P), 256, 0, c->stream>>>((const PairInfo*)c->pinfo.p, (const long long*)c->voff.p, W,
                                       Wd, (const double*)c->gbuf.p, (double*)c->bbuf.p,
                                       (const int*)c->order.p);
   c->launches += 3;

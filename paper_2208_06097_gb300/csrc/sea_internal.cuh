@@ -100,8 +100,6 @@ struct HarmCoef {
   //   D_lm(x, y, z) = sum_{a + b <= l} cart[lm][a][b] x^a y^b z^(l - a - b)
   // (the recurrence above carried out on coefficient arrays)
   double cart[SEA_NQ][SEA_LMAX + 1][SEA_LMAX + 1];
-  float gam_hi[SEA_LMAX][2 * SEA_LMAX + 1];  // gam = gam_hi + gam_lo (double-float)
-  float gam_lo[SEA_LMAX][2 * SEA_LMAX + 1];
 };
 // Each translation unit that evaluates harmonics holds its own copy (the
 // library is built without relocatable device code) and uploads it through
@@ -112,68 +110,6 @@ HarmCoef make_harmonic_coefficients();
 static inline cudaError_t upload_harmonics_here() {
   const HarmCoef h = make_harmonic_coefficients();
   return cudaMemcpyToSymbol(c_harm, &h, sizeof(h));
-}
-
-// acc[lm] += w * D_lm(x, y, z) (regular, rescaled basis), level by level.
-__device__ __forceinline__ void harm_accumulate(double w, double x, double y, double z,
-                                                double* acc) {
-  const double r2 = x * x + y * y + z * z;
-  double D[SEA_NQ];
-  D[0] = 1.0;
-  D[lmi(1, 1)] = x;
-  D[lmi(1, -1)] = y;
-  D[lmi(1, 0)] = z;
-  acc[0] += w;
-  acc[lmi(1, -1)] = fma(w, y, acc[lmi(1, -1)]);
-  acc[lmi(1, 0)] = fma(w, z, acc[lmi(1, 0)]);
-  acc[lmi(1, 1)] = fma(w, x, acc[lmi(1, 1)]);
-#pragma unroll
-  for (int l = 1; l < SEA_LMAX; ++l) {
-    D[lmi(l + 1, l + 1)] = fma(x, D[lmi(l, l)], -y * D[lmi(l, -l)]);
-    D[lmi(l + 1, -(l + 1))] = fma(y, D[lmi(l, l)], x * D[lmi(l, -l)]);
-#pragma unroll
-    for (int m = -l; m <= l; ++m) {
-      if (m >= -(l - 1) && m <= l - 1)
-        D[lmi(l + 1, m)] = fma(z, D[lmi(l, m)], -(c_harm.gam[l][m + SEA_LMAX] * r2) * D[lmi(l - 1, m)]);
-      else
-        D[lmi(l + 1, m)] = z * D[lmi(l, m)];
-    }
-#pragma unroll
-    for (int m = -(l + 1); m <= l + 1; ++m) acc[lmi(l + 1, m)] = fma(w, D[lmi(l + 1, m)], acc[lmi(l + 1, m)]);
-  }
-}
-
-// Multipole potential at r = (x, y, z) != 0 (relative to the expansion
-// centre) from the rescaled moments Qs (shared or global memory, zero beyond
-// the requested l_max): v = (1/r) sum Qs_lm D_lm(r / r^2).
-__device__ __forceinline__ double me_potential(const double* __restrict__ Q, double x,
-                                               double y, double z) {
-  const double ir2 = 1.0 / (x * x + y * y + z * z);
-  const double ux = x * ir2, uy = y * ir2, uz = z * ir2;
-  double D[SEA_NQ];
-  D[0] = 1.0;
-  D[lmi(1, 1)] = ux;
-  D[lmi(1, -1)] = uy;
-  D[lmi(1, 0)] = uz;
-  double v = Q[0];
-  v = fma(Q[lmi(1, -1)], uy, v);
-  v = fma(Q[lmi(1, 0)], uz, v);
-  v = fma(Q[lmi(1, 1)], ux, v);
-#pragma unroll
-  for (int l = 1; l < SEA_LMAX; ++l) {
-    D[lmi(l + 1, l + 1)] = fma(ux, D[lmi(l, l)], -uy * D[lmi(l, -l)]);
-    D[lmi(l + 1, -(l + 1))] = fma(uy, D[lmi(l, l)], ux * D[lmi(l, -l)]);
-#pragma unroll
-    for (int m = -l; m <= l; ++m) {
-      if (m >= -(l - 1) && m <= l - 1)
-        D[lmi(l + 1, m)] = fma(uz, D[lmi(l, m)], -(c_harm.gam[l][m + SEA_LMAX] * ir2) * D[lmi(l - 1, m)]);
-      else
-        D[lmi(l + 1, m)] = uz * D[lmi(l, m)];
-    }
-#pragma unroll
-    for (int m = -(l + 1); m <= l + 1; ++m) v = fma(Q[lmi(l + 1, m)], D[lmi(l + 1, m)], v);
-  }
-  return v * sqrt(ir2);
 }
 
 // v 2^e2 rounded to the nearest FP64 value (ties to even); 0 if below the
@@ -341,129 +277,85 @@ __device__ __forceinline__ DF df_from_double(double x) {
   return DF{s.x, s.y};
 }
 
-// me_potential in double-float: the same recurrences and summation order,
-// Q as double-float coefficients.
-__device__ __forceinline__ DF me_potential_df(const DF* __restrict__ Q, DF x, DF y, DF z) {
-  const DF r2 = df_fma(z, z, df_dot2(x, x, y, y));
-  const DF ir2 = df_rcp(r2);
-  const DF ux = df_mul(x, ir2), uy = df_mul(y, ir2), uz = df_mul(z, ir2);
-  DF Dm[2 * SEA_LMAX + 1], Dc[2 * SEA_LMAX + 1], Dn[2 * SEA_LMAX + 1];  // l-1, l, l+1
+// The multipole potential of Eq. me along grid lines.  With u = r / r^2,
+// sum_lm Qs_lm D_lm(u) = sum_abc P_abc ux^a uy^b uz^c, P_abc = sum_m Qs_lm
+// cart[lm][a][b] (l = a + b + c; formed once per pair by k_pair_moments,
+// layout mono_k), so with w = 1/r^2
+//   v(r) = (1/r) sum_l w^l S_l(r),  S_l = sum_{a+b+c=l} P_abc x^a y^b z^c.
+// On a line along axis AX the other two coordinates are fixed and S_l is a
+// polynomial of degree l in the third: its 28 coefficients take 112
+// operations once per line, a point then 21 + 6 multiply-adds instead of the
+// 84 of the full three-variable Horner form.  The evaluation is bound by the
+// FP64 unit (plain form) or by dependent FP32 chains (double-float, mixed
+// form), and a line of a window or face has 12 to 30 points.
+struct MeF64 {
+  typedef double T;
+  static __device__ __forceinline__ T mul(T a, T b) { return a * b; }
+  static __device__ __forceinline__ T fma_(T a, T b, T c) { return fma(a, b, c); }
+  // (1/r, 1/r^2) from r^2
+  static __device__ __forceinline__ void inv(T r2, T* ir, T* ir2) {
+    *ir = rsqrt(r2);
+    *ir2 = *ir * *ir;
+  }
+};
+struct MeDF {
+  typedef DF T;
+  static __device__ __forceinline__ T mul(T a, T b) { return df_mul(a, b); }
+  static __device__ __forceinline__ T fma_(T a, T b, T c) { return df_fma(a, b, c); }
+  static __device__ __forceinline__ void inv(T r2, T* ir, T* ir2) {
+    *ir2 = df_rcp(r2);
+    *ir = df_sqrt(*ir2);
+  }
+};
+constexpr int ME_LINE = (SEA_LMAX + 1) * (SEA_LMAX + 2) / 2;  // coefficients: degree l, power k <= l
+// The index of P for power k along axis AX and i, j along the other two.
+template <int AX>
+__device__ __forceinline__ constexpr int me_line_mono(int k, int i, int j) {
+  return AX == 0 ? mono_k(k, i, j) : AX == 1 ? mono_k(i, k, j) : mono_k(i, j, k);
+}
+// c[l (l + 1) / 2 + k] for the line with coordinates s, t on the other axes
+// (in axis order); P: the pair's coefficients (shared memory).
+template <class R, int AX>
+__device__ __forceinline__ void me_line(const typename R::T* __restrict__ P, typename R::T s,
+                                        typename R::T t, typename R::T (&c)[ME_LINE]) {
+  typedef typename R::T T;
+  T m[SEA_LMAX + 1];  // m[i] = s^i t^(d-i)
 #pragma unroll
-  for (int k = 0; k < 2 * SEA_LMAX + 1; ++k) Dm[k] = Dc[k] = Dn[k] = DF{0.f, 0.f};
-  Dm[SEA_LMAX] = DF{1.f, 0.f};  // l = 0
-  Dc[SEA_LMAX + 1] = ux;        // l = 1: m = 1, -1, 0
-  Dc[SEA_LMAX - 1] = uy;
-  Dc[SEA_LMAX] = uz;
-  DF v = Q[0];
-  v = df_fma(Q[lmi(1, -1)], uy, v);
-  v = df_fma(Q[lmi(1, 0)], uz, v);
-  v = df_fma(Q[lmi(1, 1)], ux, v);
+  for (int d = 0; d <= SEA_LMAX; ++d) {
+    if (d > 0) {
+      m[d] = d == 1 ? s : R::mul(m[d - 1], s);
 #pragma unroll
-  for (int l = 1; l < SEA_LMAX; ++l) {
-    Dn[SEA_LMAX + l + 1] = df_dot2(ux, Dc[SEA_LMAX + l], df_neg(uy), Dc[SEA_LMAX - l]);
-    Dn[SEA_LMAX - l - 1] = df_dot2(uy, Dc[SEA_LMAX + l], ux, Dc[SEA_LMAX - l]);
+      for (int i = d - 1; i >= 0; --i) m[i] = d == 1 ? t : R::mul(m[i], t);
+    }
 #pragma unroll
-    for (int m = -l; m <= l; ++m) {
-      if (m >= -(l - 1) && m <= l - 1) {
-        const DF g = df_mul(DF{c_harm.gam_hi[l][m + SEA_LMAX], c_harm.gam_lo[l][m + SEA_LMAX]}, ir2);
-        Dn[SEA_LMAX + m] = df_dot2(uz, Dc[SEA_LMAX + m], df_neg(g), Dm[SEA_LMAX + m]);
-      } else {
-        Dn[SEA_LMAX + m] = df_mul(uz, Dc[SEA_LMAX + m]);
+    for (int k = 0; k + d <= SEA_LMAX; ++k) {
+      const int l = k + d;
+      T a = P[me_line_mono<AX>(k, 0, d)];
+      if (d > 0) {
+        a = R::mul(a, m[0]);
+#pragma unroll
+        for (int i = 1; i <= d; ++i) a = R::fma_(P[me_line_mono<AX>(k, i, d - i)], m[i], a);
       }
-    }
-#pragma unroll
-    for (int m = -(l + 1); m <= l + 1; ++m) v = df_fma(Q[lmi(l + 1, m)], Dn[SEA_LMAX + m], v);
-#pragma unroll
-    for (int k = 0; k < 2 * SEA_LMAX + 1; ++k) {
-      Dm[k] = Dc[k];
-      Dc[k] = Dn[k];
+      c[l * (l + 1) / 2 + k] = a;
     }
   }
-  return df_mul(v, df_sqrt(ir2));
 }
-
-// The multipole potential of Eq. me from its polynomial form: with u = r /
-// r^2, sum_lm Qs_lm D_lm(u) = sum_abc P_abc ux^a uy^b uz^c, P_abc = sum_m
-// Qs_lm cart[lm][a][b] (l = a + b + c; formed once per pair by
-// k_pair_moments, layout mono_k), so v = (1/r) sum P_abc ux^a uy^b uz^c,
-// evaluated by nested Horner steps (84 multiply-adds per point).  Double-float
-// (mixed form) and FP64 versions.
-__device__ __forceinline__ DF me_potential_cart_df(const DF* __restrict__ P, DF x, DF y, DF z) {
-  const DF r2 = df_fma(z, z, df_dot2(x, x, y, y));
-  const DF ir2 = df_rcp(r2);
-  const DF ux = df_mul(x, ir2), uy = df_mul(y, ir2), uz = df_mul(z, ir2);
-  DF pa{0.f, 0.f};
+// v at coordinate x of the line, q = s^2 + t^2.
+template <class R>
+__device__ __forceinline__ typename R::T me_line_at(const typename R::T (&c)[ME_LINE],
+                                                    typename R::T x, typename R::T q) {
+  typedef typename R::T T;
+  T ir, w;
+  R::inv(R::fma_(x, x, q), &ir, &w);
+  T v = c[0];
 #pragma unroll
-  for (int a = SEA_LMAX; a >= 0; --a) {
-    DF pb{0.f, 0.f};
+  for (int l = SEA_LMAX; l >= 0; --l) {
+    T s = c[l * (l + 1) / 2 + l];
 #pragma unroll
-    for (int b = SEA_LMAX - a; b >= 0; --b) {
-      DF pc = P[mono_k(a, b, SEA_LMAX - a - b)];
-#pragma unroll
-      for (int c = SEA_LMAX - a - b - 1; c >= 0; --c) pc = df_fma(pc, uz, P[mono_k(a, b, c)]);
-      pb = (b == SEA_LMAX - a) ? pc : df_fma(pb, uy, pc);
-    }
-    pa = (a == SEA_LMAX) ? pb : df_fma(pa, ux, pb);
+    for (int k = l - 1; k >= 0; --k) s = R::fma_(s, x, c[l * (l + 1) / 2 + k]);
+    v = l == SEA_LMAX ? s : R::fma_(v, w, s);
   }
-  return df_mul(pa, df_sqrt(ir2));
-}
-__device__ __forceinline__ double me_potential_cart(const double* __restrict__ P, double x,
-                                                    double y, double z) {
-  const double ir2 = 1.0 / (x * x + y * y + z * z);
-  const double ux = x * ir2, uy = y * ir2, uz = z * ir2;
-  double pa = 0.0;
-#pragma unroll
-  for (int a = SEA_LMAX; a >= 0; --a) {
-    double pb = 0.0;
-#pragma unroll
-    for (int b = SEA_LMAX - a; b >= 0; --b) {
-      double pc = P[mono_k(a, b, SEA_LMAX - a - b)];
-#pragma unroll
-      for (int c = SEA_LMAX - a - b - 1; c >= 0; --c) pc = fma(pc, uz, P[mono_k(a, b, c)]);
-      pb = (b == SEA_LMAX - a) ? pc : fma(pb, uy, pc);
-    }
-    pa = (a == SEA_LMAX) ? pb : fma(pa, ux, pb);
-  }
-  return pa * sqrt(ir2);
-}
-
-// harm_accumulate in double-float: acc[q] += w D_q(x, y, z), the same
-// recurrences in the same order.
-__device__ __forceinline__ void harm_accumulate_df(DF w, DF x, DF y, DF z, DF* acc) {
-  const DF r2 = df_fma(z, z, df_dot2(x, x, y, y));
-  DF Dm[2 * SEA_LMAX + 1], Dc[2 * SEA_LMAX + 1], Dn[2 * SEA_LMAX + 1];  // l-1, l, l+1
-#pragma unroll
-  for (int k = 0; k < 2 * SEA_LMAX + 1; ++k) Dm[k] = Dc[k] = Dn[k] = DF{0.f, 0.f};
-  Dm[SEA_LMAX] = DF{1.f, 0.f};
-  Dc[SEA_LMAX + 1] = x;
-  Dc[SEA_LMAX - 1] = y;
-  Dc[SEA_LMAX] = z;
-  acc[0] = df_add(acc[0], w);
-  acc[lmi(1, -1)] = df_fma(w, y, acc[lmi(1, -1)]);
-  acc[lmi(1, 0)] = df_fma(w, z, acc[lmi(1, 0)]);
-  acc[lmi(1, 1)] = df_fma(w, x, acc[lmi(1, 1)]);
-#pragma unroll
-  for (int l = 1; l < SEA_LMAX; ++l) {
-    Dn[SEA_LMAX + l + 1] = df_dot2(x, Dc[SEA_LMAX + l], df_neg(y), Dc[SEA_LMAX - l]);
-    Dn[SEA_LMAX - l - 1] = df_dot2(y, Dc[SEA_LMAX + l], x, Dc[SEA_LMAX - l]);
-#pragma unroll
-    for (int m = -l; m <= l; ++m) {
-      if (m >= -(l - 1) && m <= l - 1) {
-        const DF g = df_mul(DF{c_harm.gam_hi[l][m + SEA_LMAX], c_harm.gam_lo[l][m + SEA_LMAX]}, r2);
-        Dn[SEA_LMAX + m] = df_dot2(z, Dc[SEA_LMAX + m], df_neg(g), Dm[SEA_LMAX + m]);
-      } else {
-        Dn[SEA_LMAX + m] = df_mul(z, Dc[SEA_LMAX + m]);
-      }
-    }
-#pragma unroll
-    for (int m = -(l + 1); m <= l + 1; ++m)
-      acc[lmi(l + 1, m)] = df_fma(w, Dn[SEA_LMAX + m], acc[lmi(l + 1, m)]);
-#pragma unroll
-    for (int k = 0; k < 2 * SEA_LMAX + 1; ++k) {
-      Dm[k] = Dc[k];
-      Dc[k] = Dn[k];
-    }
-  }
+  return R::mul(v, ir);
 }
 
 // Exclusive scan over the CTA of one 64-bit integer per thread (blockDim.x
@@ -704,10 +596,6 @@ struct Entry {
 };
 
 namespace sea {
-// Window points per unit of the far-field work (k_contrib's CTAs and the
-// mixed CG's far-field items).
-#define SEA_CHUNK 1024
-
 // q = floor(a / d) and *r = a - q d for 0 <= a < 2^24, 1 <= d < 2^24: the
 // FP32 product a (1/d) is within (a/d) 2^-23 < 1 of a/d, so its truncation
 // is q or q +- 1, corrected once by the sign and size of the remainder.
@@ -749,197 +637,70 @@ __host__ __device__ __forceinline__ WinSplit window_split(const Entry& e, const 
   return s;
 }
 
+// The lines along x of a window that hold points outside the pair box, in
+// window coordinates: first the whole lines (n_whole: the planes below and
+// above the box's z range, then within that range the rows below and above
+// its y range), then the n_cut lines that cross the box, whose points outside
+// are [0, b0[0]) and [b1[0], wl[0]).
+struct WinLines {
+  int n_whole, n_cut;
+};
+__host__ __device__ __forceinline__ WinLines window_lines(const WinSplit& s, const int wl[3]) {
+  WinLines n;
+  n.n_cut = (s.b1[1] - s.b0[1]) * (s.b1[2] - s.b0[2]);
+  n.n_whole = wl[1] * wl[2] - n.n_cut;
+  if (s.b1[0] - s.b0[0] == wl[0]) n.n_cut = 0;  // those lines lie inside
+  return n;
+}
+// (ty, tz) of line i < n_whole + n_cut (fewer than 2^24 lines: windows have
+// at most 1024 points per axis).
+__host__ __device__ __forceinline__ void window_outside_line(const WinSplit& s, const int wl[3],
+                                                             int i, int* ty, int* tz) {
+  const int wy = wl[1], zb = s.b1[2] - s.b0[2], yb = s.b1[1] - s.b0[1];
+  const int n1 = s.b0[2] * wy, n2 = (wl[2] - s.b1[2]) * wy;
+  const int n3 = zb * s.b0[1], n4 = zb * (wy - s.b1[1]);
+  int oy = 0, oz = 0, by = wy;
+  if (i < n1) {
+  } else if ((i -= n1) < n2) {
+    oz = s.b1[2];
+  } else {
+    i -= n2;
+    oz = s.b0[2];
+    if (i < n3) {
+      by = s.b0[1];
+    } else if ((i -= n3) < n4) {
+      oy = s.b1[1];
+      by = wy - s.b1[1];
+    } else {
+      i -= n4;
+      oy = s.b0[1];
+      by = yb;
+    }
+  }
+  int ry;
+  *tz = oz + divmod_small(i, by, &ry);
+  *ty = oy + ry;
+}
+
 // Window coordinates of point u (0 <= u < n_out, n_out < 2^24) of the window
-// points outside the pair box, numbered through six disjoint boxes: the
-// planes below and above the box's z range, then within that z range the
-// rows below and above its y range, then within that y range the runs left
-// and right of its x range; x fastest inside each.
+// points outside the pair box, line after line in the order above, on the
+// cut lines first all points left of the box, then all right of it.
 __host__ __device__ __forceinline__ void window_outside_point(const WinSplit& s, const int wl[3],
                                                               int u, int* tx, int* ty, int* tz) {
-  const int wx = wl[0], wy = wl[1], wz = wl[2];
-  const int zb = s.b1[2] - s.b0[2], yb = s.b1[1] - s.b0[1];
-  const int n1 = s.b0[2] * wx * wy, n2 = (wz - s.b1[2]) * wx * wy;
-  const int n3 = zb * s.b0[1] * wx, n4 = zb * (wy - s.b1[1]) * wx, n5 = zb * yb * s.b0[0];
-  int ox = 0, oy = 0, oz = 0, bx = wx, by = wy;
-  if (u < n1) {
-  } else if ((u -= n1) < n2) {
-    oz = s.b1[2];
-  } else if ((u -= n2) < n3) {
-    oz = s.b0[2];
-    by = s.b0[1];
-  } else if ((u -= n3) < n4) {
-    oz = s.b0[2];
-    oy = s.b1[1];
-    by = wy - s.b1[1];
-  } else if ((u -= n4) < n5) {
-    oz = s.b0[2];
-    oy = s.b0[1];
-    by = yb;
-    bx = s.b0[0];
+  const WinLines n = window_lines(s, wl);
+  const int left = s.b0[0], right = wl[0] - s.b1[0];
+  int line, rx, x0 = 0;
+  if (u < n.n_whole * wl[0]) {
+    line = divmod_small(u, wl[0], &rx);
+  } else if ((u -= n.n_whole * wl[0]) < n.n_cut * left) {
+    line = n.n_whole + divmod_small(u, left, &rx);
   } else {
-    u -= n5;
-    oz = s.b0[2];
-    oy = s.b0[1];
-    by = yb;
-    ox = s.b1[0];
-    bx = wx - s.b1[0];
+    line = n.n_whole + divmod_small(u - n.n_cut * left, right, &rx);
+    x0 = s.b1[0];
   }
-  int rx, ry;
-  const int q = divmod_small(u, bx, &rx);
-  const int qz = divmod_small(q, by, &ry);
-  *tx = ox + rx;
-  *ty = oy + ry;
-  *tz = oz + qz;
+  window_outside_line(s, wl, line, ty, tz);
+  *tx = x0 + rx;
 }
-
-// Window contributions c = v phi_partner (Eq. tDxx) of entry e (window-
-// compact output out[t], t = (tz wy + ty) wx + tx): v is the pair's CG
-// solution (v, box layout) inside the pair box and the multipole potential
-// (coefficients Pd, double-float, or Ps, FP64) outside.  part 0: every
-// window point, t = t0 + threadIdx.x, + blockDim.x, ... < t1; 1: only the
-// points outside the box (they need the moments alone), 2: only those
-// inside (they need the solution); for parts 1 and 2 with compact set, t0
-// and t1 number the points of that part alone (window_outside_point; the
-// box's points in x-fastest order), so that no lane idles on a point of the
-// other part, else they are window points and the other part's are skipped.
-// DFM: double-float products (mixed form), else FP64.
-template <bool DFM>
-__device__ __forceinline__ void contrib_range(int part, bool compact, const WinSplit& sp,
-                                              const Entry& e, const PairInfo& P,
-                                              const double* __restrict__ phi, int nx, int ny,
-                                              int nz, const double* __restrict__ v, const DF* Pd,
-                                              const double* Ps, double hx, double hy, double hz,
-                                              double* __restrict__ out, int t0, int t1) {
-  const DF Hx = df_from_double(hx), Hy = df_from_double(hy), Hz = df_from_double(hz);
-  const size_t ng = (size_t)nx * ny * nz;
-  const double* fp = phi + (size_t)e.partner * ng;
-  const double cx = 0.5 * (P.ext[0] - 1), cy = 0.5 * (P.ext[1] - 1), cz = 0.5 * (P.ext[2] - 1);
-  const float cxf = 0.5f * i2f_exact(P.ext[0] - 1), cyf = 0.5f * i2f_exact(P.ext[1] - 1),
-              czf = 0.5f * i2f_exact(P.ext[2] - 1);
-  const int wx = e.wl[0], wy = e.wl[1];
-  const int gx0 = wrapi(e.ws[0], nx), gy0 = wrapi(e.ws[1], ny), gz0 = wrapi(e.ws[2], nz);
-  const int S = blockDim.x;
-  // one window point (tx, ty, tz): its value into out[(tz wy + ty) wx + tx]
-  auto point = [&](int tx, int ty, int tz, bool inside) {
-    const int lx = e.ws[0] + tx - P.lo[0], ly = e.ws[1] + ty - P.lo[1], lz = e.ws[2] + tz - P.lo[2];
-    int gx = gx0 + tx, gy = gy0 + ty, gz = gz0 + tz;  // window lengths are at most n
-    gx -= gx >= nx ? nx : 0;
-    gy -= gy >= ny ? ny : 0;
-    gz -= gz >= nz ? nz : 0;
-    const size_t g = ((size_t)gz * ny + gy) * nx + gx;
-    const int t = (tz * wy + ty) * wx + tx;
-    if (DFM) {  // c = v phi in double-float, no FP64 instruction
-      DF val;
-      if (inside) {
-        const float2 s = split64(v[(lz * P.ext[1] + ly) * P.ext[0] + lx]);
-        val = DF{s.x, s.y};
-      } else {  // lx - cx etc. are half-integers, exact in FP32
-        val = me_potential_cart_df(Pd, df_mul_f(i2f_exact(lx) - cxf, Hx),
-                                   df_mul_f(i2f_exact(ly) - cyf, Hy), df_mul_f(i2f_exact(lz) - czf, Hz));
-      }
-      const float2 f = split64(fp[g]);
-      out[t] = df_to_double(df_mul(val, DF{f.x, f.y}));
-    } else {
-      const double val = inside ? v[(lz * P.ext[1] + ly) * P.ext[0] + lx]
-                                : me_potential_cart(Ps, (lx - cx) * hx, (ly - cy) * hy, (lz - cz) * hz);
-      out[t] = __dmul_rn(val, fp[g]);
-    }
-  };
-  // parts 0 and 2, and part 1 without compact: a box [ox, ox + bx) x
-  // [oy, oy + by) x ... (the window, or with compact part 2 the pair box
-  // within it) walked with (kx, ky, kz) advanced by the CTA stride without
-  // divisions; compact part 1: window_outside_point
-  const bool outer = compact && part == 1, box = compact && part == 2;
-  const int ox = box ? sp.b0[0] : 0, oy = box ? sp.b0[1] : 0, oz = box ? sp.b0[2] : 0;
-  const int bx = box ? sp.b1[0] - sp.b0[0] : wx, by = box ? sp.b1[1] - sp.b0[1] : wy;
-  const int bxy = bx * by;
-  const int dz = S / bxy, dy = (S - dz * bxy) / bx, dx = S - dz * bxy - dy * bx;
-  int kz = (t0 + (int)threadIdx.x) / bxy;
-  int ky = (t0 + (int)threadIdx.x - kz * bxy) / bx;
-  int kx = t0 + (int)threadIdx.x - kz * bxy - ky * bx;
-  if (box) {
-    // in-box points: the loop is bound by the latency of its two loads per
-    // point, so each thread takes CU points (t, t + S, ...) with all their
-    // loads issued before the first product; the products are those of
-    // `point`, so the results are the same bits
-    constexpr int CU = 4;
-    const int l0 = e.ws[0] - P.lo[0], l1 = e.ws[1] - P.lo[1], l2 = e.ws[2] - P.lo[2];
-    for (int t = t0 + threadIdx.x; t < t1; t += CU * S) {
-      int lq[CU], tq[CU];
-      size_t gq[CU];
-#pragma unroll
-      for (int u = 0; u < CU; ++u) {
-        const int tx = ox + kx, ty = oy + ky, tz = oz + kz;
-        kx += dx;
-        ky += dy;
-        kz += dz;
-        if (kx >= bx) {
-          kx -= bx;
-          ++ky;
-        }
-        if (ky >= by) {
-          ky -= by;
-          ++kz;
-        }
-        int gx = gx0 + tx, gy = gy0 + ty, gz = gz0 + tz;
-        gx -= gx >= nx ? nx : 0;
-        gy -= gy >= ny ? ny : 0;
-        gz -= gz >= nz ? nz : 0;
-        gq[u] = ((size_t)gz * ny + gy) * nx + gx;
-        tq[u] = (tz * wy + ty) * wx + tx;
-        lq[u] = ((l2 + tz) * P.ext[1] + (l1 + ty)) * P.ext[0] + (l0 + tx);
-      }
-      double vq[CU], fq[CU];
-#pragma unroll
-      for (int u = 0; u < CU; ++u)
-        if (t + u * S < t1) {
-          vq[u] = v[lq[u]];
-          fq[u] = fp[gq[u]];
-        }
-#pragma unroll
-      for (int u = 0; u < CU; ++u)
-        if (t + u * S < t1) {
-          if (DFM) {
-            const float2 s = split64(vq[u]), f = split64(fq[u]);
-            out[tq[u]] = df_to_double(df_mul(DF{s.x, s.y}, DF{f.x, f.y}));
-          } else {
-            out[tq[u]] = __dmul_rn(vq[u], fq[u]);
-          }
-        }
-    }
-    return;
-  }
-  for (int t = t0 + threadIdx.x; t < t1; t += S) {
-    int tx, ty, tz;
-    bool inside = box;
-    if (outer) {
-      window_outside_point(sp, e.wl, t, &tx, &ty, &tz);
-    } else {
-      tx = ox + kx;
-      ty = oy + ky;
-      tz = oz + kz;
-      kx += dx;
-      ky += dy;
-      kz += dz;
-      if (kx >= bx) {
-        kx -= bx;
-        ++ky;
-      }
-      if (ky >= by) {
-        ky -= by;
-        ++kz;
-      }
-      if (!box) {
-        const int lx = e.ws[0] + tx - P.lo[0], ly = e.ws[1] + ty - P.lo[1],
-                  lz = e.ws[2] + tz - P.lo[2];
-        inside = lx >= 0 && lx < P.ext[0] && ly >= 0 && ly < P.ext[1] && lz >= 0 && lz < P.ext[2];
-        if ((part == 1 && inside) || (part == 2 && !inside)) continue;
-      }
-    }
-    point(tx, ty, tz, inside);
-  }
-}
-
 
 // Shared-memory layout of a CG vector on a pair box: the planes of ex x ey
 // points stored row after row (so consecutive points of a warp sit in
@@ -1024,5 +785,4 @@ cudaError_t launch_cg_boxes(cudaStream_t stream, int device, const double h[3], 
                             const double* rhs, double* x, double* r, double* p, double* q,
                             int* iters, unsigned* status, int* queue, double tol, int tol_mode,
                             int max_iter, int pad_max);
-cudaError_t upload_harmonics_accum();
 }  // namespace sea
