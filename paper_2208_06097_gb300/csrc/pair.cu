@@ -1494,7 +1494,7 @@ static CgArgs fp64_args(sea_ctx* c) {
 // most the form's limit (two CTAs per SM); pairs above it solve on global
 // vectors.  Mixed form: floats of the residual; FP64 form: 8-byte fixed-point
 // values of the search direction.
-#define SEA_CG_PAD_LIMIT 13824
+#define SEA_CG_PAD_LIMIT 27000
 int cg_pad_cap(const sea_ctx* c) {
   return c->prm.precision == 1 ? std::min(c->cg_pad_max, SEA_CG_PAD_LIMIT)
                                : make_fix(c->h, c->cg_pad_max).cap;
