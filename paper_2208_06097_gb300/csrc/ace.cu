@@ -10,6 +10,8 @@
 //   V^ACE psi = -Xi Xi^T psi dV = -W L^-T L^-1 (W^T psi dV)
 // The contractions are FP64 FMA on the CUDA cores: on this part the measured
 // FP64 FMA rate is above the FP64 tensor (DMMA) rate.
+#include <type_traits>
+
 #include "sea_internal.cuh"
 
 namespace sea {
@@ -281,64 +283,81 @@ __global__ void __launch_bounds__(256)
 }
 
 // out[a * sa + o * so] = scale * sum over the tiles of o of partial[slot][a].
-// A CTA per (orbital o, 64 values of a): its four thread groups z take the
-// slots z, z + 4, z + 8, ... of o's list (eight loads in flight each, added
-// in list order), and the four sums are added in the order z = 0, 1, 2, 3.
-constexpr int GR_A = 64, GR_Z = 4;
-__global__ void __launch_bounds__(GR_A * GR_Z)
+// A CTA per (orbital o, GR_A values of a): its four thread groups z take the
+// slots z, z + 4, z + 8, ... of o's list (eight loads in flight each, the next
+// eight slots' numbers fetched beside them, added in list order), and the four
+// sums are added in the order z = 0, 1, 2, 3, whatever GR_A (8 for at most
+// eight values, where 64 would leave most threads idle).  DFM (mixed form):
+// sums in double-float (the partials split exactly to FP32 pairs, sums on the
+// FP32 pipes; FP64 adds bound the other form), one rounding to FP64 before
+// the scaling.
+constexpr int GR_Z = 4;
+template <bool DFM, int GR_A>
+__global__ void __launch_bounds__(GR_A* GR_Z)
     k_gram_reduce(const double* __restrict__ partial, int m, int n_orb,
                   const int* __restrict__ optr, const int* __restrict__ oslot, double scale,
                   double* __restrict__ out, int sa, int so) {
-  __shared__ double red[GR_Z][GR_A];
+  typedef typename std::conditional<DFM, DF, double>::type T;
+  auto add = [](T x, T y) -> T {
+    if constexpr (DFM)
+      return df_add(x, y);
+    else
+      return x + y;
+  };
+  auto in = [](double x) -> T {
+    if constexpr (DFM)
+      return df_from_double(x);
+    else
+      return x;
+  };
+  __shared__ T red[GR_Z][GR_A];
   const int o = blockIdx.y, x = threadIdx.x % GR_A, z = threadIdx.x / GR_A;
   const int a = blockIdx.x * GR_A + x;
-  double s = 0.0;
+  T s = in(0.0);
   if (a < m) {
     int k = optr[o] + z;
     const int k1 = optr[o + 1];
-    for (; k + 7 * GR_Z < k1; k += 8 * GR_Z) {
+    int idx[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) idx[u] = k + u * GR_Z < k1 ? oslot[k + u * GR_Z] : -1;
+    for (; k < k1; k += 8 * GR_Z) {
       double p[8];
+      bool use[8];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) p[u] = partial[(size_t)oslot[k + u * GR_Z] * m + a];
+      for (int u = 0; u < 8; ++u) {
+        use[u] = idx[u] >= 0;
+        p[u] = use[u] ? partial[(size_t)idx[u] * m + a] : 0.0;
+      }
 #pragma unroll
-      for (int u = 0; u < 8; ++u) s += p[u];
+      for (int u = 0; u < 8; ++u) {
+        const int kn = k + (8 + u) * GR_Z;
+        idx[u] = kn < k1 ? oslot[kn] : -1;
+      }
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        if (use[u]) s = add(s, in(p[u]));
     }
-    for (; k < k1; k += GR_Z) s += partial[(size_t)oslot[k] * m + a];
   }
   red[z][x] = s;
   __syncthreads();
-  if (z == 0 && a < m)
-    out[(size_t)a * sa + (size_t)o * so] = scale * (((red[0][x] + red[1][x]) + red[2][x]) + red[3][x]);
+  if (z == 0 && a < m) {
+#pragma unroll
+    for (int q = 1; q < GR_Z; ++q) s = add(s, red[q][x]);
+    double v;
+    if constexpr (DFM)
+      v = df_to_double(s);
+    else
+      v = s;
+    out[(size_t)a * sa + (size_t)o * so] = scale * v;
+  }
 }
-
-// The same sums in double-float for the mixed form (the partials split
-// exactly to FP32 pairs, sums on the FP32 pipes; the FP64 adds of the form
-// above bound it there), one rounding to FP64 before the scaling.
-__global__ void __launch_bounds__(GR_A * GR_Z)
-    k_gram_reduce_df(const double* __restrict__ partial, int m, int n_orb,
-                     const int* __restrict__ optr, const int* __restrict__ oslot, double scale,
-                     double* __restrict__ out, int sa, int so) {
-  __shared__ DF red[GR_Z][GR_A];
-  const int o = blockIdx.y, x = threadIdx.x % GR_A, z = threadIdx.x / GR_A;
-  const int a = blockIdx.x * GR_A + x;
-  DF s{0.f, 0.f};
-  if (a < m) {
-    int k = optr[o] + z;
-    const int k1 = optr[o + 1];
-    for (; k + 7 * GR_Z < k1; k += 8 * GR_Z) {
-      double p[8];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) p[u] = partial[(size_t)oslot[k + u * GR_Z] * m + a];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) s = df_add(s, df_from_double(p[u]));
-    }
-    for (; k < k1; k += GR_Z) s = df_add(s, df_from_double(partial[(size_t)oslot[k] * m + a]));
-  }
-  red[z][x] = s;
-  __syncthreads();
-  if (z == 0 && a < m)
-    out[(size_t)a * sa + (size_t)o * so] =
-        scale * df_to_double(df_add(df_add(df_add(red[0][x], red[1][x]), red[2][x]), red[3][x]));
+static void launch_gram_reduce(cudaStream_t st, bool df, const double* partial, int m, int n,
+                               const int* optr, const int* oslot, double scale, double* out, int sa,
+                               int so) {
+  const int A = m <= 8 ? 8 : 64;
+  auto k = m <= 8 ? (df ? k_gram_reduce<true, 8> : k_gram_reduce<false, 8>)
+                  : (df ? k_gram_reduce<true, 64> : k_gram_reduce<false, 64>);
+  k<<<dim3((m + A - 1) / A, n), A * GR_Z, 0, st>>>(partial, m, n, optr, oslot, scale, out, sa, so);
 }
 
 // -Mbar = L L^T by a blocked right-looking Cholesky (block CB = 32), and
@@ -644,61 +663,68 @@ __global__ void k_scale_rows(double* __restrict__ B, const double* __restrict__ 
 }
 
 // C[n1][n2] = op(A) B, op(A)(i, k) = A[k][i] if transA else A[i][k]; A is
-// n1 x n1 (square), B is [n1][n2].  16 x 16 shared-memory tiles.  With
-// `lower`, A's zero upper triangle is not multiplied.
-__global__ void k_small_gemm(const double* __restrict__ A, int transA, const double* __restrict__ B,
-                             int n1, int n2, double* __restrict__ C, int lower) {
-  __shared__ double As[16][17], Bs[16][17];
-  const int i = blockIdx.y * 16 + threadIdx.y, j = blockIdx.x * 16 + threadIdx.x;
-  double acc = 0.0;
-  // lower: A is lower triangular (zeros above the diagonal, exactly), so
-  // op(A)(i, k) vanishes for k > i (A B) or k < i (A^T B); those tiles are
-  // skipped (their products would add exact zeros)
-  const int kbeg = (lower && transA) ? blockIdx.y * 16 : 0;
-  const int kend = (lower && !transA) ? min(n1, (int)(blockIdx.y + 1) * 16) : n1;
-  for (int k0 = kbeg; k0 < kend; k0 += 16) {
-    const int ka = k0 + threadIdx.x, kb = k0 + threadIdx.y;
-    double av = 0.0;
-    if (i < n1 && ka < n1) av = transA ? A[(size_t)ka * n1 + i] : A[(size_t)i * n1 + ka];
-    As[threadIdx.y][threadIdx.x] = av;
-    Bs[threadIdx.y][threadIdx.x] = (kb < n1 && j < n2) ? B[(size_t)kb * n2 + j] : 0.0;
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < 16; ++k) acc = fma(As[threadIdx.y][k], Bs[k][threadIdx.x], acc);
-    __syncthreads();
-  }
-  if (i < n1 && j < n2) C[(size_t)i * n2 + j] = acc;
-}
-
-// The same product in double-float arithmetic for the mixed form (FP64
-// operands split exactly into FP32 pairs to about 2^-47, FP32 pipes instead
-// of the FP64 unit, one rounding to FP64 at the end).
+// n1 x n1 (square), B is [n1][n2].  Output tiles of 16 x 16, each element one
+// chain over k in ascending order; k in tiles of 32 through shared memory, the
+// next tile's values fetched into registers while the current one is
+// multiplied (for a few columns the loads' latency is what the product
+// takes: 12 -> 7 us at n1 = 128, n2 = 8).  With `lower` A is lower
+// triangular (zeros above the diagonal, exactly), so op(A)(i, k) vanishes for
+// k > i (A B) or k < i (A^T B); those tiles are skipped (their products would
+// add exact zeros).  DFM (mixed form): double-float arithmetic (FP64 operands
+// split exactly into FP32 pairs to about 2^-47, FP32 pipes instead of the
+// FP64 unit, one rounding to FP64 at the end).
+template <bool DFM>
 __global__ void __launch_bounds__(256)
-    k_small_gemm_df(const double* __restrict__ A, int transA, const double* __restrict__ B,
-                    int n1, int n2, double* __restrict__ C, int lower) {
-  __shared__ float Ah[16][17], Al[16][17], Bh[16][17], Bl[16][17];
-  const int i = blockIdx.y * 16 + threadIdx.y, j = blockIdx.x * 16 + threadIdx.x;
-  DF acc{0.f, 0.f};
+    k_small_gemm(const double* __restrict__ A, int transA, const double* __restrict__ B, int n1,
+                 int n2, double* __restrict__ C, int lower) {
+  constexpr int KT = 32;
+  typedef typename std::conditional<DFM, MeDF, MeF64>::type R;
+  typedef typename R::T T;
+  auto in = [](double x) -> T {
+    if constexpr (DFM)
+      return df_from_double(x);
+    else
+      return x;
+  };
+  __shared__ T As[16][KT + 1], Bs[KT][17];
+  const int tx = threadIdx.x, ty = threadIdx.y;
+  const int i = blockIdx.y * 16 + ty, j = blockIdx.x * 16 + tx;
   const int kbeg = (lower && transA) ? blockIdx.y * 16 : 0;
   const int kend = (lower && !transA) ? min(n1, (int)(blockIdx.y + 1) * 16) : n1;
-  for (int k0 = kbeg; k0 < kend; k0 += 16) {
-    const int ka = k0 + threadIdx.x, kb = k0 + threadIdx.y;
-    double av = 0.0;
-    if (i < n1 && ka < n1) av = transA ? A[(size_t)ka * n1 + i] : A[(size_t)i * n1 + ka];
-    const double bv = (kb < n1 && j < n2) ? B[(size_t)kb * n2 + j] : 0.0;
-    const float2 as = split64(av), bs = split64(bv);
-    Ah[threadIdx.y][threadIdx.x] = as.x;
-    Al[threadIdx.y][threadIdx.x] = as.y;
-    Bh[threadIdx.y][threadIdx.x] = bs.x;
-    Bl[threadIdx.y][threadIdx.x] = bs.y;
-    __syncthreads();
+  double av[2], bv[2];
+  // two A values (k = tx, tx + 16; A^T: rows along k for coalescing) and two
+  // of B (k = ty, ty + 16)
+  auto fetch = [&](int k0) {
 #pragma unroll
-    for (int k = 0; k < 16; ++k)
-      acc = df_fma(DF{Ah[threadIdx.y][k], Al[threadIdx.y][k]}, DF{Bh[k][threadIdx.x], Bl[k][threadIdx.x]},
-                   acc);
+    for (int h = 0; h < 2; ++h) {
+      const int ia = blockIdx.y * 16 + (transA ? tx : ty), ka = k0 + (transA ? ty : tx) + 16 * h;
+      av[h] = (ia < n1 && ka < kend) ? (transA ? A[(size_t)ka * n1 + ia] : A[(size_t)ia * n1 + ka]) : 0.0;
+      const int kb = k0 + ty + 16 * h;
+      bv[h] = (kb < kend && j < n2) ? B[(size_t)kb * n2 + j] : 0.0;
+    }
+  };
+  T acc = in(0.0);
+  fetch(kbeg);
+  for (int k0 = kbeg; k0 < kend; k0 += KT) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      As[transA ? tx : ty][(transA ? ty : tx) + 16 * h] = in(av[h]);
+      Bs[ty + 16 * h][tx] = in(bv[h]);
+    }
+    __syncthreads();
+    if (k0 + KT < kend) fetch(k0 + KT);
+#pragma unroll
+    for (int k = 0; k < KT; ++k) acc = R::fma_(As[ty][k], Bs[k][tx], acc);
     __syncthreads();
   }
-  if (i < n1 && j < n2) C[(size_t)i * n2 + j] = df_to_double(acc);
+  if (i < n1 && j < n2) {
+    double y;
+    if constexpr (DFM)
+      y = df_to_double(acc);
+    else
+      y = acc;
+    C[(size_t)i * n2 + j] = y;
+  }
 }
 
 // out[v][r] = sign * sum_{j in tile list} W[j][r] H(j, v), H(j, v) =
@@ -1021,9 +1047,8 @@ cudaError_t launch_ace_build(sea_ctx* c) {
                            c->wx.p, digits);
   if (err == cudaSuccess) err = cudaEventRecord(c->xev[0], c->xfer[0]);
   if (err != cudaSuccess) return err;
-  (c->prm.precision == 1 ? k_gram_reduce_df : k_gram_reduce)<<<dim3((n + GR_A - 1) / GR_A, n), GR_A * GR_Z, 0, c->stream>>>(
-      (const double*)c->partial.p, n, n, optr, oslot, c->dV, (double*)c->Mbuf.p,
-      n, 1);
+  launch_gram_reduce(c->stream, c->prm.precision == 1, (const double*)c->partial.p, n, n, optr, oslot,
+                     c->dV, (double*)c->Mbuf.p, n, 1);
   c->launches += 2;
   err = launch_chol_chain(c);
   if (err == cudaSuccess) err = cudaStreamWaitEvent(c->stream, c->xev[0], 0);
@@ -1102,13 +1127,12 @@ cudaError_t launch_ace_apply(sea_ctx* c, const double* psi, int nv, double* out)
     if (e != cudaSuccess) return e;
   }
   cudaEventRecord(c->ev[13], c->stream);
-  (c->prm.precision == 1 ? k_gram_reduce_df : k_gram_reduce)<<<dim3((nv + GR_A - 1) / GR_A, n), GR_A * GR_Z, 0, c->stream>>>(
-      (const double*)c->partial.p, nv, n, optr, oslot, c->dV, (double*)c->Gbuf.p,
-      1, nv);
+  launch_gram_reduce(c->stream, c->prm.precision == 1, (const double*)c->partial.p, nv, n, optr, oslot,
+                     c->dV, (double*)c->Gbuf.p, 1, nv);
   // H = (-Mbar)^-1 G = L^-T (L^-1 G), or Q |Lambda|^-1 Q^T G in the eigen form
   dim3 gb((nv + 15) / 16, (n + 15) / 16), tb(16, 16);
   // the mixed form's products in double-float (the FP64 unit is the bound of the FP64 ones)
-  auto small_gemm = c->prm.precision == 1 ? k_small_gemm_df : k_small_gemm;
+  auto small_gemm = c->prm.precision == 1 ? k_small_gemm<true> : k_small_gemm<false>;
   if (c->ace_eigen) {
     small_gemm<<<gb, tb, 0, c->stream>>>((const double*)c->Linv.p, 1, (const double*)c->Gbuf.p,
                                            n, nv, (double*)c->Hbuf2.p, 0);

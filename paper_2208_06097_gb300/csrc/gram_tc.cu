@@ -16,13 +16,12 @@
 //   D_d = sum_{k+l=d} sum_r dx_k(r) dw_l(r),
 // where every D_d is a sum of at most 6 x 64 products of magnitude <= 2^14,
 // hence an integer below 2^24: the tensor core's FP32 accumulation of it is
-// exact.  The epilogue combines the D_d exactly in 64-bit integers; the
-// per-thread-load kernel rounds each half tile once to FP64 and adds the
-// two halves, the TMA kernel aligns the two halves' integers on the larger
-// scale (the other truncated at its unit, 2^-54 of that segment's scale)
-// and truncates once to FP64, with no FP64 instruction.  Error: the truncation of X
-// (2^-47 of the segment maximum) and the dropped diagonals d >= S (below
-// 2^-45.7 of max|x| max|w| times the segment length).
+// exact.  The epilogue combines the D_d exactly in 64-bit integers, aligns the
+// two halves' integers on the larger scale (the other truncated at its unit,
+// 2^-55 of that segment's scale) and truncates once to FP64, with no FP64
+// instruction.  Error: the truncation of X (2^-47 of the segment maximum) and
+// the dropped diagonals d >= S (below 2^-45.7 of max|x| max|w| times the
+// segment length).
 //
 // The plain form (DIG = 7) has seven digits per operand: 55-bit integers for W,
 // 56-bit ones for A's bytes, seven diagonals (each still below 2^24), each
@@ -45,17 +44,15 @@
 // planes 0..5-k (N = (6 - k) P) adds every product of plane k to the
 // diagonals k..5 at once: 24 tcgen05.mma instructions (M = 128, K = 16) per
 // unit.  After the second half tile the converting warps read the
-// accumulators back with tcgen05.ld for the epilogue.  Two versions:
-//   k_gram_tc_ldg  512 threads load the A rows themselves and form their
-//                  digits in registers while the previous unit's MMAs run
-//                  (issued by thread 0); used when the rows are not
-//                  16-byte strided (odd nx) or A is unaligned;
-//   k_gram_tc      A rows by TMA per K half, 16 converting warps and one
-//                  MMA-issuing warp (described above the kernel).
+// accumulators back with tcgen05.ld for the epilogue (k_gram_tc).  A few rows
+// take k_gram_few, whose partials are the same bits.
 // Every wait on a completion barrier is bounded: on expiry the kernel sets
 // SEA_FLAG_WAIT, waits once more (bounded) for work in flight, frees its
 // tensor memory and ends.
 #include <cuda.h>
+
+#include <climits>
+#include <cstring>
 
 #include "cg_fixed.cuh"
 #include "sea_internal.cuh"
@@ -67,9 +64,6 @@ namespace {
 // DIG digits per operand: 6 in the mixed form, 7 in the plain form
 constexpr int KH = 64;                          // points per half tile
 constexpr int MBLK = 128;                       // A rows per block
-constexpr int GT_THREADS = 512;
-constexpr uint32_t A_PLANE = MBLK * KH * 2;     // bytes per digit plane of A
-constexpr uint32_t A_LBO = (MBLK / 8) * 128;    // K-adjacent core matrices of A
 constexpr uint32_t CORE_SBO = 128;              // row-group-adjacent core matrices
 constexpr uint32_t TMEM_COLS = 512;
 template <int DIG>
@@ -78,9 +72,7 @@ struct GramSizes {
   // for 16 (all but 92 of the 6912 tiles of 256 orbitals on 96^3 have no more)
   static constexpr int NBLK = DIG == 6 ? 32 : 16;
   static constexpr uint32_t W_HALF = DIG * NBLK * KH * 2;  // bytes of W digits per half tile
-  static constexpr uint32_t SMEM_A = DIG * A_PLANE;        // 96 KB with six digits
   static constexpr uint32_t SMEM_W = 2 * W_HALF;           // 48 KB (both halves)
-  static constexpr size_t GT_SMEM = SMEM_A + 2 * SMEM_W + 128;  // A digits, two W buffers
   static constexpr uint32_t TMEM_HALF = DIG * NBLK;        // accumulator columns per half tile
 };
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool valid) {
@@ -191,25 +183,6 @@ __device__ __forceinline__ void make_digits(const double* __restrict__ rp, const
     }
 }
 
-// Digit planes of the group to shared memory (core matrices: row group g
-// 128 B apart, run u one lbo apart, row l % 8 at 16 B), and the exponent
-// (lanes 0..7) to emax_row[l % 8].
-template <int DIG>
-__device__ __forceinline__ void store_digits(const GroupDigits<DIG>& o, unsigned char* plane0,
-                                             uint32_t plane_bytes, uint32_t lbo, int g,
-                                             int* emax_row) {
-  const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int q = 0; q < 2; ++q) {
-    unsigned char* dst = plane0 + g * CORE_SBO + ((lane >> 3) + 4 * q) * lbo + (lane & 7) * 16;
-#pragma unroll
-    for (int k = 0; k < DIG; ++k)
-      *reinterpret_cast<uint4*>(dst + k * plane_bytes) =
-          make_uint4(o.w[q][k][0], o.w[q][k][1], o.w[q][k][2], o.w[q][k][3]);
-  }
-  if (lane < 8) emax_row[lane] = o.emax;
-}
-
 // Integer value of an integer-valued FP32 number at most 2^22 in magnitude:
 // adding 1.5 2^23 puts it in the low mantissa bits.
 __device__ __forceinline__ int small_float_int(uint32_t f) {
@@ -225,16 +198,6 @@ __device__ __forceinline__ double scaled_i64_rz_cvt(long long v, int e2) {
   const int ex = (int)((b >> 52) & 0x7FF) + e2;  // biased exponent of the result
   return (v == 0 || ex <= 0) ? 0.0 : __longlong_as_double(b + ((long long)e2 << 52));
 }
-
-// Exact value of an integer-valued float below 2^24 in magnitude.
-__device__ __forceinline__ int float_int(float f) {
-  const unsigned u = __float_as_uint(f);
-  const int e = (int)((u >> 23) & 255);
-  if (e < 127) return 0;
-  const int mag = (int)(((u & 0x7FFFFFu) | 0x800000u) >> (150 - e));
-  return (u >> 31) ? -mag : mag;
-}
-
 
 // Seven diagonal sums (integer-valued floats, |D_0|, |D_1| < 2^22, the others
 // below 2^24) as y = sum_d D_d 256^(6-d) 2^e0, |y| < 2^(e0 + 62 + DROP): the
@@ -291,237 +254,18 @@ __global__ void __launch_bounds__(256, DIG == 6 ? 4 : 3)
   }
 }
 
-// A unit of work: half h of A block mb against W block jb of tile T, whose
-// W digits are in buffer wb.
+// A unit of work: half h of A block mb against W block jb of tile T, whose W
+// exponents are in buffer wb.
 struct Unit {
   int T, j0, nJ, jb, mb, h, wb;
-  int ab;  // parity of the A block in processing order (TMA kernel: its exponent buffer)
+  int ab;  // parity of the A block in processing order (its exponent buffer)
 };
 
-
-template <int DIG>
-__global__ void __launch_bounds__(GT_THREADS, 1)
-    k_gram_tc_ldg(const double* __restrict__ A, int m, TileGeom G, size_t ng, int n_tiles,
-              const int* __restrict__ tptr, const uint4* __restrict__ wdig,
-              const int* __restrict__ wexp, double* __restrict__ partial, int* __restrict__ queue,
-              unsigned* __restrict__ status) {
-  using Z = GramSizes<DIG>;
-  constexpr int NBLK = Z::NBLK;
-  constexpr uint32_t W_HALF = Z::W_HALF, SMEM_A = Z::SMEM_A, SMEM_W = Z::SMEM_W,
-                     TMEM_HALF = Z::TMEM_HALF;
-  extern __shared__ unsigned char gt_raw[];
-  unsigned char* sA = gt_raw + ((128 - (smem_addr(gt_raw) & 127)) & 127);
-  unsigned char* sW = sA + SMEM_A;  // two buffers of SMEM_W
-  __shared__ int Aexp[2][MBLK], Wexp[2][2][NBLK];  // [half][row], [buffer][half][row]
-  __shared__ __align__(8) unsigned long long mbar;
-  __shared__ uint32_t tmem_base;
-  __shared__ int s_tile, s_fail;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const uint32_t bar = smem_addr(&mbar);
-
-  if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
-                     smem_addr(&tmem_base)),
-                 "r"(TMEM_COLS));
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
-  }
-  if (tid == 0) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar));
-    asm volatile("fence.mbarrier_init.release.cluster;");
-    s_fail = 0;
-  }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem = tmem_base;
-  const uint32_t a_base = smem_addr(sA), w_base = smem_addr(sW);
-  const int nmb = (m + MBLK - 1) / MBLK;
-
-  // first unit of the next tile with a non-empty list; uniform, contains
-  // __syncthreads (false: no tile left)
-  auto claim = [&](Unit& u) -> bool {
-    __syncthreads();
-    if (tid == 0) {
-      int t;
-      do {
-        t = atomicAdd(queue, 1);
-      } while (t < n_tiles && tptr[t + 1] == tptr[t]);
-      s_tile = t;
-    }
-    __syncthreads();
-    const int T = s_tile;
-    if (T >= n_tiles) return false;
-    u.T = T;
-    u.j0 = tptr[T];
-    u.nJ = tptr[T + 1] - u.j0;
-    u.jb = 0;
-    u.mb = 0;
-    u.h = 0;
-    u.wb ^= 1;
-    return true;
-  };
-  // the unit after u; *new_block: it starts another W block
-  auto advance = [&](Unit& u, bool* new_block) -> bool {
-    *new_block = false;
-    if (u.h == 0) {
-      u.h = 1;
-      return true;
-    }
-    u.h = 0;
-    if (++u.mb < nmb) return true;
-    u.mb = 0;
-    *new_block = true;
-    u.jb += NBLK;
-    if (u.jb < u.nJ) {
-      u.wb ^= 1;
-      return true;
-    }
-    return claim(u);
-  };
-  auto a_row = [&](const Unit& u) -> const double* {
-    const int a = u.mb * MBLK + 8 * warp + (lane & 7);
-    return a < m ? A + (size_t)a * ng : nullptr;
-  };
-  // W digits of u's block (both halves) into buffer u.wb, planes stacked
-  // along N with row stride P (16 or 32): row l P + slot of half h at core
-  // matrix (row / 8, run), K-adjacent ones 6 P 16 bytes apart.  16-byte
-  // asynchronous copies, zeros beyond the list (completed before the next
-  // __syncthreads that precedes the MMAs reading them).
-  auto load_w = [&](const Unit& u) {
-    const int nj = min(NBLK, u.nJ - u.jb), P = nj <= 16 ? 16 : 32;
-    const uint32_t lbo = DIG * P * 16;
-    const uint32_t dst0 = w_base + u.wb * SMEM_W;
-    for (int p = tid; p < P * 2 * DIG * 8; p += GT_THREADS) {
-      const int run = p & 7, k = (p >> 3) % DIG, h = (p / (8 * DIG)) & 1, sl = p / (16 * DIG);
-      const bool ok = sl < nj;
-      const uint4* src = ok ? wdig + ((size_t)(u.j0 + u.jb + sl) * 2 + h) * DIG * 8 + k * 8 + run : wdig;
-      const int row = k * P + sl;
-      cp_async16(dst0 + h * W_HALF + (row >> 3) * CORE_SBO + run * lbo + (row & 7) * 16, src, ok);
-    }
-    if (tid < 2 * NBLK) {
-      const int h = tid / NBLK, sl = tid % NBLK;
-      Wexp[u.wb][h][sl] = sl < nj ? wexp[(size_t)(u.j0 + u.jb + sl) * 2 + h] : 0;
-    }
-  };
-  // partials of u's A block (both halves done): warp = (lane quarter q,
-  // column class g), columns g, g + 4, ... of the block
-  auto epilogue = [&](const Unit& u) {
-    const int nj = min(NBLK, u.nJ - u.jb), P = nj <= 16 ? 16 : 32;
-    const int quarter = warp & 3, g = warp >> 2;
-    const int a = u.mb * MBLK + 32 * quarter + lane;
-    const uint32_t lane_addr = tmem + ((uint32_t)(32 * quarter) << 16);
-    const int ea0 = Aexp[0][32 * quarter + lane] - 1022, ea1 = Aexp[1][32 * quarter + lane] - 1022;
-#pragma unroll 1
-    for (int c = g; c < nj; c += 4) {
-      uint32_t f[2 * DIG];
-#pragma unroll
-      for (int q = 0; q < 2 * DIG; ++q)
-        f[q] = tmem_ld1(lane_addr + (uint32_t)((q / DIG) * TMEM_HALF + (q % DIG) * P + c));
-      tmem_wait_ld();
-      double sum = 0.0;
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int ea = h ? ea1 : ea0, ew = Wexp[u.wb][h][c];
-        if constexpr (DIG == 7) {
-          const bool bad = ea + 1022 == EXP_NONFINITE || ew == EXP_NONFINITE;
-          sum += bad ? quiet_nan() : combine7<6>(f + h * DIG, ea + ew - 1022 - 62);
-        } else {
-          long long acc = 0;
-#pragma unroll
-          for (int d = 0; d < DIG; ++d)
-            acc += (long long)float_int(__uint_as_float(f[h * DIG + d])) << (8 * (DIG - 1 - d));
-          sum += scaled_i64(acc, ea + (ew - 1022) - 54);
-        }
-      }
-      if (a < m) partial[(size_t)(u.j0 + u.jb + c) * m + a] = sum;
-    }
-  };
-  // the MMAs of unit u (half u.h), then the commit: for K step q and A
-  // plane k, one MMA against W planes 0..5-k into diagonals k..5
-  auto issue = [&](const Unit& u) {
-    const int nj = min(NBLK, u.nJ - u.jb), P = nj <= 16 ? 16 : 32;
-    const uint32_t lbo = DIG * P * 16;
-    // descriptors differ only in the start address (low 14 bits, no
-    // carry: shared addresses are below 2^18)
-    const uint64_t a0 = sdesc(a_base, A_LBO, CORE_SBO);
-    const uint64_t w0 = sdesc(w_base + u.wb * SMEM_W + u.h * W_HALF, lbo, CORE_SBO);
-    const uint32_t dcol = tmem + (uint32_t)(u.h * TMEM_HALF);
-#pragma unroll
-    for (int q = 0; q < KH / 16; ++q)
-#pragma unroll
-      for (int k = 0; k < DIG; ++k)
-        mma_kf16(dcol + (uint32_t)(k * P), a0 + ((k * A_PLANE + q * 2 * A_LBO) >> 4),
-                 w0 + ((q * 2 * lbo) >> 4), idesc_kf16((DIG - k) * P, MBLK, false), (k > 0 || q > 0) ? 1u : 0u);
-    asm volatile(
-        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
-        : "memory");
-  };
-
-  Unit cur;
-  cur.wb = 1;
-  if (claim(cur)) {
-    load_w(cur);
-    GroupDigits<DIG> dg;
-    make_digits(a_row(cur), G, cur.T, cur.h, dg);
-    Unit prev = cur;
-    bool have_prev = false;
-    uint32_t phase = 0;
-    for (;;) {
-      if (have_prev) {
-        // prev's MMAs done: the A digits and the accumulators are free
-        const bool ok = mbar_wait(bar, phase);
-        if (!ok) s_fail = 1;
-        __syncthreads();
-        if (s_fail) break;
-        phase ^= 1;
-        tc_fence_after();
-        if (prev.h == 1) {
-          epilogue(prev);
-          __syncthreads();  // the exponents are read before they are replaced
-        }
-      }
-      store_digits(dg, sA, A_PLANE, A_LBO, warp, &Aexp[cur.h][8 * warp]);
-      cp_async_wait_all();
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      tc_fence_before();
-      __syncthreads();
-      tc_fence_after();
-      if (tid == 0) issue(cur);
-      prev = cur;
-      have_prev = true;
-      // while the MMAs run: the next unit's W digits (a new block goes to
-      // the other buffer, whose MMAs are done) and A digits
-      bool new_block;
-      if (!advance(cur, &new_block)) break;
-      if (new_block) load_w(cur);
-      make_digits(a_row(cur), G, cur.T, cur.h, dg);
-    }
-    // the last unit: its MMAs (bounded wait) and epilogue
-    if (!s_fail) {
-      const bool ok = mbar_wait(bar, phase);
-      if (!ok) s_fail = 1;
-      __syncthreads();
-      if (!s_fail) {
-        tc_fence_after();
-        if (prev.h == 1) epilogue(prev);
-      }
-    }
-    if (s_fail) mbar_wait(bar, phase);  // once more, bounded, before freeing
-  }
-  cp_async_wait_all();
-  if (s_fail && tid == 0) atomicOr(status, SEA_FLAG_WAIT);
-  tc_fence_before();
-  __syncthreads();
-  if (warp == 0) {
-    tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
-                 "r"(TMEM_COLS));
-  }
-}
-
 // ---------------------------------------------------------------------------
-// The same contraction with A's rows brought in by the tensor memory
-// accelerator.  Per unit two 4D boxes (x 8, y 4, z 1, rows 128): the two
+// The contraction's kernel.  A's rows come in by the tensor memory accelerator
+// or, where the rows are not 16-byte strided (odd nx) or A is unaligned (TMA =
+// false), by 8-byte asynchronous copies of every warp's own rows into the same
+// places.  Per unit two 4D boxes (x 8, y 4, z 1, rows 128): the two
 // z-planes of the half tile (K halves 0 and 1) for the whole A block, 32 KB
 // each, written with the 64-byte swizzle so that the reads below are free
 // of bank conflicts.  Thread t takes row t / 4 and the x-run y = t % 4 of
@@ -687,9 +431,10 @@ __device__ __forceinline__ bool conv_sync_or(bool v) {
   return r != 0;
 }
 
-template <int DIG>
+template <int DIG, bool TMA>
 __global__ void __launch_bounds__(GT2_THREADS, 1)
-    k_gram_tc(const __grid_constant__ CUtensorMap tmA, int m, TileGeom G, int n_tiles,
+    k_gram_tc(const __grid_constant__ CUtensorMap tmA, const double* __restrict__ A, size_t ng, int m,
+              TileGeom G, int n_tiles,
               const int* __restrict__ tptr, const uint4* __restrict__ wdig,
               const int* __restrict__ wexp, double* __restrict__ partial, int* __restrict__ queue,
               unsigned* __restrict__ status) {
@@ -725,7 +470,8 @@ __global__ void __launch_bounds__(GT2_THREADS, 1)
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(rb[q]));
     }
     asm volatile("fence.mbarrier_init.release.cluster;");
-    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmA)) : "memory");
+    if (TMA)
+      asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmA)) : "memory");
     s_fail = 0;
     s_ifail = 0;
   }
@@ -857,6 +603,31 @@ __global__ void __launch_bounds__(GT2_THREADS, 1)
       u.jb += NBLK;
       if (u.jb < u.nJ) return true;
       return claim(u);
+    };
+    // the same without the accelerator: every warp copies its own eight rows
+    // (a row's 4 x 8 points of a plane per instruction; zeros outside the grid
+    // and beyond m), in flight until cp_async_wait_all and a warp barrier
+    auto raw_copy = [&](const Unit& u) {
+      const int txi = u.T % G.ntx, tyi = (u.T / G.ntx) % G.nty, tzi = u.T / (G.ntx * G.nty);
+      const int rn = lane >> 3, x = lane & 7, gx = txi * TX + x, gy = tyi * TY + rn;
+      const uint32_t dx = (uint32_t)(rn * 64 + 8 * (x & 1));
+      __syncwarp();  // the lanes have read the values that are replaced
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const int z = tzi * TZ + 2 * u.h + q;
+        const bool in = gx < G.nx && gy < G.ny && z < G.nz;
+        const double* src = A + (in ? ((size_t)z * G.ny + gy) * G.nx + gx : 0);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const int r = 8 * warp + i, a = u.mb * MBLK + r;
+          const uint32_t swz = (uint32_t)((((r & 1) << 1) | (rn >> 1)) << 4);
+          const bool ok = in && a < m;
+          asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(
+                           r_base + q * RAW_KHALF + r * 256 + dx + (((uint32_t)(x >> 1) << 4) ^ swz)),
+                       "l"(ok ? src + (size_t)a * ng : A), "r"(ok ? 8 : 0)
+                       : "memory");
+        }
+      }
     };
     // K half q (z-plane 2 h + q of the half tile) of unit u's A block (thread 0)
     auto tma_issue = [&](const Unit& u, int q) {
@@ -1004,15 +775,23 @@ __global__ void __launch_bounds__(GT2_THREADS, 1)
     // the MMA completion barriers, the A exponents double-buffered by A block.
     if (claim(cur)) {
       load_w(cur);
-      if (tid == TMA_TID) {
+      if (!TMA) {
+        raw_copy(cur);
+      } else if (tid == TMA_TID) {
         tma_issue(cur, 0);
         tma_issue(cur, 1);
       }
       bool need_w = false;
       for (;;) {
         // both K halves of cur to registers; the row's exponent
-        bool ok = wait_raw(0);
-        ok = wait_raw(1) && ok;
+        bool ok = true;
+        if (TMA) {
+          ok = wait_raw(0);
+          ok = wait_raw(1) && ok;
+        } else {
+          cp_async_wait_all();
+          __syncwarp();
+        }
         double v[2][8];
         uint32_t emf = 0;  // largest exponent field (high-word bits 20..30) of the row segment
 #pragma unroll
@@ -1031,14 +810,16 @@ __global__ void __launch_bounds__(GT2_THREADS, 1)
         const int em = (int)(emf >> 20);
         const uint32_t em_sh = DIG == 6 ? (em < 64 ? 0xF0000000u : emf + (5u << 20)) : emf;
         if (tid == 0) q_step();
-        if (conv_sync_or(!ok)) {  // B1: both raw buffers consumed
+        if (TMA && conv_sync_or(!ok)) {  // B1: both raw buffers consumed
           fail = true;
           break;
         }
         Unit next = cur;
         bool new_block = false;
         const bool has_next = advance(next, &new_block);  // may claim (uniform, syncs)
-        if (tid == TMA_TID && has_next) {
+        if (!TMA) {
+          if (has_next) raw_copy(next);
+        } else if (tid == TMA_TID && has_next) {
           tma_issue(next, 0);
           tma_issue(next, 1);
         }
@@ -1056,7 +837,7 @@ __global__ void __launch_bounds__(GT2_THREADS, 1)
         // above) and its exponents sit in the other buffer
         if (need_w) load_w(cur);
         if (run == 0) Aexp[cur.ab][cur.h][row] = em;
-        cp_async_wait_all();
+        if (TMA || need_w || !have_prev) cp_async_wait_all();  // W's digits
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         tc_fence_before();
         if (conv_sync_or(!ok)) {  // B2: digits, W and exponents in place
@@ -1104,6 +885,138 @@ __global__ void __launch_bounds__(GT2_THREADS, 1)
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
                  "r"(TMEM_COLS));
+  }
+}
+
+// ---------------------------------------------------------------------------
+// A few rows of A (an operator applied to one or a handful of vectors): the
+// kernel above works on 128 rows per unit whatever their number, so up to
+// GRAM_FEW rows each warp takes 16 list entries of a tile against eight rows
+// with the warp-wide mma.sync.m16n8k16 (FP16 operands, FP32 accumulators): W's
+// digits straight from their global image as the A fragments, the rows'
+// digits formed in registers as the B fragments.  The contraction index is
+// permuted so that a thread's four fragment words are one 16-byte piece of
+// the image.  Digits, diagonals and the final combination are those of
+// k_gram_tc, every D_d the same exact integer, so the partials are the same
+// bits.  Bound by the latency of its loads and conversions; 8 rows of 75^3
+// against 128 orbitals 320 -> 46 us.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void mma_16816(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2,
+                                          uint32_t a3, uint32_t b0, uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, "
+      "{%8, %9}, {%0, %1, %2, %3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+// acc of the six diagonals (k_gram_tc's epilogue): sum_d D_d 256^(5-d)
+__device__ __forceinline__ long long combine6(const uint32_t* f) {
+  const int t01 = small_float_int(f[0]) * 256 + small_float_int(f[1]);
+  const int t23 =
+      __float2int_rz(__uint_as_float(f[2])) * 256 + __float2int_rz(__uint_as_float(f[3]));
+  return ((long long)t01 << 32) + ((long long)t23 << 16) +
+         ((long long)__float2int_rz(__uint_as_float(f[4])) << 8) +
+         (long long)__float2int_rz(__uint_as_float(f[5]));
+}
+// two half tiles' sums on the larger scale, one truncation
+__device__ __forceinline__ double join6(long long a0, int e0, long long a1, int e1) {
+  const bool b0 = e0 >= e1;
+  const int sh = min(b0 ? e0 - e1 : e1 - e0, 63);
+  return scaled_i64_rz_cvt((b0 ? a0 : a1) + ((b0 ? a1 : a0) >> sh), b0 ? e0 : e1);
+}
+
+constexpr int FEW_WARPS = 4;
+// Rows (GRAM_FEW) and vectors (EXPAND_FEW) up to which the warp-wide kernels are
+// the faster ones.  Measured (128 orbitals on 76^3, six digits): contraction of
+// 8, 24, 32 rows 51, 98, 125 us against 169 to 171 (256 orbitals on 96^3: 32
+// rows 302 against 316); expansion of 8 and 16 vectors 49 and 88 us against 83.
+constexpr int GRAM_FEW = 32, EXPAND_FEW = 8;
+template <int DIG>
+__global__ void __launch_bounds__(32 * FEW_WARPS)
+    k_gram_few(const double* __restrict__ A, int m, TileGeom G, size_t ng, int n_tiles,
+               const int* __restrict__ tptr, const uint4* __restrict__ wdig,
+               const int* __restrict__ wexp, double* __restrict__ partial) {
+  const int T = blockIdx.x * FEW_WARPS + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (T >= n_tiles) return;  // warp-uniform
+  const int j0 = tptr[T], nJ = tptr[T + 1] - j0;
+  if (nJ == 0) return;
+  const int a0 = blockIdx.y * 8, g = lane >> 2, q = lane & 3;
+  const int txi = T % G.ntx, tyi = (T / G.ntx) % G.nty, tzi = T / (G.ntx * G.nty);
+  const int x0 = txi * TX, y = tyi * TY + q;
+  double lead[4][2];   // seven digits: the first half's values [entry half, row pair]
+  long long acc0[4];   // six digits: the first half's integers
+  int e0[4];
+  for (int s0 = 0; s0 < nJ; s0 += 16) {
+#pragma unroll 1
+    for (int h = 0; h < 2; ++h) {
+      // row a0 + g: x-runs y = q of the planes 2h, 2h + 1
+      uint4 d[2][DIG];
+      double v[2][8];
+      uint32_t emf = 0;
+#pragma unroll
+      for (int qq = 0; qq < 2; ++qq) {
+        const int z = tzi * TZ + 2 * h + qq;
+        const bool in = a0 + g < m && y < G.ny && z < G.nz;
+        const double* src = A + (in ? (size_t)(a0 + g) * ng + ((size_t)z * G.ny + y) * G.nx + x0 : 0);
+#pragma unroll
+        for (int x = 0; x < 8; ++x) {
+          v[qq][x] = (in && x0 + x < G.nx) ? src[x] : 0.0;
+          emf = max(emf, (uint32_t)__double2hiint(v[qq][x]) & 0x7FF00000u);
+        }
+      }
+      emf = max(emf, __shfl_xor_sync(0xffffffffu, emf, 1));
+      emf = max(emf, __shfl_xor_sync(0xffffffffu, emf, 2));
+      const int em = (int)(emf >> 20);
+      const uint32_t em_sh = DIG == 6 ? (em < 64 ? 0xF0000000u : emf + (5u << 20)) : emf;
+      digits8_u<DIG>(v[0], em_sh, d[0]);
+      digits8_u<DIG>(v[1], em_sh, d[1]);
+      float c[DIG][4];
+#pragma unroll
+      for (int k = 0; k < DIG; ++k) c[k][0] = c[k][1] = c[k][2] = c[k][3] = 0.f;
+      // entries s0 + g and s0 + g + 8 (zeros beyond the list)
+      const bool in0 = s0 + g < nJ, in1 = s0 + g + 8 < nJ;
+      const uint4* w0 = wdig + ((size_t)(j0 + s0 + (in0 ? g : 0)) * 2 + h) * DIG * 8 + q;
+      const uint4* w1 = wdig + ((size_t)(j0 + s0 + (in1 ? g + 8 : 0)) * 2 + h) * DIG * 8 + q;
+#pragma unroll
+      for (int l = 0; l < DIG; ++l) {
+        const uint4 z4 = make_uint4(0, 0, 0, 0);
+#pragma unroll
+        for (int qq = 0; qq < 2; ++qq) {
+          const uint4 u0 = in0 ? w0[l * 8 + 4 * qq] : z4, u1 = in1 ? w1[l * 8 + 4 * qq] : z4;
+#pragma unroll
+          for (int k = 0; k + l < DIG; ++k) {
+            mma_16816(c[k + l], u0.x, u1.x, u0.y, u1.y, d[qq][k].x, d[qq][k].y);
+            mma_16816(c[k + l], u0.z, u1.z, u0.w, u1.w, d[qq][k].z, d[qq][k].w);
+          }
+        }
+      }
+      // c[d][i]: entry s0 + g + 8 (i / 2), row a0 + 2 q + (i & 1)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int s = s0 + g + 8 * (i >> 1), a = a0 + 2 * q + (i & 1);
+        const int ea = __shfl_sync(0xffffffffu, em, 8 * q + 4 * (i & 1));
+        const int ew = s < nJ ? wexp[(size_t)(j0 + s) * 2 + h] : 0;
+        uint32_t f[DIG];
+#pragma unroll
+        for (int k = 0; k < DIG; ++k) f[k] = __float_as_uint(c[k][i]);
+        double y0 = 0.0;
+        if constexpr (DIG == 7) {
+          const bool bad = ea == EXP_NONFINITE || ew == EXP_NONFINITE;
+          const double yh = bad ? quiet_nan() : combine7<7>(f, ea - 1022 + ew - 1022 - 63);
+          if (h == 0) lead[i][0] = 0.0 + yh;
+          y0 = lead[i][0] + yh;
+        } else {
+          const long long ac = combine6(f);
+          const int e = ea - 1022 + ew - 1022 - 55;
+          if (h == 0) {
+            acc0[i] = ac;
+            e0[i] = e;
+          }
+          y0 = join6(acc0[i], e0[i], ac, e);
+        }
+        if (h == 1 && s < nJ && a < m) partial[(size_t)(j0 + s) * m + a] = y0;
+      }
+    }
   }
 }
 
@@ -1587,6 +1500,83 @@ __global__ void __launch_bounds__(XE_THREADS, 1)
   }
 }
 
+// The expansion for a few vectors, the counterpart of k_gram_few: CTA per
+// tile, warp w the points 16 w .. + 15 against eight vectors, W's image as the
+// A fragments, H's digits formed in registers as the B fragments, E_v over the
+// tile's list by the warp itself.  The outputs are k_expand_tc's bits.
+template <int DIG>
+__global__ void __launch_bounds__(256)
+    k_expand_few(const uint4* __restrict__ wx, const int* __restrict__ wxexp, TileGeom G, size_t ng,
+                 const int* __restrict__ tptr, const int* __restrict__ tlist,
+                 const double* __restrict__ H, long long hj, long long hv, int m, int negate,
+                 double* __restrict__ out) {
+  constexpr uint32_t XA_STEP = ExpandSizes<DIG>::XA_STEP, XA_TILE = 2 * XA_STEP;
+  const int T = blockIdx.x, v0 = blockIdx.y * 8;
+  const int j0 = tptr[T], nJ = tptr[T + 1] - j0;
+  if (nJ > XJ) return;  // uniform: the long-list kernel's
+  const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3, p0 = 16 * (threadIdx.x >> 5);
+  const long long o0 = tile_point(G, T, p0 + g), o1 = tile_point(G, T, p0 + g + 8);
+  float c[DIG][4];
+#pragma unroll
+  for (int k = 0; k < DIG; ++k) c[k][0] = c[k][1] = c[k][2] = c[k][3] = 0.f;
+  // entries j = 16 s + {2q, 2q + 1, 8 + 2q, 9 + 2q} of vector v0 + g
+  double hval[2][4];
+  int sh[2][4], em = 0;
+#pragma unroll
+  for (int s = 0; s < 2; ++s)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int j = 16 * s + 2 * q + (i & 1) + 8 * (i >> 1);
+      const bool in = j < nJ && v0 + g < m;
+      double h = in ? H[(long long)tlist[j0 + j] * hj + (long long)(v0 + g) * hv] : 0.0;
+      const int e = (__double2hiint(h) >> 20) & 0x7FF, w = j < nJ ? wxexp[j0 + j] : 0;
+      if (e) em = max(em, e + w - 1022);
+      if (DIG == 7 && in && (e == EXP_NONFINITE || w == EXP_NONFINITE)) em = EV_NONFINITE;
+      if (negate) h = __longlong_as_double(__double_as_longlong(h) ^ (long long)0x8000000000000000ULL);
+      hval[s][i] = h;
+      sh[s][i] = j < nJ ? w - 1022 : INT_MIN;
+    }
+  em = max(em, __shfl_xor_sync(0xffffffffu, em, 1));
+  em = max(em, __shfl_xor_sync(0xffffffffu, em, 2));
+  const unsigned char* base = reinterpret_cast<const unsigned char*>(wx) + (size_t)T * XA_TILE;
+#pragma unroll
+  for (int s = 0; s < 2; ++s) {
+    if (16 * s >= nJ) break;  // uniform
+    uint32_t pk[DIG][2];
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const int s0 = sh[s][2 * e], s1 = sh[s][2 * e + 1];
+      digits2_u<DIG>(hval[s][2 * e], hval[s][2 * e + 1], s0 != INT_MIN ? em - s0 : 0,
+                     s1 != INT_MIN ? em - s1 : 0, pk, e);
+    }
+#pragma unroll
+    for (int k = 0; k < DIG; ++k) {
+      const unsigned char* a = base + (s * DIG + k) * XA_BLOCK + (p0 >> 3) * 128 + g * 16 + q * 4;
+      auto word = [&](uint32_t off) { return __ldg(reinterpret_cast<const uint32_t*>(a + off)); };
+      const uint32_t a0 = word(0), a1 = word(128), a2 = word(XA_LBO), a3 = word(XA_LBO + 128);
+#pragma unroll
+      for (int l = 0; k + l < DIG; ++l) mma_16816(c[k + l], a0, a1, a2, a3, pk[l][0], pk[l][1]);
+    }
+  }
+  // c[d][i]: point p0 + g + 8 (i / 2), vector v0 + 2 q + (i & 1)
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int v = v0 + 2 * q + (i & 1);
+    const long long o = i < 2 ? o0 : o1;
+    const int ev = __shfl_sync(0xffffffffu, em, 8 * q + 4 * (i & 1));
+    uint32_t f[DIG];
+#pragma unroll
+    for (int k = 0; k < DIG; ++k) f[k] = __float_as_uint(c[k][i]);
+    double val;
+    if constexpr (DIG == 7)
+      val = ev >= EV_NONFINITE ? quiet_nan() : combine7<6>(f, ev - 1022 - 63);
+    else
+      val = scaled_i64_rz_cvt(combine6(f), ev - 1022 - 55);
+    if (nJ == 0) val = 0.0;
+    if (o >= 0 && v < m) out[(size_t)v * ng + o] = val;
+  }
+}
+
 }  // namespace
 
 
@@ -1678,6 +1668,11 @@ static cudaError_t expand_tc(cudaStream_t st, int device, const void* wxbuf, con
   if (n_tiles <= 0 || m <= 0) return cudaSuccess;
   const uint4* wx = (const uint4*)wxbuf;
   const int* wxexp = (const int*)((const unsigned char*)wxbuf + (size_t)n_tiles * xa_tile(DIG));
+  if (m <= EXPAND_FEW) {
+    k_expand_few<DIG><<<dim3(n_tiles, (m + 7) / 8), 256, 0, st>>>(wx, wxexp, G, ng, tptr, tlist, H, hj,
+                                                                  hv, m, negate ? 1 : 0, out);
+    return cudaGetLastError();
+  }
   int nsm = 0;
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, device);
   e = cudaMemsetAsync(queue, 0, sizeof(int), st);
@@ -1704,28 +1699,27 @@ template <int DIG>
 static cudaError_t gram_tc(cudaStream_t st, int device, const double* A, int m, const TileGeom& G,
                            size_t ng, int n_tiles, const int* tptr, long long slots,
                            const void* wbuf, double* partial, int* queue, unsigned* status) {
-  constexpr size_t smem_ldg = GramSizes<DIG>::GT_SMEM, smem_tma = GramTmaSizes<DIG>::SMEM;
-  static_assert(smem_ldg <= 232448 - 4096 && smem_tma <= 232448 - 4096, "shared memory of an SM");
-  cudaError_t e = cudaFuncSetAttribute(k_gram_tc_ldg<DIG>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_ldg);
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_gram_tc<DIG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)smem_tma);
-  if (e != cudaSuccess) return e;
+  constexpr size_t smem = GramTmaSizes<DIG>::SMEM;
+  static_assert(smem <= 232448 - 4096, "shared memory of an SM");
   const uint4* wdig = (const uint4*)wbuf;
   const int* wexp = w_digits_exp(wbuf, slots, DIG);
+  if (m <= GRAM_FEW) {
+    k_gram_few<DIG><<<dim3((n_tiles + FEW_WARPS - 1) / FEW_WARPS, (m + 7) / 8), 32 * FEW_WARPS, 0, st>>>(
+        A, m, G, ng, n_tiles, tptr, wdig, wexp, partial);
+    return cudaGetLastError();
+  }
   int nsm = 0;
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, device);
-  e = cudaMemsetAsync(queue, 0, sizeof(int), st);
-  if (e != cudaSuccess) return e;
-  const int grid = std::min(nsm, std::max(n_tiles, 1));
   alignas(64) CUtensorMap map;
-  if (make_a_map(A, m, G, &map))
-    k_gram_tc<DIG><<<grid, GT2_THREADS, smem_tma, st>>>(map, m, G, n_tiles, tptr, wdig, wexp,
-                                                       partial, queue, status);
-  else
-    k_gram_tc_ldg<DIG><<<grid, GT_THREADS, smem_ldg, st>>>(A, m, G, ng, n_tiles, tptr, wdig, wexp,
-                                                          partial, queue, status);
+  memset(&map, 0, sizeof(map));
+  const bool tma = make_a_map(A, m, G, &map);
+  auto kern = tma ? k_gram_tc<DIG, true> : k_gram_tc<DIG, false>;
+  cudaError_t e =
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e == cudaSuccess) e = cudaMemsetAsync(queue, 0, sizeof(int), st);
+  if (e != cudaSuccess) return e;
+  kern<<<std::min(nsm, std::max(n_tiles, 1)), GT2_THREADS, smem, st>>>(
+      map, A, ng, m, G, n_tiles, tptr, wdig, wexp, partial, queue, status);
   return cudaGetLastError();
 }
 

@@ -78,3 +78,26 @@ def test_non_finite_vectors_are_not_hidden(bad, nx):
         ctx.apply_ace(psi, y)
         assert torch.isnan(y[1]).all()
         assert torch.isfinite(y[0]).all() and torch.isfinite(y[2]).all()
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("nx", [24, 23])
+def test_vector_count_does_not_change_the_bits(precision, nx):
+    # a few vectors go through warp-wide kernels, more through the 128-row
+    # ones: the same digits and sums, hence the same bits
+    from paper_2208_06097_gb300 import sea
+    grid = (nx, 21, 22)
+    F, dV = _orthonormal(19, grid, 2, 1.0)
+    shape = (19, 22, 21, nx)
+    W = -F - 0.3 * np.roll(F, 1, axis=0) - 0.3 * np.roll(F, -1, axis=0)
+    with sea.Context((L,) * 3, grid, precision=precision) as ctx:
+        ctx.set_orbitals(torch.from_numpy(F.reshape(shape).copy()).cuda())
+        ctx.build_ace_from(torch.from_numpy(W.reshape(shape).copy()).cuda())
+        psi = torch.randn((41, 22, 21, nx), dtype=torch.float64, device="cuda")
+        whole = torch.empty_like(psi)
+        ctx.apply_ace(psi, whole)
+        for m in (1, 8, 9, 32, 33):
+            y = torch.full((m,) + shape[1:], float("nan"), dtype=torch.float64, device="cuda")
+            ctx.apply_ace(psi[:m].contiguous(), y)
+            torch.cuda.synchronize()
+            assert torch.equal(y, whole[:m]), m
