@@ -284,8 +284,8 @@ __global__ void __launch_bounds__(256)
 
 // out[a * sa + o * so] = scale * sum over the tiles of o of partial[slot][a].
 // A CTA per (orbital o, GR_A values of a): its four thread groups z take the
-// slots z, z + 4, z + 8, ... of o's list (eight loads in flight each, the next
-// eight slots' numbers fetched beside them, added in list order), and the four
+// slots z, z + 4, z + 8, ... of o's list (eight loads in flight each, added in
+// list order), and the four
 // sums are added in the order z = 0, 1, 2, 3, whatever GR_A (8 for at most
 // eight values, where 64 would leave most threads idle).  DFM (mixed form):
 // sums in double-float (the partials split exactly to FP32 pairs, sums on the
@@ -317,25 +317,37 @@ __global__ void __launch_bounds__(GR_A* GR_Z)
   if (a < m) {
     int k = optr[o] + z;
     const int k1 = optr[o + 1];
-    int idx[8];
+    if (GR_A >= 64) {
+      for (; k + 7 * GR_Z < k1; k += 8 * GR_Z) {
+        double p[8];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) idx[u] = k + u * GR_Z < k1 ? oslot[k + u * GR_Z] : -1;
-    for (; k < k1; k += 8 * GR_Z) {
-      double p[8];
-      bool use[8];
+        for (int u = 0; u < 8; ++u) p[u] = partial[(size_t)oslot[k + u * GR_Z] * m + a];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        use[u] = idx[u] >= 0;
-        p[u] = use[u] ? partial[(size_t)idx[u] * m + a] : 0.0;
+        for (int u = 0; u < 8; ++u) s = add(s, in(p[u]));
       }
+      for (; k < k1; k += GR_Z) s = add(s, in(partial[(size_t)oslot[k] * m + a]));
+    } else {
+      // one warp per CTA: latency-bound, the next slots' numbers beside the loads
+      int idx[8];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int kn = k + (8 + u) * GR_Z;
-        idx[u] = kn < k1 ? oslot[kn] : -1;
+      for (int u = 0; u < 8; ++u) idx[u] = k + u * GR_Z < k1 ? oslot[k + u * GR_Z] : -1;
+      for (; k < k1; k += 8 * GR_Z) {
+        double p[8];
+        bool use[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          use[u] = idx[u] >= 0;
+          p[u] = use[u] ? partial[(size_t)idx[u] * m + a] : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const int kn = k + (8 + u) * GR_Z;
+          idx[u] = kn < k1 ? oslot[kn] : -1;
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+          if (use[u]) s = add(s, in(p[u]));
       }
-#pragma unroll
-      for (int u = 0; u < 8; ++u)
-        if (use[u]) s = add(s, in(p[u]));
     }
   }
   red[z][x] = s;

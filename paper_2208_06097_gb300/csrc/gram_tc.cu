@@ -24,8 +24,8 @@
 // segment length).
 //
 // The plain form (DIG = 7) has seven digits per operand: 55-bit integers for W,
-// 56-bit ones for A's bytes, seven diagonals (each still below 2^24), each
-// half tile rounded to nearest and the two added in FP64.  Values within a
+// 56-bit ones for A's bytes, seven diagonals (each still below 2^24), the two
+// halves' sums to 2^-55 of the larger scale, one rounding.  Values within a
 // factor of 8 (A) or 4 (W) of their segment's largest are kept whole, the
 // others to 2^-56 and 2^-55 of it, and the dropped diagonals stay below 2^-54
 // of max|x| max|w| per product: the error of a partial is below the rounding
@@ -200,24 +200,34 @@ __device__ __forceinline__ double scaled_i64_rz_cvt(long long v, int e2) {
 }
 
 // Seven diagonal sums (integer-valued floats, |D_0|, |D_1| < 2^22, the others
-// below 2^24) as y = sum_d D_d 256^(6-d) 2^e0, |y| < 2^(e0 + 62 + DROP): the
-// sum's lowest DROP bits truncated so that 64 bits hold it, one rounding to
-// nearest (the conversion instruction, on the FP64 pipe that the integer
-// epilogues leave idle), the scaling added to the exponent field.
+// below 2^24) as the integer sum_d D_d 256^(6-d) with its lowest DROP bits
+// truncated, so that 64 bits hold it.
 template <int DROP>
-__device__ __forceinline__ double combine7(const uint32_t* f, int e0) {
+__device__ __forceinline__ long long combine7(const uint32_t* f) {
   auto big = [](uint32_t x) { return __float2int_rz(__uint_as_float(x)); };
   const long long hi = (long long)(small_float_int(f[0]) * 256 + small_float_int(f[1])) * 4096 +
                        (long long)big(f[2]) * 16;
   const long long lo = (long long)big(f[3]) * 16777216 + (long long)big(f[4]) * 65536 +
                        (long long)big(f[5]) * 256 + (long long)big(f[6]);
-  const long long v = (hi << (28 - DROP)) + (lo >> DROP);
-  const int e2 = e0 + DROP;
+  return (hi << (28 - DROP)) + (lo >> DROP);
+}
+// v 2^e2 rounded to nearest: the conversion instruction (on the FP64 pipe that
+// the integer epilogues leave idle), the scaling added to the exponent field;
+// 0 below the normal range, infinite above it.
+__device__ __forceinline__ double scaled_i64_rn_cvt(long long v, int e2) {
   const long long b = __double_as_longlong(__ll2double_rn(v));
   const int ex = (int)((b >> 52) & 0x7FF) + e2;  // biased exponent of the result
   if (v == 0 || ex <= 0) return 0.0;
   if (ex >= 0x7FF) return __longlong_as_double((b & (1LL << 63)) | 0x7FF0000000000000LL);
   return __longlong_as_double(b + ((long long)e2 << 52));
+}
+// Two half tiles' sums (combine7<8>: below 2^61, units 2^e0 and 2^e1) on the
+// larger scale, one rounding; NaN if `bad`.
+__device__ __forceinline__ double join7(long long a0, int e0, long long a1, int e1, bool bad) {
+  const bool b0 = e0 >= e1;
+  const int sh = min(b0 ? e0 - e1 : e1 - e0, 63);
+  const double y = scaled_i64_rn_cvt((b0 ? a0 : a1) + ((b0 ? a1 : a0) >> sh), b0 ? e0 : e1);
+  return bad ? __longlong_as_double(0x7FF8000000000000LL) : y;
 }
 __device__ __forceinline__ double quiet_nan() { return __longlong_as_double(0x7FF8000000000000LL); }
 constexpr int EXP_NONFINITE = 0x7FF;
@@ -691,8 +701,8 @@ __global__ void __launch_bounds__(GT2_THREADS, 1)
         // magnitude, 64 points): D_0, D_1 (< 2^22) by the 2^22 conversion on
         // the FP32 pipe, the others by the conversion unit (exact: integer
         // values below 2^24); D_0 256 + D_1 and D_2 256 + D_3 stay below 2^31
-        if constexpr (DIG == 7) {  // each half rounded to FP64, then added
-          double y[2] = {0.0, 0.0};
+        if constexpr (DIG == 7) {
+          long long s7[2][2];  // [half][column]
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
             uint32_t f[2][DIG];
@@ -704,17 +714,21 @@ __global__ void __launch_bounds__(GT2_THREADS, 1)
               f[1][d] = t[1];
             }
             tmem_wait_ld();
-            const int ea = h ? ea1 : ea0;
+            s7[h][0] = combine7<8>(f[0]);
+            s7[h][1] = combine7<8>(f[1]);
+          }
+          // sum_r x w = 2^(E_x + E_w - 63 + 8) s7
 #pragma unroll
-            for (int cc = 0; cc < 2; ++cc) {
-              const int ew = Wexp[u.wb][h][min(c0 + cc, NBLK - 1)];
-              const bool bad = ea + 1022 == EXP_NONFINITE || ew == EXP_NONFINITE;
-              y[cc] += bad ? quiet_nan() : combine7<7>(f[cc], ea + ew - 1022 - 63);
+          for (int cc = 0; cc < 2; ++cc) {
+            const int c = c0 + cc;
+            if (c < nj && a < m) {
+              const int w0 = Wexp[u.wb][0][c], w1 = Wexp[u.wb][1][c];
+              const bool bad = ea0 + 1022 == EXP_NONFINITE || ea1 + 1022 == EXP_NONFINITE ||
+                               w0 == EXP_NONFINITE || w1 == EXP_NONFINITE;
+              partial[(size_t)(u.j0 + u.jb + c) * m + a] =
+                  join7(s7[0][cc], ea0 + w0 - 1022 - 55, s7[1][cc], ea1 + w1 - 1022 - 55, bad);
             }
           }
-#pragma unroll
-          for (int cc = 0; cc < 2; ++cc)
-            if (c0 + cc < nj && a < m) partial[(size_t)(u.j0 + u.jb + c0 + cc) * m + a] = y[cc];
         } else {
           long long acc[2][2];  // [half][column]
 #pragma unroll
@@ -943,9 +957,9 @@ __global__ void __launch_bounds__(32 * FEW_WARPS)
   const int a0 = blockIdx.y * 8, g = lane >> 2, q = lane & 3;
   const int txi = T % G.ntx, tyi = (T / G.ntx) % G.nty, tzi = T / (G.ntx * G.nty);
   const int x0 = txi * TX, y = tyi * TY + q;
-  double lead[4][2];   // seven digits: the first half's values [entry half, row pair]
-  long long acc0[4];   // six digits: the first half's integers
+  long long acc0[4];  // the first half's integers, units and non-finite marks
   int e0[4];
+  bool bad0[4];
   for (int s0 = 0; s0 < nJ; s0 += 16) {
 #pragma unroll 1
     for (int h = 0; h < 2; ++h) {
@@ -999,21 +1013,20 @@ __global__ void __launch_bounds__(32 * FEW_WARPS)
         uint32_t f[DIG];
 #pragma unroll
         for (int k = 0; k < DIG; ++k) f[k] = __float_as_uint(c[k][i]);
-        double y0 = 0.0;
-        if constexpr (DIG == 7) {
-          const bool bad = ea == EXP_NONFINITE || ew == EXP_NONFINITE;
-          const double yh = bad ? quiet_nan() : combine7<7>(f, ea - 1022 + ew - 1022 - 63);
-          if (h == 0) lead[i][0] = 0.0 + yh;
-          y0 = lead[i][0] + yh;
-        } else {
-          const long long ac = combine6(f);
-          const int e = ea - 1022 + ew - 1022 - 55;
-          if (h == 0) {
-            acc0[i] = ac;
-            e0[i] = e;
-          }
-          y0 = join6(acc0[i], e0[i], ac, e);
+        long long ac;
+        if constexpr (DIG == 7)
+          ac = combine7<8>(f);
+        else
+          ac = combine6(f);
+        const int e = ea - 1022 + ew - 1022 - 55;
+        const bool bad = ea == EXP_NONFINITE || ew == EXP_NONFINITE;
+        if (h == 0) {
+          acc0[i] = ac;
+          e0[i] = e;
+          bad0[i] = bad;
         }
+        const double y0 = DIG == 7 ? join7(acc0[i], e0[i], ac, e, bad || bad0[i])
+                                   : join6(acc0[i], e0[i], ac, e);
         if (h == 1 && s < nJ && a < m) partial[(size_t)(j0 + s) * m + a] = y0;
       }
     }
@@ -1465,7 +1478,7 @@ __global__ void __launch_bounds__(XE_THREADS, 1)
 #pragma unroll
               for (int d = 0; d < DIG; ++d) fd[d] = f[d][u];
               const int e = ev[4 * hh + u];
-              val = e >= EV_NONFINITE ? quiet_nan() : combine7<6>(fd, e - 1022 - 63);
+              val = e >= EV_NONFINITE ? quiet_nan() : scaled_i64_rn_cvt(combine7<6>(fd), e - 1022 - 63 + 6);
             } else {
               // sum_d D_d 256^(5 - d) in three 32-bit pairs; |D_d| < 2^22 except
               // D_4 and D_5 of lists longer than 16 (below 2^23): those by the
@@ -1569,7 +1582,7 @@ __global__ void __launch_bounds__(256)
     for (int k = 0; k < DIG; ++k) f[k] = __float_as_uint(c[k][i]);
     double val;
     if constexpr (DIG == 7)
-      val = ev >= EV_NONFINITE ? quiet_nan() : combine7<6>(f, ev - 1022 - 63);
+      val = ev >= EV_NONFINITE ? quiet_nan() : scaled_i64_rn_cvt(combine7<6>(f), ev - 1022 - 63 + 6);
     else
       val = scaled_i64_rz_cvt(combine6(f), ev - 1022 - 55);
     if (nJ == 0) val = 0.0;
