@@ -315,6 +315,12 @@ sea_status sea_create(const double cell[3], const int grid[3], const sea_params*
       sea_destroy(c);
       return SEA_ERR_CUDA;
     }
+  if (cudaStreamCreateWithFlags(&c->aux.stream, cudaStreamNonBlocking) != cudaSuccess ||
+      cudaEventCreateWithFlags(&c->aux.fork, cudaEventDisableTiming) != cudaSuccess ||
+      cudaEventCreateWithFlags(&c->aux.join, cudaEventDisableTiming) != cudaSuccess) {
+    sea_destroy(c);
+    return SEA_ERR_CUDA;
+  }
   if (!sea_ensure(c, c->status, 64) || !sea_ensure(c, c->counts, 128) ||
       !sea_ensure(c, c->exx_dev, 64) || !sea_ensure(c, c->queue, 64)) {
     sea_destroy(c);
@@ -487,6 +493,7 @@ sea_status sea_apply_vxx(sea_ctx* c, double* vxx_phi, int on_device, double* exx
   memcpy(&c->WC, hc + 6, sizeof(long long));
   memcpy(&c->max_window, hc + 8, sizeof(long long));
   c->cg_pad_max = hc[10];
+  c->n_large = hc[3];
   SEA_CK(cudaEventRecord(c->ev[1], c->stream), "event");
   const size_t U = (size_t)std::max<long long>(c->U, 1);
   SEA_ALLOC(vbuf, U * sizeof(double));
@@ -855,8 +862,6 @@ sea_status sea_poisson_batch(const double h[3], int n_box, const int* ext, const
   if (!(tol > 0.0) || max_iter < 1 || (tol_mode != 0 && tol_mode != 1)) return SEA_ERR_ARG;
   if (n_box == 0) return SEA_OK;
   cudaStream_t st = (cudaStream_t)cuda_stream;
-  int device = 0;
-  if (cudaGetDevice(&device) != cudaSuccess) return SEA_ERR_CUDA;
   PairInfo* hb = (PairInfo*)malloc((size_t)n_box * sizeof(PairInfo));
   long long* ho = (long long*)malloc((size_t)n_box * sizeof(long long));
   int* hord = (int*)malloc((size_t)n_box * sizeof(int));
@@ -867,7 +872,7 @@ sea_status sea_poisson_batch(const double h[3], int n_box, const int* ext, const
     return SEA_ERR_OOM;
   }
   long long tot = 0;
-  int pad_max = 0;
+  int pad_max = 0, n_large = 0;
   sea_status rs = SEA_OK;
   for (int b = 0; b < n_box && rs == SEA_OK; ++b) {
     PairInfo P;
@@ -878,6 +883,7 @@ sea_status sea_poisson_batch(const double h[3], int n_box, const int* ext, const
     }
     P.n = P.ext[0] * P.ext[1] * P.ext[2];
     pad_max = std::max(pad_max, sea::cg_pad_volume(P.ext[0], P.ext[1], P.ext[2]));
+    n_large += P.n > SEA_CG_SPLIT;
     hb[b] = P;
     ho[b] = tot;
     tot += P.n;
@@ -920,8 +926,8 @@ sea_status sea_poisson_batch(const double h[3], int n_box, const int* ext, const
   if (e == cudaSuccess) e = cudaMemcpyAsync(dord, hord, n_box * sizeof(int), cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(dst, 0, sizeof(unsigned), st);
   if (e == cudaSuccess)
-    e = sea::launch_cg_boxes(st, device, h, n_box, dbox, dvoff, dord, rhs, x, r, pp, qq, dit, dst,
-                             dq, tol, tol_mode, max_iter, pad_max);
+    e = sea::launch_cg_boxes(st, h, n_box, dbox, dvoff, dord, rhs, x, r, pp, qq, dit, dst,
+                             dq, tol, tol_mode, max_iter, pad_max, n_large);
   unsigned hst = 0;
   if (e == cudaSuccess && iters)
     e = cudaMemcpyAsync(iters, dit, n_box * sizeof(int), cudaMemcpyDeviceToHost, st);
@@ -963,6 +969,12 @@ void sea_destroy(sea_ctx* c) {
       cudaStreamSynchronize(c->xfer[k]);
       cudaStreamDestroy(c->xfer[k]);
     }
+  if (c->aux.stream) {
+    cudaStreamSynchronize(c->aux.stream);
+    cudaStreamDestroy(c->aux.stream);
+  }
+  for (cudaEvent_t e : {c->aux.fork, c->aux.join})
+    if (e) cudaEventDestroy(e);
   for (cudaEvent_t e : c->xev)
     if (e) cudaEventDestroy(e);
   sea_batch_cache_free(c);

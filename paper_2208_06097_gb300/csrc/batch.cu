@@ -150,6 +150,7 @@ extern "C" sea_status sea_apply_vxx_batch(sea_ctx* const* ctxs, int n, double* c
     memcpy(&c->WC, h + 6, sizeof(long long));
     memcpy(&c->max_window, h + 8, sizeof(long long));
     c->cg_pad_max = h[10];
+    c->n_large = h[3];
     const size_t U = (size_t)(c->U > 1 ? c->U : 1);
     const size_t P = (size_t)(c->P > 1 ? c->P : 1);
     if (!sea_ensure(c, c->vbuf, U * sizeof(double)) || !sea_ensure(c, c->bbuf, U * sizeof(double)) ||
@@ -166,10 +167,12 @@ extern "C" sea_status sea_apply_vxx_batch(sea_ctx* const* ctxs, int n, double* c
   // descriptors and items (longest-first ranks dealt round-robin)
   const size_t db = sea::batch_desc_bytes();
   std::vector<unsigned char> hdesc((size_t)n * db);
-  int pad_cap = 0, pad_cap_f = 0;  // of the mixed-form and FP64 configurations
+  // largest padded boxes and large-class pairs of the mixed-form and FP64 configurations
+  int pad_m = 0, pad_f = 0, large_m = 0, large_f = 0;
   for (int k = 0; k < n; ++k) {
-    int& cap = ctxs[k]->prm.precision == 1 ? pad_cap : pad_cap_f;
-    cap = std::max(cap, sea::cg_pad_cap(ctxs[k]));
+    int& pad = ctxs[k]->prm.precision == 1 ? pad_m : pad_f;
+    pad = std::max(pad, ctxs[k]->cg_pad_max);
+    (ctxs[k]->prm.precision == 1 ? large_m : large_f) += ctxs[k]->n_large;
     ctxs[k]->cg_warm = false;  // the batched form solves from zero
     sea::make_batch_desc(ctxs[k], &hdesc[(size_t)k * db]);
   }
@@ -181,6 +184,7 @@ extern "C" sea_status sea_apply_vxx_batch(sea_ctx* const* ctxs, int n, double* c
     wsig.push_back(c->P);
     wsig.push_back(c->U);
     wsig.push_back(c->cg_pad_max);
+    wsig.push_back(c->n_large);
     wsig.push_back(c->prm.precision);
     for (int a = 0; a < 3; ++a) wsig.push_back(c->N[a]);
   }
@@ -250,6 +254,7 @@ extern "C" sea_status sea_apply_vxx_batch(sea_ctx* const* ctxs, int n, double* c
     sig.push_back(c->WC);
     sig.push_back(c->max_window);
     sig.push_back(c->cg_pad_max);
+    sig.push_back(c->n_large);
     sig.push_back(c->prm.precision);
     sig.push_back((long long)(uintptr_t)outs[k]);
     const SeaBuf* bufs[] = {&c->phi, &c->vxx_dev, &c->pinfo, &c->voff, &c->order, &c->Q,
@@ -267,13 +272,13 @@ extern "C" sea_status sea_apply_vxx_batch(sea_ctx* const* ctxs, int n, double* c
       cudaError_t e = sea::launch_pair_setup(ctxs[k]);
       if (e != cudaSuccess) return e;
     }
-    cudaError_t e = sea::launch_cg_batch(st, c0->device, c0->bdesc.p, (const int2*)c0->bitems.p,
-                                         (int)total_mixed, (int*)c0->queue.p, pad_cap, true,
+    cudaError_t e = sea::launch_cg_batch(st, &c0->aux, c0->bdesc.p, (const int2*)c0->bitems.p,
+                                         (int)total_mixed, large_m, (int*)c0->queue.p, pad_m, true,
                                          tuned.per_sm_mixed);
     if (e != cudaSuccess) return e;
-    e = sea::launch_cg_batch(st, c0->device, c0->bdesc.p,
+    e = sea::launch_cg_batch(st, &c0->aux, c0->bdesc.p,
                              (const int2*)c0->bitems.p + total_mixed, (int)(total - total_mixed),
-                             (int*)c0->queue.p, pad_cap_f, false, tuned.per_sm_fp64);
+                             large_f, (int*)c0->queue.p, pad_f, false, tuned.per_sm_fp64);
     if (e != cudaSuccess) return e;
     c0->launches += (total_mixed > 0) + (total > total_mixed);
     for (int k = 0; k < n; ++k) {
@@ -296,8 +301,8 @@ extern "C" sea_status sea_apply_vxx_batch(sea_ctx* const* ctxs, int n, double* c
     for (int q = 0; q < 3; ++q) SEA_BCK(cudaEventCreate(&ev[q]), "event");
     SEA_BCK(cudaEventRecord(ev[2], st), "event");
     for (int k = 0; k < n; ++k) SEA_BCK(sea::launch_pair_setup(ctxs[k]), "pair setup (tuning)");
-    const int occ_m = sea::cg_batch_max_ctas_per_sm(c0->device, pad_cap, true);
-    const int occ_f = sea::cg_batch_max_ctas_per_sm(c0->device, pad_cap_f, false);
+    const int occ_m = sea::cg_batch_max_ctas_per_sm(pad_m, true);
+    const int occ_f = sea::cg_batch_max_ctas_per_sm(pad_f, false);
     double best = 1e300;
     std::vector<int2> items;
     for (int o = 0; o < N_ORDERS; ++o) {
@@ -315,8 +320,8 @@ extern "C" sea_status sea_apply_vxx_batch(sea_ctx* const* ctxs, int n, double* c
         const int occ = mixed ? occ_m : occ_f;
         for (int j = (o == 0 ? 0 : 1); j <= occ; ++j) {  // j = 0: the warm-up launch
           SEA_BCK(cudaEventRecord(ev[0], st), "event");
-          SEA_BCK(sea::launch_cg_batch(st, c0->device, c0->bdesc.p, it0, (int)cnt,
-                                       (int*)c0->queue.p, mixed ? pad_cap : pad_cap_f, mixed, j < 1 ? 1 : j),
+          SEA_BCK(sea::launch_cg_batch(st, &c0->aux, c0->bdesc.p, it0, (int)cnt,
+                                       mixed ? large_m : large_f, (int*)c0->queue.p, mixed ? pad_m : pad_f, mixed, j < 1 ? 1 : j),
                   "batched CG (tuning)");
           SEA_BCK(cudaEventRecord(ev[1], st), "event");
           SEA_BCK(cudaEventSynchronize(ev[1]), "tuning");

@@ -163,7 +163,6 @@ struct FixScal {
 struct FixArgs {
   double s[3];  // 1 / (831600 h_a^2)
   int mode;     // 0: not used; 1: three axes; 2: equal spacings
-  int cap;      // padded points that fit the launch's shared memory
 };
 
 // sum_a (s_a / s_0) I_a with I_a = axis a's integer stencil sum at padded

@@ -143,7 +143,7 @@ extern "C" sea_status sea_poisson_batch_noalloc(const double h[3], int n_box, co
   if (!(tol > 0.0) || max_iter < 1 || (tol_mode != 0 && tol_mode != 1)) return SEA_ERR_ARG;
   if (n_box > SEA_NOALLOC_MAX_BOXES) return SEA_ERR_LIMIT;
   long long total = 0;
-  int pad_max = 0;
+  int pad_max = 0, n_large = 0;
   for (int b = 0; b < n_box; ++b) {
     long long nb = 1;
     for (int a = 0; a < 3; ++a) {
@@ -152,6 +152,7 @@ extern "C" sea_status sea_poisson_batch_noalloc(const double h[3], int n_box, co
       nb *= e;
     }
     pad_max = std::max(pad_max, sea::cg_pad_volume(ext[3 * b], ext[3 * b + 1], ext[3 * b + 2]));
+    n_large += nb > SEA_CG_SPLIT;
     total += nb;
   }
   if (total > SEA_NOALLOC_MAX_UNKNOWNS) return SEA_ERR_LIMIT;
@@ -162,8 +163,6 @@ extern "C" sea_status sea_poisson_batch_noalloc(const double h[3], int n_box, co
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) return SEA_ERR_CUDA;
   if (cap != cudaStreamCaptureStatusNone) return SEA_ERR_ARG;
-  int device = 0;
-  if (cudaGetDevice(&device) != cudaSuccess) return SEA_ERR_CUDA;
   unsigned char* base = nullptr;
   if (scratch_for_current_device(&base) != cudaSuccess) return SEA_ERR_CUDA;
   double* r = (double*)(base + kOffR);
@@ -186,8 +185,8 @@ extern "C" sea_status sea_poisson_batch_noalloc(const double h[3], int n_box, co
     e = cudaGetLastError();
   }
   if (e == cudaSuccess)
-    e = sea::launch_cg_boxes(st, device, h, n_box, boxes, voff, order, rhs, x, r, p, q, dit,
-                             status, queue, tol, tol_mode, max_iter, pad_max);
+    e = sea::launch_cg_boxes(st, h, n_box, boxes, voff, order, rhs, x, r, p, q, dit,
+                             status, queue, tol, tol_mode, max_iter, pad_max, n_large);
   unsigned hst = 0;
   if (e == cudaSuccess && iters)
     e = cudaMemcpyAsync(iters, dit, (size_t)n_box * sizeof(int), cudaMemcpyDeviceToHost, st);

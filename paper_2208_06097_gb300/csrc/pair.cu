@@ -483,6 +483,7 @@ struct CgArgs {
   int warm;  // x holds an initial guess (else the solve starts from 0)
   unsigned long long budget_ns;  // time budget of the launch (0: none)
   FixArgs fix;
+  int cap[2];  // padded points that fit the launch's shared memory, per class
 };
 
 // After a pair's solve (the whole CTA): the pair integral of Eq. exxGen_mlwf
@@ -750,11 +751,12 @@ __device__ __forceinline__ bool cg_pair_fix(const CgArgs& A, const StencilW& W, 
   return true;
 }
 
+template <bool LARGE>
 __device__ __forceinline__ void cg_pair_plain(const CgArgs& A, const StencilW& W, int pidx,
                                               double (*red)[32], int4* slots, int2* Ps) {
   const int* e = A.pinfo[pidx].ext;
   bool solved = false;
-  if (A.fix.mode && cg_pad_volume(e[0], e[1], e[2]) <= A.fix.cap)
+  if (A.fix.mode && cg_pad_volume(e[0], e[1], e[2]) <= A.cap[LARGE])
     solved = A.fix.mode == 2 ? cg_pair_fix<true>(A, W, pidx, red, slots, Ps)
                              : cg_pair_fix<false>(A, W, pidx, red, slots, Ps);
   if (!solved) cg_pair_fp64(A, W, pidx, red);
@@ -780,24 +782,27 @@ __device__ __forceinline__ int claim_item(int* queue, int P, unsigned long long 
   return atomicAdd(queue, 1);
 }
 
-// CTA size of the plain CG.
-#define SEA_FIX_THREADS 512
-// Padded points of a pair box that two CTAs per SM can hold (8 bytes each).
-#define SEA_FIX_PAD_LIMIT 13824
+__host__ __device__ constexpr int cg_threads(bool large) { return large ? 1024 : 512; }
+// Padded points of a box that fit shared memory, 8 bytes (plain form) or 4
+// (mixed form) each.
+__host__ __device__ constexpr int cg_pad_limit(bool mixed, bool large) {
+  return mixed ? (large ? 56000 : 27000) : (large ? 28000 : 13824);
+}
 
-__global__ void __launch_bounds__(SEA_FIX_THREADS, 2) k_cg(CgArgs A, StencilW W) {
+template <bool LARGE>
+__global__ void __launch_bounds__(cg_threads(LARGE), LARGE ? 1 : 2) k_cg(CgArgs A, StencilW W) {
   __shared__ double red[2][32];
   __shared__ int4 slots[64];
   __shared__ int s_item;
-  extern __shared__ int2 Ps[];  // A.fix.cap points
+  extern __shared__ int2 Ps[];  // A.cap[LARGE] points
   const unsigned long long t0 = A.budget_ns ? global_ns() : 0ull;
   for (;;) {
-    if (threadIdx.x == 0) s_item = claim_item(A.queue, A.P, A.budget_ns, t0, A.status);
+    if (threadIdx.x == 0) s_item = claim_item(A.queue + LARGE, A.P, A.budget_ns, t0, A.status);
     __syncthreads();
     const int item = s_item;
     if (item >= A.P) break;
     const int pidx = A.order[item];
-    cg_pair_plain(A, W, pidx, red, slots, Ps);
+    if ((A.pinfo[pidx].n > SEA_CG_SPLIT) == LARGE) cg_pair_plain<LARGE>(A, W, pidx, red, slots, Ps);
     __syncthreads();
   }
 }
@@ -819,8 +824,6 @@ __global__ void __launch_bounds__(SEA_FIX_THREADS, 2) k_cg(CgArgs A, StencilW W)
 // meets the same bound as the FP64 solver.
 // ---------------------------------------------------------------------------
 #define SEA_MIXED_INNER 1e-4f
-// CTA size of the mixed CG (one pair per CTA at a time)
-#define SEA_CG_THREADS 512
 #define SEA_MIXED_MAX_OUTER 30
 // smallest relative tolerance for which the true residual is formed in
 // double-float (below it, in FP64)
@@ -1067,7 +1070,7 @@ struct CgMixedArgs {
   unsigned* status;
   int* queue;
   int warm;       // x holds an initial guess (else the solve starts from 0)
-  int pad_cap;    // floats of shared memory for the padded search direction
+  int cap[2];     // floats of shared memory for the padded residual, per class
   unsigned long long budget_ns;  // time budget of the launch (0: none)
 };
 
@@ -1091,6 +1094,7 @@ __device__ __forceinline__ double block_sum_1w(double v, double* slots, double* 
 }
 
 // One pair's mixed-precision solve (the whole CTA).
+template <bool LARGE>
 __device__ __forceinline__ void cg_pair_mixed(const CgMixedArgs& A, const StencilW& W,
                                               const StencilWf& Wf, int pidx, double (*red)[32],
                                               double* bc, float* pS) {
@@ -1169,7 +1173,7 @@ __device__ __forceinline__ void cg_pair_mixed(const CgMixedArgs& A, const Stenci
     // reductions (compensated partials) all in FP32
     float2* fs0 = reinterpret_cast<float2*>(red[0]);
     float2* fs1 = reinterpret_cast<float2*>(red[1]);
-    if (cg_pad_volume(ex, ey, ez) <= A.pad_cap) {
+    if (cg_pad_volume(ex, ey, ez) <= A.cap[LARGE]) {
       inner_total = dres ? inner_cg_smem<true>(r, rnorm, x, d, pf, rf, qf, pS, n, ex, ey, ez, Wf,
                                                fs0, fs1, inner_total, A.max_iter)
                          : inner_cg_smem<false>(r, rnorm, x, d, pf, rf, qf, pS, n, ex, ey, ez, Wf,
@@ -1286,19 +1290,21 @@ __device__ __forceinline__ void cg_pair_mixed(const CgMixedArgs& A, const Stenci
   }
 }
 
-__global__ void __launch_bounds__(SEA_CG_THREADS, 1024 / SEA_CG_THREADS) k_cg_mixed(CgMixedArgs A, StencilW W, StencilWf Wf) {
+template <bool LARGE>
+__global__ void __launch_bounds__(cg_threads(LARGE), LARGE ? 1 : 2)
+    k_cg_mixed(CgMixedArgs A, StencilW W, StencilWf Wf) {
   __shared__ double red[2][32];
   __shared__ int s_item;
   __shared__ double bc;
-  extern __shared__ float pS[];  // A.pad_cap floats
+  extern __shared__ float pS[];  // A.cap[LARGE] floats
   const unsigned long long t0 = A.budget_ns ? global_ns() : 0ull;
   for (;;) {
-    if (threadIdx.x == 0) s_item = claim_item(A.queue, A.P, A.budget_ns, t0, A.status);
+    if (threadIdx.x == 0) s_item = claim_item(A.queue + LARGE, A.P, A.budget_ns, t0, A.status);
     __syncthreads();
     const int item = s_item;
     if (item >= A.P) break;
     const int pidx = A.order[item];
-    cg_pair_mixed(A, W, Wf, pidx, red, &bc, pS);
+    if ((A.pinfo[pidx].n > SEA_CG_SPLIT) == LARGE) cg_pair_mixed<LARGE>(A, W, Wf, pidx, red, &bc, pS);
     __syncthreads();
   }
 }
@@ -1319,12 +1325,10 @@ struct BatchCg {
   int mixed;
 };
 
-// MIXED: the items are all mixed-form (CTA of SEA_CG_THREADS, as k_cg_mixed)
-// or all FP64 (CTA of SEA_FIX_THREADS, as k_cg), so every pair is solved with
-// the same CTA size, hence the same bits, as in its own configuration's launch.
-template <bool MIXED>
-__global__ void __launch_bounds__(MIXED ? SEA_CG_THREADS : SEA_FIX_THREADS,
-                                  MIXED ? 1024 / SEA_CG_THREADS : 2)
+// MIXED: the items are all mixed-form or all FP64; the class is as in their own
+// launches (k_cg_mixed, k_cg), so every pair gives the same bits.
+template <bool MIXED, bool LARGE>
+__global__ void __launch_bounds__(cg_threads(LARGE), LARGE ? 1 : 2)
     k_cg_batch(const BatchCg* __restrict__ descs, const int2* __restrict__ items, int total,
                int* __restrict__ queue) {
   __shared__ double red[2][32];
@@ -1335,7 +1339,7 @@ __global__ void __launch_bounds__(MIXED ? SEA_CG_THREADS : SEA_FIX_THREADS,
   extern __shared__ int2 Ps[];  // the largest capacity of the descriptors
   float* pS = reinterpret_cast<float*>(Ps);
   for (;;) {
-    if (threadIdx.x == 0) s_item = atomicAdd(queue, 1);
+    if (threadIdx.x == 0) s_item = atomicAdd(queue + LARGE, 1);
     __syncthreads();
     const int item = s_item;
     if (item >= total) break;
@@ -1347,10 +1351,13 @@ __global__ void __launch_bounds__(MIXED ? SEA_CG_THREADS : SEA_FIX_THREADS,
         dst[w] = src[w];
     }
     __syncthreads();
-    if (MIXED)
-      cg_pair_mixed(d.m, d.W, d.Wf, d.m.order[it.y], red, &bc, pS);
-    else
-      cg_pair_plain(d.a, d.W, d.a.order[it.y], red, slots, Ps);
+    const int pidx = MIXED ? d.m.order[it.y] : d.a.order[it.y];
+    if (((MIXED ? d.m.pinfo : d.a.pinfo)[pidx].n > SEA_CG_SPLIT) == LARGE) {
+      if (MIXED)
+        cg_pair_mixed<LARGE>(d.m, d.W, d.Wf, pidx, red, &bc, pS);
+      else
+        cg_pair_plain<LARGE>(d.a, d.W, pidx, red, slots, Ps);
+    }
     __syncthreads();
   }
 }
@@ -1413,6 +1420,58 @@ static StencilWf make_weights_f(const StencilW& W) {
   return F;
 }
 
+// Points of a class's launch in shared memory: the largest padded pair box
+// pad_max, at most the class's limit; boxes above it solve on global vectors.
+static int cg_pad_cap(int pad_max, bool mixed, bool large) {
+  return std::min(pad_max, cg_pad_limit(mixed, large));
+}
+static size_t cg_smem_bytes(int cap, bool mixed) {
+  return (size_t)cap * (mixed ? sizeof(float) : sizeof(int2));
+}
+// The launch of a class's kernel: shared memory, CTAs (at most per_sm an SM
+// when that is positive) for `items` items.
+struct CgLaunch {
+  int grid, threads;
+  size_t smem;
+};
+static cudaError_t cg_shape(const void* kernel, int pad_max, bool mixed, bool large, int items,
+                            int per_sm, CgLaunch* L) {
+  int dev = 0, nsm = 0, occ = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)cg_smem_bytes(cg_pad_limit(mixed, large), mixed));
+  if (e != cudaSuccess) return e;
+  L->threads = cg_threads(large);
+  L->smem = cg_smem_bytes(cg_pad_cap(pad_max, mixed, large), mixed);
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, L->threads, L->smem);
+  if (e != cudaSuccess) return e;
+  occ = std::max(occ, 1);
+  if (per_sm > 0) occ = std::min(occ, per_sm);
+  L->grid = std::min(items, nsm * occ);
+  return cudaSuccess;
+}
+// A launch of n pairs, `large` of them of the large class: both classes side by
+// side, the large boxes' kernel on st, the others' on aux (after it on st when
+// null), which take the SMs that the large ones leave.
+template <class LaunchFn>
+static cudaError_t cg_both(cudaStream_t st, const CgAux* aux, int n, int large, LaunchFn launch) {
+  if (large == 0) return launch(false, st);
+  if (large == n) return launch(true, st);
+  if (!aux) {
+    const cudaError_t e = launch(true, st);
+    return e == cudaSuccess ? launch(false, st) : e;
+  }
+  cudaError_t e = cudaEventRecord(aux->fork, st);
+  if (e == cudaSuccess) e = cudaStreamWaitEvent(aux->stream, aux->fork, 0);
+  if (e == cudaSuccess) e = launch(true, st);
+  if (e == cudaSuccess) e = launch(false, aux->stream);
+  if (e == cudaSuccess) e = cudaEventRecord(aux->join, aux->stream);
+  if (e == cudaSuccess) e = cudaStreamWaitEvent(st, aux->join, 0);
+  return e;
+}
+
 static CgMixedArgs mixed_args(sea_ctx* c) {
   CgMixedArgs A;
   memset(&A, 0, sizeof(A));
@@ -1441,22 +1500,21 @@ static CgMixedArgs mixed_args(sea_ctx* c) {
   A.outers = nullptr;
   A.status = (unsigned*)c->status.p;
   A.queue = (int*)c->queue.p;
-  A.pad_cap = cg_pad_cap(c);
+  for (int l = 0; l < 2; ++l) A.cap[l] = cg_pad_cap(c->cg_pad_max, true, l);
   A.warm = c->cg_warm ? 1 : 0;
   A.budget_ns = (unsigned long long)(c->prm.timeout_ms * 1e6);
   return A;
 }
 
-// The fixed-point stencil's arguments for spacings h and boxes of at most
-// pad_max padded points; not used for spacings whose weights leave 1e+-30.
-static FixArgs make_fix(const double h[3], int pad_max) {
+// The fixed-point stencil's arguments for spacings h; not used for spacings
+// whose weights leave 1e+-30.
+static FixArgs make_fix(const double h[3]) {
   FixArgs F;
   F.mode = h[0] == h[1] && h[1] == h[2] ? 2 : 1;
   for (int a = 0; a < 3; ++a) {
     F.s[a] = 1.0 / (SEA_FIX_DEN * h[a] * h[a]);
     if (!(F.s[a] > 1e-30 && F.s[a] < 1e30)) F.mode = 0;
   }
-  F.cap = F.mode ? std::min(pad_max, SEA_FIX_PAD_LIMIT) : 0;
   return F;
 }
 
@@ -1486,52 +1544,31 @@ static CgArgs fp64_args(sea_ctx* c) {
   A.queue = (int*)c->queue.p;
   A.warm = c->cg_warm ? 1 : 0;
   A.budget_ns = (unsigned long long)(c->prm.timeout_ms * 1e6);
-  A.fix = make_fix(c->h, c->cg_pad_max);
+  A.fix = make_fix(c->h);
+  for (int l = 0; l < 2; ++l) A.cap[l] = cg_pad_cap(c->cg_pad_max, false, l);
   return A;
-}
-
-// Shared memory of the CG's padded vector: the largest padded pair box, at
-// most the form's limit (two CTAs per SM); pairs above it solve on global
-// vectors.  Mixed form: floats of the residual; FP64 form: 8-byte fixed-point
-// values of the search direction.
-#define SEA_CG_PAD_LIMIT 27000
-int cg_pad_cap(const sea_ctx* c) {
-  return c->prm.precision == 1 ? std::min(c->cg_pad_max, SEA_CG_PAD_LIMIT)
-                               : make_fix(c->h, c->cg_pad_max).cap;
-}
-static size_t cg_smem_bytes(int pad_cap, bool mixed) {
-  return (size_t)pad_cap * (mixed ? sizeof(float) : sizeof(int2));
-}
-static cudaError_t cg_allow_smem(const void* kernel, bool mixed) {
-  return cudaFuncSetAttribute(
-      kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-      (int)(mixed ? SEA_CG_PAD_LIMIT * sizeof(float) : SEA_FIX_PAD_LIMIT * sizeof(int2)));
 }
 
 cudaError_t launch_cg(sea_ctx* c) {
   if (c->P == 0) return cudaSuccess;
-  int nsm = 0, occ = 0;
-  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device);
   const bool mixed = c->prm.precision == 1;
-  const size_t smem = cg_smem_bytes(cg_pad_cap(c), mixed);
-  {
-    const cudaError_t e = cg_allow_smem(mixed ? (const void*)k_cg_mixed : (const void*)k_cg, mixed);
-    if (e != cudaSuccess) return e;
-  }
-  if (mixed)
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_cg_mixed, SEA_CG_THREADS, smem);
-  else
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_cg, SEA_FIX_THREADS, smem);
-  if (occ < 1) occ = 1;
-  const int grid = min(c->P, nsm * occ);
-  cudaMemsetAsync(c->queue.p, 0, sizeof(int), c->stream);
+  cudaError_t e = cudaMemsetAsync(c->queue.p, 0, 2 * sizeof(int), c->stream);
+  if (e != cudaSuccess) return e;
   const StencilW W = make_weights(c);
-  if (mixed)
-    k_cg_mixed<<<grid, SEA_CG_THREADS, smem, c->stream>>>(mixed_args(c), W, make_weights_f(W));
-  else
-    k_cg<<<grid, SEA_FIX_THREADS, smem, c->stream>>>(fp64_args(c), W);
-  c->launches += 1;
-  return cudaGetLastError();
+  return cg_both(c->stream, &c->aux, c->P, c->n_large, [&](bool large, cudaStream_t st) {
+    auto km = large ? k_cg_mixed<true> : k_cg_mixed<false>;
+    auto kf = large ? k_cg<true> : k_cg<false>;
+    CgLaunch L;
+    const cudaError_t e1 = cg_shape(mixed ? (const void*)km : (const void*)kf, c->cg_pad_max, mixed,
+                                    large, large ? c->n_large : c->P - c->n_large, 0, &L);
+    if (e1 != cudaSuccess) return e1;
+    if (mixed)
+      km<<<L.grid, L.threads, L.smem, st>>>(mixed_args(c), W, make_weights_f(W));
+    else
+      kf<<<L.grid, L.threads, L.smem, st>>>(fp64_args(c), W);
+    c->launches += 1;
+    return cudaGetLastError();
+  });
 }
 
 // Damped Jacobi sweeps on every pair's starting vector x (CTA per pair):
@@ -1580,42 +1617,43 @@ void make_batch_desc(sea_ctx* c, void* out) {
 
 size_t batch_desc_bytes() { return sizeof(BatchCg); }
 
-int cg_batch_max_ctas_per_sm(int device, int pad_cap, bool mixed) {
-  const size_t smem = cg_smem_bytes(pad_cap, mixed);
-  const int threads = mixed ? SEA_CG_THREADS : SEA_FIX_THREADS;
-  auto kern = mixed ? k_cg_batch<true> : k_cg_batch<false>;
-  if (cg_allow_smem((const void*)kern, mixed) != cudaSuccess) return 1;
+int cg_batch_max_ctas_per_sm(int pad_max, bool mixed) {
+  auto kern = mixed ? k_cg_batch<true, false> : k_cg_batch<false, false>;
+  CgLaunch L;
   int occ = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, threads, smem);
-  (void)device;
-  return occ < 1 ? 1 : occ;
+  if (cg_shape((const void*)kern, pad_max, mixed, false, 1, 0, &L) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, L.threads, L.smem) != cudaSuccess)
+    return 1;
+  return std::max(occ, 1);
 }
 
-cudaError_t launch_cg_batch(cudaStream_t st, int device, const void* descs, const int2* items,
-                            int total, int* queue, int pad_cap, bool mixed, int ctas_per_sm) {
+cudaError_t launch_cg_batch(cudaStream_t st, const CgAux* aux, const void* descs, const int2* items,
+                            int total, int n_large, int* queue, int pad_max, bool mixed,
+                            int ctas_per_sm) {
   if (total == 0) return cudaSuccess;
-  int nsm = 0;
-  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, device);
-  const size_t smem = cg_smem_bytes(pad_cap, mixed);
-  const int threads = mixed ? SEA_CG_THREADS : SEA_FIX_THREADS;
-  auto kern = mixed ? k_cg_batch<true> : k_cg_batch<false>;
-  const int occ = cg_batch_max_ctas_per_sm(device, pad_cap, mixed);
-  const int per_sm = ctas_per_sm >= 1 ? min(ctas_per_sm, occ) : occ;
-  cudaError_t e = cudaMemsetAsync(queue, 0, sizeof(int), st);
+  cudaError_t e = cudaMemsetAsync(queue, 0, 2 * sizeof(int), st);
   if (e != cudaSuccess) return e;
-  kern<<<min(total, nsm * per_sm), threads, smem, st>>>((const BatchCg*)descs, items, total, queue);
-  return cudaGetLastError();
+  return cg_both(st, aux, total, n_large, [&](bool large, cudaStream_t s) {
+    auto kern = mixed ? (large ? k_cg_batch<true, true> : k_cg_batch<true, false>)
+                      : (large ? k_cg_batch<false, true> : k_cg_batch<false, false>);
+    CgLaunch L;
+    const cudaError_t e1 = cg_shape((const void*)kern, pad_max, mixed, large,
+                                    large ? n_large : total - n_large, large ? 0 : ctas_per_sm, &L);
+    if (e1 != cudaSuccess) return e1;
+    kern<<<L.grid, L.threads, L.smem, s>>>((const BatchCg*)descs, items, total, queue);
+    return cudaGetLastError();
+  });
 }
 
 // Batched solve of -Lap_h x = rhs on independent boxes (no pair energies):
 // boxes[] and voff[] on the device, order[] the processing order; r, p, q
 // scratch of the same total length as x; pad_max the boxes' largest
-// cg_pad_volume.
-cudaError_t launch_cg_boxes(cudaStream_t stream, int device, const double h[3], int nbox,
+// cg_pad_volume, n_large how many have more than SEA_CG_SPLIT points.
+cudaError_t launch_cg_boxes(cudaStream_t stream, const double h[3], int nbox,
                             const PairInfo* boxes, const long long* voff, const int* order,
                             const double* rhs, double* x, double* r, double* p, double* q,
                             int* iters, unsigned* status, int* queue, double tol, int tol_mode,
-                            int max_iter, int pad_max) {
+                            int max_iter, int pad_max, int n_large) {
   if (nbox == 0) return cudaSuccess;
   double w[SEA_FDP + 1];
   fornberg_weights(w);
@@ -1629,18 +1667,12 @@ cudaError_t launch_cg_boxes(cudaStream_t stream, int device, const double h[3], 
     }
     W.center += -w[0] * ih2;
   }
-  int nsm = 0, occ = 0;
-  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, device);
+  const cudaError_t e = cudaMemsetAsync(queue, 0, 2 * sizeof(int), stream);
+  if (e != cudaSuccess) return e;
   CgArgs A;
   memset(&A, 0, sizeof(A));
-  A.fix = make_fix(h, pad_max);
-  const size_t smem = cg_smem_bytes(A.fix.cap, false);
-  cudaError_t e = cg_allow_smem((const void*)k_cg, false);
-  if (e != cudaSuccess) return e;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_cg, SEA_FIX_THREADS, smem);
-  if (occ < 1) occ = 1;
-  e = cudaMemsetAsync(queue, 0, sizeof(int), stream);
-  if (e != cudaSuccess) return e;
+  A.fix = make_fix(h);
+  for (int l = 0; l < 2; ++l) A.cap[l] = cg_pad_cap(pad_max, false, l);
   A.phi = nullptr;
   A.nx = A.ny = A.nz = 1;
   A.pinfo = boxes;
@@ -1660,8 +1692,15 @@ cudaError_t launch_cg_boxes(cudaStream_t stream, int device, const double h[3], 
   A.iters = iters;
   A.status = status;
   A.queue = queue;
-  k_cg<<<min(nbox, nsm * occ), SEA_FIX_THREADS, smem, stream>>>(A, W);
-  return cudaGetLastError();
+  return cg_both(stream, nullptr, nbox, n_large, [&](bool large, cudaStream_t st) {
+    auto kern = large ? k_cg<true> : k_cg<false>;
+    CgLaunch L;
+    const cudaError_t e1 = cg_shape((const void*)kern, pad_max, false, large,
+                                    large ? n_large : nbox - n_large, 0, &L);
+    if (e1 != cudaSuccess) return e1;
+    kern<<<L.grid, L.threads, L.smem, st>>>(A, W);
+    return cudaGetLastError();
+  });
 }
 
 cudaError_t upload_harmonics_pair() { return upload_harmonics_here(); }

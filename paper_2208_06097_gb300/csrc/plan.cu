@@ -539,29 +539,34 @@ __global__ void k_fill_pairs(const int* __restrict__ kept, const int* __restrict
 }
 
 // Single-CTA exclusive scan of P sizes into 64-bit offsets; total in *tot,
-// and the largest pair box in the mixed CG's padded shared-memory layout
-// (ex (ey + F)(ez + 2F) floats, F = SEA_FDP) in *maxpad.
+// the largest pair box in the CG's padded shared-memory layout
+// (cg_pad_volume points) in *maxpad and the boxes of the CG's large class in
+// *large.
 __global__ void k_scan_sizes(const int* __restrict__ sz, const int* __restrict__ count,
                              const PairInfo* __restrict__ pinfo, long long* __restrict__ off,
-                             long long* __restrict__ tot, int* __restrict__ maxpad) {
+                             long long* __restrict__ tot, int* __restrict__ maxpad,
+                             int* __restrict__ large) {
   __shared__ long long part[32];
   const int n = *count;
   const int T = blockDim.x;
   const int chunk = (n + T - 1) / T;
   const int b = chunk * threadIdx.x, e = min(n, b + chunk);
-  long long s = 0;
+  long long s = 0, nl = 0;
   int pm = 0;
   for (int x = b; x < e; ++x) {
     s += sz[x];
+    nl += sz[x] > SEA_CG_SPLIT;
     const PairInfo P = pinfo[x];
-    pm = max(pm, P.ext[0] * (P.ext[1] + SEA_FDP) * (P.ext[2] + 2 * SEA_FDP));
+    pm = max(pm, cg_pad_volume(P.ext[0], P.ext[1], P.ext[2]));
   }
-  long long acc = 0;
+  long long acc = 0, nlarge = 0;
   long long pos = block_exscan_ll(s, part, &acc);
+  block_exscan_ll(nl, part, &nlarge);
   const int m = (int)block_max_ll(pm, part);
   if (threadIdx.x == 0) {
     *tot = acc;
     *maxpad = m;
+    *large = (int)nlarge;
   }
   for (int x = b; x < e; ++x) {
     off[x] = pos;
@@ -663,7 +668,7 @@ cudaError_t launch_plan_pairs(sea_ctx* c) {
                                           (double*)c->pS.p, (int*)c->psize.p);
   k_scan_sizes<<<1, 1024, 0, c->stream>>>((const int*)c->psize.p, counts + 1,
                                           (const PairInfo*)c->pinfo.p, (long long*)c->voff.p,
-                                          (long long*)(counts + 4), counts + 10);
+                                          (long long*)(counts + 4), counts + 10, counts + 3);
   k_lpt_order<<<gc, 256, 0, c->stream>>>((const int*)c->psize.p, counts + 1, (int*)c->order.p);
   c->launches += 7;
   return cudaGetLastError();

@@ -472,6 +472,13 @@ struct LaunchGraph {
   long long launches = 0;
 };
 
+// A stream that runs a second kernel beside one on the context stream, and the
+// events that fork and join it.
+struct CgAux {
+  cudaStream_t stream = nullptr;
+  cudaEvent_t fork = nullptr, join = nullptr;
+};
+
 struct sea_ctx {
   int device = 0;
   cudaStream_t stream = nullptr;
@@ -496,7 +503,8 @@ struct sea_ctx {
   // plan sizes (host copies)
   int P = 0, Pproto = 0, E = 0;
   long long U = 0, WC = 0, max_window = 0;
-  int cg_pad_max = 0;  // largest zero-padded pair box (floats), for the mixed CG
+  int cg_pad_max = 0;  // largest padded pair box (points), for the CG
+  int n_large = 0;     // pairs of the CG's large class
 
   sea_stats stats{};
 
@@ -530,6 +538,7 @@ struct sea_ctx {
   // host-buffer transfers: copy streams (host to device, device to host) and
   // per-chunk events, created with the context
   cudaStream_t xfer[2] = {};
+  CgAux aux;  // the CG's second class of pairs
   std::vector<int> h_eptr;  // entry offsets per orbital, host copy (last plan)
   struct sea_unet* unet = nullptr;  // learned warm start (attached model, not owned)
   bool cg_warm = false;             // the next CG starts from the guess in vbuf
@@ -714,6 +723,19 @@ __host__ __device__ __forceinline__ int cg_pad_volume(int ex, int ey, int ez) {
   return v > 2147483647LL ? 2147483647 : (int)v;
 }
 
+// The pairs of a launch in two classes, each a kernel of its own (the class is
+// the pair's alone, so a pair is solved by the same CTA size, hence with the
+// same bits, in every launch).  Boxes of at most SEA_CG_SPLIT points: CTAs of
+// 512 threads, two per SM, where one fills the other's waits at the step's
+// barriers.  Larger boxes: CTAs of 1024 threads, one per SM: a step of a large
+// box takes several rounds of its CTA's points, a launch seldom has two of
+// them per SM, and one may hold a padded box twice as large in shared memory.
+// (H2O)16 on 81^3, most boxes large: mixed CG 2.33 -> 1.40 ms; FP64 26.7 -> 3.05
+// ms, since the padded boxes no longer miss the fixed-point stencil.  With the
+// line at 3072 or 2048 points the 96^3 workloads, whose boxes lie below it,
+// lose 0 to 0.4 and 0.2 to 0.75 ms.
+#define SEA_CG_SPLIT 4096
+
 // Launch wrappers (each file implements its own).
 cudaError_t launch_plan_boxes(sea_ctx* c);
 cudaError_t launch_plan_pairs(sea_ctx* c);
@@ -727,12 +749,13 @@ cudaError_t launch_chol_flow(cudaStream_t st, int device, const double* M, int n
                              double* Linv, void* scratch, unsigned* status, double* exx);
 void make_batch_desc(sea_ctx* c, void* out);
 size_t batch_desc_bytes();
-// The persistent batched CG: ctas_per_sm CTAs per SM (0 or above the
-// occupancy limit: the limit).
-cudaError_t launch_cg_batch(cudaStream_t st, int device, const void* descs, const int2* items,
-                            int total, int* queue, int pad_cap, bool mixed, int ctas_per_sm);
-int cg_batch_max_ctas_per_sm(int device, int pad_cap, bool mixed);
-int cg_pad_cap(const sea_ctx* c);
+// The persistent batched CG: ctas_per_sm CTAs per SM for the smaller boxes (0
+// or above the occupancy limit: the limit); queue: two counters; pad_max: the
+// largest padded pair box.
+cudaError_t launch_cg_batch(cudaStream_t st, const CgAux* aux, const void* descs, const int2* items,
+                            int total, int n_large, int* queue, int pad_max, bool mixed,
+                            int ctas_per_sm);
+int cg_batch_max_ctas_per_sm(int pad_max, bool mixed);
 cudaError_t launch_entries(sea_ctx* c);
 // V_xx phi into out (the context's W) and, when out2 is not null, also into
 // out2 (the caller's device buffer), both written by the same stores.
@@ -780,9 +803,9 @@ cudaError_t launch_ace_apply(sea_ctx* c, const double* psi, int n_vec, double* o
 cudaError_t launch_ace_vectors(sea_ctx* c, double* xi);
 cudaError_t upload_harmonics_pair();
 void fornberg_weights(double* w);
-cudaError_t launch_cg_boxes(cudaStream_t stream, int device, const double h[3], int nbox,
+cudaError_t launch_cg_boxes(cudaStream_t stream, const double h[3], int nbox,
                             const PairInfo* boxes, const long long* voff, const int* order,
                             const double* rhs, double* x, double* r, double* p, double* q,
                             int* iters, unsigned* status, int* queue, double tol, int tol_mode,
-                            int max_iter, int pad_max);
+                            int max_iter, int pad_max, int n_large);
 }  // namespace sea
