@@ -170,6 +170,7 @@ __global__ void k_scdm_downdate(const double* __restrict__ phi, int n, size_t N,
 // ---- pivots among the candidates --------------------------------------
 constexpr int SC_CLASSES = 24;   // quarter octaves below the largest density
 constexpr int SC_THREADS = 512;  // of k_scdm_step
+constexpr int SC_ROW = 4;        // its registers for a candidate's row
 
 // The class of density c against the largest cmax: floor(4 log2(cmax / c)),
 // decided on cmax 2^(-m/4) (edge m: the lower edge of class m - 1).
@@ -180,32 +181,34 @@ __device__ __forceinline__ double sc_edge(double cmax, int m) {
   return cmax * f * (1.0 / (double)(1 << (m >> 2)));
 }
 
-// cmax over the block maxima of k_argmax1; one CTA.  cnt[0..SC_CLASSES] = 0.
+// The classes' edges edge[0..SC_CLASSES] from the block maxima of k_argmax1; one
+// CTA.  cnt[0..SC_CLASSES] = 0.
 __global__ void __launch_bounds__(1024)
-    k_scdm_cmax(const double* __restrict__ bv, int nb, double* __restrict__ cmax,
-                int* __restrict__ cnt) {
+    k_scdm_edges(const double* __restrict__ bv, int nb, double* __restrict__ edge,
+                 int* __restrict__ cnt) {
   __shared__ double red[32];
   double v = -2.0;
   for (int b = threadIdx.x; b < nb; b += blockDim.x) v = fmax(v, bv[b]);
   for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
   __syncthreads();
-  if (threadIdx.x == 0) {
+  if (threadIdx.x <= SC_CLASSES) {
+    v = red[0];
     for (int w = 1; w < (int)blockDim.x / 32; ++w) v = fmax(v, red[w]);
-    *cmax = v;
+    edge[threadIdx.x] = sc_edge(v, threadIdx.x);
+    cnt[threadIdx.x] = 0;
   }
-  if (threadIdx.x <= SC_CLASSES) cnt[threadIdx.x] = 0;
 }
 
 // mode 0: counts the grid points per class; mode 1: writes their indices to
 // list at the classes' places (cnt then holds running positions).  The order
 // within a class does not matter: a pivot is chosen by value, then index.
 __global__ void __launch_bounds__(256)
-    k_scdm_classes(const double* __restrict__ c, size_t N, const double* __restrict__ cmax_p,
+    k_scdm_classes(const double* __restrict__ c, size_t N, const double* __restrict__ edge_g,
                    int mode, int cap, int* __restrict__ cnt, int* __restrict__ list) {
   __shared__ int n_of[SC_CLASSES], at[SC_CLASSES];
   __shared__ double edge[SC_CLASSES + 1];
-  if (threadIdx.x <= SC_CLASSES) edge[threadIdx.x] = sc_edge(*cmax_p, threadIdx.x);
+  if (threadIdx.x <= SC_CLASSES) edge[threadIdx.x] = edge_g[threadIdx.x];
   const size_t per = (N + gridDim.x - 1) / gridDim.x;
   const size_t b0 = min(N, per * blockIdx.x), b1 = min(N, b0 + per);
   if (threadIdx.x < SC_CLASSES) n_of[threadIdx.x] = 0;
@@ -259,8 +262,11 @@ struct ScMax {
   double v;
   int r, a;  // grid index, candidate
 };
+// FP64 values compared as integers (no FP64 instruction), which is their order
+// wherever one of them is positive, as every pivot's is.
 __device__ __forceinline__ bool sc_better(const ScMax& x, const ScMax& y) {
-  return x.v > y.v || (x.v == y.v && x.r < y.r);
+  const long long a = __double_as_longlong(x.v), b = __double_as_longlong(y.v);
+  return a > b || (a == b && x.r < y.r);
 }
 
 // One step of the greedy pivot choice (a launch each; the launch boundary is
@@ -271,18 +277,35 @@ __device__ __forceinline__ bool sc_better(const ScMax& x, const ScMax& y) {
 // and c_r -= L[r][k]^2; else the next class is opened and its candidates'
 // L[r][0..k) formed.  A warp per candidate, the lanes over the orbitals; the
 // lanes' sums are added as integers (no FP64 instruction).
+// A step is a chain of latencies: the loads that need no result of the step
+// before come first, the CTAs of the next step are resident before this one
+// ends (programmatic launch: only the wait for the predecessor's results
+// remains), and the maxima are compared as integers (as FP64, every warp's
+// twenty compares took as long as the dot products).  128 pivots on 72x75x76:
+// 14.3 -> 8.3 us a step.
 __global__ void __launch_bounds__(SC_THREADS)
     k_scdm_step(const double* __restrict__ A, int n, const int* __restrict__ list,
                 const int* __restrict__ start, const int* __restrict__ n_kept,
-                const double* __restrict__ cmax_p, double* __restrict__ cA, double* __restrict__ L,
-                const ScMax* __restrict__ mx_in, ScMax* __restrict__ mx_out,
-                const ScState* __restrict__ st_in, ScState* __restrict__ st_out, int first_open,
-                int* __restrict__ piv_a, long long* __restrict__ C) {
+                const double* __restrict__ edge, double* cA, double* L,
+                const ScMax* mx_in, ScMax* mx_out, const ScState* st_in, ScState* st_out,
+                int first_open, int* piv_a, long long* __restrict__ C) {
   extern __shared__ double sp[];  // pivot's a_p [n], -L[p] [n], 1 / sqrt(c_p)
   __shared__ ScMax wb[SC_THREADS / 32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int gw = blockIdx.x * (SC_THREADS / 32) + warp, nw = gridDim.x * (SC_THREADS / 32);
-  ScState st = *st_in;
+  const int kept = *n_kept;
+  // this warp's first candidate: its row and index do not change between steps
+  const bool has = gw < kept;
+  double row[SC_ROW];
+#pragma unroll
+  for (int u = 0; u < SC_ROW; ++u)
+    row[u] = has && lane + 32 * u < n ? A[(size_t)gw * n + lane + 32 * u] : 0.0;
+  const int r0 = has ? list[gw] : 0;
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // the step before has ended
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const ScState st0 = *st_in;
+  const double c0 = has ? cA[gw] : 0.0;
+  ScState st = st0;
   if (st.k >= n || st.stop) {
     if (threadIdx.x == 0 && blockIdx.x == 0) *st_out = st;
     return;
@@ -305,14 +328,13 @@ __global__ void __launch_bounds__(SC_THREADS)
     if (sc_better(y, best)) best = y;
   }
   best = warp_best(best);
-  const double cmax = *cmax_p;
   // a pivot must not lie below the open classes' lower edge (a closed
   // candidate could be larger)
-  const bool decide = st.open > 0 && best.v >= sc_edge(cmax, st.open);
-  const int kept = *n_kept;
+  const bool decide = st.open > 0 && __double_as_longlong(best.v) >=
+                                         __double_as_longlong(edge[st.open]);
   ScMax mine{-2.0, 0x7fffffff, -1};
   auto keep = [&](double v, int a) {
-    const ScMax y{v, list[a], a};
+    const ScMax y{v, a == gw ? r0 : list[a], a};
     if (sc_better(y, mine)) mine = y;
   };
   auto dot = [&](const double* x, const double* y, int m, double s, double f) {
@@ -335,11 +357,18 @@ __global__ void __launch_bounds__(SC_THREADS)
     const double inv = sp[2 * n];
     const int end = min(start[st.open], kept);
     for (int a = gw; a < end; a += nw) {
-      double c = cA[a];
+      double c = a == gw ? c0 : cA[a];
       if (a == best.a) {
         c = -1.0;
-      } else if (c >= 0.0) {
-        double s = dot(A + (size_t)a * n, sp, n, 0.0, 1.0);
+      } else if (__double2hiint(c) >= 0) {
+        double s = 0.0;
+        if (a == gw && n <= 32 * SC_ROW) {
+#pragma unroll
+          for (int u = 0; u < SC_ROW; ++u)
+            if (lane + 32 * u < n) s = fma(row[u], sp[lane + 32 * u], s);
+        } else {
+          s = dot(A + (size_t)a * n, sp, n, 0.0, 1.0);
+        }
         s = dot(L + (size_t)a * n, sp + n, st.k, s, 1.0);
         const double d = total(s) * inv;
         c = fma(-d, d, c);
@@ -496,19 +525,19 @@ static cudaError_t pivots_lazy(sea_ctx* c, const double* cn, const double* bv, i
   *done = false;
   int nsm = 0;
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device);
-  // small state: cmax, class counts and starts, step states and maxima
+  // small state: class edges, counts and starts, step states and maxima
   const size_t small = 256 + 4 * (SC_CLASSES + 1) * 4 + 64 + 2 * (size_t)nsm * sizeof(ScMax) + n * 4;
   if (!sea_ensure(c, c->scdm_s, small)) return cudaErrorMemoryAllocation;
   char* q = (char*)c->scdm_s.p;
-  double* cmax = (double*)q;
-  int* cnt = (int*)(q + 64);
+  double* edge = (double*)q;
+  int* cnt = (int*)(q + 256);
   int* start = cnt + SC_CLASSES + 1;
   int* kept = start + SC_CLASSES + 1;
   ScState* state = (ScState*)(kept + 1);
-  ScMax* mx = (ScMax*)(q + ((64 + (2 * (SC_CLASSES + 1) + 1) * 4 + 2 * sizeof(ScState) + 15) & ~(size_t)15));
+  ScMax* mx = (ScMax*)(q + ((256 + (2 * (SC_CLASSES + 1) + 1) * 4 + 2 * sizeof(ScState) + 15) & ~(size_t)15));
   int* piv_a = (int*)(mx + 2 * nsm);
-  k_scdm_cmax<<<1, 1024, 0, st>>>(bv, nb, cmax, cnt);
-  k_scdm_classes<<<4 * nsm, 256, 0, st>>>(cn, N, cmax, 0, 0, cnt, nullptr);
+  k_scdm_edges<<<1, 1024, 0, st>>>(bv, nb, edge, cnt);
+  k_scdm_classes<<<4 * nsm, 256, 0, st>>>(cn, N, edge, 0, 0, cnt, nullptr);
   k_scdm_starts<<<1, 1, 0, st>>>(cnt, start);
   int hs[SC_CLASSES + 1];
   cudaMemcpyAsync(hs, start, sizeof(hs), cudaMemcpyDeviceToHost, st);
@@ -527,7 +556,7 @@ static cudaError_t pivots_lazy(sea_ctx* c, const double* cn, const double* bv, i
   double* L = A + (size_t)na * n;
   double* cA = L + (size_t)na * n;
   int* list = (int*)(cA + na + n);
-  k_scdm_classes<<<4 * nsm, 256, 0, st>>>(cn, N, cmax, 1, na, cnt, list);
+  k_scdm_classes<<<4 * nsm, 256, 0, st>>>(cn, N, edge, 1, na, cnt, list);
   k_scdm_collect<<<(na + 7) / 8, 256, 0, st>>>((const double*)c->vxx_dev.p, n, N, list, na, cn, A, cA);
   const int smem = (2 * n + 1) * (int)sizeof(double);
   if (smem > 48 * 1024) {
@@ -543,10 +572,24 @@ static cudaError_t pivots_lazy(sea_ctx* c, const double* cn, const double* bv, i
   int first = 1;
   while (first < m && hs[first + 1] <= 2 * nsm * (SC_THREADS / 32)) ++first;
   const int launches = n + m - first + 1;  // every pivot, every opening
-  for (int l = 0; l < launches; ++l)
-    k_scdm_step<<<nsm, SC_THREADS, smem, st>>>(A, n, list, start, kept, cmax, cA, L,
-                                               mx + (l & 1) * nsm, mx + ((l + 1) & 1) * nsm,
-                                               state + (l & 1), state + ((l + 1) & 1), first, piv_a, C_dev);
+  for (int l = 0; l < launches; ++l) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(nsm);
+    cfg.blockDim = dim3(SC_THREADS);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute early;
+    early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    early.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &early;
+    cfg.numAttrs = l > 0;  // the first step reads what ordinary launches wrote
+    e = cudaLaunchKernelEx(&cfg, k_scdm_step, (const double*)A, n, (const int*)list,
+                           (const int*)start, (const int*)kept, (const double*)edge, cA, L,
+                           (const ScMax*)(mx + (l & 1) * nsm), mx + ((l + 1) & 1) * nsm,
+                           (const ScState*)(state + (l & 1)), state + ((l + 1) & 1), first, piv_a,
+                           C_dev);
+    if (e != cudaSuccess) return e;
+  }
   ScState hst;
   cudaMemcpyAsync(&hst, state + (launches & 1), sizeof(hst), cudaMemcpyDeviceToHost, st);
   e = cudaStreamSynchronize(st);
