@@ -882,7 +882,6 @@ sea_status sea_poisson_batch(const double h[3], int n_box, const int* ext, const
       if (P.ext[a] < 1 || P.ext[a] > 1024) rs = SEA_ERR_ARG;
     }
     P.n = P.ext[0] * P.ext[1] * P.ext[2];
-    pad_max = std::max(pad_max, sea::cg_pad_volume(P.ext[0], P.ext[1], P.ext[2]));
     n_large += P.n > SEA_CG_SPLIT;
     hb[b] = P;
     ho[b] = tot;
@@ -895,6 +894,9 @@ sea_status sea_poisson_batch(const double h[3], int n_box, const int* ext, const
     free(hord);
     return rs;
   }
+  const int team = sea::cg_box_team(n_box, ext);
+  for (int b = 0; b < n_box; ++b)
+    pad_max = std::max(pad_max, sea::cg_pad_volume(ext[3 * b], ext[3 * b + 1], ext[3 * b + 2], team));
   // longest boxes first (ties by index).  k_noalloc_order (noalloc.cu) ranks
   // the boxes of sea_poisson_batch_noalloc the same way; the two orders must
   // stay identical, since the solutions and iteration counts of the two entry
@@ -927,7 +929,7 @@ sea_status sea_poisson_batch(const double h[3], int n_box, const int* ext, const
   if (e == cudaSuccess) e = cudaMemsetAsync(dst, 0, sizeof(unsigned), st);
   if (e == cudaSuccess)
     e = sea::launch_cg_boxes(st, h, n_box, dbox, dvoff, dord, rhs, x, r, pp, qq, dit, dst,
-                             dq, tol, tol_mode, max_iter, pad_max, n_large);
+                             dq, tol, tol_mode, max_iter, team, pad_max, n_large);
   unsigned hst = 0;
   if (e == cudaSuccess && iters)
     e = cudaMemcpyAsync(iters, dit, n_box * sizeof(int), cudaMemcpyDeviceToHost, st);

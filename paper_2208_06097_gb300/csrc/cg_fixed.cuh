@@ -98,24 +98,72 @@ __device__ __forceinline__ FixSum fix_warp_sum(double v) {
   return FixSum{fix_warp_add(X), (int)em};
 }
 
-// The warp's part of a block sum and a block maximum: lane 0 posts them.
-__device__ __forceinline__ void fix_post(double v, unsigned vmax, int4* slots) {
-  const FixSum w = fix_warp_sum(v);
-  const unsigned wm = __reduce_max_sync(0xffffffffu, vmax);
-  if ((threadIdx.x & 31) == 0)
-    slots[threadIdx.x >> 5] = make_int4((int)(unsigned)w.X, (int)(w.X >> 32), w.e, (int)wm);
+// The CTAs that share a box: cluster rank and size.  TEAM: the size, or (3 and
+// more) the largest size of a launch.
+struct CgTeam {
+  int rank, size;
+};
+template <int TEAM>
+__device__ __forceinline__ CgTeam cg_team() {
+  if (TEAM == 1) return CgTeam{0, 1};
+  unsigned r, n = TEAM;
+  asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  if (TEAM > 2) asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(n));
+  return CgTeam{(int)r, (int)n};
+}
+// p's counterpart in the shared memory of the team's CTA `rank`.
+template <class T>
+__device__ __forceinline__ T* team_ptr(T* p, int rank) {
+  unsigned long long a;
+  asm("mapa.u64 %0, %1, %2;" : "=l"(a) : "l"((unsigned long long)p), "r"(rank));
+  return (T*)a;
+}
+// Barrier of the team's threads, shared-memory writes to the others included.
+__device__ __forceinline__ void team_sync(const CgTeam& T) {
+  if (T.size == 1) {
+    __syncthreads();
+    return;
+  }
+  asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
 }
 
-// The block's sum (and maximum) from the warps' posts, by one whole warp.
-__device__ __forceinline__ FixSum fix_combine(const int4* slots, unsigned* bmax) {
-  const int lane = threadIdx.x & 31, nw = (blockDim.x + 31) >> 5;
+// The warp's part of a team's sum and maximum, posted to every CTA of the team.
+__device__ __forceinline__ void fix_post(const CgTeam& T, double v, unsigned vmax, int4* slots) {
+  const FixSum w = fix_warp_sum(v);
+  const unsigned wm = __reduce_max_sync(0xffffffffu, vmax);
+  const int lane = threadIdx.x & 31, at = T.rank * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const int4 v4 = make_int4((int)(unsigned)w.X, (int)(w.X >> 32), w.e, (int)wm);
+  if (T.size == 1) {
+    if (lane == 0) slots[at] = v4;
+  } else if (lane < T.size) {
+    team_ptr(slots, lane)[at] = v4;
+  }
+}
+
+// The team's sum (and maximum) from the warps' posts, by one whole warp.
+__device__ __forceinline__ FixSum fix_combine(const CgTeam& T, const int4* slots, unsigned* bmax) {
+  const int lane = threadIdx.x & 31, nw = T.size * (int)(blockDim.x >> 5);
   int4 s = make_int4(0, 0, 0, 0);
   if (lane < nw) s = slots[lane];
-  const int E = (int)__reduce_max_sync(0xffffffffu, (unsigned)s.z);
-  *bmax = __reduce_max_sync(0xffffffffu, (unsigned)s.w);
-  const long long X = ((long long)s.y << 32) | (long long)(unsigned)s.x;
-  // 5 bits of room for 32 warps
-  return FixSum{fix_warp_add(X >> min(E - s.z + 5, 63)), E + 5};
+  int E = s.z, room = 5;  // bits for 32 warps
+  unsigned m = (unsigned)s.w;
+  if (T.size > 1)
+    for (int k = lane + 32; k < nw; k += 32) {
+      E = max(E, slots[k].z);
+      m = max(m, (unsigned)slots[k].w);
+    }
+  E = (int)__reduce_max_sync(0xffffffffu, (unsigned)E);
+  *bmax = __reduce_max_sync(0xffffffffu, m);
+  if (T.size > 1)
+    while ((1 << room) < nw) ++room;
+  long long X = (((long long)s.y << 32) | (long long)(unsigned)s.x) >> min(E - s.z + room, 63);
+  if (T.size > 1)
+    for (int k = lane + 32; k < nw; k += 32) {
+      s = slots[k];
+      X += (((long long)s.y << 32) | (long long)(unsigned)s.x) >> min(E - s.z + room, 63);
+    }
+  return FixSum{fix_warp_add(X), E + room};
 }
 
 // 1 / b as Y 2^e for a positive sum b (Y = 0 if it is not), good to 2^-59:
@@ -157,6 +205,48 @@ __device__ __forceinline__ float fix_upper(unsigned h, int k) {
 struct FixScal {
   double as, beta;
   int E, done;
+};
+
+// What the lead warp of a CTA keeps between a solve's steps: rr, its
+// reciprocal, and the bound M 2^k0 of |p| (M FP32, kept from below by rounding
+// up): the next |p| <= |r| + beta |p|.
+struct FixLead {
+  FixSum rr{0, 0};
+  FixRecip irr{0, 0};
+  float M = 0.f;
+  int k0 = 0;
+  // from the posts of (r, r) and the largest |r| at the start: E
+  __device__ __forceinline__ void start(const CgTeam& T, const int4* slots, bool post, FixScal& sc) {
+    unsigned rmax;
+    rr = fix_combine(T, slots, &rmax);
+    irr = fix_recip(rr);
+    k0 = (int)(rmax >> 20) - 1023;
+    M = fix_upper(rmax, k0);
+    if (post) sc.E = k0 + (int)(__float_as_uint(M) >> 23) - 126;
+  }
+  // from the posts of (p, q): alpha s_x
+  __device__ __forceinline__ void step(const CgTeam& T, const int4* slots, bool post, FixScal& sc) {
+    unsigned none;
+    const double as = fix_ratio(rr, fix_recip(fix_combine(T, slots, &none)));
+    if (post) sc.as = as;
+  }
+  // from the posts of the new (r, r): beta, the next E and whether to stop;
+  // next() follows, off the critical path
+  __device__ __forceinline__ void turn(const CgTeam& T, const int4* slots, double target2, bool post,
+                                       FixScal& sc) {
+    unsigned rmax;
+    rr = fix_combine(T, slots, &rmax);
+    const double beta = fix_ratio(rr, irr);
+    M = __fmaf_ru(fix_upper((unsigned)__double2hiint(beta), 0), M, fix_upper(rmax, k0));
+    if (post) {
+      sc.beta = beta;
+      sc.E = k0 + (int)(__float_as_uint(M) >> 23) - 126;
+      // non-negative FP64 values compare as their bit patterns
+      sc.done = __double_as_longlong(scaled_i64(rr.X, rr.e - 1080)) <=
+                __double_as_longlong(target2);
+    }
+  }
+  __device__ __forceinline__ void next() { irr = fix_recip(rr); }
 };
 
 // What the fixed-point solve needs beside the CG's own arguments.

@@ -151,11 +151,13 @@ extern "C" sea_status sea_poisson_batch_noalloc(const double h[3], int n_box, co
       if (e < 1 || e > 1024) return SEA_ERR_ARG;
       nb *= e;
     }
-    pad_max = std::max(pad_max, sea::cg_pad_volume(ext[3 * b], ext[3 * b + 1], ext[3 * b + 2]));
     n_large += nb > SEA_CG_SPLIT;
     total += nb;
   }
   if (total > SEA_NOALLOC_MAX_UNKNOWNS) return SEA_ERR_LIMIT;
+  const int team = sea::cg_box_team(n_box, ext);
+  for (int b = 0; b < n_box; ++b)
+    pad_max = std::max(pad_max, sea::cg_pad_volume(ext[3 * b], ext[3 * b + 1], ext[3 * b + 2], team));
   if (n_box == 0) return SEA_OK;
   cudaStream_t st = (cudaStream_t)cuda_stream;
   // a stream under capture cannot take the synchronous copies and the wait
@@ -186,7 +188,7 @@ extern "C" sea_status sea_poisson_batch_noalloc(const double h[3], int n_box, co
   }
   if (e == cudaSuccess)
     e = sea::launch_cg_boxes(st, h, n_box, boxes, voff, order, rhs, x, r, p, q, dit,
-                             status, queue, tol, tol_mode, max_iter, pad_max, n_large);
+                             status, queue, tol, tol_mode, max_iter, team, pad_max, n_large);
   unsigned hst = 0;
   if (e == cudaSuccess && iters)
     e = cudaMemcpyAsync(iters, dit, (size_t)n_box * sizeof(int), cudaMemcpyDeviceToHost, st);

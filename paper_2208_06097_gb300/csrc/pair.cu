@@ -486,28 +486,29 @@ struct CgArgs {
   int cap[2];  // padded points that fit the launch's shared memory, per class
 };
 
-// After a pair's solve (the whole CTA): the pair integral of Eq. exxGen_mlwf
-// over Omega_ij (skipped for a bare batch of boxes, phi == nullptr), the
-// iteration count (negative: capped) and the cap flag.
-__device__ __forceinline__ void cg_finish(const CgArgs& A, const PairInfo& P, int pidx,
-                                          const double* __restrict__ x, int iters, double* slots) {
+// After a pair's solve, by the whole CTA: the pair integral of Eq. exxGen_mlwf
+// over Omega_ij (n points; 0 for a bare batch of boxes, phi == nullptr).
+__device__ __forceinline__ double cg_integral(const CgArgs& A, const PairInfo& P,
+                                              const double* __restrict__ x, int n, double* slots) {
   const size_t ng = (size_t)A.nx * A.ny * A.nz;
   const int ex = P.ext[0], ey = P.ext[1];
   const double* fi = A.phi ? A.phi + (size_t)P.i * ng : nullptr;
   const double* fj = A.phi ? A.phi + (size_t)P.j * ng : nullptr;
   double e = 0.0;
-  for (int t = threadIdx.x; fi && t < P.n; t += blockDim.x) {
+  for (int t = threadIdx.x; fi && t < n; t += blockDim.x) {
     const int xx = t % ex, yy = (t / ex) % ey, zz = t / (ex * ey);
     const size_t g = ((size_t)wrapi(P.lo[2] + zz, A.nz) * A.ny + wrapi(P.lo[1] + yy, A.ny)) * A.nx +
                      wrapi(P.lo[0] + xx, A.nx);
     e = fma(fi[g] * fj[g], x[t], e);
   }
-  e = block_sum(e, slots);
-  if (threadIdx.x == 0) {
-    if (A.epair) A.epair[pidx] = e * A.dV;
-    A.iters[pidx] = iters;
-    if (iters < 0) atomicOr(A.status, SEA_FLAG_CG_CAP);
-  }
+  return block_sum(e, slots);
+}
+// One thread: the pair integral, the iteration count (negative: capped) and the
+// cap flag.
+__device__ __forceinline__ void cg_finish(const CgArgs& A, int pidx, double e, int iters) {
+  if (A.epair) A.epair[pidx] = e * A.dV;
+  A.iters[pidx] = iters;
+  if (iters < 0) atomicOr(A.status, SEA_FLAG_CG_CAP);
 }
 
 // One pair's FP64 CG (the whole CTA), results into A's per-pair arrays.
@@ -585,25 +586,29 @@ __device__ __forceinline__ void cg_pair_fp64(const CgArgs& A, const StencilW& W,
     for (int t = threadIdx.x; t < n; t += blockDim.x) pv[t] = fma(beta, pv[t], r[t]);
     __syncthreads();
   }
-  cg_finish(A, P, pidx, x, done ? it : -it, red[1]);
+  const double e = cg_integral(A, P, x, n, red[1]);
+  if (threadIdx.x == 0) cg_finish(A, pidx, e, done ? it : -it);
 }
 
 // The same CG with the stencil in fixed point (cg_fixed.cuh): the search
 // direction's integers live in shared memory in the padded layout (8 bytes a
 // point), the FP64 vectors x, r, p and q in global memory (L1 and L2; holding
-// r and q in registers measured the same).  Same iteration, stopping rule and
-// counts as cg_pair_fp64; q is kept without the factor s_x, which goes into
-// the step.  The step's scalars are formed by the last warp, whose share of
-// the points is the smallest, in integer arithmetic: one warp's FP64
-// instruction takes as long as a full one's, and every warp dividing took
-// more of the FP64 unit than the vector updates.  `slots`: 2 x 32 int4.
+// r and q in registers measured the same with a CTA per box).  Same iteration,
+// stopping rule and counts as cg_pair_fp64; q is kept without the factor s_x,
+// which goes into the step.  The step's scalars are formed by the last warp,
+// whose share of the points is the smallest, in integer arithmetic: one warp's
+// FP64 instruction takes as long as a full one's, and every warp dividing took
+// more of the FP64 unit than the vector updates.  `slots`, `slots2`: an int4 for
+// each warp.
 // Returns the iterations (negative: capped).
 template <bool ISO>
 __device__ __forceinline__ int cg_fix_loop(const CgArgs& A, int n, int ex, int ey, int ez,
                                            double* __restrict__ x, double* __restrict__ r,
                                            double* __restrict__ p, double* __restrict__ q,
-                                           double target2, int2* __restrict__ Ps, int4* slots) {
+                                           double target2, int2* __restrict__ Ps, int4* slots,
+                                           int4* slots2) {
   __shared__ FixScal sc;
+  const CgTeam T{0, 1};
   const int S = blockDim.x;
   const int PXY = ex * (ey + SEA_FDP), gap = SEA_FDP * ex, org = SEA_FDP * PXY;
   const int Vp = PXY * (ez + 2 * SEA_FDP);
@@ -617,25 +622,14 @@ __device__ __forceinline__ int cg_fix_loop(const CgArgs& A, int n, int ex, int e
     v = fma(rt, rt, v);
     rmax = max(rmax, (unsigned)__double2hiint(rt) & 0x7FFFFFFFu);
   };
-  // lead warp: rr, its reciprocal, and the bound M 2^k0 of |p| (M FP32, kept
-  // from below by rounding up): the next |p| <= |r| + beta |p|
-  FixSum rr{0, 0};
-  FixRecip irr{0, 0};
-  float M = 0.f;
-  int k0 = 0;
+  FixLead L;
   {
     double v = 0.0;
     unsigned rmax = 0;
     for (int t = threadIdx.x; t < n; t += S) square(r[t], v, rmax);
-    fix_post(v, rmax, slots);
+    fix_post(T, v, rmax, slots);
     __syncthreads();
-    if (lead) {
-      rr = fix_combine(slots, &rmax);
-      irr = fix_recip(rr);
-      k0 = (int)(rmax >> 20) - 1023;
-      M = fix_upper(rmax, k0);
-      if (post) sc.E = k0 + (int)(__float_as_uint(M) >> 23) - 126;
-    }
+    if (lead) L.start(T, slots, post, sc);
     __syncthreads();
   }
   int E = sc.E;
@@ -652,13 +646,9 @@ __device__ __forceinline__ int cg_fix_loop(const CgArgs& A, int n, int ex, int e
       q[w.t] = qt;
       v = fma(pt, qt, v);
     }
-    fix_post(v, 0u, slots);
+    fix_post(T, v, 0u, slots);
     __syncthreads();
-    if (lead) {
-      unsigned none;
-      const double as = fix_ratio(rr, fix_recip(fix_combine(slots, &none)));
-      if (post) sc.as = as;
-    }
+    if (lead) L.step(T, slots, post, sc);
     __syncthreads();
     const double as = sc.as;
     v = 0.0;
@@ -676,21 +666,10 @@ __device__ __forceinline__ int cg_fix_loop(const CgArgs& A, int n, int ex, int e
         square(y1, v, rmax);
       }
     }
-    fix_post(v, rmax, slots + 32);
+    fix_post(T, v, rmax, slots2);
     __syncthreads();
     ++it;
-    if (lead) {
-      rr = fix_combine(slots + 32, &rmax);
-      const double beta = fix_ratio(rr, irr);
-      M = __fmaf_ru(fix_upper((unsigned)__double2hiint(beta), 0), M, fix_upper(rmax, k0));
-      if (post) {
-        sc.beta = beta;
-        sc.E = k0 + (int)(__float_as_uint(M) >> 23) - 126;
-        // non-negative FP64 values compare as their bit patterns
-        sc.done = __double_as_longlong(scaled_i64(rr.X, rr.e - 1080)) <=
-                  __double_as_longlong(target2);
-      }
-    }
+    if (lead) L.turn(T, slots2, target2, post, sc);
     __syncthreads();
     const double alpha = as * inv_s0, beta = sc.beta;
     E = sc.E;
@@ -707,59 +686,244 @@ __device__ __forceinline__ int cg_fix_loop(const CgArgs& A, int n, int ex, int e
       p[w.t] = pn;
       Ps[org + w.t + w.z * gap] = fix_quant(pn, E);
     }
-    if (lead) irr = fix_recip(rr);
+    if (lead) L.next();
     __syncthreads();
   }
 }
 
-// One pair's FP64-form solve (the whole CTA): the fixed-point stencil where
-// the padded box fits the launch's shared memory and the values stay far
-// from the ends of the FP64 range (also where they are finite), else
-// cg_pair_fp64.
-template <bool ISO>
-__device__ __forceinline__ bool cg_pair_fix(const CgArgs& A, const StencilW& W, int pidx,
-                                            double (*red)[32], int4* slots, int2* Ps) {
+// The points t0 <= t < t1 of CTA `rank` of a box's n, shared by `size` CTAs, and the
+// planes z0 <= z <= z1 they lie in (none: z1 far below z0).
+struct CgPart {
+  int t0, t1, z0, z1;
+};
+__device__ __forceinline__ CgPart cg_part(int n, int area, int size, int rank) {
+  const int m = cg_share(n, size);
+  CgPart q;
+  q.t0 = min(n, m * rank);
+  q.t1 = min(n, q.t0 + m);
+  q.z0 = q.t0 / area;
+  q.z1 = q.t1 > q.t0 ? (q.t1 - 1) / area : -1000;
+  return q;
+}
+
+// The same solve by a team of CTAs (a cluster), each with an equal share of the
+// box's points (part; x and r: the whole box's; p starts as r) and their planes
+// in shared memory with the six on either side: a point's integers are written
+// here and to the CTAs whose stencils reach it.  The vectors stay in registers,
+// NP points a thread: the team's barriers order memory across SMs, so writes to
+// global memory would have to reach L2 at each (with them there, pairs of CTAs
+// took 1.5 times the time of single ones on 640 boxes).  The scalars are formed
+// by every CTA from the same posts, so all agree.  `slots`, `slots2`: an int4 for
+// each warp of the team.
+template <bool ISO, int NP>
+__device__ __forceinline__ int cg_fix_team(const CgArgs& A, const CgTeam& T, const CgPart& part,
+                                           int n, int ex, int ey, double* __restrict__ x,
+                                           const double* __restrict__ r, double target2, int2* Ps,
+                                           int4* slots, int4* slots2) {
+  __shared__ FixScal sc;
+  const int S = blockDim.x;
+  const int PXY = ex * (ey + SEA_FDP), gap = SEA_FDP * ex;
+  const int org = (SEA_FDP - part.z0) * PXY;
+  const int Vp = PXY * (max(part.z1 - part.z0 + 1, 0) + 2 * SEA_FDP);
+  const double s0 = A.fix.s[0], inv_s0 = 1.0 / s0;
+  const double ry = A.fix.s[1] / s0, rz = A.fix.s[2] / s0;
+  const bool lead = (threadIdx.x >> 5) == (blockDim.x >> 5) - 1;
+  const bool post = (threadIdx.x & 31) == 0;
+  for (int t = threadIdx.x; t < Vp; t += S) Ps[t] = make_int2(0, 0);
+  double xv[NP], rv[NP], pv[NP], qv[NP];
+  // padded index (-1: no point); x, and from bit 16 the CTAs that the point's
+  // integers go to, where they lie `far` from the own place
+  int at[NP], xm[NP];
+  __shared__ int far[SEA_CG_TEAM_MAX];
+  if ((int)threadIdx.x < T.size)
+    far[threadIdx.x] = (part.z0 - cg_part(n, ex * ey, T.size, threadIdx.x).z0) * PXY;
+  double v = 0.0;
+  unsigned rmax = 0;
+  {
+    BoxWalk w(part.t0 + threadIdx.x, S, ex, ey);
+#pragma unroll
+    for (int u = 0; u < NP; ++u, w.next(S)) {
+      const bool in = w.t < part.t1;
+      at[u] = in ? org + w.t + w.z * gap : -1;
+      xm[u] = w.x;
+      rv[u] = pv[u] = in ? r[w.t] : 0.0;
+      xv[u] = in ? x[w.t] : 0.0;
+      v = fma(rv[u], rv[u], v);
+      rmax = max(rmax, (unsigned)__double2hiint(rv[u]) & 0x7FFFFFFFu);
+    }
+  }
+  for (int o = 0; o < T.size; ++o) {
+    const CgPart q = cg_part(n, ex * ey, T.size, o);
+    BoxWalk w(part.t0 + threadIdx.x, S, ex, ey);
+#pragma unroll
+    for (int u = 0; u < NP; ++u, w.next(S))
+      if (o != T.rank && at[u] >= 0 && w.z >= q.z0 - SEA_FDP && w.z <= q.z1 + SEA_FDP)
+        xm[u] |= 1 << (16 + o);
+  }
+  // the direction of point u, here and where another CTA's stencil reaches it
+  auto put = [&](int u, int E) {
+    if (at[u] < 0) return;
+    const int2 P = fix_quant(pv[u], E);
+    Ps[at[u]] = P;
+    for (unsigned m = (unsigned)xm[u] >> 16; m; m &= m - 1) {
+      const int o = __ffs(m) - 1;
+      team_ptr(Ps, o)[at[u] + far[o]] = P;
+    }
+  };
+  FixLead L;
+  fix_post(T, v, rmax, slots);
+  team_sync(T);  // also: every CTA's Ps is zero
+  if (lead) L.start(T, slots, post, sc);
+  __syncthreads();
+  int E = sc.E;
+#pragma unroll
+  for (int u = 0; u < NP; ++u) put(u, E);
+  team_sync(T);
+  int it = 0;
+  for (;;) {
+    v = 0.0;
+#pragma unroll
+    for (int u = 0; u < NP; ++u)
+      if (at[u] >= 0) {
+        qv[u] = fix_stencil<ISO>(Ps, at[u], xm[u] & 0xFFFF, ex, PXY, ry, rz, E - FIX_BITS);
+        v = fma(pv[u], qv[u], v);
+      }
+    fix_post(T, v, 0u, slots);
+    team_sync(T);
+    if (lead) L.step(T, slots, post, sc);
+    __syncthreads();
+    const double as = sc.as;
+    v = 0.0;
+    rmax = 0;
+#pragma unroll
+    for (int u = 0; u < NP; ++u)
+      if (at[u] >= 0) {
+        rv[u] = fma(-as, qv[u], rv[u]);
+        v = fma(rv[u], rv[u], v);
+        rmax = max(rmax, (unsigned)__double2hiint(rv[u]) & 0x7FFFFFFFu);
+      }
+    fix_post(T, v, rmax, slots2);
+    team_sync(T);
+    ++it;
+    if (lead) L.turn(T, slots2, target2, post, sc);
+    __syncthreads();
+    const double alpha = as * inv_s0, beta = sc.beta;
+    E = sc.E;
+    const bool done = sc.done;
+    const bool last = done || it >= A.max_iter;
+#pragma unroll
+    for (int u = 0; u < NP; ++u)
+      if (at[u] >= 0) {
+        xv[u] = fma(alpha, pv[u], xv[u]);
+        if (last) {
+          x[part.t0 + threadIdx.x + u * S] = xv[u];
+        } else {
+          pv[u] = fma(beta, pv[u], rv[u]);
+          put(u, E);
+        }
+      }
+    if (last) {
+      __syncthreads();  // sc is free for the next box
+      return done ? it : -it;
+    }
+    if (lead) L.next();
+    team_sync(T);
+  }
+}
+
+// Shared memory of a CTA of `warps` warps beside the padded direction.
+template <int TEAM, int WARPS>
+struct CgShared {
+  double red[2][32];
+  double sums[2][TEAM];
+  int4 slots[2][TEAM * WARPS];
+};
+// v (the same in all threads of a CTA) of every CTA of the team, in sums[rank]
+// after the next team_sync.
+__device__ __forceinline__ void team_post(const CgTeam& T, double v, double* sums) {
+  if ((int)threadIdx.x < T.size) team_ptr(sums, threadIdx.x)[T.rank] = v;
+}
+__device__ __forceinline__ double team_total(const CgTeam& T, const double* sums) {
+  double s = sums[0];
+  for (int k = 1; k < T.size; ++k) s += sums[k];
+  return s;
+}
+
+// Points of a team's CTA in registers: the largest of cg_fix_team's forms.
+#define SEA_CG_TEAM_NP 4
+
+// One pair's FP64-form solve (all CTAs of its team; teams solve bare boxes
+// only): the fixed-point stencil
+// where the padded planes fit the launch's shared memory (and a team's points
+// its registers) and the values stay far from the ends of the FP64 range (also
+// where they are finite), else cg_pair_fp64 by the first CTA.
+template <bool ISO, int TEAM, int WARPS>
+__device__ __forceinline__ bool cg_pair_fix(const CgArgs& A, const CgTeam& T, const StencilW& W,
+                                            int pidx, CgShared<TEAM, WARPS>& M, int2* Ps) {
   const PairInfo P = A.pinfo[pidx];
-  const int ex = P.ext[0], ey = P.ext[1], ez = P.ext[2], n = P.n;
+  const int ex = P.ext[0], ey = P.ext[1], ez = P.ext[2];
+  const CgPart part = cg_part(P.n, ex * ey, T.size, T.rank);
   const long long off = A.voff[pidx];
   double *x = A.x + off, *r = A.r + off, *pv = A.p + off, *q = A.q + off;
   const double* b = A.b + off;
   double rr = 0.0, bb = 0.0;
-  for (int t = threadIdx.x; t < n; t += blockDim.x) {
+  for (int t = part.t0 + threadIdx.x; t < part.t1; t += blockDim.x) {
     const double bt = b[t];
     double rt = bt;
-    if (A.warm)  // r = b - A x0
+    if (TEAM == 1 && A.warm)  // r = b - A x0
       rt = bt - neg_lap(x, t, t % ex, (t / ex) % ey, t / (ex * ey), ex, ey, ez, W);
     r[t] = rt;
-    pv[t] = rt;
+    if (TEAM == 1) pv[t] = rt;
     rr = fma(rt, rt, rr);
     bb = fma(bt, bt, bb);
   }
-  rr = block_sum(rr, red[0]);
-  bb = block_sum(bb, red[1]);
-  __syncthreads();  // both slot arrays are read before their next use
+  rr = block_sum(rr, M.red[0]);
+  bb = block_sum(bb, M.red[1]);
+  if (TEAM > 1) {
+    team_post(T, rr, M.sums[0]);
+    team_post(T, bb, M.sums[1]);
+  }
+  team_sync(T);  // also: both slot arrays are read before their next use
+  if (TEAM > 1) {
+    rr = team_total(T, M.sums[0]);
+    bb = team_total(T, M.sums[1]);
+  }
   const double target = A.tol_mode == 0 ? A.tol * sqrt(bb)
-                                        : A.tol * 4.0 * 3.14159265358979323846 * sqrt((double)n);
+                                        : A.tol * 4.0 * 3.14159265358979323846 * sqrt((double)P.n);
   const double target2 = target * target;
   if (!(target2 >= 1e-260 && target2 >= 1e-60 * rr && rr <= 1e200 && bb <= 1e200)) return false;
-  if (!A.warm)
-    for (int t = threadIdx.x; t < n; t += blockDim.x) x[t] = 0.0;
+  if (TEAM > 1 || !A.warm)
+    for (int t = part.t0 + threadIdx.x; t < part.t1; t += blockDim.x) x[t] = 0.0;
   int it = 0;
-  if (sqrt(rr) > target)
-    it = cg_fix_loop<ISO>(A, n, ex, ey, ez, x, r, pv, q, target2, Ps, slots);
-  cg_finish(A, P, pidx, x, it, red[1]);
+  if (sqrt(rr) > target) {
+    if constexpr (TEAM > 1) {
+      const int most = cg_share(P.n, T.size), S = blockDim.x;
+#define SEA_TEAM_LOOP(NP) \
+  cg_fix_team<ISO, NP>(A, T, part, P.n, ex, ey, x, r, target2, Ps, M.slots[0], M.slots[1])
+      it = most <= S ? SEA_TEAM_LOOP(1)
+                     : (most <= 2 * S ? SEA_TEAM_LOOP(2) : SEA_TEAM_LOOP(SEA_CG_TEAM_NP));
+#undef SEA_TEAM_LOOP
+    } else {
+      it = cg_fix_loop<ISO>(A, P.n, ex, ey, ez, x, r, pv, q, target2, Ps, M.slots[0], M.slots[1]);
+    }
+  }
+  double e = 0.0;
+  if (TEAM == 1) e = cg_integral(A, P, x, P.n, M.red[1]);
+  if (T.rank == 0 && threadIdx.x == 0) cg_finish(A, pidx, e, it);
   return true;
 }
 
-template <bool LARGE>
-__device__ __forceinline__ void cg_pair_plain(const CgArgs& A, const StencilW& W, int pidx,
-                                              double (*red)[32], int4* slots, int2* Ps) {
-  const int* e = A.pinfo[pidx].ext;
+template <int TEAM, int WARPS>
+__device__ __forceinline__ void cg_pair_plain(const CgArgs& A, const CgTeam& T, int cap,
+                                              const StencilW& W, int pidx,
+                                              CgShared<TEAM, WARPS>& M, int2* Ps) {
+  const PairInfo& P = A.pinfo[pidx];
   bool solved = false;
-  if (A.fix.mode && cg_pad_volume(e[0], e[1], e[2]) <= A.cap[LARGE])
-    solved = A.fix.mode == 2 ? cg_pair_fix<true>(A, W, pidx, red, slots, Ps)
-                             : cg_pair_fix<false>(A, W, pidx, red, slots, Ps);
-  if (!solved) cg_pair_fp64(A, W, pidx, red);
+  if (A.fix.mode && cg_pad_volume(P.ext[0], P.ext[1], P.ext[2], T.size) <= cap &&
+      (TEAM == 1 || cg_share(P.n, T.size) <= SEA_CG_TEAM_NP * (int)blockDim.x))
+    solved = A.fix.mode == 2 ? cg_pair_fix<true, TEAM, WARPS>(A, T, W, pidx, M, Ps)
+                             : cg_pair_fix<false, TEAM, WARPS>(A, T, W, pidx, M, Ps);
+  if (!solved && T.rank == 0) cg_pair_fp64(A, W, pidx, M.red);
 }
 
 // The device's nanosecond clock (the same on every SM).
@@ -785,25 +949,31 @@ __device__ __forceinline__ int claim_item(int* queue, int P, unsigned long long 
 __host__ __device__ constexpr int cg_threads(bool large) { return large ? 1024 : 512; }
 // Padded points of a box that fit shared memory, 8 bytes (plain form) or 4
 // (mixed form) each.
-__host__ __device__ constexpr int cg_pad_limit(bool mixed, bool large) {
-  return mixed ? (large ? 56000 : 27000) : (large ? 28000 : 13824);
+__host__ __device__ constexpr int cg_pad_limit(bool mixed, bool large, bool team = false) {
+  return mixed ? (large ? 56000 : 27000) : (large ? (team ? 27000 : 28000) : 13824);
 }
 
-template <bool LARGE>
+// Each item's box is solved by the CTAs of a cluster (TEAM > 1) or one CTA.
+template <bool LARGE, int TEAM>
 __global__ void __launch_bounds__(cg_threads(LARGE), LARGE ? 1 : 2) k_cg(CgArgs A, StencilW W) {
-  __shared__ double red[2][32];
-  __shared__ int4 slots[64];
+  __shared__ CgShared<TEAM, cg_threads(LARGE) / 32> M;
   __shared__ int s_item;
   extern __shared__ int2 Ps[];  // A.cap[LARGE] points
+  const CgTeam T = cg_team<TEAM>();
+  team_sync(T);  // the team's CTAs have started
   const unsigned long long t0 = A.budget_ns ? global_ns() : 0ull;
   for (;;) {
-    if (threadIdx.x == 0) s_item = claim_item(A.queue + LARGE, A.P, A.budget_ns, t0, A.status);
-    __syncthreads();
+    if (T.rank == 0 && threadIdx.x == 0) {
+      s_item = claim_item(A.queue + LARGE, A.P, A.budget_ns, t0, A.status);
+      for (int o = 1; o < T.size; ++o) *team_ptr(&s_item, o) = s_item;
+    }
+    team_sync(T);
     const int item = s_item;
-    if (item >= A.P) break;
+    if (item >= A.P) break;  // no CTA writes to another from here on
     const int pidx = A.order[item];
-    if ((A.pinfo[pidx].n > SEA_CG_SPLIT) == LARGE) cg_pair_plain<LARGE>(A, W, pidx, red, slots, Ps);
-    __syncthreads();
+    if ((A.pinfo[pidx].n > SEA_CG_SPLIT) == LARGE)
+      cg_pair_plain(A, T, A.cap[LARGE], W, pidx, M, Ps);
+    team_sync(T);
   }
 }
 
@@ -1173,7 +1343,7 @@ __device__ __forceinline__ void cg_pair_mixed(const CgMixedArgs& A, const Stenci
     // reductions (compensated partials) all in FP32
     float2* fs0 = reinterpret_cast<float2*>(red[0]);
     float2* fs1 = reinterpret_cast<float2*>(red[1]);
-    if (cg_pad_volume(ex, ey, ez) <= A.cap[LARGE]) {
+    if (cg_pad_volume(ex, ey, ez, 1) <= A.cap[LARGE]) {
       inner_total = dres ? inner_cg_smem<true>(r, rnorm, x, d, pf, rf, qf, pS, n, ex, ey, ez, Wf,
                                                fs0, fs1, inner_total, A.max_iter)
                          : inner_cg_smem<false>(r, rnorm, x, d, pf, rf, qf, pS, n, ex, ey, ez, Wf,
@@ -1331,11 +1501,10 @@ template <bool MIXED, bool LARGE>
 __global__ void __launch_bounds__(cg_threads(LARGE), LARGE ? 1 : 2)
     k_cg_batch(const BatchCg* __restrict__ descs, const int2* __restrict__ items, int total,
                int* __restrict__ queue) {
-  __shared__ double red[2][32];
+  __shared__ CgShared<1, cg_threads(LARGE) / 32> M;
   __shared__ int s_item;
   __shared__ BatchCg d;
   __shared__ double bc;
-  __shared__ int4 slots[64];
   extern __shared__ int2 Ps[];  // the largest capacity of the descriptors
   float* pS = reinterpret_cast<float*>(Ps);
   for (;;) {
@@ -1354,9 +1523,9 @@ __global__ void __launch_bounds__(cg_threads(LARGE), LARGE ? 1 : 2)
     const int pidx = MIXED ? d.m.order[it.y] : d.a.order[it.y];
     if (((MIXED ? d.m.pinfo : d.a.pinfo)[pidx].n > SEA_CG_SPLIT) == LARGE) {
       if (MIXED)
-        cg_pair_mixed<LARGE>(d.m, d.W, d.Wf, pidx, red, &bc, pS);
+        cg_pair_mixed<LARGE>(d.m, d.W, d.Wf, pidx, M.red, &bc, pS);
       else
-        cg_pair_plain<LARGE>(d.a, d.W, pidx, red, slots, Ps);
+        cg_pair_plain(d.a, cg_team<1>(), d.a.cap[LARGE], d.W, pidx, M, Ps);
     }
     __syncthreads();
   }
@@ -1422,8 +1591,8 @@ static StencilWf make_weights_f(const StencilW& W) {
 
 // Points of a class's launch in shared memory: the largest padded pair box
 // pad_max, at most the class's limit; boxes above it solve on global vectors.
-static int cg_pad_cap(int pad_max, bool mixed, bool large) {
-  return std::min(pad_max, cg_pad_limit(mixed, large));
+static int cg_pad_cap(int pad_max, bool mixed, bool large, bool team = false) {
+  return std::min(pad_max, cg_pad_limit(mixed, large, team));
 }
 static size_t cg_smem_bytes(int cap, bool mixed) {
   return (size_t)cap * (mixed ? sizeof(float) : sizeof(int2));
@@ -1431,26 +1600,43 @@ static size_t cg_smem_bytes(int cap, bool mixed) {
 // The launch of a class's kernel: shared memory, CTAs (at most per_sm an SM
 // when that is positive) for `items` items.
 struct CgLaunch {
-  int grid, threads;
+  int grid, threads, team;
   size_t smem;
 };
 static cudaError_t cg_shape(const void* kernel, int pad_max, bool mixed, bool large, int items,
-                            int per_sm, CgLaunch* L) {
+                            int per_sm, int team, CgLaunch* L) {
   int dev = 0, nsm = 0, occ = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)cg_smem_bytes(cg_pad_limit(mixed, large), mixed));
+                             (int)cg_smem_bytes(cg_pad_limit(mixed, large, team > 1), mixed));
   if (e != cudaSuccess) return e;
   L->threads = cg_threads(large);
-  L->smem = cg_smem_bytes(cg_pad_cap(pad_max, mixed, large), mixed);
+  L->smem = cg_smem_bytes(cg_pad_cap(pad_max, mixed, large, team > 1), mixed);
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, L->threads, L->smem);
   if (e != cudaSuccess) return e;
   occ = std::max(occ, 1);
   if (per_sm > 0) occ = std::min(occ, per_sm);
-  L->grid = std::min(items, nsm * occ);
+  L->grid = team * std::max(1, std::min(items, nsm * occ / team));
+  L->team = team;
   return cudaSuccess;
+}
+// The launch itself, its CTAs in clusters of a team each.
+template <class... Par, class... Arg>
+static cudaError_t cg_run(void (*kernel)(Par...), const CgLaunch& L, cudaStream_t st, Arg... arg) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(L.grid);
+  cfg.blockDim = dim3(L.threads);
+  cfg.dynamicSmemBytes = L.smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = L.team;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = L.team > 1;
+  return cudaLaunchKernelEx(&cfg, kernel, Par(arg)...);
 }
 // A launch of n pairs, `large` of them of the large class: both classes side by
 // side, the large boxes' kernel on st, the others' on aux (after it on st when
@@ -1557,17 +1743,15 @@ cudaError_t launch_cg(sea_ctx* c) {
   const StencilW W = make_weights(c);
   return cg_both(c->stream, &c->aux, c->P, c->n_large, [&](bool large, cudaStream_t st) {
     auto km = large ? k_cg_mixed<true> : k_cg_mixed<false>;
-    auto kf = large ? k_cg<true> : k_cg<false>;
+    auto kf = large ? k_cg<true, 1> : k_cg<false, 1>;
     CgLaunch L;
     const cudaError_t e1 = cg_shape(mixed ? (const void*)km : (const void*)kf, c->cg_pad_max, mixed,
-                                    large, large ? c->n_large : c->P - c->n_large, 0, &L);
+                                    large, large ? c->n_large : c->P - c->n_large, 0,
+                                    1, &L);
     if (e1 != cudaSuccess) return e1;
-    if (mixed)
-      km<<<L.grid, L.threads, L.smem, st>>>(mixed_args(c), W, make_weights_f(W));
-    else
-      kf<<<L.grid, L.threads, L.smem, st>>>(fp64_args(c), W);
     c->launches += 1;
-    return cudaGetLastError();
+    return mixed ? cg_run(km, L, st, mixed_args(c), W, make_weights_f(W))
+                 : cg_run(kf, L, st, fp64_args(c), W);
   });
 }
 
@@ -1621,7 +1805,7 @@ int cg_batch_max_ctas_per_sm(int pad_max, bool mixed) {
   auto kern = mixed ? k_cg_batch<true, false> : k_cg_batch<false, false>;
   CgLaunch L;
   int occ = 0;
-  if (cg_shape((const void*)kern, pad_max, mixed, false, 1, 0, &L) != cudaSuccess ||
+  if (cg_shape((const void*)kern, pad_max, mixed, false, 1, 0, 1, &L) != cudaSuccess ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, L.threads, L.smem) != cudaSuccess)
     return 1;
   return std::max(occ, 1);
@@ -1638,22 +1822,48 @@ cudaError_t launch_cg_batch(cudaStream_t st, const CgAux* aux, const void* descs
                       : (large ? k_cg_batch<false, true> : k_cg_batch<false, false>);
     CgLaunch L;
     const cudaError_t e1 = cg_shape((const void*)kern, pad_max, mixed, large,
-                                    large ? n_large : total - n_large, large ? 0 : ctas_per_sm, &L);
+                                    large ? n_large : total - n_large, large ? 0 : ctas_per_sm,
+                                    1, &L);
     if (e1 != cudaSuccess) return e1;
-    kern<<<L.grid, L.threads, L.smem, s>>>((const BatchCg*)descs, items, total, queue);
-    return cudaGetLastError();
+    return cg_run(kern, L, s, (const BatchCg*)descs, items, total, queue);
   });
+}
+
+// The rule: as many CTAs a box (8 at most, the portable cluster size) as fill two
+// places per SM, fewer where a box that one CTA solves in fixed point would not
+// fit the team's registers and shared memory.  Time of a call with teams of 1, 2,
+// 4 and 8, us, boxes of 9 to 16 points an edge: 16 boxes 1019, 873, 770, 689; 48
+// boxes 1376, 1045, 933, 1055; 100 boxes 1335, 1337, 1136, 1721; 150 boxes 1450,
+// 1412, 1659, 2480; 450 boxes 1884, 2185, 3500, 6410 (there the teams' barriers
+// only delay SMs that have other boxes to work on).
+int cg_box_team(int n_box, const int* ext) {
+  int dev = 0, nsm = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return 1;
+  int team = SEA_CG_TEAM_MAX;
+  while (team > 1 && (long long)team * n_box > 2LL * nsm) team /= 2;
+  for (int b = 0; b < n_box && team > 1; ++b) {
+    const int* e = ext + 3 * b;
+    const int n = e[0] * e[1] * e[2];
+    const bool large = n > SEA_CG_SPLIT;
+    if (cg_pad_volume(e[0], e[1], e[2], 1) > cg_pad_limit(false, large)) continue;
+    while (team > 1 && (cg_share(n, team) > SEA_CG_TEAM_NP * cg_threads(large) ||
+                        cg_pad_volume(e[0], e[1], e[2], team) > cg_pad_limit(false, large, true)))
+      team /= 2;
+  }
+  return team;
 }
 
 // Batched solve of -Lap_h x = rhs on independent boxes (no pair energies):
 // boxes[] and voff[] on the device, order[] the processing order; r, p, q
-// scratch of the same total length as x; pad_max the boxes' largest
-// cg_pad_volume, n_large how many have more than SEA_CG_SPLIT points.
+// scratch of the same total length as x; team the CTAs a box
+// (cg_box_team), pad_max the boxes' largest cg_pad_volume of it, n_large how many have more than SEA_CG_SPLIT points.
 cudaError_t launch_cg_boxes(cudaStream_t stream, const double h[3], int nbox,
                             const PairInfo* boxes, const long long* voff, const int* order,
                             const double* rhs, double* x, double* r, double* p, double* q,
                             int* iters, unsigned* status, int* queue, double tol, int tol_mode,
-                            int max_iter, int pad_max, int n_large) {
+                            int max_iter, int team, int pad_max, int n_large) {
   if (nbox == 0) return cudaSuccess;
   double w[SEA_FDP + 1];
   fornberg_weights(w);
@@ -1672,7 +1882,7 @@ cudaError_t launch_cg_boxes(cudaStream_t stream, const double h[3], int nbox,
   CgArgs A;
   memset(&A, 0, sizeof(A));
   A.fix = make_fix(h);
-  for (int l = 0; l < 2; ++l) A.cap[l] = cg_pad_cap(pad_max, false, l);
+  for (int l = 0; l < 2; ++l) A.cap[l] = cg_pad_cap(pad_max, false, l, team > 1);
   A.phi = nullptr;
   A.nx = A.ny = A.nz = 1;
   A.pinfo = boxes;
@@ -1693,13 +1903,14 @@ cudaError_t launch_cg_boxes(cudaStream_t stream, const double h[3], int nbox,
   A.status = status;
   A.queue = queue;
   return cg_both(stream, nullptr, nbox, n_large, [&](bool large, cudaStream_t st) {
-    auto kern = large ? k_cg<true> : k_cg<false>;
+    auto kern = team > 2    ? (large ? k_cg<true, SEA_CG_TEAM_MAX> : k_cg<false, SEA_CG_TEAM_MAX>)
+                : team == 2 ? (large ? k_cg<true, 2> : k_cg<false, 2>)
+                            : (large ? k_cg<true, 1> : k_cg<false, 1>);
     CgLaunch L;
     const cudaError_t e1 = cg_shape((const void*)kern, pad_max, false, large,
-                                    large ? n_large : nbox - n_large, 0, &L);
+                                    large ? n_large : nbox - n_large, 0, team, &L);
     if (e1 != cudaSuccess) return e1;
-    kern<<<L.grid, L.threads, L.smem, st>>>(A, W);
-    return cudaGetLastError();
+    return cg_run(kern, L, st, A, W);
   });
 }
 

@@ -557,7 +557,7 @@ __global__ void k_scan_sizes(const int* __restrict__ sz, const int* __restrict__
     s += sz[x];
     nl += sz[x] > SEA_CG_SPLIT;
     const PairInfo P = pinfo[x];
-    pm = max(pm, cg_pad_volume(P.ext[0], P.ext[1], P.ext[2]));
+    pm = max(pm, cg_pad_volume(P.ext[0], P.ext[1], P.ext[2], 1));
   }
   long long acc = 0, nlarge = 0;
   long long pos = block_exscan_ll(s, part, &acc);

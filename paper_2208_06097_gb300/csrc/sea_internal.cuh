@@ -717,9 +717,14 @@ __host__ __device__ __forceinline__ void window_outside_point(const WinSplit& s,
 // serve as the y halo on both sides, and F zero planes before and after the
 // box for the z halo.  Box point t = (z ey + y) ex + x sits at
 // F ex (ey + F) + t + z F ex.  Neighbours along y and z outside the box read
-// zeros; along x they are masked.  Points of the layout (INT_MAX above that):
-__host__ __device__ __forceinline__ int cg_pad_volume(int ex, int ey, int ez) {
-  const long long v = (long long)ex * (ey + SEA_FDP) * (ez + 2 * SEA_FDP);
+// zeros; along x they are masked.  Points of the layout of one of `team` CTAs
+// that share the box's points (cg_share; INT_MAX above that):
+__host__ __device__ __forceinline__ int sea_min(int a, int b) { return a < b ? a : b; }
+__host__ __device__ __forceinline__ int cg_share(int n, int team) { return (n + team - 1) / team; }
+__host__ __device__ __forceinline__ int cg_pad_volume(int ex, int ey, int ez, int team) {
+  const int area = ex * ey;
+  const int nz = team == 1 ? ez : sea_min(ez, (cg_share(area * ez, team) + area - 1) / area + 1);
+  const long long v = (long long)ex * (ey + SEA_FDP) * (nz + 2 * SEA_FDP);
   return v > 2147483647LL ? 2147483647 : (int)v;
 }
 
@@ -735,6 +740,11 @@ __host__ __device__ __forceinline__ int cg_pad_volume(int ex, int ey, int ez) {
 // line at 3072 or 2048 points the 96^3 workloads, whose boxes lie below it,
 // lose 0 to 0.4 and 0.2 to 0.75 ms.
 #define SEA_CG_SPLIT 4096
+
+// CTAs (a cluster, at most SEA_CG_TEAM_MAX) that share a box of a bare batch of
+// n_box boxes on the current device.
+#define SEA_CG_TEAM_MAX 8
+int cg_box_team(int n_box, const int* ext);
 
 // Launch wrappers (each file implements its own).
 cudaError_t launch_plan_boxes(sea_ctx* c);
@@ -807,5 +817,5 @@ cudaError_t launch_cg_boxes(cudaStream_t stream, const double h[3], int nbox,
                             const PairInfo* boxes, const long long* voff, const int* order,
                             const double* rhs, double* x, double* r, double* p, double* q,
                             int* iters, unsigned* status, int* queue, double tol, int tol_mode,
-                            int max_iter, int pad_max, int n_large);
+                            int max_iter, int team, int pad_max, int n_large);
 }  // namespace sea
