@@ -140,12 +140,12 @@ __global__ void __launch_bounds__(256)
 
 // |dV sum_b part[o][b] - 1| > tol for some orbital o: SEA_FLAG_NORM (the
 // chunks added in index order).
-__global__ void k_check_norms(const double* __restrict__ part, int n, double dV, double tol,
+__global__ void k_check_norms(const double* __restrict__ part, int n, int parts, double dV, double tol,
                               unsigned* __restrict__ st) {
   const int o = blockIdx.x * blockDim.x + threadIdx.x;
   if (o >= n) return;
   double s = 0.0;
-  for (int b = 0; b < SEA_NORM_CHUNKS; ++b) s += part[(size_t)o * SEA_NORM_CHUNKS + b];
+  for (int b = 0; b < parts; ++b) s += part[(size_t)o * parts + b];
   if (!(fabs(s * dV - 1.0) <= tol)) atomicOr(st, SEA_FLAG_NORM);
 }
 
@@ -361,14 +361,28 @@ static sea_status load_orbitals(sea_ctx* c, const double* phi, int n_orb, int on
   SEA_ALLOC(eptr, (size_t)(n_orb + 1) * sizeof(int));
   SEA_ALLOC(ewin, (size_t)2 * ncand * sizeof(Entry));
   SEA_ALLOC(coff, (size_t)2 * ncand * sizeof(long long));
-  SEA_ALLOC(onorm, (size_t)n_orb * SEA_NORM_CHUNKS * sizeof(double));
+  SEA_ALLOC(onorm, (size_t)n_orb * std::max(SEA_NORM_CHUNKS, c->N[2]) * sizeof(double));
   double* npart = (double*)c->onorm.p;
   SEA_CK(cudaMemsetAsync(c->status.p, 0, sizeof(unsigned), c->stream), "memset");
   double* pd = (double*)(c->*into).p;
-  if (on_device) {
-    sea::k_check_orbitals<true><<<dim3(SEA_NORM_CHUNKS, n_orb), 256, 0, c->stream>>>(
-        phi, pd, c->ng, (unsigned*)c->status.p, npart);
+  // the plan's sums in the same pass, for orbitals that stay as they are
+  c->sums_ready = into == &sea_ctx::phi && c->N[0] <= SEA_SUMS_REG_MAX;
+  const int parts = c->sums_ready ? c->N[2] : SEA_NORM_CHUNKS;
+  auto check = [&](const double* from, size_t o0, size_t o1, double* dst) {
+    if (c->sums_ready)
+      return sea::launch_row_col_sums(c, from, (int)o0, (int)o1, dst, npart + o0 * parts);
+    const dim3 grid(SEA_NORM_CHUNKS, (unsigned)(o1 - o0));
+    unsigned* status = (unsigned*)c->status.p;
+    double* part = npart + o0 * parts;
+    if (dst)
+      sea::k_check_orbitals<true><<<grid, 256, 0, c->stream>>>(from, dst, c->ng, status, part);
+    else
+      sea::k_check_orbitals<false><<<grid, 256, 0, c->stream>>>(from, dst, c->ng, status, part);
     c->launches += 1;
+    return cudaGetLastError();
+  };
+  if (on_device) {
+    SEA_CK(check(phi, 0, n_orb, pd), "input check");
   } else {
     // orbital ranges copied in on the copy stream, each checked on the
     // context stream once it has arrived
@@ -386,15 +400,11 @@ static sea_status load_orbitals(sea_ctx* c, const double* phi, int n_orb, int on
     for (int k = 0; k < nch; ++k) {
       const size_t o0 = (size_t)n_orb * k / nch, o1 = (size_t)n_orb * (k + 1) / nch;
       SEA_CK(cudaStreamWaitEvent(c->stream, c->xev[k], 0), "wait");
-      sea::k_check_orbitals<false><<<dim3(SEA_NORM_CHUNKS, (unsigned)(o1 - o0)), 256, 0,
-                                     c->stream>>>(pd + o0 * c->ng, nullptr, c->ng,
-                                                  (unsigned*)c->status.p,
-                                                  npart + o0 * SEA_NORM_CHUNKS);
-      c->launches += 1;
+      SEA_CK(check(pd + o0 * c->ng, o0, o1, nullptr), "input check");
     }
   }
   if (c->prm.orth_tol > 0.0) {
-    sea::k_check_norms<<<(n_orb + 127) / 128, 128, 0, c->stream>>>(npart, n_orb, c->dV,
+    sea::k_check_norms<<<(n_orb + 127) / 128, 128, 0, c->stream>>>(npart, n_orb, parts, c->dV,
                                                                     c->prm.orth_tol,
                                                                     (unsigned*)c->status.p);
     c->launches += 1;
@@ -459,7 +469,7 @@ sea_status sea_apply_vxx(sea_ctx* c, double* vxx_phi, int on_device, double* exx
   {
     // the plan: a fixed launch sequence for the context's sizes and buffers
     const std::vector<uintptr_t> sig = {
-        (uintptr_t)c->n_orb, (uintptr_t)c->N[0], (uintptr_t)c->N[1], (uintptr_t)c->N[2],
+        (uintptr_t)c->n_orb, (uintptr_t)c->sums_ready, (uintptr_t)c->N[0], (uintptr_t)c->N[1], (uintptr_t)c->N[2],
         (uintptr_t)c->device, sea::bits_of(c->prm.eps), sea::bits_of(c->prm.delta),
         sea::bits_of(c->dV),
         (uintptr_t)c->phi.p, (uintptr_t)c->rowsum.p, (uintptr_t)c->colsum.p, (uintptr_t)c->marg.p,

@@ -156,38 +156,59 @@ __global__ void __launch_bounds__(128)
   for (int x = threadIdx.x; x < nx; x += blockDim.x) C[((size_t)i * nz + z) * nx + x] = col[x];
 }
 
-// The same sums without a shared-memory tile, for rows of at most 32 KX
+// A warp's sum of 48-bit limb sums below 2^52 (two parts of 26 bits: 32 lanes
+// stay below 2^31).
+__device__ __forceinline__ unsigned long long warp_sum52(unsigned long long v) {
+  const unsigned a = __reduce_add_sync(0xffffffffu, (unsigned)v & 0x3FFFFFFu);
+  const unsigned b = __reduce_add_sync(0xffffffffu, (unsigned)(v >> 26));
+  return ((unsigned long long)b << 26) + a;
+}
+
+// The same sums without a shared-memory tile, for rows of at most 32 KX <= 256
 // points: warp w takes the rows y = w, w + 4, ... (two at a time), lane l
-// the points x = l + 32 k; a row's sum is a warp butterfly, a column's
-// partial sums stay in the lane's registers until one exchange between the
-// four warps at the end of the plane.  All sums are exact, so the order is
-// free.
-template <int KX>
+// the points x = l + 32 k; a row's sum is four integer reductions of the warp,
+// a column's partial sums stay in the lane's registers until one exchange
+// between the four warps at the end of the plane.  All sums are exact, so the
+// order is free.
+// CHECK: as sea_set_orbitals' pass over the caller's orbitals it also copies
+// them (dst, where not null), flags non-finite values and writes the plane's
+// FP64 sum of squares to part[orbital][z] (a fixed order), so that they are
+// read once instead of twice: bound by HBM (16 bytes a point with the copy).
+// 256 orbitals on 96^3, whole exchange: 2.99 -> 2.70 ms (two passes took 0.55 + 0.34 ms).
+template <int KX, bool CHECK>
 __global__ void __launch_bounds__(128)
     k_row_col_sums_reg(const double* __restrict__ phi, int nx, int ny, int nz,
-                       ulonglong2* __restrict__ R, ulonglong2* __restrict__ C) {
+                       ulonglong2* __restrict__ R, ulonglong2* __restrict__ C,
+                       double* __restrict__ dst, unsigned* __restrict__ st,
+                       double* __restrict__ part) {
   __shared__ ulonglong2 cpart[4][32 * KX];  // per warp: column partial sums
+  __shared__ double red[32];
   const int z = blockIdx.x, i = blockIdx.y;
-  const double* plane = phi + ((size_t)i * nz + z) * (size_t)ny * nx;
+  const size_t base = ((size_t)i * nz + z) * (size_t)ny * nx;
+  const double* plane = phi + base;
   ulonglong2* Rp = R + ((size_t)i * nz + z) * ny;
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   unsigned long long clo[KX], chi[KX];
+  unsigned emax = 0;  // largest exponent field
+  double sum = 0.0;
 #pragma unroll
   for (int k = 0; k < KX; ++k) clo[k] = chi[k] = 0;
-  for (int y0 = w; y0 < ny; y0 += 8) {
-    double v[2][KX];
+  constexpr int TR = CHECK && KX <= 4 ? 4 : 2;  // rows at a time
+  for (int y0 = w; y0 < ny; y0 += 4 * TR) {
+    double v[TR][KX];
 #pragma unroll
-    for (int t = 0; t < 2; ++t) {
+    for (int t = 0; t < TR; ++t) {
       const int y = y0 + 4 * t;
       const double* row = plane + (size_t)y * nx;
 #pragma unroll
       for (int k = 0; k < KX; ++k) {
         const int x = lane + 32 * k;
-        v[t][k] = (y < ny && x < nx) ? row[x] : 0.0;
+        v[t][k] = (y < ny && x < nx) ? (CHECK ? __ldcs(row + x) : row[x]) : 0.0;
       }
     }
 #pragma unroll
-    for (int t = 0; t < 2; ++t) {
+    for (int t = 0; t < TR; ++t) {
+      const int y = y0 + 4 * t;
       unsigned long long rlo = 0, rhi = 0;
 #pragma unroll
       for (int k = 0; k < KX; ++k) {
@@ -197,13 +218,15 @@ __global__ void __launch_bounds__(128)
         chi[k] += hi;
         rlo += lo;
         rhi += hi;
+        if (CHECK) {
+          const int x = lane + 32 * k;
+          if (dst && y < ny && x < nx) dst[base + (size_t)y * nx + x] = v[t][k];
+          emax = max(emax, (unsigned)__double2hiint(v[t][k]) & 0x7FF00000u);
+          sum = fma(v[t][k], v[t][k], sum);
+        }
       }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        rlo += __shfl_xor_sync(0xffffffffu, rlo, o);
-        rhi += __shfl_xor_sync(0xffffffffu, rhi, o);
-      }
-      const int y = y0 + 4 * t;
+      rlo = warp_sum52(rlo);
+      rhi = warp_sum52(rhi);
       if (lane == 0 && y < ny) Rp[y] = make_ulonglong2(rlo, rhi);
     }
   }
@@ -218,6 +241,12 @@ __global__ void __launch_bounds__(128)
       c.y += cpart[u][x].y;
     }
     C[((size_t)i * nz + z) * nx + x] = c;
+  }
+  if (CHECK) {
+    if (__syncthreads_or(emax == 0x7FF00000u) && threadIdx.x == 0)
+      atomicOr(st, SEA_FLAG_NONFINITE);
+    sum = block_sum(sum, red);
+    if (threadIdx.x == 0) part[(size_t)i * nz + z] = sum;
   }
 }
 
@@ -599,29 +628,41 @@ __global__ void __launch_bounds__(256) k_lpt_order(const int* __restrict__ sz,
   if (p < n) order[rank] = p;
 }
 
+// Row and column sums of F(phi) for orbitals [o0, o1) at `phi` (the first of
+// them); with part not null also the checks and, with dst, the copy of
+// sea_set_orbitals (rows of at most SEA_SUMS_REG_MAX points).
+cudaError_t launch_row_col_sums(sea_ctx* c, const double* phi, int o0, int o1, double* dst,
+                                double* part) {
+  const int nx = c->N[0], ny = c->N[1], nz = c->N[2];
+  const dim3 grid(nz, o1 - o0);
+  ulonglong2* Rs = (ulonglong2*)c->rowsum.p + (size_t)o0 * nz * ny;
+  ulonglong2* Cs = (ulonglong2*)c->colsum.p + (size_t)o0 * nz * nx;
+  unsigned* st = (unsigned*)c->status.p;
+  c->launches += 1;
+  auto run = [&](auto plain, auto check) {
+    (part ? check : plain)<<<grid, 128, 0, c->stream>>>(phi, nx, ny, nz, Rs, Cs, dst, st, part);
+    return cudaGetLastError();
+  };
+  if (nx <= 64) return run(k_row_col_sums_reg<2, false>, k_row_col_sums_reg<2, true>);
+  if (nx <= 96) return run(k_row_col_sums_reg<3, false>, k_row_col_sums_reg<3, true>);
+  if (nx <= 128) return run(k_row_col_sums_reg<4, false>, k_row_col_sums_reg<4, true>);
+  if (nx <= 192) return run(k_row_col_sums_reg<6, false>, k_row_col_sums_reg<6, true>);
+  if (nx <= SEA_SUMS_REG_MAX) return run(k_row_col_sums_reg<8, false>, k_row_col_sums_reg<8, true>);
+  const size_t rc_smem = rc_smem_bytes(nx);
+  const cudaError_t e = cudaFuncSetAttribute(
+      k_row_col_sums, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rc_smem);
+  if (e != cudaSuccess) return e;
+  k_row_col_sums<<<grid, 128, rc_smem, c->stream>>>(phi, nx, ny, nz, Rs, Cs);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_plan_boxes(sea_ctx* c) {
   const int n = c->n_orb, nx = c->N[0], ny = c->N[1], nz = c->N[2];
   const int Nmax = max(nx, max(ny, nz));
-  const dim3 rc_grid(nz, n);
   const double* phi = (const double*)c->phi.p;
-  ulonglong2* Rs = (ulonglong2*)c->rowsum.p;
-  ulonglong2* Cs = (ulonglong2*)c->colsum.p;
-  if (nx <= 64)
-    k_row_col_sums_reg<2><<<rc_grid, 128, 0, c->stream>>>(phi, nx, ny, nz, Rs, Cs);
-  else if (nx <= 96)
-    k_row_col_sums_reg<3><<<rc_grid, 128, 0, c->stream>>>(phi, nx, ny, nz, Rs, Cs);
-  else if (nx <= 128)
-    k_row_col_sums_reg<4><<<rc_grid, 128, 0, c->stream>>>(phi, nx, ny, nz, Rs, Cs);
-  else if (nx <= 192)
-    k_row_col_sums_reg<6><<<rc_grid, 128, 0, c->stream>>>(phi, nx, ny, nz, Rs, Cs);
-  else if (nx <= 256)
-    k_row_col_sums_reg<8><<<rc_grid, 128, 0, c->stream>>>(phi, nx, ny, nz, Rs, Cs);
-  else {
-    const size_t rc_smem = rc_smem_bytes(nx);
-    cudaError_t e = cudaFuncSetAttribute(k_row_col_sums, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)rc_smem);
+  if (!c->sums_ready) {
+    const cudaError_t e = launch_row_col_sums(c, phi, 0, n, nullptr, nullptr);
     if (e != cudaSuccess) return e;
-    k_row_col_sums<<<rc_grid, 128, rc_smem, c->stream>>>(phi, nx, ny, nz, Rs, Cs);
   }
   {
     const int mmin = std::max(1, std::min(nx, ny));
@@ -637,7 +678,7 @@ cudaError_t launch_plan_boxes(sea_ctx* c) {
   }
   k_box_fit<<<n * 3, 128, Nmax * sizeof(double), c->stream>>>(
       (const double*)c->marg.p, nx, ny, nz, Nmax, c->prm.eps / 3.0, (int*)c->box.p);
-  c->launches += 3;
+  c->launches += 2;
   return cudaGetLastError();
 }
 

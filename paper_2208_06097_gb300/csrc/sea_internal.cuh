@@ -511,6 +511,7 @@ struct sea_ctx {
   // device buffers
   SeaBuf phi, vxx_dev, psi_dev, out_dev;
   SeaBuf rowsum, colsum, marg, box;
+  bool sums_ready = false;  // rowsum and colsum are those of phi (formed as it was read)
   SeaBuf cand_flag, cand_geom, list_a, list_b, cand_S, counts;
   SeaBuf pinfo, pS, psize, voff, order, Q, epair, iters;
   SeaBuf vbuf, bbuf, rbuf, pbuf, qbuf;
@@ -747,6 +748,10 @@ __host__ __device__ __forceinline__ int cg_pad_volume(int ex, int ey, int ez, in
 int cg_box_team(int n_box, const int* ext);
 
 // Launch wrappers (each file implements its own).
+// Rows that the plan's sums are formed of in registers.
+#define SEA_SUMS_REG_MAX 256
+cudaError_t launch_row_col_sums(sea_ctx* c, const double* phi, int o0, int o1, double* dst,
+                                double* part);
 cudaError_t launch_plan_boxes(sea_ctx* c);
 cudaError_t launch_plan_pairs(sea_ctx* c);
 cudaError_t launch_pair_setup(sea_ctx* c);
