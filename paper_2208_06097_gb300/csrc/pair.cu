@@ -950,7 +950,7 @@ __host__ __device__ constexpr int cg_threads(bool large) { return large ? 1024 :
 // Padded points of a box that fit shared memory, 8 bytes (plain form) or 4
 // (mixed form) each.
 __host__ __device__ constexpr int cg_pad_limit(bool mixed, bool large, bool team = false) {
-  return mixed ? (large ? 56000 : 27000) : (large ? (team ? 27000 : 28000) : 13824);
+  return mixed ? (large ? 56000 : SEA_CG_SINGLE) : (large ? (team ? 27000 : 28000) : 13824);
 }
 
 // Each item's box is solved by the CTAs of a cluster (TEAM > 1) or one CTA.
@@ -971,7 +971,7 @@ __global__ void __launch_bounds__(cg_threads(LARGE), LARGE ? 1 : 2) k_cg(CgArgs 
     const int item = s_item;
     if (item >= A.P) break;  // no CTA writes to another from here on
     const int pidx = A.order[item];
-    if ((A.pinfo[pidx].n > SEA_CG_SPLIT) == LARGE)
+    if (cg_large(A.pinfo[pidx].ext, false) == LARGE)
       cg_pair_plain(A, T, A.cap[LARGE], W, pidx, M, Ps);
     team_sync(T);
   }
@@ -1223,6 +1223,64 @@ __device__ __forceinline__ int inner_cg_smem(const double* __restrict__ r, doubl
   return inner_total;
 }
 
+// Inner solve by CG with two reductions per iteration and compensated dot
+// products, the search direction in shared memory in the same padded layout
+// (r, q and d in global memory): the boxes over SEA_CG_SINGLE padded points.  Its
+// iterates are those of the form on global vectors below, whatever the CTA
+// size; the single-reduction arrangement on 1024 threads stopped some of their
+// inner solves an iteration apart, which moved V_xx phi by up to 2.4e-9 of its
+// norm (19 waters on 91^3).  rf holds r / ||r||.  Returns the new total of inner
+// iterations.
+__device__ __forceinline__ int inner_cg2_smem(float* __restrict__ d, float* __restrict__ rf,
+                                              float* __restrict__ qf, float* __restrict__ pS, int n,
+                                              int ex, int ey, int ez, const StencilWf& Wf,
+                                              float2* fs0, float2* fs1, int inner_total,
+                                              int max_iter) {
+  const int S = blockDim.x;
+  const int PXY = ex * (ey + SEA_FDP), gap = SEA_FDP * ex, org = SEA_FDP * PXY;
+  const int Vp = PXY * (ez + 2 * SEA_FDP);
+  for (int t = threadIdx.x; t < Vp; t += S) pS[t] = 0.f;
+  __syncthreads();
+  DotF rr0;
+  for (BoxWalk w(threadIdx.x, S, ex, ey); w.t < n; w.next(S)) {
+    const float v = rf[w.t];
+    pS[org + w.t + w.z * gap] = v;
+    d[w.t] = 0.f;
+    rr0.add(v, v);
+  }
+  float rr = block_sum_f(rr0.hi, rr0.lo, fs1);  // also: pS is complete
+  const float stop = (float)SEA_MIXED_INNER * (float)SEA_MIXED_INNER * rr;  // on ||r||^2
+  while (rr > stop && inner_total < max_iter) {
+    DotF pq0;
+    for (BoxWalk w(threadIdx.x, S, ex, ey); w.t < n; w.next(S)) {
+      const int tp = org + w.t + w.z * gap;
+      const float q0 = neg_lap_pad(pS, tp, w.x, ex, PXY, Wf);
+      qf[w.t] = q0;
+      pq0.add(pS[tp], q0);
+    }
+    const float pq = block_sum_f(pq0.hi, pq0.lo, fs0);
+    const float alpha = rr / pq;
+    DotF rn0;
+    for (BoxWalk w(threadIdx.x, S, ex, ey); w.t < n; w.next(S)) {
+      d[w.t] = fmaf(alpha, pS[org + w.t + w.z * gap], d[w.t]);
+      const float rt = fmaf(-alpha, qf[w.t], rf[w.t]);
+      rf[w.t] = rt;
+      rn0.add(rt, rt);
+    }
+    const float rn = block_sum_f(rn0.hi, rn0.lo, fs1);
+    ++inner_total;
+    const float beta = rn / rr;
+    rr = rn;
+    if (rn <= stop) break;
+    for (BoxWalk w(threadIdx.x, S, ex, ey); w.t < n; w.next(S)) {
+      const int tp = org + w.t + w.z * gap;
+      pS[tp] = fmaf(beta, pS[tp], rf[w.t]);
+    }
+    __syncthreads();
+  }
+  return inner_total;
+}
+
 struct CgMixedArgs {
   const double* phi;
   int nx, ny, nz;
@@ -1261,6 +1319,16 @@ __device__ __forceinline__ double block_sum_1w(double v, double* slots, double* 
   }
   __syncthreads();
   return *bc;
+}
+
+// This thread's part of sum hi^2 over the n points of r, in the order of a CTA of
+// 512 threads whatever the CTA's (the FP32 sum depends on it); all threads call.
+__device__ __forceinline__ float square512(const float2* r, int n) {
+  __syncthreads();  // r is written
+  float s = 0.f;
+  if (threadIdx.x < 512)
+    for (int t = threadIdx.x; t < n; t += 512) s = fmaf(r[t].x, r[t].x, s);
+  return s;
 }
 
 // One pair's mixed-precision solve (the whole CTA).
@@ -1309,9 +1377,9 @@ __device__ __forceinline__ void cg_pair_mixed(const CgMixedArgs& A, const Stenci
       if (A.warm) rt = df_add(rt, df_neg(neg_lap_df(xd, w.t, w.x, w.y, w.z, ex, ey, ez, Wo)));
       rd[w.t] = make_float2(rt.hi, rt.lo);
       bb = fma(bt, bt, bb);
-      rr0f = fmaf(rt.hi, rt.hi, rr0f);
+      if (!LARGE) rr0f = fmaf(rt.hi, rt.hi, rr0f);
     }
-    rr0 = (double)rr0f;
+    rr0 = (double)(LARGE ? square512(rd, n) : rr0f);
   } else {
     for (int t = threadIdx.x; t < n; t += S) {
       const double bt = b[t];
@@ -1343,7 +1411,8 @@ __device__ __forceinline__ void cg_pair_mixed(const CgMixedArgs& A, const Stenci
     // reductions (compensated partials) all in FP32
     float2* fs0 = reinterpret_cast<float2*>(red[0]);
     float2* fs1 = reinterpret_cast<float2*>(red[1]);
-    if (cg_pad_volume(ex, ey, ez, 1) <= A.cap[LARGE]) {
+    const int pad = cg_pad_volume(ex, ey, ez, 1);
+    if (!LARGE) {
       inner_total = dres ? inner_cg_smem<true>(r, rnorm, x, d, pf, rf, qf, pS, n, ex, ey, ez, Wf,
                                                fs0, fs1, inner_total, A.max_iter)
                          : inner_cg_smem<false>(r, rnorm, x, d, pf, rf, qf, pS, n, ex, ey, ez, Wf,
@@ -1358,7 +1427,11 @@ __device__ __forceinline__ void cg_pair_mixed(const CgMixedArgs& A, const Stenci
       d[t] = 0.f;
       rr0.add(v, v);
     }
-    float rr = block_sum_f(rr0.hi, rr0.lo, fs1);
+    const bool fits = pad <= A.cap[LARGE];
+    if (fits)
+      inner_total = inner_cg2_smem(d, rf, qf, pS, n, ex, ey, ez, Wf, fs0, fs1, inner_total,
+                                   A.max_iter);
+    float rr = fits ? 0.f : block_sum_f(rr0.hi, rr0.lo, fs1);
     const float stop = (float)SEA_MIXED_INNER * (float)SEA_MIXED_INNER * rr;  // on ||r||^2
     while (rr > stop && inner_total < A.max_iter) {
       DotF pq0, pq1;
@@ -1419,9 +1492,9 @@ __device__ __forceinline__ void cg_pair_mixed(const CgMixedArgs& A, const Stenci
         const DF rt = df_add(DF{bs.x, bs.y},
                              df_neg(neg_lap_df(xd, w0.t, w0.x, w0.y, w0.z, ex, ey, ez, Wo)));
         rd[w0.t] = make_float2(rt.hi, rt.lo);
-        r2f = fmaf(rt.hi, rt.hi, r2f);
+        if (!LARGE) r2f = fmaf(rt.hi, rt.hi, r2f);
       }
-      r2 = (double)r2f;
+      r2 = (double)(LARGE ? square512(rd, n) : r2f);
     } else {
       BoxWalk w0(threadIdx.x, S, ex, ey);
       for (; w0.t < n; w0.next(S)) {
@@ -1474,7 +1547,7 @@ __global__ void __launch_bounds__(cg_threads(LARGE), LARGE ? 1 : 2)
     const int item = s_item;
     if (item >= A.P) break;
     const int pidx = A.order[item];
-    if ((A.pinfo[pidx].n > SEA_CG_SPLIT) == LARGE) cg_pair_mixed<LARGE>(A, W, Wf, pidx, red, &bc, pS);
+    if (cg_large(A.pinfo[pidx].ext, true) == LARGE) cg_pair_mixed<LARGE>(A, W, Wf, pidx, red, &bc, pS);
     __syncthreads();
   }
 }
@@ -1521,7 +1594,7 @@ __global__ void __launch_bounds__(cg_threads(LARGE), LARGE ? 1 : 2)
     }
     __syncthreads();
     const int pidx = MIXED ? d.m.order[it.y] : d.a.order[it.y];
-    if (((MIXED ? d.m.pinfo : d.a.pinfo)[pidx].n > SEA_CG_SPLIT) == LARGE) {
+    if (cg_large((MIXED ? d.m.pinfo : d.a.pinfo)[pidx].ext, MIXED) == LARGE) {
       if (MIXED)
         cg_pair_mixed<LARGE>(d.m, d.W, d.Wf, pidx, M.red, &bc, pS);
       else

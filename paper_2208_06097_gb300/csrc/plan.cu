@@ -574,7 +574,7 @@ __global__ void k_fill_pairs(const int* __restrict__ kept, const int* __restrict
 __global__ void k_scan_sizes(const int* __restrict__ sz, const int* __restrict__ count,
                              const PairInfo* __restrict__ pinfo, long long* __restrict__ off,
                              long long* __restrict__ tot, int* __restrict__ maxpad,
-                             int* __restrict__ large) {
+                             int* __restrict__ large, bool mixed) {
   __shared__ long long part[32];
   const int n = *count;
   const int T = blockDim.x;
@@ -584,8 +584,8 @@ __global__ void k_scan_sizes(const int* __restrict__ sz, const int* __restrict__
   int pm = 0;
   for (int x = b; x < e; ++x) {
     s += sz[x];
-    nl += sz[x] > SEA_CG_SPLIT;
     const PairInfo P = pinfo[x];
+    nl += cg_large(P.ext, mixed);
     pm = max(pm, cg_pad_volume(P.ext[0], P.ext[1], P.ext[2], 1));
   }
   long long acc = 0, nlarge = 0;
@@ -709,7 +709,8 @@ cudaError_t launch_plan_pairs(sea_ctx* c) {
                                           (double*)c->pS.p, (int*)c->psize.p);
   k_scan_sizes<<<1, 1024, 0, c->stream>>>((const int*)c->psize.p, counts + 1,
                                           (const PairInfo*)c->pinfo.p, (long long*)c->voff.p,
-                                          (long long*)(counts + 4), counts + 10, counts + 3);
+                                          (long long*)(counts + 4), counts + 10, counts + 3,
+                                          c->prm.precision == 1);
   k_lpt_order<<<gc, 256, 0, c->stream>>>((const int*)c->psize.p, counts + 1, (int*)c->order.p);
   c->launches += 7;
   return cudaGetLastError();

@@ -736,11 +736,19 @@ __host__ __device__ __forceinline__ int cg_pad_volume(int ex, int ey, int ez, in
 // barriers.  Larger boxes: CTAs of 1024 threads, one per SM: a step of a large
 // box takes several rounds of its CTA's points, a launch seldom has two of
 // them per SM, and one may hold a padded box twice as large in shared memory.
-// (H2O)16 on 81^3, most boxes large: mixed CG 2.33 -> 1.40 ms; FP64 26.7 -> 3.05
-// ms, since the padded boxes no longer miss the fixed-point stencil.  With the
+// (H2O)16 on 81^3, most boxes large: FP64 CG 26.7 -> 3.05 ms, since the padded
+// boxes no longer miss the fixed-point stencil.  With the
 // line at 3072 or 2048 points the 96^3 workloads, whose boxes lie below it,
 // lose 0 to 0.4 and 0.2 to 0.75 ms.
 #define SEA_CG_SPLIT 4096
+// In the mixed form the line is at SEA_CG_SINGLE padded points, where its inner
+// solve changes its arrangement: its FP32 sums depend on the CTA size, so each
+// arrangement keeps one.
+#define SEA_CG_SINGLE 13824
+__host__ __device__ __forceinline__ bool cg_large(const int* ext, bool mixed) {
+  return mixed ? cg_pad_volume(ext[0], ext[1], ext[2], 1) > SEA_CG_SINGLE
+               : ext[0] * ext[1] * ext[2] > SEA_CG_SPLIT;
+}
 
 // CTAs (a cluster, at most SEA_CG_TEAM_MAX) that share a box of a bare batch of
 // n_box boxes on the current device.
