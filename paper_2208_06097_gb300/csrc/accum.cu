@@ -394,17 +394,22 @@ __device__ __forceinline__ bool cyc_hits(int s, int L, int a, int b, int n) {
   return a < min(b, s + L - n);  // the wrapped part [0, s + L - n)
 }
 
-// Shared-memory form: CTA per (orbital, z-plane), the plane (nx*ny
-// doubles) in dynamic shared memory.  A thread walks the window rows of an
-// entry with its (tx, ty) advanced by the CTA stride, without divisions.
+// Shared-memory form: CTA per (orbital, z-plane, slab of `rows` rows), the slab
+// (nx*rows doubles) in dynamic shared memory: whole planes where three CTAs of
+// them fit an SM, else as few slabs as let three fit, so that one's stores
+// overlap the others' window reads (far field and accumulation of 128 orbitals:
+// 100^2 planes 0.284 -> 0.272 ms, 112^2 0.370 -> 0.335, 128^2 0.749 -> 0.495, 159^2
+// with 64 0.897 -> 0.670; on 96^2, 74 KB, slabs only add window walks).  A thread walks the window rows of an entry with its (tx, ty) advanced
+// by the CTA stride, without divisions.
 // With a second output (the caller's copy, written in full), the context's
 // copy is stored only on the tiles (TX x TY x TZ) that a window of the
 // orbital touches: the tiles of the orbital's W lists, the only places the
 // ACE kernels read it (tile mask after the plane, in shared memory).
 #define SEA_ACC_MAXE 64
 #define SEA_ACC_THREADS 512
+#define SEA_ACC_SMEM_SLAB 75000  // three CTAs and their static shared memory per SM
 __global__ void __launch_bounds__(SEA_ACC_THREADS)
-    k_accumulate(int nx, int ny, int nz, int o_begin, const int* __restrict__ eptr,
+    k_accumulate(int nx, int ny, int nz, int rows, int o_begin, const int* __restrict__ eptr,
                  const Entry* __restrict__ ent, const long long* __restrict__ coff,
                  const double* __restrict__ cbuf, double* __restrict__ out,
                  double* __restrict__ out2, int bulk) {
@@ -412,7 +417,8 @@ __global__ void __launch_bounds__(SEA_ACC_THREADS)
   __shared__ int es[SEA_ACC_MAXE][5];  // x start, x length, y start, y length, meets the z tile
   const int o = o_begin + blockIdx.x;
   const int z = blockIdx.y;
-  const int plane = nx * ny;
+  const int ya = blockIdx.z * rows, yb = min(ny, ya + rows);  // ya: a multiple of TY
+  const int plane = nx * (yb - ya);                           // points of the slab
   unsigned char* tmask = reinterpret_cast<unsigned char*>(sp + plane);
   if ((plane & 1) == 0) {
     double2* sp2 = reinterpret_cast<double2*>(sp);
@@ -427,22 +433,25 @@ __global__ void __launch_bounds__(SEA_ACC_THREADS)
     if (tz >= e.wl[2]) continue;  // uniform over the CTA
     __syncthreads();
     const int wx = e.wl[0], wy = e.wl[1];
-    const int rowpts = wx * wy;
-    const double* c = cbuf + coff[k] + (size_t)tz * rowpts;
+    const double* c = cbuf + coff[k] + (size_t)tz * (wx * wy);
     const int x0 = wrapi(e.ws[0], nx), y0 = wrapi(e.ws[1], ny);
     const int sy = blockDim.x / wx, sx = blockDim.x - sy * wx;  // stride as (rows, columns)
-    int ty = threadIdx.x / wx, tx = threadIdx.x - ty * wx;
-    for (int r = threadIdx.x; r < rowpts; r += blockDim.x) {
-      int gx = x0 + tx, gy = y0 + ty;
-      gx -= gx >= nx ? nx : 0;
-      gy -= gy >= ny ? ny : 0;
-      const int g = gy * nx + gx;
-      sp[g] = __dsub_rn(sp[g], c[r]);
-      tx += sx;
-      ty += sy;
-      if (tx >= wx) {
-        tx -= wx;
-        ++ty;
+    // window rows in the slab: before and after the cell's edge
+    for (int ys = y0; ys > y0 - 2 * ny; ys -= ny) {
+      const int r0 = max(0, ya - ys), r1 = min(wy, yb - ys);
+      int ty = threadIdx.x / wx, tx = threadIdx.x - ty * wx;
+      ty += r0;
+      for (int r = r0 * wx + threadIdx.x; r < r1 * wx; r += blockDim.x) {
+        int gx = x0 + tx;
+        gx -= gx >= nx ? nx : 0;
+        const int g = (ys + ty - ya) * nx + gx;
+        sp[g] = __dsub_rn(sp[g], c[r]);
+        tx += sx;
+        ty += sy;
+        if (tx >= wx) {
+          tx -= wx;
+          ++ty;
+        }
       }
     }
   }
@@ -460,10 +469,10 @@ __global__ void __launch_bounds__(SEA_ACC_THREADS)
       es[t][4] = cyc_hits(wrapi(e.ws[2], nz), e.wl[2], zs, min(nz, zs + TZ), nz);
     }
     __syncthreads();
-    const int nty = (ny + TY - 1) / TY;
+    const int nty = (yb - ya + TY - 1) / TY;
     for (int q = threadIdx.x; q < ntx * nty; q += blockDim.x) {
       const int qy = q / ntx, qx = q - qy * ntx;
-      const int ax = qx * TX, bx = min(nx, ax + TX), ay = qy * TY, by = min(ny, ay + TY);
+      const int ax = qx * TX, bx = min(nx, ax + TX), ay = ya + qy * TY, by = min(ny, ay + TY);
       bool hit = false;
       for (int k = 0; k < e1 - e0; ++k)
         hit = hit || (es[k][4] && cyc_hits(es[k][0], es[k][1], ax, bx, nx) &&
@@ -471,10 +480,10 @@ __global__ void __launch_bounds__(SEA_ACC_THREADS)
       tmask[q] = hit ? 1 : 0;
     }
   }
-  const size_t base = ((size_t)o * nz + z) * plane;
+  const size_t base = (((size_t)o * nz + z) * ny + ya) * nx;
   // The output stored in full (out2, else out when every tile is wanted) by
-  // one bulk copy of the plane from shared memory when `bulk` (the plane is
-  // a multiple of 16 bytes and the outputs 16-byte aligned): the generic
+  // one bulk copy of the slab from shared memory when `bulk` (planes and
+  // four rows are multiples of 16 bytes and the outputs 16-byte aligned): the generic
   // writes are made visible to the copy engine, then thread 0 issues it and
   // waits, before the CTA ends, until the plane has been read.
   double* full = out2 ? out2 : (all ? out : nullptr);
@@ -487,7 +496,7 @@ __global__ void __launch_bounds__(SEA_ACC_THREADS)
                  : "memory");
     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
   }
-  const int nty = (ny + TY - 1) / TY;
+  const int nty = (yb - ya + TY - 1) / TY;
   if (by_copy && out2 != nullptr && !all) {
     // the context's copy on the marked tiles only: a thread per tile, its
     // rows as 16-byte pieces when rows and outputs allow it
@@ -495,7 +504,7 @@ __global__ void __launch_bounds__(SEA_ACC_THREADS)
     for (int q = threadIdx.x; q < ntx * nty; q += blockDim.x) {
       if (!tmask[q]) continue;
       const int qy = q / ntx, qx = q - qy * ntx;
-      const int x0 = qx * TX, x1 = min(nx, x0 + TX), y1 = min(ny, qy * TY + TY);
+      const int x0 = qx * TX, x1 = min(nx, x0 + TX), y1 = min(yb - ya, qy * TY + TY);
       for (int y = qy * TY; y < y1; ++y) {
         const int g0 = y * nx;
         if (v2) {
@@ -612,10 +621,19 @@ cudaError_t launch_accumulate_range(sea_ctx* c, double* out, int o_begin, int o_
       const cudaError_t e = cudaStreamWaitEvent(c->stream, c->xev[1], 0);
       if (e != cudaSuccess) return e;
     }
-    // the plane, then one tile-mask byte per (x tile, y tile)
-    const size_t smem = (size_t)c->N[0] * c->N[1] * sizeof(double) +
-                        (size_t)((c->N[0] + TX - 1) / TX) * ((c->N[1] + TY - 1) / TY);
-    if (smem <= SEA_ACC_SMEM_MAX) {
+    // a slab of rows, then one tile-mask byte per (x tile, y tile)
+    auto bytes = [&](int rows) {
+      return (size_t)c->N[0] * rows * sizeof(double) +
+             (size_t)((c->N[0] + TX - 1) / TX) * ((rows + TY - 1) / TY);
+    };
+    if (bytes(c->N[1]) <= SEA_ACC_SMEM_MAX) {
+      int slabs = 1, rows = c->N[1];
+      while (bytes(rows) > SEA_ACC_SMEM_SLAB) {
+        ++slabs;
+        rows = ((c->N[1] + slabs - 1) / slabs + TY - 1) / TY * TY;
+      }
+      slabs = (c->N[1] + rows - 1) / rows;
+      const size_t smem = bytes(rows);
       cudaError_t e = cudaFuncSetAttribute(k_accumulate, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            (int)smem);
       if (e != cudaSuccess) return e;
@@ -623,8 +641,8 @@ cudaError_t launch_accumulate_range(sea_ctx* c, double* out, int o_begin, int o_
       // aligned outputs
       const bool plane16 = ((size_t)c->N[0] * c->N[1] * sizeof(double)) % 16 == 0;
       const bool al16 = ((uintptr_t)out % 16 == 0) && ((uintptr_t)out2 % 16 == 0);
-      k_accumulate<<<dim3(o_end - o_begin, c->N[2]), SEA_ACC_THREADS, smem, c->stream>>>(
-          c->N[0], c->N[1], c->N[2], o_begin, (const int*)c->eptr.p, (const Entry*)c->ewin.p,
+      k_accumulate<<<dim3(o_end - o_begin, c->N[2], slabs), SEA_ACC_THREADS, smem, c->stream>>>(
+          c->N[0], c->N[1], c->N[2], rows, o_begin, (const int*)c->eptr.p, (const Entry*)c->ewin.p,
           (const long long*)c->coff.p, (const double*)c->cbuf.p, out, out2,
           plane16 && al16 ? 1 : 0);
     } else {
