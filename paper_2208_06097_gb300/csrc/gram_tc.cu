@@ -1123,8 +1123,9 @@ __global__ void __launch_bounds__(MBLK)
 
 // E_v of the expansion for every (tile, vector): the largest biased
 // exponent of H(j, v) 2^(E_j) over the tile's list (0 where all are zero);
-// thread = vector, grid y = tile.  Tiles with an empty list or more than XJ
-// entries are skipped (not read).  STRICT: EV_NONFINITE where a factor is not
+// thread = vector, grid x = tile (grid y ends at 65535, a 204^3 grid has more
+// tiles).  Tiles with an empty list or more than XJ entries are skipped (not
+// read).  STRICT: EV_NONFINITE where a factor is not
 // finite.
 constexpr int EV_NONFINITE = 1 << 20;
 template <bool STRICT>
@@ -1132,7 +1133,7 @@ __global__ void __launch_bounds__(128)
     k_expand_ev(const int* __restrict__ tptr, const int* __restrict__ tlist,
                 const int* __restrict__ wxexp, const double* __restrict__ H, long long hj,
                 long long hv, int m, int* __restrict__ ev) {
-  const int T = blockIdx.y, v = blockIdx.x * 128 + threadIdx.x;
+  const int T = blockIdx.x, v = blockIdx.y * 128 + threadIdx.x;
   const int j0 = tptr[T], nJ = tptr[T + 1] - j0;
   if (v >= m || nJ == 0 || nJ > XJ) return;
   int em = 0;
@@ -1690,7 +1691,7 @@ static cudaError_t expand_tc(cudaStream_t st, int device, const void* wxbuf, con
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, device);
   e = cudaMemsetAsync(queue, 0, sizeof(int), st);
   if (e != cudaSuccess) return e;
-  k_expand_ev<DIG == 7><<<dim3((m + 127) / 128, n_tiles), 128, 0, st>>>(tptr, tlist, wxexp, H, hj,
+  k_expand_ev<DIG == 7><<<dim3(n_tiles, (m + 127) / 128), 128, 0, st>>>(tptr, tlist, wxexp, H, hj,
                                                                        hv, m, evbuf);
   k_expand_tc<DIG><<<std::min(nsm, n_tiles), XE_THREADS, smem, st>>>(
       wx, wxexp, G, ng, n_tiles, tptr, tlist, H, hj, hv, m, negate ? 1 : 0, out, evbuf, queue,
