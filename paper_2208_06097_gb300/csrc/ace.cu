@@ -170,6 +170,38 @@ __global__ void k_scan_small(const int* __restrict__ in, int n, int* __restrict_
   if (threadIdx.x == T - 1) out[n] = (int)pos;
 }
 
+// Exclusive scans of the tiles' list lengths and of the K steps of their images
+// for the expansion (both totals below 2^31: one scan, the steps in the upper
+// half).
+__global__ void k_scan_tiles(const int* __restrict__ cnt, int n, int* __restrict__ ptr,
+                             int* __restrict__ xoff, int* __restrict__ tot,
+                             int* __restrict__ steps) {
+  __shared__ long long part[32];
+  const int T = blockDim.x, chunk = (n + T - 1) / T;
+  const int b = min(n, chunk * (int)threadIdx.x), e = min(n, b + chunk);
+  auto both = [&](int x) {
+    const int c = cnt[x];
+    return (long long)wx_tile_steps(c) << 32 | (long long)c;
+  };
+  long long s = 0;
+  for (int x = b; x < e; ++x) s += both(x);
+  long long acc = 0;
+  long long pos = block_exscan_ll(s, part, &acc);
+  if (threadIdx.x == 0) {
+    *tot = (int)acc;
+    *steps = (int)(acc >> 32);
+  }
+  for (int x = b; x < e; ++x) {
+    ptr[x] = (int)pos;
+    xoff[x] = (int)(pos >> 32);
+    pos += both(x);
+  }
+  if (threadIdx.x == T - 1) {
+    ptr[n] = (int)pos;
+    xoff[n] = (int)(pos >> 32);
+  }
+}
+
 __global__ void k_max_int(const int* __restrict__ in, int n, int* __restrict__ out) {
   __shared__ int part[1024];
   int m = 0;
@@ -850,31 +882,94 @@ static cudaError_t launch_exx_ace(sea_ctx* c, int transA, const double* d) {
 // in the mixed form, 55- and 56-bit ones in the plain form.
 static int ace_digits(const sea_ctx* c) { return c->prm.precision == 1 ? 6 : 7; }
 
-// The contraction with W on the tensor cores (exact digit splitting).
-static cudaError_t launch_gram(sea_ctx* c, const double* A, int m, const TileGeom& G,
-                               const int* tptr) {
-  return launch_gram_tc(c->stream, c->device, A, m, G, c->ng, c->n_tiles, tptr, c->tile_inc,
-                        c->wdig.p, (double*)c->partial.p, (int*)c->counts.p + 20,
-                        (unsigned*)c->status.p, ace_digits(c));
+bool sea_ensure_first(sea_ctx* c, SeaBuf& b, size_t bytes) {
+  if (sea_ensure(c, b, bytes)) return true;
+  c->wx_ready = false;
+  for (SeaBuf* spare : {&c->wx, &c->wdig}) {
+    if (!spare->p || spare == &b) continue;
+    if (spare == &c->wdig) c->wparts.clear();
+    cudaStreamSynchronize(c->stream);
+    cudaFree(spare->p);
+    *spare = SeaBuf();
+    if (sea_ensure(c, b, bytes)) return true;
+  }
+  return false;
 }
 
-// The expansion W H: tiles with at most expand_tc_max_list() W rows on the
-// tensor cores, longer lists (if any) in FP64, or FP32 pairs (mixed form).
+// The parts of W whose digits are held at a time: all of W if device memory
+// allows it, else as large parts as it does (of whole tiles).  A part of
+// several is formed again at each contraction.
+static cudaError_t plan_w_parts(sea_ctx* c, const int* tptr) {
+  if (!c->wparts.empty()) return cudaSuccess;
+  const int nt = c->n_tiles;
+  int cap = std::max(c->tile_inc, 1);
+  while (!sea_ensure(c, c->wdig, w_digits_bytes(cap, ace_digits(c)))) {
+    if (cap <= c->max_tile_list) return cudaErrorMemoryAllocation;
+    cap = std::max(cap / 2, c->max_tile_list);
+  }
+  c->wparts.push_back(make_int2(0, 0));
+  if (cap < c->tile_inc) {
+    std::vector<int> ptr((size_t)nt + 1);
+    cudaError_t e = cudaMemcpyAsync(ptr.data(), tptr, ptr.size() * sizeof(int),
+                                    cudaMemcpyDeviceToHost, c->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+    if (e != cudaSuccess) {
+      c->wparts.clear();
+      return e;
+    }
+    for (int t = 0; t < nt; ++t)
+      if (ptr[t + 1] - c->wparts.back().y > cap) c->wparts.push_back(make_int2(t, ptr[t]));
+  }
+  c->wparts.push_back(make_int2(nt, c->tile_inc));
+  return cudaSuccess;
+}
+
+static cudaError_t form_w_digits(sea_ctx* c, const TileGeom& G, const int* tptr, const int* tlist,
+                                 size_t part) {
+  c->launches += 1;
+  return launch_w_digits(c->stream, (const double*)c->vxx_dev.p, G, c->ng, c->wparts[part],
+                         c->wparts[part + 1], c->max_tile_list, tptr, tlist, c->wdig.p,
+                         ace_digits(c));
+}
+
+// The contraction with W on the tensor cores (exact digit splitting), part
+// after part.
+static cudaError_t launch_gram(sea_ctx* c, const double* A, int m, const TileGeom& G,
+                               const int* tptr, const int* tlist) {
+  const bool planned = !c->wparts.empty();
+  cudaError_t e = plan_w_parts(c, tptr);
+  for (size_t k = 0; e == cudaSuccess && k + 1 < c->wparts.size(); ++k) {
+    if (!planned || c->wparts.size() > 2) e = form_w_digits(c, G, tptr, tlist, k);
+    if (e == cudaSuccess)
+      e = launch_gram_tc(c->stream, c->device, A, m, G, c->ng, c->wparts[k], c->wparts[k + 1], tptr,
+                         c->wdig.p, (double*)c->partial.p, (int*)c->counts.p + 20,
+                         (unsigned*)c->status.p, ace_digits(c));
+  }
+  return e;
+}
+
+// The expansion W H: tiles with at most SEA_XJ W rows on the tensor cores,
+// longer lists (if any) in FP64, or FP32 pairs (mixed form); so all tiles
+// where device memory does not hold the images.
 static cudaError_t launch_expand(sea_ctx* c, const TileGeom& G, const int* tptr,
                                  const int* tlist, const int* tsub, const double* H, long long hj,
                                  long long hv, int m, double sign, double* out) {
-  if (!sea_ensure(c, c->xevb, (size_t)max(c->n_tiles, 1) * m * sizeof(int)))
-    return cudaErrorMemoryAllocation;
-  const cudaError_t e = launch_expand_tc(
-      c->stream, c->device, c->wx.p, G, c->ng, c->n_tiles, tptr, tlist, H, hj, hv, m, sign < 0.0, out,
-      (int*)c->xevb.p, (int*)c->counts.p + 24, (unsigned*)c->status.p, ace_digits(c));
-  if (e != cudaSuccess) return e;
-  if (c->max_tile_list > expand_tc_max_list()) {
+  const int* xoff = tptr + (c->n_tiles + 1);
+  const bool images =
+      c->wx_ready && sea_ensure(c, c->xevb, (size_t)max(c->n_tiles, 1) * m * sizeof(int));
+  if (images) {
+    const cudaError_t e = launch_expand_tc(
+        c->stream, c->device, c->wx.p, G, c->ng, c->n_tiles, tptr, tlist, xoff, c->wx_steps, H, hj, hv,
+        m, sign < 0.0, out, (int*)c->xevb.p, (int*)c->counts.p + 24, (unsigned*)c->status.p,
+        ace_digits(c));
+    if (e != cudaSuccess) return e;
+  }
+  if (!images || c->max_tile_list > SEA_XJ) {
     const size_t smem = (size_t)c->max_tile_list * EV * sizeof(double);
     (c->prm.precision == 1 ? k_tile_expand_x : k_tile_expand)<<<
         dim3(c->n_tiles, (m + EV - 1) / EV), 256, smem, c->stream>>>(
         (const double*)c->vxx_dev.p, G, c->ng, tptr, tlist, tsub, H, hj, hv, m, sign,
-        expand_tc_max_list(), out);
+        images ? SEA_XJ : -1, out);
     c->launches += 1;
   }
   return cudaGetLastError();
@@ -951,7 +1046,9 @@ static cudaError_t launch_chol_chain(sea_ctx* c) {
 // (orbital, tile) incidences, per-tile counts and their scan, the lists.
 // The list arrays are sized for every (orbital, tile) pair (list_cap), so no
 // count has to reach the host before the lists are formed; the incidence
-// count and the longest tile list land in counts[10] and counts[12].
+// count, the longest tile list and the K steps of the expansion's images land in
+// counts[10], counts[12] and counts[13].  tptr_t holds three arrays of n_tiles + 1
+// entries: list lengths, list starts and first K steps.
 cudaError_t launch_ace_lists(sea_ctx* c, cudaStream_t st) {
   const int n = c->n_orb;
   const TileGeom G = make_tile_geom(c->N);
@@ -959,7 +1056,7 @@ cudaError_t launch_ace_lists(sea_ctx* c, cudaStream_t st) {
   const long long ninc = (long long)n * nt;
   const long long cap = std::max(ninc, 1LL);
   if (!sea_ensure(c, c->tmask, ninc * sizeof(int) * 3) ||
-      !sea_ensure(c, c->tptr_t, (size_t)(nt + 1) * sizeof(int) * 2) ||
+      !sea_ensure(c, c->tptr_t, (size_t)(nt + 1) * sizeof(int) * 3) ||
       !sea_ensure(c, c->tptr_o, (size_t)(n + 1) * sizeof(int) * 2) ||
       !sea_ensure(c, c->tlist_t, (size_t)cap * sizeof(int) * 2) ||
       !sea_ensure(c, c->tlist_o, (size_t)cap * sizeof(int) * 2))
@@ -971,6 +1068,7 @@ cudaError_t launch_ace_lists(sea_ctx* c, cudaStream_t st) {
   int* sub = inc + 2 * ninc;
   int* tcnt = (int*)c->tptr_t.p;
   int* tptr = tcnt + (nt + 1);
+  int* xoff = tptr + (nt + 1);
   int* ocnt = (int*)c->tptr_o.p;
   int* optr = ocnt + (n + 1);
   int* counts = (int*)c->counts.p;
@@ -982,7 +1080,7 @@ cudaError_t launch_ace_lists(sea_ctx* c, cudaStream_t st) {
       (const Entry*)c->ewin.p, (const int*)c->eptr.p, n, G, nt, c->w_dense ? 1 : 0, inc, sub);
   k_tile_lists<<<(nt + 7) / 8, 256, 0, st>>>(inc, sub, n, nt, 0, tcnt, nullptr, nullptr, nullptr,
                                              nullptr);
-  k_scan_small<<<1, 1024, 0, st>>>(tcnt, nt, tptr, counts + 10);
+  k_scan_tiles<<<1, 1024, 0, st>>>(tcnt, nt, tptr, xoff, counts + 10, counts + 13);
   k_max_int<<<1, 1024, 0, st>>>(tcnt, nt, counts + 12);
   k_tile_lists<<<(nt + 7) / 8, 256, 0, st>>>(inc, sub, n, nt, 1, nullptr, tptr, tlist, tsub, gidx);
   k_orb_lists<<<(n * 32 + 127) / 128, 128, 0, st>>>(gidx, n, nt, 0, ocnt, nullptr, nullptr,
@@ -1009,12 +1107,13 @@ cudaError_t launch_ace_build(sea_ctx* c) {
     c->lists_ready = false;
     err = launch_ace_lists(c, c->stream);
     if (err != cudaSuccess) return err;
-    int hc[3] = {0, 0, 0};
+    int hc[4] = {0, 0, 0, 0};
     cudaMemcpyAsync(hc, (int*)c->counts.p + 10, sizeof(hc), cudaMemcpyDeviceToHost, c->stream);
     err = cudaStreamSynchronize(c->stream);
     if (err != cudaSuccess) return err;
     c->tile_inc = hc[0];
     c->max_tile_list = hc[2];
+    c->wx_steps = hc[3];
   }
   const int nt = c->n_tiles;
   const int hinc = c->tile_inc;
@@ -1036,27 +1135,26 @@ cudaError_t launch_ace_build(sea_ctx* c) {
   const int* tlist = (const int*)c->tlist_t.p;
   const int* tsub = tlist + c->list_cap;
   const int* oslot = (const int*)c->tlist_o.p + c->list_cap;
-  // M = Phi^T W dV
-  // from W's digits
-  const int digits = ace_digits(c);
-  if (!sea_ensure(c, c->wdig, w_digits_bytes(hinc, digits)) ||
-      !sea_ensure(c, c->wx, wx_digits_bytes(nt, hinc, digits)))
-    return cudaErrorMemoryAllocation;
-  err = launch_w_digits(c->stream, (const double*)c->vxx_dev.p, G, c->ng, nt, c->max_tile_list, tptr,
-                        tlist, hinc, c->wdig.p, digits);
+  // M = Phi^T W dV from W's digits (formed before the contraction is timed
+  // where they are formed once)
+  c->wparts.clear();
+  err = plan_w_parts(c, tptr);
+  if (err == cudaSuccess && c->wparts.size() == 2) err = form_w_digits(c, G, tptr, tlist, 0);
   if (err != cudaSuccess) return err;
-  c->launches += 2;
+  const int digits = ace_digits(c);
+  c->wx_ready = sea_ensure(c, c->wx, wx_digits_bytes(c->wx_steps, hinc, digits));
+  c->launches += 1;
   cudaEventRecord(c->ev[10], c->stream);
-  err = launch_gram(c, (const double*)c->phi.p, n, G, tptr);
+  err = launch_gram(c, (const double*)c->phi.p, n, G, tptr, tlist);
   if (err != cudaSuccess) return err;
   cudaEventRecord(c->ev[11], c->stream);
   // W's per-tile images for the expansion (used by sea_apply_ace only) on
   // a second stream, beside the latency-bound Cholesky chain below; the
   // context stream waits for them before the build ends
   err = cudaStreamWaitEvent(c->xfer[0], c->ev[11], 0);
-  if (err == cudaSuccess)
+  if (err == cudaSuccess && c->wx_ready)
     err = launch_wx_digits(c->xfer[0], (const double*)c->vxx_dev.p, G, c->ng, nt, tptr, tlist, tsub,
-                           c->wx.p, digits);
+                           tptr + (nt + 1), c->wx_steps, c->wx.p, digits);
   if (err == cudaSuccess) err = cudaEventRecord(c->xev[0], c->xfer[0]);
   if (err != cudaSuccess) return err;
   launch_gram_reduce(c->stream, c->prm.precision == 1, (const double*)c->partial.p, n, n, optr, oslot,
@@ -1120,11 +1218,11 @@ cudaError_t launch_ace_apply(sea_ctx* c, const double* psi, int nv, double* out)
   const TileGeom G = make_tile_geom(c->N);
   const int nt = c->n_tiles;
   const int hinc = c->tile_inc;
-  if (!sea_ensure(c, c->partial,
-                  (size_t)max(hinc, 1) * max(n, nv) * sizeof(double)) ||
-      !sea_ensure(c, c->Gbuf, (size_t)n * nv * sizeof(double)) ||
-      !sea_ensure(c, c->Hbuf, (size_t)n * nv * sizeof(double)) ||
-      !sea_ensure(c, c->Hbuf2, (size_t)n * nv * sizeof(double)))
+  if (!sea_ensure_first(c, c->partial,
+                        (size_t)max(hinc, 1) * max(n, nv) * sizeof(double)) ||
+      !sea_ensure_first(c, c->Gbuf, (size_t)n * nv * sizeof(double)) ||
+      !sea_ensure_first(c, c->Hbuf, (size_t)n * nv * sizeof(double)) ||
+      !sea_ensure_first(c, c->Hbuf2, (size_t)n * nv * sizeof(double)))
     return cudaErrorMemoryAllocation;
   const int* tptr = (const int*)c->tptr_t.p + (nt + 1);
   const int* tlist = (const int*)c->tlist_t.p;
@@ -1135,7 +1233,7 @@ cudaError_t launch_ace_apply(sea_ctx* c, const double* psi, int nv, double* out)
   // G[o][v] = <W_o|psi_v> dV
   cudaEventRecord(c->ev[12], c->stream);
   {
-    const cudaError_t e = launch_gram(c, psi, nv, G, tptr);
+    const cudaError_t e = launch_gram(c, psi, nv, G, tptr, tlist);
     if (e != cudaSuccess) return e;
   }
   cudaEventRecord(c->ev[13], c->stream);

@@ -577,7 +577,7 @@ sea_status sea_apply_vxx(sea_ctx* c, double* vxx_phi, int on_device, double* exx
   struct {
     double res[5];
     unsigned st;
-    int lists[3];
+    int lists[4];
   } r;
   SEA_CK(cudaStreamWaitEvent(c->stream, c->xev[2], 0), "wait");
   SEA_CK(cudaMemcpyAsync(r.res, c->exx_dev.p, sizeof(r.res), cudaMemcpyDeviceToHost, c->stream),
@@ -590,6 +590,7 @@ sea_status sea_apply_vxx(sea_ctx* c, double* vxx_phi, int on_device, double* exx
   SEA_CK(cudaStreamSynchronize(c->stream), "apply_vxx");
   c->tile_inc = r.lists[0];
   c->max_tile_list = r.lists[2];
+  c->wx_steps = r.lists[3];
   c->lists_ready = true;
   float t01 = 0, t12 = 0, t23 = 0, t34 = 0;
   cudaEventElapsedTime(&t01, c->ev[0], c->ev[1]);
@@ -720,8 +721,8 @@ sea_status sea_apply_ace(sea_ctx* c, const double* psi, int n_vec, double* out, 
   // of vectors: chunk k is copied in on one copy stream, applied on the
   // context stream and copied out on the other copy stream, so the two
   // transfer directions and the kernels overlap.
-  SEA_ALLOC(psi_dev, bytes);
-  SEA_ALLOC(out_dev, bytes);
+  if (!sea::sea_ensure_first(c, c->psi_dev, bytes) || !sea::sea_ensure_first(c, c->out_dev, bytes))
+    return sea_fail(c, SEA_ERR_OOM, "device allocation failed: vectors");
   // chunk starts: a half-size first and last chunk (the copy-in before the
   // first kernels and the copy-out after the last ones are not overlapped)
   const int per = std::max(32, (n_vec + SEA_XCHUNKS_MAX - 1) / SEA_XCHUNKS_MAX);
@@ -810,7 +811,8 @@ sea_status sea_get_ace_vectors(sea_ctx* c, double* xi, int on_device) {
   const size_t bytes = (size_t)c->n_orb * c->ng * sizeof(double);
   double* dst = xi;
   if (!on_device) {
-    SEA_ALLOC(out_dev, bytes);
+    if (!sea::sea_ensure_first(c, c->out_dev, bytes))
+      return sea_fail(c, SEA_ERR_OOM, "device allocation failed: out_dev");
     dst = (double*)c->out_dev.p;
   }
   SEA_CK(sea::launch_ace_vectors(c, dst), "ace vectors");

@@ -235,17 +235,18 @@ constexpr int EXP_NONFINITE = 0x7FF;
 // W digits, once per W: for every slot s of every tile list and half h,
 // wdig[((s * 2 + h) * DIG + k) * 8 + u] = the 8 BF16 digits (16 bytes) of
 // plane k, x-run u of W row list[s] on that half tile, and wexp[2 s + h]
-// the row segment's largest biased exponent.  Warp per (tile, half, group
-// of 8 slots).  Four CTAs per SM: the warps wait on their row loads, so
+// the row segment's largest biased exponent, s counted from slot s0, for the
+// n_tiles tiles from t0.  Warp per (tile, half, group of 8 slots).  Four CTAs per SM: the warps wait on their row loads, so
 // occupancy is what hides the latency.
 template <int DIG>
 __global__ void __launch_bounds__(256, DIG == 6 ? 4 : 3)
-    k_w_digits(const double* __restrict__ W, TileGeom G, size_t ng, int n_tiles, int ngroups,
-               const int* __restrict__ tptr, const int* __restrict__ tlist, uint4* __restrict__ wdig,
-               int* __restrict__ wexp) {
+    k_w_digits(const double* __restrict__ W, TileGeom G, size_t ng, int t0, int n_tiles, int s0,
+               int ngroups, const int* __restrict__ tptr, const int* __restrict__ tlist,
+               uint4* __restrict__ wdig, int* __restrict__ wexp) {
   const long long gw = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (gw >= (long long)n_tiles * 2 * ngroups) return;  // warp-uniform
-  const int g = (int)(gw % ngroups), h = (int)((gw / ngroups) % 2), T = (int)(gw / (2 * ngroups));
+  const int g = (int)(gw % ngroups), h = (int)((gw / ngroups) % 2),
+            T = t0 + (int)(gw / (2 * ngroups));
   const int j0 = tptr[T], nJ = tptr[T + 1] - j0;
   if (8 * g >= nJ) return;  // warp-uniform
   const int lane = threadIdx.x & 31, r = lane & 7, s = 8 * g + r;
@@ -253,14 +254,14 @@ __global__ void __launch_bounds__(256, DIG == 6 ? 4 : 3)
   GroupDigits<DIG> d;
   make_digits(rp, G, T, h, d);
   if (s < nJ) {
-    uint4* dst = wdig + ((size_t)(j0 + s) * 2 + h) * DIG * 8;
+    uint4* dst = wdig + ((size_t)(j0 + s - s0) * 2 + h) * DIG * 8;
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
       const int u = (lane >> 3) + 4 * q;
 #pragma unroll
       for (int k = 0; k < DIG; ++k) dst[k * 8 + u] = make_uint4(d.w[q][k][0], d.w[q][k][1], d.w[q][k][2], d.w[q][k][3]);
     }
-    if (lane < 8) wexp[(size_t)(j0 + s) * 2 + h] = d.emax;
+    if (lane < 8) wexp[(size_t)(j0 + s - s0) * 2 + h] = d.emax;
   }
 }
 
@@ -444,8 +445,8 @@ __device__ __forceinline__ bool conv_sync_or(bool v) {
 template <int DIG, bool TMA>
 __global__ void __launch_bounds__(GT2_THREADS, 1)
     k_gram_tc(const __grid_constant__ CUtensorMap tmA, const double* __restrict__ A, size_t ng, int m,
-              TileGeom G, int n_tiles,
-              const int* __restrict__ tptr, const uint4* __restrict__ wdig,
+              TileGeom G, int t0, int n_tiles,  // tiles [t0, n_tiles)
+              const int* __restrict__ tptr, const uint4* __restrict__ wdig, int slot0,
               const int* __restrict__ wexp, double* __restrict__ partial, int* __restrict__ queue,
               unsigned* __restrict__ status) {
   using Z = GramSizes<DIG>;
@@ -562,10 +563,10 @@ __global__ void __launch_bounds__(GT2_THREADS, 1)
         }
       } else if (q_stage == 2) {
         if (q_j1 == q_j0) {
-          q_t = atomicAdd(queue, 1);
+          q_t = t0 + atomicAdd(queue, 1);
           q_stage = 1;
         } else {
-          bulk_prefetch_l2(wdig + (size_t)q_j0 * 2 * DIG * 8,
+          bulk_prefetch_l2(wdig + (size_t)(q_j0 - slot0) * 2 * DIG * 8,
                            (uint32_t)min(q_j1 - q_j0, NBLK) * 2 * DIG * 8 * 16);
           q_stage = 3;
         }
@@ -575,7 +576,7 @@ __global__ void __launch_bounds__(GT2_THREADS, 1)
       conv_sync();
       if (tid == 0) {
         if (q_stage == 0) {
-          q_t = atomicAdd(queue, 1);
+          q_t = t0 + atomicAdd(queue, 1);
           q_stage = 1;
         }
         while (q_stage != 3) q_step();
@@ -583,7 +584,7 @@ __global__ void __launch_bounds__(GT2_THREADS, 1)
         s_j[0] = q_j0;
         s_j[1] = q_j1;
         if (q_t < n_tiles) {
-          q_t = atomicAdd(queue, 1);
+          q_t = t0 + atomicAdd(queue, 1);
           q_stage = 1;
         }
       }
@@ -655,13 +656,13 @@ __global__ void __launch_bounds__(GT2_THREADS, 1)
         const int rn = p & 7, k = (p >> 3) % DIG, h = (p / (8 * DIG)) & 1, sl = p / (16 * DIG);
         const bool ok = sl < nj;
         const uint4* src =
-            ok ? wdig + ((size_t)(u.j0 + u.jb + sl) * 2 + h) * DIG * 8 + k * 8 + rn : wdig;
+            ok ? wdig + ((size_t)(u.j0 - slot0 + u.jb + sl) * 2 + h) * DIG * 8 + k * 8 + rn : wdig;
         const int r = k * P + sl;
         cp_async16(w_base + h * W_HALF + (r >> 3) * CORE_SBO + rn * lbo + (r & 7) * 16, src, ok);
       }
       if (tid < 2 * NBLK) {
         const int h = tid / NBLK, sl = tid % NBLK;
-        Wexp[u.wb][h][sl] = sl < nj ? wexp[(size_t)(u.j0 + u.jb + sl) * 2 + h] : 0;
+        Wexp[u.wb][h][sl] = sl < nj ? wexp[(size_t)(u.j0 - slot0 + u.jb + sl) * 2 + h] : 0;
       }
     };
     // bounded waits; false on expiry
@@ -947,10 +948,10 @@ constexpr int FEW_WARPS = 4;
 constexpr int GRAM_FEW = 32, EXPAND_FEW = 8;
 template <int DIG>
 __global__ void __launch_bounds__(32 * FEW_WARPS)
-    k_gram_few(const double* __restrict__ A, int m, TileGeom G, size_t ng, int n_tiles,
-               const int* __restrict__ tptr, const uint4* __restrict__ wdig,
+    k_gram_few(const double* __restrict__ A, int m, TileGeom G, size_t ng, int t0, int n_tiles,
+               const int* __restrict__ tptr, const uint4* __restrict__ wdig, int slot0,
                const int* __restrict__ wexp, double* __restrict__ partial) {
-  const int T = blockIdx.x * FEW_WARPS + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  const int T = t0 + blockIdx.x * FEW_WARPS + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (T >= n_tiles) return;  // warp-uniform
   const int j0 = tptr[T], nJ = tptr[T + 1] - j0;
   if (nJ == 0) return;
@@ -989,8 +990,9 @@ __global__ void __launch_bounds__(32 * FEW_WARPS)
       for (int k = 0; k < DIG; ++k) c[k][0] = c[k][1] = c[k][2] = c[k][3] = 0.f;
       // entries s0 + g and s0 + g + 8 (zeros beyond the list)
       const bool in0 = s0 + g < nJ, in1 = s0 + g + 8 < nJ;
-      const uint4* w0 = wdig + ((size_t)(j0 + s0 + (in0 ? g : 0)) * 2 + h) * DIG * 8 + q;
-      const uint4* w1 = wdig + ((size_t)(j0 + s0 + (in1 ? g + 8 : 0)) * 2 + h) * DIG * 8 + q;
+      const uint4* ws = wdig + ((size_t)(j0 - slot0 + s0) * 2 + h) * DIG * 8 + q;
+      const uint4* w0 = ws + (in0 ? g : 0) * 2 * DIG * 8;
+      const uint4* w1 = ws + (in1 ? g + 8 : 0) * 2 * DIG * 8;
 #pragma unroll
       for (int l = 0; l < DIG; ++l) {
         const uint4 z4 = make_uint4(0, 0, 0, 0);
@@ -1009,7 +1011,7 @@ __global__ void __launch_bounds__(32 * FEW_WARPS)
       for (int i = 0; i < 4; ++i) {
         const int s = s0 + g + 8 * (i >> 1), a = a0 + 2 * q + (i & 1);
         const int ea = __shfl_sync(0xffffffffu, em, 8 * q + 4 * (i & 1));
-        const int ew = s < nJ ? wexp[(size_t)(j0 + s) * 2 + h] : 0;
+        const int ew = s < nJ ? wexp[(size_t)(j0 - slot0 + s) * 2 + h] : 0;
         uint32_t f[DIG];
 #pragma unroll
         for (int k = 0; k < DIG; ++k) f[k] = __float_as_uint(c[k][i]);
@@ -1055,7 +1057,7 @@ __global__ void __launch_bounds__(32 * FEW_WARPS)
 // its buffer back, and the digits of the following chunks are formed
 // meanwhile by warps of their own.
 // ---------------------------------------------------------------------------
-constexpr int XJ = 32, XKS = 16, XN = 32;
+constexpr int XJ = SEA_XJ, XKS = SEA_XKS, XN = 32;
 constexpr uint32_t XA_BLOCK = MBLK * XKS * 2;          // 4 KB: one plane, one K step
 constexpr uint32_t XA_LBO = (MBLK / 8) * 128;          // 2048
 constexpr int XR = 4;                                  // ring slots (chunks of XN vectors)
@@ -1071,15 +1073,18 @@ struct ExpandSizes {  // with six digits
 };
 
 // W's digit image: CTA per tile (thread = point p), for tiles whose list has
-// 1..XJ entries.  wx[T][(q 6 + k) 4096 + (p / 8) 128 + (jq / 8) 2048 +
+// 1..XJ entries; only the K steps in use are stored, tile T's from step xoff[T]
+// on (a step of every tile would be 448 bytes a grid point in the plain form,
+// 60 GB at 512^3).  wx[step xoff[T]][(q 6 + k) 4096 + (p / 8) 128 + (jq / 8) 2048 +
 // (p % 8) 16 + (jq % 8) 2] = digit k of W[list(16 q + jq)] at point p (zero
 // outside the entry's sub-box and beyond the list), wxexp[slot] = E_j + 1022.
 template <int DIG>
 __global__ void __launch_bounds__(MBLK)
     k_wx_digits(const double* __restrict__ W, TileGeom G, size_t ng, int n_tiles,
                 const int* __restrict__ tptr, const int* __restrict__ tlist,
-                const int* __restrict__ tsub, uint4* __restrict__ wx, int* __restrict__ wxexp) {
-  constexpr uint32_t XA_STEP = ExpandSizes<DIG>::XA_STEP, XA_TILE = 2 * XA_STEP;
+                const int* __restrict__ tsub, const int* __restrict__ xoff,
+                uint4* __restrict__ wx, int* __restrict__ wxexp) {
+  constexpr uint32_t XA_STEP = ExpandSizes<DIG>::XA_STEP;
   const int T = blockIdx.x;
   const int j0 = tptr[T], nJ = tptr[T + 1] - j0;
   if (nJ == 0 || nJ > XJ) return;  // uniform
@@ -1101,7 +1106,7 @@ __global__ void __launch_bounds__(MBLK)
   __syncthreads();
   if (p < nJ) wxexp[j0 + p] = emx[p];
   const int nq = (nJ + XKS - 1) / XKS;
-  unsigned char* base = reinterpret_cast<unsigned char*>(wx) + (size_t)T * XA_TILE;
+  unsigned char* base = reinterpret_cast<unsigned char*>(wx) + (size_t)xoff[T] * XA_STEP;
   for (int grp = 0; grp < 2 * nq; ++grp) {  // 8 list entries at a time
     uint32_t pk[DIG][4];
 #pragma unroll
@@ -1179,8 +1184,9 @@ template <int DIG>
 __global__ void __launch_bounds__(XE_THREADS, 1)
     k_expand_tc(const uint4* __restrict__ wx, const int* __restrict__ wxexp, TileGeom G, size_t ng,
                 int n_tiles, const int* __restrict__ tptr, const int* __restrict__ tlist,
-                const double* __restrict__ H, long long hj, long long hv, int m, int negate,
-                double* __restrict__ out, const int* __restrict__ evp, int* __restrict__ queue,
+                const int* __restrict__ xoff, const double* __restrict__ H, long long hj,
+                long long hv, int m, int negate, double* __restrict__ out,
+                const int* __restrict__ evp, int* __restrict__ queue,
                 unsigned* __restrict__ status) {
   using Z = ExpandSizes<DIG>;
   constexpr uint32_t XA_STEP = Z::XA_STEP, XA_TILE = Z::XA_TILE, XB_LBO = Z::XB_LBO,
@@ -1269,7 +1275,7 @@ __global__ void __launch_bounds__(XE_THREADS, 1)
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
           mbar_expect_tx(smem_addr(&bar_a[ab]), bytes);
           bulk_load(a_base + ab * XA_TILE,
-                    reinterpret_cast<const unsigned char*>(wx) + (size_t)T * XA_TILE, bytes,
+                    reinterpret_cast<const unsigned char*>(wx) + (size_t)xoff[T] * XA_STEP, bytes,
                     smem_addr(&bar_a[ab]));
           a_pend |= 1u << ab;
           a_par = (a_par & ~(1u << ab)) | ((uint32_t)((tseq >> 1) & 1) << ab);
@@ -1522,11 +1528,11 @@ template <int DIG>
 __global__ void __launch_bounds__(256)
     k_expand_few(const uint4* __restrict__ wx, const int* __restrict__ wxexp, TileGeom G, size_t ng,
                  const int* __restrict__ tptr, const int* __restrict__ tlist,
-                 const double* __restrict__ H, long long hj, long long hv, int m, int negate,
-                 double* __restrict__ out) {
-  constexpr uint32_t XA_STEP = ExpandSizes<DIG>::XA_STEP, XA_TILE = 2 * XA_STEP;
+                 const int* __restrict__ xoff, const double* __restrict__ H, long long hj,
+                 long long hv, int m, int negate, double* __restrict__ out) {
+  constexpr uint32_t XA_STEP = ExpandSizes<DIG>::XA_STEP;
   const int T = blockIdx.x, v0 = blockIdx.y * 8;
-  const int j0 = tptr[T], nJ = tptr[T + 1] - j0;
+  const int j0 = tptr[T], nJ = tptr[T + 1] - j0, x0 = xoff[T];
   if (nJ > XJ) return;  // uniform: the long-list kernel's
   const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3, p0 = 16 * (threadIdx.x >> 5);
   const long long o0 = tile_point(G, T, p0 + g), o1 = tile_point(G, T, p0 + g + 8);
@@ -1552,7 +1558,7 @@ __global__ void __launch_bounds__(256)
     }
   em = max(em, __shfl_xor_sync(0xffffffffu, em, 1));
   em = max(em, __shfl_xor_sync(0xffffffffu, em, 2));
-  const unsigned char* base = reinterpret_cast<const unsigned char*>(wx) + (size_t)T * XA_TILE;
+  const unsigned char* base = reinterpret_cast<const unsigned char*>(wx) + (size_t)x0 * XA_STEP;
 #pragma unroll
   for (int s = 0; s < 2; ++s) {
     if (16 * s >= nJ) break;  // uniform
@@ -1603,13 +1609,14 @@ static int* w_digits_exp(const void* wbuf, long long slots, int digits) {
 }
 
 cudaError_t launch_w_digits(cudaStream_t st, const double* W, const TileGeom& G, size_t ng,
-                            int n_tiles, int max_list, const int* tptr, const int* tlist,
-                            long long slots, void* wbuf, int digits) {
-  if (n_tiles <= 0 || max_list <= 0) return cudaSuccess;
+                            int2 a, int2 b, int max_list, const int* tptr, const int* tlist,
+                            void* wbuf, int digits) {
+  if (b.x <= a.x || max_list <= 0) return cudaSuccess;
   const int ngroups = (max_list + 7) / 8;
-  const long long warps = (long long)n_tiles * 2 * ngroups;
+  const long long warps = (long long)(b.x - a.x) * 2 * ngroups;
   (digits == 7 ? k_w_digits<7> : k_w_digits<6>)<<<(unsigned)((warps + 7) / 8), 256, 0, st>>>(
-      W, G, ng, n_tiles, ngroups, tptr, tlist, (uint4*)wbuf, w_digits_exp(wbuf, slots, digits));
+      W, G, ng, a.x, b.x - a.x, a.y, ngroups, tptr, tlist, (uint4*)wbuf,
+      w_digits_exp(wbuf, b.y - a.y, digits));
   return cudaGetLastError();
 }
 
@@ -1651,40 +1658,40 @@ static bool make_a_map(const double* A, int m, const TileGeom& G, CUtensorMap* m
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-static size_t xa_tile(int digits) {
-  return digits == 7 ? ExpandSizes<7>::XA_TILE : ExpandSizes<6>::XA_TILE;
+static size_t xa_step(int digits) {
+  return digits == 7 ? ExpandSizes<7>::XA_STEP : ExpandSizes<6>::XA_STEP;
 }
-size_t wx_digits_bytes(int n_tiles, long long slots, int digits) {
-  return (size_t)std::max(n_tiles, 1) * xa_tile(digits) +
-         (size_t)std::max(slots, 1LL) * sizeof(int);
+size_t wx_digits_bytes(long long steps, long long slots, int digits) {
+  return (size_t)steps * xa_step(digits) + (size_t)std::max(slots, 1LL) * sizeof(int);
 }
 
 cudaError_t launch_wx_digits(cudaStream_t st, const double* W, const TileGeom& G, size_t ng,
                              int n_tiles, const int* tptr, const int* tlist, const int* tsub,
-                             void* wxbuf, int digits) {
+                             const int* xoff, long long steps, void* wxbuf, int digits) {
   if (n_tiles <= 0) return cudaSuccess;
   uint4* wx = (uint4*)wxbuf;
-  int* wxexp = (int*)((unsigned char*)wxbuf + (size_t)n_tiles * xa_tile(digits));
-  (digits == 7 ? k_wx_digits<7> : k_wx_digits<6>)<<<n_tiles, MBLK, 0, st>>>(W, G, ng, n_tiles, tptr,
-                                                                           tlist, tsub, wx, wxexp);
+  int* wxexp = (int*)((unsigned char*)wxbuf + (size_t)steps * xa_step(digits));
+  (digits == 7 ? k_wx_digits<7> : k_wx_digits<6>)<<<n_tiles, MBLK, 0, st>>>(
+      W, G, ng, n_tiles, tptr, tlist, tsub, xoff, wx, wxexp);
   return cudaGetLastError();
 }
 
 template <int DIG>
 static cudaError_t expand_tc(cudaStream_t st, int device, const void* wxbuf, const TileGeom& G,
                              size_t ng, int n_tiles, const int* tptr, const int* tlist,
-                             const double* H, long long hj, long long hv, int m, bool negate,
-                             double* out, int* evbuf, int* queue, unsigned* status) {
+                             const int* xoff, long long steps, const double* H, long long hj,
+                             long long hv, int m, bool negate, double* out, int* evbuf, int* queue,
+                             unsigned* status) {
   constexpr size_t smem = ExpandSizes<DIG>::XE_SMEM;
   cudaError_t e =
       cudaFuncSetAttribute(k_expand_tc<DIG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   if (n_tiles <= 0 || m <= 0) return cudaSuccess;
   const uint4* wx = (const uint4*)wxbuf;
-  const int* wxexp = (const int*)((const unsigned char*)wxbuf + (size_t)n_tiles * xa_tile(DIG));
+  const int* wxexp = (const int*)((const unsigned char*)wxbuf + (size_t)steps * xa_step(DIG));
   if (m <= EXPAND_FEW) {
-    k_expand_few<DIG><<<dim3(n_tiles, (m + 7) / 8), 256, 0, st>>>(wx, wxexp, G, ng, tptr, tlist, H, hj,
-                                                                  hv, m, negate ? 1 : 0, out);
+    k_expand_few<DIG><<<dim3(n_tiles, (m + 7) / 8), 256, 0, st>>>(wx, wxexp, G, ng, tptr, tlist, xoff,
+                                                                  H, hj, hv, m, negate ? 1 : 0, out);
     return cudaGetLastError();
   }
   int nsm = 0;
@@ -1694,32 +1701,34 @@ static cudaError_t expand_tc(cudaStream_t st, int device, const void* wxbuf, con
   k_expand_ev<DIG == 7><<<dim3(n_tiles, (m + 127) / 128), 128, 0, st>>>(tptr, tlist, wxexp, H, hj,
                                                                        hv, m, evbuf);
   k_expand_tc<DIG><<<std::min(nsm, n_tiles), XE_THREADS, smem, st>>>(
-      wx, wxexp, G, ng, n_tiles, tptr, tlist, H, hj, hv, m, negate ? 1 : 0, out, evbuf, queue,
+      wx, wxexp, G, ng, n_tiles, tptr, tlist, xoff, H, hj, hv, m, negate ? 1 : 0, out, evbuf, queue,
       status);
   return cudaGetLastError();
 }
 
 cudaError_t launch_expand_tc(cudaStream_t st, int device, const void* wxbuf, const TileGeom& G,
                              size_t ng, int n_tiles, const int* tptr, const int* tlist,
-                             const double* H, long long hj, long long hv, int m, bool negate,
-                             double* out, int* evbuf, int* queue, unsigned* status, int digits) {
+                             const int* xoff, long long steps, const double* H, long long hj,
+                             long long hv, int m, bool negate, double* out, int* evbuf, int* queue,
+                             unsigned* status, int digits) {
   return (digits == 7 ? expand_tc<7> : expand_tc<6>)(st, device, wxbuf, G, ng, n_tiles, tptr, tlist,
-                                                     H, hj, hv, m, negate, out, evbuf, queue, status);
+                                                     xoff, steps, H, hj, hv, m, negate, out, evbuf,
+                                                     queue, status);
 }
-
-int expand_tc_max_list() { return XJ; }
 
 template <int DIG>
 static cudaError_t gram_tc(cudaStream_t st, int device, const double* A, int m, const TileGeom& G,
-                           size_t ng, int n_tiles, const int* tptr, long long slots,
-                           const void* wbuf, double* partial, int* queue, unsigned* status) {
+                           size_t ng, int2 a, int2 b, const int* tptr, const void* wbuf,
+                           double* partial, int* queue, unsigned* status) {
   constexpr size_t smem = GramTmaSizes<DIG>::SMEM;
   static_assert(smem <= 232448 - 4096, "shared memory of an SM");
   const uint4* wdig = (const uint4*)wbuf;
-  const int* wexp = w_digits_exp(wbuf, slots, DIG);
+  const int* wexp = w_digits_exp(wbuf, b.y - a.y, DIG);
+  const int n_tiles = b.x - a.x;
+  if (n_tiles <= 0) return cudaSuccess;
   if (m <= GRAM_FEW) {
     k_gram_few<DIG><<<dim3((n_tiles + FEW_WARPS - 1) / FEW_WARPS, (m + 7) / 8), 32 * FEW_WARPS, 0, st>>>(
-        A, m, G, ng, n_tiles, tptr, wdig, wexp, partial);
+        A, m, G, ng, a.x, b.x, tptr, wdig, a.y, wexp, partial);
     return cudaGetLastError();
   }
   int nsm = 0;
@@ -1732,17 +1741,16 @@ static cudaError_t gram_tc(cudaStream_t st, int device, const double* A, int m, 
       cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e == cudaSuccess) e = cudaMemsetAsync(queue, 0, sizeof(int), st);
   if (e != cudaSuccess) return e;
-  kern<<<std::min(nsm, std::max(n_tiles, 1)), GT2_THREADS, smem, st>>>(
-      map, A, ng, m, G, n_tiles, tptr, wdig, wexp, partial, queue, status);
+  kern<<<std::min(nsm, n_tiles), GT2_THREADS, smem, st>>>(
+      map, A, ng, m, G, a.x, b.x, tptr, wdig, a.y, wexp, partial, queue, status);
   return cudaGetLastError();
 }
 
 cudaError_t launch_gram_tc(cudaStream_t st, int device, const double* A, int m, const TileGeom& G,
-                           size_t ng, int n_tiles, const int* tptr, long long slots,
-                           const void* wbuf, double* partial, int* queue, unsigned* status,
-                           int digits) {
-  return (digits == 7 ? gram_tc<7> : gram_tc<6>)(st, device, A, m, G, ng, n_tiles, tptr, slots, wbuf,
-                                                 partial, queue, status);
+                           size_t ng, int2 a, int2 b, const int* tptr, const void* wbuf,
+                           double* partial, int* queue, unsigned* status, int digits) {
+  return (digits == 7 ? gram_tc<7> : gram_tc<6>)(st, device, A, m, G, ng, a, b, tptr, wbuf, partial,
+                                                 queue, status);
 }
 
 }  // namespace sea

@@ -519,8 +519,14 @@ struct sea_ctx {
   SeaBuf status, exx_dev, queue;
   SeaBuf onorm;  // per-orbital partial sums of phi^2 (input check of sea_set_orbitals)
   // ACE
-  SeaBuf wdig;  // the mixed form's W digits (tensor-core contraction)
-  SeaBuf wx;    // the mixed form's per-tile W digit images (tensor-core expansion)
+  SeaBuf wdig;  // W's digits (tensor-core contraction)
+  SeaBuf wx;    // W's per-tile digit images (tensor-core expansion)
+  // (tile, slot) bounds of the parts of W whose digits fit wdig at a time: one
+  // part, formed once per build, where device memory allows it; empty: not
+  // planned for the present W
+  std::vector<int2> wparts;
+  int wx_steps = 0;       // K steps of all images
+  bool wx_ready = false;  // the images are those of the present W
   SeaBuf xevb;  // the expansion's H exponents per (tile, vector)
   SeaBuf gbuf;  // ghost (boundary) values of the pair boxes, 36 voff per pair
   SeaBuf flowbuf;  // the mixed form's one-launch Cholesky chain: DF blocks and task flags
@@ -797,28 +803,38 @@ cudaError_t launch_rotate(sea_ctx* c, const double* phi, int n, size_t N, const 
                           double* out);
 // Damped Jacobi sweeps on every pair's starting vector (pair.cu).
 cudaError_t launch_smooth(sea_ctx* c, int sweeps, double omega);
-// The contraction with W on the tensor cores.  launch_w_digits
-// splits W's rows on every tile of every list once into wbuf
-// (w_digits_bytes(slots), slots = total list length); launch_gram_tc then
-// forms partial[slot m + a] for A's m rows.  *queue is reset on the stream.
+// The contraction with W on the tensor cores.  launch_w_digits splits W's rows
+// on the lists of tiles [a.x, b.x), slots [a.y, b.y), into wbuf
+// (w_digits_bytes(b.y - a.y)); launch_gram_tc then forms partial[slot m + a]
+// of those slots for A's m rows.  *queue is reset on the stream.
 // digits: 6 (mixed form) or 7 (plain form).
 size_t w_digits_bytes(long long slots, int digits);
 cudaError_t launch_w_digits(cudaStream_t st, const double* W, const TileGeom& G, size_t ng,
-                            int n_tiles, int max_list, const int* tptr, const int* tlist,
-                            long long slots, void* wbuf, int digits);
-size_t wx_digits_bytes(int n_tiles, long long slots, int digits);
+                            int2 a, int2 b, int max_list, const int* tptr, const int* tlist,
+                            void* wbuf, int digits);
+// The expansion's images: SEA_XKS list entries a K step, for tiles of 1 to
+// SEA_XJ entries; tile T's first step is xoff[T], `steps` in all, `slots` the
+// total list length.
+#define SEA_XJ 32
+#define SEA_XKS 16
+__host__ __device__ __forceinline__ int wx_tile_steps(int list) {
+  return list > SEA_XJ ? 0 : (list + SEA_XKS - 1) / SEA_XKS;
+}
+size_t wx_digits_bytes(long long steps, long long slots, int digits);
 cudaError_t launch_wx_digits(cudaStream_t st, const double* W, const TileGeom& G, size_t ng,
                              int n_tiles, const int* tptr, const int* tlist, const int* tsub,
-                             void* wxbuf, int digits);
+                             const int* xoff, long long steps, void* wxbuf, int digits);
 cudaError_t launch_expand_tc(cudaStream_t st, int device, const void* wxbuf, const TileGeom& G,
                              size_t ng, int n_tiles, const int* tptr, const int* tlist,
-                             const double* H, long long hj, long long hv, int m, bool negate,
-                             double* out, int* evbuf, int* queue, unsigned* status, int digits);
-int expand_tc_max_list();
+                             const int* xoff, long long steps, const double* H, long long hj,
+                             long long hv, int m, bool negate, double* out, int* evbuf, int* queue,
+                             unsigned* status, int digits);
 cudaError_t launch_gram_tc(cudaStream_t st, int device, const double* A, int m, const TileGeom& G,
-                           size_t ng, int n_tiles, const int* tptr, long long slots,
-                           const void* wbuf, double* partial, int* queue, unsigned* status,
-                           int digits);
+                           size_t ng, int2 a, int2 b, const int* tptr, const void* wbuf,
+                           double* partial, int* queue, unsigned* status, int digits);
+// sea_ensure; where memory is short the digits and images of W are given up
+// first (they are formed again, or done without).
+bool sea_ensure_first(sea_ctx* c, SeaBuf& b, size_t bytes);
 cudaError_t launch_ace_lists(sea_ctx* c, cudaStream_t st);
 cudaError_t launch_ace_build(sea_ctx* c);
 cudaError_t launch_ace_eigen(sea_ctx* c);
