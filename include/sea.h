@@ -91,10 +91,11 @@ typedef struct {
   double self_scale;
   int precision;  /* 0: FP64, 1: mixed (FP32 CG inside FP64 refinement) */
   int warm_start; /* 0: none; 1: the attached sea_unet's guesses (sea_unet_attach) */
-  double timeout_ms; /* time budget of sea_apply_vxx's persistent CG launch
-                        (0: none).  Once it is spent no CTA takes another
-                        pair; the call then returns SEA_ERR_TIMEOUT and its
-                        results are not valid (the context stays usable). */
+  double timeout_ms; /* time budget of sea_apply_vxx's CG (0: none), counted
+                        from the start of its first CTA.  Once it is spent no
+                        CTA takes another pair; a call whose CG outlasts it
+                        returns SEA_ERR_TIMEOUT and its results are not valid
+                        (the context stays usable). */
   int ace_decomp; /* 0: Cholesky, eigen form of App. A if a pivot fails;
                      1: Cholesky only (SEA_ERR_NOT_PD on failure); 2: eigen form */
   double orth_tol; /* sea_set_orbitals returns SEA_ERR_INPUT when some

@@ -479,9 +479,9 @@ struct CgArgs {
   double* epair;
   int* iters;
   unsigned* status;
-  int* queue;
+  int* queue;  // the classes' counters; with a time budget a CgQueue
   int warm;  // x holds an initial guess (else the solve starts from 0)
-  unsigned long long budget_ns;  // time budget of the launch (0: none)
+  unsigned long long budget_ns;  // time budget from the first CTA's start (0: none)
   FixArgs fix;
   int cap[2];  // padded points that fit the launch's shared memory, per class
 };
@@ -933,13 +933,27 @@ __device__ __forceinline__ unsigned long long global_ns() {
   return t;
 }
 
+// The two classes' queue counters, and when the first CTA of either started (0
+// before; set where there is a time budget).
+struct CgQueue {
+  int next[2];
+  unsigned long long start;
+};
+// One start for all CTAs of both classes: those of the small class that wait for
+// SMs which the large class holds start late.
+__device__ __forceinline__ unsigned long long cg_start(CgQueue* q) {
+  const unsigned long long now = global_ns(), first = atomicCAS(&q->start, 0ull, now);
+  return first ? first : now;
+}
+
 // Next queue item for the CTA (thread 0).  With a time budget, once more
-// than budget_ns have passed since the CTA started (t0) no further pair is
+// than budget_ns have passed since the start t0 no further pair is
 // taken: the status gets SEA_FLAG_TIMEOUT and the returned item ends the
 // CTA's loop (the pairs not taken keep no solution).
 __device__ __forceinline__ int claim_item(int* queue, int P, unsigned long long budget_ns,
                                           unsigned long long t0, unsigned* status) {
-  if (budget_ns && global_ns() - t0 > budget_ns) {
+  // signed: another SM's clock may have been read a little later than this one's
+  if (budget_ns && (long long)(global_ns() - t0) > (long long)budget_ns) {
     atomicOr(status, SEA_FLAG_TIMEOUT);
     return P;
   }
@@ -961,7 +975,8 @@ __global__ void __launch_bounds__(cg_threads(LARGE), LARGE ? 1 : 2) k_cg(CgArgs 
   extern __shared__ int2 Ps[];  // A.cap[LARGE] points
   const CgTeam T = cg_team<TEAM>();
   team_sync(T);  // the team's CTAs have started
-  const unsigned long long t0 = A.budget_ns ? global_ns() : 0ull;
+  const unsigned long long t0 =
+      A.budget_ns && T.rank == 0 && threadIdx.x == 0 ? cg_start((CgQueue*)A.queue) : 0ull;
   for (;;) {
     if (T.rank == 0 && threadIdx.x == 0) {
       s_item = claim_item(A.queue + LARGE, A.P, A.budget_ns, t0, A.status);
@@ -1296,10 +1311,10 @@ struct CgMixedArgs {
   int* iters;     // total inner iterations (negative if capped)
   int* outers;    // refinement steps
   unsigned* status;
-  int* queue;
+  int* queue;  // the classes' counters; with a time budget a CgQueue
   int warm;       // x holds an initial guess (else the solve starts from 0)
   int cap[2];     // floats of shared memory for the padded residual, per class
-  unsigned long long budget_ns;  // time budget of the launch (0: none)
+  unsigned long long budget_ns;  // time budget from the first CTA's start (0: none)
 };
 
 // block_sum with the serial combine done by one warp (the same order, so the
@@ -1540,7 +1555,8 @@ __global__ void __launch_bounds__(cg_threads(LARGE), LARGE ? 1 : 2)
   __shared__ int s_item;
   __shared__ double bc;
   extern __shared__ float pS[];  // A.cap[LARGE] floats
-  const unsigned long long t0 = A.budget_ns ? global_ns() : 0ull;
+  const unsigned long long t0 =
+      A.budget_ns && threadIdx.x == 0 ? cg_start((CgQueue*)A.queue) : 0ull;
   for (;;) {
     if (threadIdx.x == 0) s_item = claim_item(A.queue + LARGE, A.P, A.budget_ns, t0, A.status);
     __syncthreads();
@@ -1811,7 +1827,7 @@ static CgArgs fp64_args(sea_ctx* c) {
 cudaError_t launch_cg(sea_ctx* c) {
   if (c->P == 0) return cudaSuccess;
   const bool mixed = c->prm.precision == 1;
-  cudaError_t e = cudaMemsetAsync(c->queue.p, 0, 2 * sizeof(int), c->stream);
+  cudaError_t e = cudaMemsetAsync(c->queue.p, 0, sizeof(CgQueue), c->stream);
   if (e != cudaSuccess) return e;
   const StencilW W = make_weights(c);
   return cg_both(c->stream, &c->aux, c->P, c->n_large, [&](bool large, cudaStream_t st) {
