@@ -329,9 +329,10 @@ __global__ void __launch_bounds__(SC_THREADS)
   }
   best = warp_best(best);
   // a pivot must not lie below the open classes' lower edge (a closed
-  // candidate could be larger)
-  const bool decide = st.open > 0 && __double_as_longlong(best.v) >=
-                                         __double_as_longlong(edge[st.open]);
+  // candidate could be larger) and be positive (with no density at all every
+  // edge is 0: the classes then run out and the pass over all points reports it)
+  const long long bits = __double_as_longlong(best.v);
+  const bool decide = st.open > 0 && bits > 0 && bits >= __double_as_longlong(edge[st.open]);
   ScMax mine{-2.0, 0x7fffffff, -1};
   auto keep = [&](double v, int a) {
     const ScMax y{v, a == gw ? r0 : list[a], a};
