@@ -934,16 +934,21 @@ __device__ __forceinline__ unsigned long long global_ns() {
 }
 
 // The two classes' queue counters, and when the first CTA of either started (0
-// before; set where there is a time budget).
+// before; set where both classes are launched with a time budget).
 struct CgQueue {
   int next[2];
   unsigned long long start;
 };
-// One start for all CTAs of both classes: those of the small class that wait for
-// SMs which the large class holds start late.
-__device__ __forceinline__ unsigned long long cg_start(CgQueue* q) {
-  const unsigned long long now = global_ns(), first = atomicCAS(&q->start, 0ull, now);
-  return first ? first : now;
+// Start of the time budget.  The CTAs of one launch start together; of two, those
+// of the small class wait for SMs which the large class holds, so all take the
+// start of the first (BOTH; kernels of their own, since the stamp's registers
+// cost the solve 1 to 3%).
+template <bool BOTH>
+__device__ __forceinline__ unsigned long long cg_start(int* queue) {
+  if (!BOTH) return global_ns();
+  const unsigned long long now = global_ns(),
+                           first = atomicCAS(&((CgQueue*)queue)->start, 0ull, now);
+  return first && first < now ? first : now;  // not after what this SM's clock shows
 }
 
 // Next queue item for the CTA (thread 0).  With a time budget, once more
@@ -952,8 +957,7 @@ __device__ __forceinline__ unsigned long long cg_start(CgQueue* q) {
 // CTA's loop (the pairs not taken keep no solution).
 __device__ __forceinline__ int claim_item(int* queue, int P, unsigned long long budget_ns,
                                           unsigned long long t0, unsigned* status) {
-  // signed: another SM's clock may have been read a little later than this one's
-  if (budget_ns && (long long)(global_ns() - t0) > (long long)budget_ns) {
+  if (budget_ns && global_ns() - t0 > budget_ns) {
     atomicOr(status, SEA_FLAG_TIMEOUT);
     return P;
   }
@@ -968,15 +972,14 @@ __host__ __device__ constexpr int cg_pad_limit(bool mixed, bool large, bool team
 }
 
 // Each item's box is solved by the CTAs of a cluster (TEAM > 1) or one CTA.
-template <bool LARGE, int TEAM>
+template <bool LARGE, int TEAM, bool BOTH>
 __global__ void __launch_bounds__(cg_threads(LARGE), LARGE ? 1 : 2) k_cg(CgArgs A, StencilW W) {
   __shared__ CgShared<TEAM, cg_threads(LARGE) / 32> M;
   __shared__ int s_item;
   extern __shared__ int2 Ps[];  // A.cap[LARGE] points
   const CgTeam T = cg_team<TEAM>();
   team_sync(T);  // the team's CTAs have started
-  const unsigned long long t0 =
-      A.budget_ns && T.rank == 0 && threadIdx.x == 0 ? cg_start((CgQueue*)A.queue) : 0ull;
+  const unsigned long long t0 = A.budget_ns ? cg_start<BOTH>(A.queue) : 0ull;
   for (;;) {
     if (T.rank == 0 && threadIdx.x == 0) {
       s_item = claim_item(A.queue + LARGE, A.P, A.budget_ns, t0, A.status);
@@ -1548,15 +1551,14 @@ __device__ __forceinline__ void cg_pair_mixed(const CgMixedArgs& A, const Stenci
   }
 }
 
-template <bool LARGE>
+template <bool LARGE, bool BOTH>
 __global__ void __launch_bounds__(cg_threads(LARGE), LARGE ? 1 : 2)
     k_cg_mixed(CgMixedArgs A, StencilW W, StencilWf Wf) {
   __shared__ double red[2][32];
   __shared__ int s_item;
   __shared__ double bc;
   extern __shared__ float pS[];  // A.cap[LARGE] floats
-  const unsigned long long t0 =
-      A.budget_ns && threadIdx.x == 0 ? cg_start((CgQueue*)A.queue) : 0ull;
+  const unsigned long long t0 = A.budget_ns ? cg_start<BOTH>(A.queue) : 0ull;
   for (;;) {
     if (threadIdx.x == 0) s_item = claim_item(A.queue + LARGE, A.P, A.budget_ns, t0, A.status);
     __syncthreads();
@@ -1831,8 +1833,11 @@ cudaError_t launch_cg(sea_ctx* c) {
   if (e != cudaSuccess) return e;
   const StencilW W = make_weights(c);
   return cg_both(c->stream, &c->aux, c->P, c->n_large, [&](bool large, cudaStream_t st) {
-    auto km = large ? k_cg_mixed<true> : k_cg_mixed<false>;
-    auto kf = large ? k_cg<true, 1> : k_cg<false, 1>;
+    const bool both = c->prm.timeout_ms > 0.0 && c->n_large > 0 && c->n_large < c->P;
+    auto km = large ? (both ? k_cg_mixed<true, true> : k_cg_mixed<true, false>)
+                    : (both ? k_cg_mixed<false, true> : k_cg_mixed<false, false>);
+    auto kf = large ? (both ? k_cg<true, 1, true> : k_cg<true, 1, false>)
+                    : (both ? k_cg<false, 1, true> : k_cg<false, 1, false>);
     CgLaunch L;
     const cudaError_t e1 = cg_shape(mixed ? (const void*)km : (const void*)kf, c->cg_pad_max, mixed,
                                     large, large ? c->n_large : c->P - c->n_large, 0,
@@ -1992,9 +1997,10 @@ cudaError_t launch_cg_boxes(cudaStream_t stream, const double h[3], int nbox,
   A.status = status;
   A.queue = queue;
   return cg_both(stream, nullptr, nbox, n_large, [&](bool large, cudaStream_t st) {
-    auto kern = team > 2    ? (large ? k_cg<true, SEA_CG_TEAM_MAX> : k_cg<false, SEA_CG_TEAM_MAX>)
-                : team == 2 ? (large ? k_cg<true, 2> : k_cg<false, 2>)
-                            : (large ? k_cg<true, 1> : k_cg<false, 1>);
+    constexpr int M = SEA_CG_TEAM_MAX;
+    auto kern = team > 2    ? (large ? k_cg<true, M, false> : k_cg<false, M, false>)
+                : team == 2 ? (large ? k_cg<true, 2, false> : k_cg<false, 2, false>)
+                            : (large ? k_cg<true, 1, false> : k_cg<false, 1, false>);
     CgLaunch L;
     const cudaError_t e1 = cg_shape((const void*)kern, pad_max, false, large,
                                     large ? n_large : nbox - n_large, 0, team, &L);
