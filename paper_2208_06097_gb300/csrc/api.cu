@@ -381,8 +381,13 @@ static sea_status load_orbitals(sea_ctx* c, const double* phi, int n_orb, int on
     c->launches += 1;
     return cudaGetLastError();
   };
-  if (on_device) {
+  cudaPointerAttributes at = {};
+  if (on_device && cudaPointerGetAttributes(&at, phi) != cudaSuccess) cudaGetLastError();
+  if (on_device && sea_reads_in_place(at, c->device)) {
     SEA_CK(check(phi, 0, n_orb, pd), "input check");
+  } else if (on_device) {
+    SEA_CK(cudaMemcpyAsync(pd, phi, bytes, cudaMemcpyDeviceToDevice, c->stream), "copy orbitals");
+    SEA_CK(check(pd, 0, n_orb, nullptr), "input check");
   } else {
     // orbital ranges copied in on the copy stream, each checked on the
     // context stream once it has arrived

@@ -592,6 +592,13 @@ inline cudaError_t run_graph(sea_ctx* c, LaunchGraph& gc, const std::vector<uint
 }
 
 
+// Whether a kernel on `device` may read memory of these attributes where it
+// lies: memory of the device itself.  Memory of another GPU (which needs peer
+// access) or of the host goes through a copy by the runtime.
+inline bool sea_reads_in_place(const cudaPointerAttributes& a, int device) {
+  return a.type == cudaMemoryTypeDevice && a.device == device;
+}
+
 // Host-side helpers implemented in api.cu.
 sea_status sea_fail(sea_ctx* c, sea_status s, const char* msg);
 void sea_batch_cache_free(sea_ctx* c);
