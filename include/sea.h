@@ -65,7 +65,17 @@ typedef enum {
  * decomposition of App. A -- -Mbar = Q Lambda Q^T, operator
  * -W Q |Lambda|^-1 Q^T W^T (the complex zeta of App. A under a Hermitian
  * inner product), eigenvalues within 1e-13 max|lambda| of zero dropped --
- * when a Cholesky pivot is not positive), precision = 0 (FP64 everywhere; 1: the mixed form --
+ * when a Cholesky pivot is not positive), precision = 0 (FP64 inputs, sums and
+ * results; four steps hold their operands as integers against a shared power of
+ * two 2^E above the values named, instead of each against its own: the CG's
+ * search direction, 2^-56 of a bound on the box's largest |p|; the two
+ * contractions with W (M = Phi^T W dV, W^T psi), 2^-56 of each 64-point
+ * segment's 2^E for either factor; W H, 2^-56 of the largest value at the point,
+ * each orbital's scale on the 8 x 4 x 4 tile taken out; the SCDM rotation, 2^-55
+ * of the largest orbital value at the point and of U's column.  Their errors
+ * against the norm of the result are at most those of FP64 multiply-adds; a
+ * component that is smaller than the operands of its segment by 2^k keeps about
+ * 53 - k bits; 1: the mixed form --
  * FP32 stencil sweeps and CG vectors inside an iterative refinement of
  * each pair's solve, whose true residual and solution are FP64 for
  * cg_tol < 1e-10 and double-float (pairs of FP32 values, about 48 bits)

@@ -959,8 +959,8 @@ static cudaError_t launch_expand(sea_ctx* c, const TileGeom& G, const int* tptr,
       c->wx_ready && sea_ensure(c, c->xevb, (size_t)max(c->n_tiles, 1) * m * sizeof(int));
   if (images) {
     const cudaError_t e = launch_expand_tc(
-        c->stream, c->device, c->wx.p, G, c->ng, c->n_tiles, tptr, tlist, xoff, c->wx_steps, H, hj, hv,
-        m, sign < 0.0, out, (int*)c->xevb.p, (int*)c->counts.p + 24, (unsigned*)c->status.p,
+        c->stream, c->device, c->wx.p, G, c->ng, c->n_tiles, tptr, tlist, xoff, c->wx_steps,
+        c->tile_inc, H, hj, hv, m, sign < 0.0, out, (int*)c->xevb.p, (int*)c->counts.p + 24, (unsigned*)c->status.p,
         ace_digits(c));
     if (e != cudaSuccess) return e;
   }
@@ -1154,7 +1154,7 @@ cudaError_t launch_ace_build(sea_ctx* c) {
   err = cudaStreamWaitEvent(c->xfer[0], c->ev[11], 0);
   if (err == cudaSuccess && c->wx_ready)
     err = launch_wx_digits(c->xfer[0], (const double*)c->vxx_dev.p, G, c->ng, nt, tptr, tlist, tsub,
-                           tptr + (nt + 1), c->wx_steps, c->wx.p, digits);
+                           tptr + (nt + 1), c->wx_steps, hinc, c->wx.p, digits);
   if (err == cudaSuccess) err = cudaEventRecord(c->xev[0], c->xfer[0]);
   if (err != cudaSuccess) return err;
   launch_gram_reduce(c->stream, c->prm.precision == 1, (const double*)c->partial.p, n, n, optr, oslot,

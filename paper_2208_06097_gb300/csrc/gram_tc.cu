@@ -5,33 +5,40 @@
 // (s a slot of tile T's W list); the per-orbital sums of M = Phi^T W and of
 // W^T psi add these partials afterwards in FP64.
 //
-// Precision: FP64 operands, FP64-accurate result from BF16 tensor-core
-// products by exact splitting (the Ozaki scheme).  Each row segment x (the
-// 64 points of one half tile, 8 x 4 x 2, of an A row or a W row) shares one
-// exponent E (|x| < 2^E); x 2^-E is truncated to an integer X on a 2^-47
-// grid and written in S = 6 balanced base-256 digits, x 2^-E ~ sum_k d_k
-// 2^(-7-8k) with |d_k| <= 128, each exactly a BF16 value.  For a pair of
-// segments,
-//   sum_r x_r w_r ~ 2^(Ex+Ew) sum_{d=0}^{S-1} 2^(-14-8d) D_d,
+// Precision: FP64 operands, FP16 tensor-core products by exact splitting (the
+// Ozaki scheme).  Each row segment x (the 64 points of one half tile, 8 x 4 x 2,
+// of an A row or a W row) shares one exponent E (|x| < 2^E); x 2^-E is taken to
+// an integer X on a 2^-47 grid and written in S = 6 base-256 digits (W's
+// balanced, |d_k| <= 128, A's the bytes of |x| on a 2^-48 grid with x's sign),
+// each exactly an FP16 value.  For a pair of segments,
+//   sum_r x_r w_r ~ 2^(Ex+Ew) sum_{d=0}^{S-1} 2^(-15-8d) D_d,
 //   D_d = sum_{k+l=d} sum_r dx_k(r) dw_l(r),
-// where every D_d is a sum of at most 6 x 64 products of magnitude <= 2^14,
+// where every D_d is a sum of at most 6 x 64 products of magnitude < 2^15,
 // hence an integer below 2^24: the tensor core's FP32 accumulation of it is
 // exact.  The epilogue combines the D_d exactly in 64-bit integers, aligns the
 // two halves' integers on the larger scale (the other truncated at its unit,
 // 2^-55 of that segment's scale) and truncates once to FP64, with no FP64
-// instruction.  Error: the truncation of X (2^-47 of the segment maximum) and
-// the dropped diagonals d >= S (below 2^-45.7 of max|x| max|w| times the
-// segment length).
+// instruction.  Error: the truncation of X (2^-47 and 2^-48 of the segment's
+// power of two) and the dropped diagonals d >= S (below 2^-45.7 of max|x| max|w|
+// times the segment length).
 //
-// The plain form (DIG = 7) has seven digits per operand: 55-bit integers for W,
-// 56-bit ones for A's bytes, seven diagonals (each still below 2^24), the two
-// halves' sums to 2^-55 of the larger scale, one rounding.  Values within a
-// factor of 8 (A) or 4 (W) of their segment's largest are kept whole, the
-// others to 2^-56 and 2^-55 of it, and the dropped diagonals stay below 2^-54
-// of max|x| max|w| per product: the error of a partial is below the rounding
-// of an FP64 chain of its 64 products.  The FP64 unit took 3.68 ms per
-// contraction (256 rows, 96^3) and 3.51 ms for the expansion.  Segments with
-// a non-finite value give NaN.
+// The plain form (DIG = 7) has seven digits per operand and eight diagonals
+// (each still below 2^24): W rounded to 55 bits, A's bytes to 56, both against
+// their segment's power of two 2^E, the diagonals d >= 8 dropped (2^-61 a point),
+// the two halves' sums to 2^-55 of the larger scale, one rounding.  So a product
+// errs by at most 2^-56 (|x| 2^Ew + |w| 2^Ex): an absolute bound per segment, not
+// one relative to the product as an FP64 multiply-add has it.  Values within a
+// factor of 8 (A) or 4 (W) of 2^E are kept whole; where large x meets small w
+// throughout a segment the sum keeps fewer digits than an FP64 chain (W falling
+// by 2^8 where A rises by as much: errors 2^5 times those of a chain, and at
+// 2^56 nothing is left), which matters only to sums that are as small against
+// the operands.  The expansion holds W against the largest value at each point
+// (k_wx_digits).  Errors of V^ACE psi against extended precision, relative to its
+// norm, 16 to 256 orbitals, 27^3 to 101^3: 3.3 to 6.0e-16, with FP64 multiply-adds
+// 3.9 to 6.3e-16 (with the seven diagonals, W truncated and the tile's scale in
+// the expansion 4.3 to 6.6e-16).  The FP64 unit took 3.68 ms per contraction (256
+// rows, 96^3) and 3.51 ms for the expansion.  Segments with a non-finite value
+// give NaN.
 //
 // Kernel shape: persistent CTAs (one per SM) take tiles from a queue and
 // walk units (W block of up to 32 slots, A block of 128 rows, half tile).
@@ -43,7 +50,7 @@
 // tensor-memory columns d P, so one MMA of A plane k against the stacked W
 // planes 0..5-k (N = (6 - k) P) adds every product of plane k to the
 // diagonals k..5 at once: 24 tcgen05.mma instructions (M = 128, K = 16) per
-// unit.  After the second half tile the converting warps read the
+// unit (28 with seven digits, N = (8 - k) P).  After the second half tile the converting warps read the
 // accumulators back with tcgen05.ld for the epilogue (k_gram_tc).  A few rows
 // take k_gram_few, whose partials are the same bits.
 // Every wait on a completion barrier is bounded: on expiry the kernel sets
@@ -66,14 +73,21 @@ constexpr int KH = 64;                          // points per half tile
 constexpr int MBLK = 128;                       // A rows per block
 constexpr uint32_t CORE_SBO = 128;              // row-group-adjacent core matrices
 constexpr uint32_t TMEM_COLS = 512;
+// Diagonals d = k + l of the digit planes' products that are formed.  Seven digits
+// keep an eighth: the products of diagonal 7, 2^-56.3 of max|x| max|w| a point
+// (rms), were the largest error of a partial, 3.5 times the digits' own.  B then
+// has an eighth plane of zeros, so that every diagonal's accumulator is set by
+// the first MMA.
+constexpr int diagonals(int digits) { return digits == 7 ? 8 : 6; }
 template <int DIG>
 struct GramSizes {
   // W rows per block: seven digit planes of A beside the raw rows leave room
   // for 16 (all but 92 of the 6912 tiles of 256 orbitals on 96^3 have no more)
   static constexpr int NBLK = DIG == 6 ? 32 : 16;
-  static constexpr uint32_t W_HALF = DIG * NBLK * KH * 2;  // bytes of W digits per half tile
-  static constexpr uint32_t SMEM_W = 2 * W_HALF;           // 48 KB (both halves)
-  static constexpr uint32_t TMEM_HALF = DIG * NBLK;        // accumulator columns per half tile
+  static constexpr int ND = diagonals(DIG);
+  static constexpr uint32_t W_HALF = ND * NBLK * KH * 2;  // bytes of W digits per half tile
+  static constexpr uint32_t SMEM_W = 2 * W_HALF;          // 48 KB (both halves)
+  static constexpr uint32_t TMEM_HALF = ND * NBLK;        // accumulator columns per half tile
 };
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool valid) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst), "l"(src),
@@ -83,9 +97,9 @@ __device__ __forceinline__ void cp_async_wait_all() {
   asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;\n" ::: "memory");
 }
 
-// x 2^-E on the 2^-(8 DIG - 1) grid (truncated toward zero), E = emax - 1022
-// for the segment's largest biased exponent emax: a signed integer below
-// 2^(8 DIG - 1).  Integer operations only.
+// x 2^-E on the 2^-(8 DIG - 1) grid, E = emax - 1022 for the segment's largest
+// biased exponent emax: a signed integer below 2^(8 DIG - 1), truncated toward
+// zero with six digits, rounded with seven.  Integer operations only.
 template <int DIG>
 __device__ __forceinline__ long long fixed_bal(double v, int emax) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(v);
@@ -97,7 +111,7 @@ __device__ __forceinline__ long long fixed_bal(double v, int emax) {
     X = ((b & 0xFFFFFFFFFFFFFULL) | (1ULL << 52)) >> sh;
   } else {
     if (e == 0) return 0;
-    X = shr64c(((b & 0xFFFFFFFFFFFFFULL) | (1ULL << 52)) << 2, (unsigned)(emax - e));
+    X = (shr64c(((b & 0xFFFFFFFFFFFFFULL) | (1ULL << 52)) << 3, (unsigned)(emax - e)) + 1) >> 1;
   }
   return (b >> 63) ? -(long long)X : (long long)X;
 }
@@ -199,16 +213,18 @@ __device__ __forceinline__ double scaled_i64_rz_cvt(long long v, int e2) {
   return (v == 0 || ex <= 0) ? 0.0 : __longlong_as_double(b + ((long long)e2 << 52));
 }
 
-// Seven diagonal sums (integer-valued floats, |D_0|, |D_1| < 2^22, the others
-// below 2^24) as the integer sum_d D_d 256^(6-d) with its lowest DROP bits
-// truncated, so that 64 bits hold it.
+// Eight diagonal sums (integer-valued floats, |D_0|, |D_1| < 2^22, the others
+// below 2^24) as the integer sum_d D_d 256^(6-d) rounded at its lowest DROP bits,
+// so that 64 bits hold it.
 template <int DROP>
 __device__ __forceinline__ long long combine7(const uint32_t* f) {
   auto big = [](uint32_t x) { return __float2int_rz(__uint_as_float(x)); };
   const long long hi = (long long)(small_float_int(f[0]) * 256 + small_float_int(f[1])) * 4096 +
                        (long long)big(f[2]) * 16;
+  // D_7 to D_6's unit, half a unit of the result for the rounding
+  const int last = big(f[6]) + (big(f[7]) >> 8) + (1 << (DROP - 1));
   const long long lo = (long long)big(f[3]) * 16777216 + (long long)big(f[4]) * 65536 +
-                       (long long)big(f[5]) * 256 + (long long)big(f[6]);
+                       (long long)big(f[5]) * 256 + (long long)last;
   return (hi << (28 - DROP)) + (lo >> DROP);
 }
 // v 2^e2 rounded to nearest: the conversion instruction (on the FP64 pipe that
@@ -233,7 +249,7 @@ __device__ __forceinline__ double quiet_nan() { return __longlong_as_double(0x7F
 constexpr int EXP_NONFINITE = 0x7FF;
 
 // W digits, once per W: for every slot s of every tile list and half h,
-// wdig[((s * 2 + h) * DIG + k) * 8 + u] = the 8 BF16 digits (16 bytes) of
+// wdig[((s * 2 + h) * DIG + k) * 8 + u] = the 8 FP16 digits (16 bytes) of
 // plane k, x-run u of W row list[s] on that half tile, and wexp[2 s + h]
 // the row segment's largest biased exponent, s counted from slot s0, for the
 // n_tiles tiles from t0.  Warp per (tile, half, group of 8 slots).  Four CTAs per SM: the warps wait on their row loads, so
@@ -336,8 +352,9 @@ __device__ __forceinline__ uint32_t hfma2_u(uint32_t a, uint32_t b, uint32_t c) 
   return r;
 }
 
-// With seven digits X = floor(|x| 2^(56 - E)) = 8 m >> (emax - e) < 2^56, the
-// bytes 6 - k; em_sh = emax << 20, nothing but zeros and subnormals (taken
+// With seven digits X = floor(|x| 2^(56 - E)) = 8 m >> (emax - e) < 2^56
+// (truncated: rounding it costs the converting warps two 64-bit operations a
+// value and W's error is twice as large), the bytes 6 - k; em_sh = emax << 20, nothing but zeros and subnormals (taken
 // as zero) when emax is 0.
 
 // X of one value: the significand of v (bits h, l) shifted onto the grid.
@@ -414,7 +431,7 @@ __device__ __forceinline__ void digits2_u(double v0, double v1, int emax0, int e
     auto fixed = [](uint32_t h, uint32_t l, int emax) -> unsigned long long {
       const int ex = (int)((h >> 20) & 0x7FFu);
       const unsigned long long m = ((unsigned long long)((h & 0xFFFFFu) | 0x100000u) << 32) | l;
-      return ex ? shr64c(m << 3, (unsigned)max(emax - ex, 0)) : 0ULL;
+      return ex ? (shr64c(m << 4, (unsigned)max(emax - ex, 0)) + 1) >> 1 : 0ULL;
     };
     X0 = fixed(h0, (uint32_t)b0, emax0);
     X1 = fixed(h1, (uint32_t)b1, emax1);
@@ -450,7 +467,7 @@ __global__ void __launch_bounds__(GT2_THREADS, 1)
               const int* __restrict__ wexp, double* __restrict__ partial, int* __restrict__ queue,
               unsigned* __restrict__ status) {
   using Z = GramSizes<DIG>;
-  constexpr int NBLK = Z::NBLK;
+  constexpr int NBLK = Z::NBLK, ND = Z::ND;
   constexpr uint32_t W_HALF = Z::W_HALF, TMEM_HALF = Z::TMEM_HALF,
                      SMEM_A2 = GramTmaSizes<DIG>::SMEM_A2;
   extern __shared__ unsigned char gt_raw[];
@@ -505,7 +522,7 @@ __global__ void __launch_bounds__(GT2_THREADS, 1)
         const int nj = u_ring[seq & 1][0], h = u_ring[seq & 1][1];
         if (nj == 0) break;
         const int P = nj <= 16 ? 16 : 32;
-        const uint32_t lbo = DIG * P * 16;
+        const uint32_t lbo = ND * P * 16;
         const uint64_t a0 = sdesc(a_base, A2_LBO, CORE_SBO);
         const uint64_t w0 = sdesc(w_base + h * W_HALF, lbo, CORE_SBO);
         const uint32_t dcol = tmem + (uint32_t)(h * TMEM_HALF);
@@ -524,7 +541,7 @@ __global__ void __launch_bounds__(GT2_THREADS, 1)
 #pragma unroll
             for (int k = 0; k < DIG; ++k)
               mma_kf16(dcol + (uint32_t)(k * P), a0 + ((k * A2_PLANE + q * 2 * A2_LBO) >> 4),
-                       w0 + ((q * 2 * lbo) >> 4), idesc_kf16((DIG - k) * P, MBLK, false),
+                       w0 + ((q * 2 * lbo) >> 4), idesc_kf16((ND - k) * P, MBLK, false),
                        (k > 0 || q > 0) ? 1u : 0u);
           }
           asm volatile(
@@ -651,7 +668,7 @@ __global__ void __launch_bounds__(GT2_THREADS, 1)
     };
     auto load_w = [&](const Unit& u) {
       const int nj = min(NBLK, u.nJ - u.jb), P = nj <= 16 ? 16 : 32;
-      const uint32_t lbo = DIG * P * 16;
+      const uint32_t lbo = ND * P * 16;
       for (int p = tid; p < P * 2 * DIG * 8; p += GT2_CONV) {
         const int rn = p & 7, k = (p >> 3) % DIG, h = (p / (8 * DIG)) & 1, sl = p / (16 * DIG);
         const bool ok = sl < nj;
@@ -706,9 +723,9 @@ __global__ void __launch_bounds__(GT2_THREADS, 1)
           long long s7[2][2];  // [half][column]
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
-            uint32_t f[2][DIG];
+            uint32_t f[2][ND];
 #pragma unroll
-            for (int d = 0; d < DIG; ++d) {
+            for (int d = 0; d < ND; ++d) {
               uint32_t t[2];
               tmem_ld2(lane_addr + (uint32_t)(h * TMEM_HALF + d * P + c0), t);
               f[0][d] = t[0];
@@ -777,6 +794,14 @@ __global__ void __launch_bounds__(GT2_THREADS, 1)
       }
     };
 
+    if (ND > DIG) {  // the zero plane of both halves (blocks of NBLK = 16 alone)
+      static_assert(ND == DIG || NBLK == 16, "one layout of the stack");
+      for (int p = tid; p < 2 * 8 * NBLK; p += GT2_CONV) {
+        const int r = DIG * NBLK + p % NBLK, rn = (p / NBLK) & 7, h = p / (8 * NBLK);
+        *reinterpret_cast<uint4*>(sW + h * W_HALF + (r >> 3) * CORE_SBO + rn * (ND * NBLK * 16) +
+                                  (r & 7) * 16) = make_uint4(0, 0, 0, 0);
+      }
+    }
     Unit cur;
     cur.wb = 0;
     cur.ab = 0;
@@ -914,7 +939,10 @@ __global__ void __launch_bounds__(GT2_THREADS, 1)
 // the image.  Digits, diagonals and the final combination are those of
 // k_gram_tc, every D_d the same exact integer, so the partials are the same
 // bits.  Bound by the latency of its loads and conversions; 8 rows of 75^3
-// against 128 orbitals 320 -> 46 us.
+// against 128 orbitals 320 -> 46 us.  Three CTAs an SM (168 registers, 80 in
+// k_expand_few) where the registers left alone allow two: apply of 8 vectors on
+// 75^3 141 -> 122 us mixed, 208 -> 170 us plain (164 with seven diagonals; four
+// CTAs 175).
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void mma_16816(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2,
                                           uint32_t a3, uint32_t b0, uint32_t b1) {
@@ -947,10 +975,11 @@ constexpr int FEW_WARPS = 4;
 // rows 302 against 316); expansion of 8 and 16 vectors 49 and 88 us against 83.
 constexpr int GRAM_FEW = 32, EXPAND_FEW = 8;
 template <int DIG>
-__global__ void __launch_bounds__(32 * FEW_WARPS)
+__global__ void __launch_bounds__(32 * FEW_WARPS, 3)
     k_gram_few(const double* __restrict__ A, int m, TileGeom G, size_t ng, int t0, int n_tiles,
                const int* __restrict__ tptr, const uint4* __restrict__ wdig, int slot0,
                const int* __restrict__ wexp, double* __restrict__ partial) {
+  constexpr int ND = GramSizes<DIG>::ND;
   const int T = t0 + blockIdx.x * FEW_WARPS + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (T >= n_tiles) return;  // warp-uniform
   const int j0 = tptr[T], nJ = tptr[T + 1] - j0;
@@ -985,9 +1014,9 @@ __global__ void __launch_bounds__(32 * FEW_WARPS)
       const uint32_t em_sh = DIG == 6 ? (em < 64 ? 0xF0000000u : emf + (5u << 20)) : emf;
       digits8_u<DIG>(v[0], em_sh, d[0]);
       digits8_u<DIG>(v[1], em_sh, d[1]);
-      float c[DIG][4];
+      float c[ND][4];
 #pragma unroll
-      for (int k = 0; k < DIG; ++k) c[k][0] = c[k][1] = c[k][2] = c[k][3] = 0.f;
+      for (int k = 0; k < ND; ++k) c[k][0] = c[k][1] = c[k][2] = c[k][3] = 0.f;
       // entries s0 + g and s0 + g + 8 (zeros beyond the list)
       const bool in0 = s0 + g < nJ, in1 = s0 + g + 8 < nJ;
       const uint4* ws = wdig + ((size_t)(j0 - slot0 + s0) * 2 + h) * DIG * 8 + q;
@@ -1000,7 +1029,7 @@ __global__ void __launch_bounds__(32 * FEW_WARPS)
         for (int qq = 0; qq < 2; ++qq) {
           const uint4 u0 = in0 ? w0[l * 8 + 4 * qq] : z4, u1 = in1 ? w1[l * 8 + 4 * qq] : z4;
 #pragma unroll
-          for (int k = 0; k + l < DIG; ++k) {
+          for (int k = 0; k < DIG && k + l < ND; ++k) {
             mma_16816(c[k + l], u0.x, u1.x, u0.y, u1.y, d[qq][k].x, d[qq][k].y);
             mma_16816(c[k + l], u0.z, u1.z, u0.w, u1.w, d[qq][k].z, d[qq][k].w);
           }
@@ -1012,9 +1041,9 @@ __global__ void __launch_bounds__(32 * FEW_WARPS)
         const int s = s0 + g + 8 * (i >> 1), a = a0 + 2 * q + (i & 1);
         const int ea = __shfl_sync(0xffffffffu, em, 8 * q + 4 * (i & 1));
         const int ew = s < nJ ? wexp[(size_t)(j0 - slot0 + s) * 2 + h] : 0;
-        uint32_t f[DIG];
+        uint32_t f[ND];
 #pragma unroll
-        for (int k = 0; k < DIG; ++k) f[k] = __float_as_uint(c[k][i]);
+        for (int k = 0; k < ND; ++k) f[k] = __float_as_uint(c[k][i]);
         long long ac;
         if constexpr (DIG == 7)
           ac = combine7<8>(f);
@@ -1036,10 +1065,10 @@ __global__ void __launch_bounds__(32 * FEW_WARPS)
 }
 
 // ---------------------------------------------------------------------------
-// The mixed form's expansion y[v][r] = sign sum_j W[list(j)][r] H(j, v) on
-// the tensor cores, per tile (M = the tile's 128 points, N = vectors, K =
-// the tile's W list, at most XJ = 32 entries; longer lists go to the FP32
-// kernel).  Scales: W's digits are taken per (tile, list entry j) with the
+// The expansion y[v][r] = sign sum_j W[list(j)][r] H(j, v) on the tensor cores,
+// per tile (M = the tile's 128 points, N = vectors, K = the tile's W list, at
+// most XJ = 32 entries; longer lists go to the general kernels of ace.cu).  With
+// six digits (mixed form; seven as in k_wx_digits):  scales: W's digits are taken per (tile, list entry j) with the
 // exponent E_j of that W row on the tile (six balanced FP16 digits a_k,
 // |a_k| <= 128, on the 2^-47 grid); H(j, v) is scaled exactly by 2^E_j and
 // measured against one exponent E_v per (tile, vector v) over the list, its
@@ -1065,9 +1094,10 @@ template <int DIG>
 struct ExpandSizes {  // with six digits
   static constexpr uint32_t XA_STEP = DIG * XA_BLOCK;       // 24 KB
   static constexpr uint32_t XA_TILE = 2 * XA_STEP;          // 48 KB
-  static constexpr uint32_t XB_LBO = (DIG * XN / 8) * 128;  // 3072
+  static constexpr int ND = diagonals(DIG);
+  static constexpr uint32_t XB_LBO = (ND * XN / 8) * 128;   // 3072
   static constexpr uint32_t XB_CHUNK = 2 * XB_LBO;          // 6 KB: 192 rows x 16 K
-  static constexpr uint32_t XT_COLS = DIG * XN;             // 192
+  static constexpr uint32_t XT_COLS = ND * XN;              // 192
   static constexpr uint32_t XS_SLOT = 2 * XB_CHUNK;         // 12 KB: both K steps of one chunk
   static constexpr size_t XE_SMEM = 2 * XA_TILE + XR * XS_SLOT + 128;
 };
@@ -1078,12 +1108,17 @@ struct ExpandSizes {  // with six digits
 // 60 GB at 512^3).  wx[step xoff[T]][(q 6 + k) 4096 + (p / 8) 128 + (jq / 8) 2048 +
 // (p % 8) 16 + (jq % 8) 2] = digit k of W[list(16 q + jq)] at point p (zero
 // outside the entry's sub-box and beyond the list), wxexp[slot] = E_j + 1022.
+// Seven digits: the digits are those of W 2^(-E_j - e_p), e_p = wxpe[step][p] <= 0
+// the point's largest exponent of W 2^(-E_j) over the list, so that points where
+// all of W is small against the tile (an orbital's tail falls by 2^20 and more
+// across a tile) keep their digits; exact, and e_p goes into the output's
+// exponent.
 template <int DIG>
 __global__ void __launch_bounds__(MBLK)
     k_wx_digits(const double* __restrict__ W, TileGeom G, size_t ng, int n_tiles,
                 const int* __restrict__ tptr, const int* __restrict__ tlist,
                 const int* __restrict__ tsub, const int* __restrict__ xoff,
-                uint4* __restrict__ wx, int* __restrict__ wxexp) {
+                uint4* __restrict__ wx, int* __restrict__ wxexp, int* __restrict__ wxpe) {
   constexpr uint32_t XA_STEP = ExpandSizes<DIG>::XA_STEP;
   const int T = blockIdx.x;
   const int j0 = tptr[T], nJ = tptr[T + 1] - j0;
@@ -1105,6 +1140,16 @@ __global__ void __launch_bounds__(MBLK)
     atomicMax(&emx[jl], (int)((__double_as_longlong(wval(jl)) >> 52) & 0x7FF));
   __syncthreads();
   if (p < nJ) wxexp[j0 + p] = emx[p];
+  int ep = 0;
+  if (DIG == 7) {
+    ep = INT_MIN;
+    for (int jl = 0; jl < nJ; ++jl) {
+      const int e = (int)((__double_as_longlong(wval(jl)) >> 52) & 0x7FF);
+      if (e) ep = max(ep, e - emx[jl]);
+    }
+    if (ep == INT_MIN) ep = 0;  // no value
+    wxpe[(size_t)xoff[T] * MBLK + p] = ep;
+  }
   const int nq = (nJ + XKS - 1) / XKS;
   unsigned char* base = reinterpret_cast<unsigned char*>(wx) + (size_t)xoff[T] * XA_STEP;
   for (int grp = 0; grp < 2 * nq; ++grp) {  // 8 list entries at a time
@@ -1113,8 +1158,8 @@ __global__ void __launch_bounds__(MBLK)
     for (int e = 0; e < 8; e += 2) {
       const int jl = 8 * grp + e;
       float f0[DIG], f1[DIG];
-      digit_floats<DIG>(jl < nJ ? fixed_bal<DIG>(wval(jl), emx[jl]) : 0, f0);
-      digit_floats<DIG>(jl + 1 < nJ ? fixed_bal<DIG>(wval(jl + 1), emx[jl + 1]) : 0, f1);
+      digit_floats<DIG>(jl < nJ ? fixed_bal<DIG>(wval(jl), emx[jl] + ep) : 0, f0);
+      digit_floats<DIG>(jl + 1 < nJ ? fixed_bal<DIG>(wval(jl + 1), emx[jl + 1] + ep) : 0, f1);
 #pragma unroll
       for (int k = 0; k < DIG; ++k) pk[k][e / 2] = pack_f16(f0[k], f1[k]);
     }
@@ -1182,19 +1227,21 @@ constexpr int XF_FIRST = 1, XF_LAST = 2, XF_END = 4;    // slot flags
 // SEA_FLAG_WAIT after the MMAs and copies in flight are done.
 template <int DIG>
 __global__ void __launch_bounds__(XE_THREADS, 1)
-    k_expand_tc(const uint4* __restrict__ wx, const int* __restrict__ wxexp, TileGeom G, size_t ng,
-                int n_tiles, const int* __restrict__ tptr, const int* __restrict__ tlist,
+    k_expand_tc(const uint4* __restrict__ wx, const int* __restrict__ wxexp,
+                const int* __restrict__ wxpe, TileGeom G, size_t ng, int n_tiles, const int* __restrict__ tptr, const int* __restrict__ tlist,
                 const int* __restrict__ xoff, const double* __restrict__ H, long long hj,
                 long long hv, int m, int negate, double* __restrict__ out,
                 const int* __restrict__ evp, int* __restrict__ queue,
                 unsigned* __restrict__ status) {
   using Z = ExpandSizes<DIG>;
+  constexpr int ND = Z::ND;
+  static_assert(2 * Z::XT_COLS <= TMEM_COLS, "two accumulator buffers");
   constexpr uint32_t XA_STEP = Z::XA_STEP, XA_TILE = Z::XA_TILE, XB_LBO = Z::XB_LBO,
                      XB_CHUNK = Z::XB_CHUNK, XT_COLS = Z::XT_COLS, XS_SLOT = Z::XS_SLOT;
   extern __shared__ unsigned char xe_raw[];
   unsigned char* sA = xe_raw + ((128 - (smem_addr(xe_raw) & 127)) & 127);  // two tile images
   unsigned char* sS = sA + 2 * XA_TILE;                                     // XR chunk slots
-  __shared__ int s_T[XR], s_nJ[XR], s_v0[XR], s_fl[XR], s_ab[XR];
+  __shared__ int s_T[XR], s_nJ[XR], s_v0[XR], s_fl[XR], s_ab[XR], s_xo[XR];
   __shared__ __align__(16) int s_ev[XR][XN];
   __shared__ int p_lj[XJ], p_shj[XJ], p_tile;
   __shared__ __align__(8) unsigned long long bar_full[XR], bar_free[XR], bar_md[2], bar_tf[2],
@@ -1245,6 +1292,12 @@ __global__ void __launch_bounds__(XE_THREADS, 1)
           : "memory");
       return r != 0;
     };
+    if (ND > DIG)  // the zero plane of every slot and K step: 32 rows of two core matrices
+      for (int z = ptid; z < XR * 2 * 2 * XN; z += 32 * XP_WARPS) {
+        const int row = DIG * XN + z % XN, jj = (z / XN) & 1, st = z / (2 * XN);
+        *reinterpret_cast<uint4*>(sS + st * XB_CHUNK + jj * XB_LBO + (row >> 3) * 128 +
+                                  (row & 7) * 16) = make_uint4(0, 0, 0, 0);
+      }
     int pseq = 0, tseq = 0;               // chunks published; tiles whose W image was loaded
     uint32_t a_pend = 0, a_par = 0;       // ptid 0, bit b: a load into image buffer b was
                                           // issued; the parity of its completion
@@ -1262,6 +1315,7 @@ __global__ void __launch_bounds__(XE_THREADS, 1)
       const bool end = T >= n_tiles;
       const int j0 = end ? 0 : tptr[T], nJ = end ? 0 : tptr[T + 1] - j0;
       const int nq = (nJ + XKS - 1) / XKS, ab = tseq & 1, jp = 2 * nq, jb = jp * pw;
+      const int xo = nJ > 0 ? xoff[T] : 0;
       if (ptid < nJ) {
         p_lj[ptid] = tlist[j0 + ptid];
         p_shj[ptid] = wxexp[j0 + ptid] - 1022;
@@ -1275,7 +1329,7 @@ __global__ void __launch_bounds__(XE_THREADS, 1)
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
           mbar_expect_tx(smem_addr(&bar_a[ab]), bytes);
           bulk_load(a_base + ab * XA_TILE,
-                    reinterpret_cast<const unsigned char*>(wx) + (size_t)xoff[T] * XA_STEP, bytes,
+                    reinterpret_cast<const unsigned char*>(wx) + (size_t)xo * XA_STEP, bytes,
                     smem_addr(&bar_a[ab]));
           a_pend |= 1u << ab;
           a_par = (a_par & ~(1u << ab)) | ((uint32_t)((tseq >> 1) & 1) << ab);
@@ -1350,6 +1404,7 @@ __global__ void __launch_bounds__(XE_THREADS, 1)
           s_v0[slot] = c * XN;
           s_fl[slot] = end ? XF_END : ((c == 0 ? XF_FIRST : 0) | (c == nch - 1 ? XF_LAST : 0));
           s_ab[slot] = ab;
+          if (DIG == 7) s_xo[slot] = xo;
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // digits -> tensor core
         __syncwarp();
@@ -1411,7 +1466,7 @@ __global__ void __launch_bounds__(XE_THREADS, 1)
           for (int k = 0; k < DIG; ++k) {
             const uint64_t a = sdesc(a_base + ab * XA_TILE + qq * XA_STEP + k * XA_BLOCK, XA_LBO, 128);
             const uint64_t b = sdesc(s_base + slot * XS_SLOT + qq * XB_CHUNK, XB_LBO, 128);
-            mma_kf16(dcol + (uint32_t)(k * XN), a, b, idesc_kf16((DIG - k) * XN, MBLK, false),
+            mma_kf16(dcol + (uint32_t)(k * XN), a, b, idesc_kf16((ND - k) * XN, MBLK, false),
                      (k > 0 || qq > 0) ? 1u : 0u);
           }
         mma_commit(smem_addr(&bar_md[tb]));
@@ -1431,7 +1486,7 @@ __global__ void __launch_bounds__(XE_THREADS, 1)
     const int vv0 = 8 * (warp >> 2);
     const uint32_t lane_q = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)vv0;
     long long cgm = 0, g = -1;
-    int lastT = -1;
+    int lastT = -1, ep = 0;  // seven digits: the point's exponent
     bool fail = false;
     for (int seq = 0;; ++seq) {
       const int slot = seq % XR, use = seq / XR;
@@ -1443,12 +1498,14 @@ __global__ void __launch_bounds__(XE_THREADS, 1)
       const int fl = s_fl[slot], nJ = s_nJ[slot], T = s_T[slot], v0 = s_v0[slot];
       const int4 e4[2] = {*reinterpret_cast<const int4*>(&s_ev[slot][vv0]),
                           *reinterpret_cast<const int4*>(&s_ev[slot][vv0 + 4])};
+      const int xo = DIG == 7 ? s_xo[slot] : 0;
       __syncwarp();
       if (fl & XF_END) break;
       if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(&bar_free[slot])) : "memory");
       if (T != lastT) {
         g = tile_point(G, T, p);
         lastT = T;
+        if (DIG == 7) ep = nJ > 0 ? wxpe[(size_t)xo * MBLK + p] : 0;
       }
       const int vbase = v0 + vv0;  // this warp's first vector of the chunk
       double* o = out + (size_t)vbase * ng + (g >= 0 ? g : 0);
@@ -1468,9 +1525,9 @@ __global__ void __launch_bounds__(XE_THREADS, 1)
         // four vectors at a time: six diagonal sums each
 #pragma unroll
         for (int hh = 0; hh < 2; ++hh) {
-          uint32_t f[DIG][4];
+          uint32_t f[ND][4];
 #pragma unroll
-          for (int d = 0; d < DIG; ++d) tmem_ld4(la + (uint32_t)(d * XN + 4 * hh), f[d]);
+          for (int d = 0; d < ND; ++d) tmem_ld4(la + (uint32_t)(d * XN + 4 * hh), f[d]);
           tmem_wait_ld();
           if (hh == 1) {  // the buffer is read: the next MMAs may overwrite it
             tc_fence_before();
@@ -1481,11 +1538,12 @@ __global__ void __launch_bounds__(XE_THREADS, 1)
           for (int u = 0; u < 4; ++u) {
             double val;
             if constexpr (DIG == 7) {
-              uint32_t fd[DIG];
+              uint32_t fd[ND];
 #pragma unroll
-              for (int d = 0; d < DIG; ++d) fd[d] = f[d][u];
+              for (int d = 0; d < ND; ++d) fd[d] = f[d][u];
               const int e = ev[4 * hh + u];
-              val = e >= EV_NONFINITE ? quiet_nan() : scaled_i64_rn_cvt(combine7<6>(fd), e - 1022 - 63 + 6);
+              val = e >= EV_NONFINITE ? quiet_nan()
+                                      : scaled_i64_rn_cvt(combine7<6>(fd), e + ep - 1022 - 63 + 6);
             } else {
               // sum_d D_d 256^(5 - d) in three 32-bit pairs; |D_d| < 2^22 except
               // D_4 and D_5 of lists longer than 16 (below 2^23): those by the
@@ -1525,20 +1583,24 @@ __global__ void __launch_bounds__(XE_THREADS, 1)
 // A fragments, H's digits formed in registers as the B fragments, E_v over the
 // tile's list by the warp itself.  The outputs are k_expand_tc's bits.
 template <int DIG>
-__global__ void __launch_bounds__(256)
-    k_expand_few(const uint4* __restrict__ wx, const int* __restrict__ wxexp, TileGeom G, size_t ng,
-                 const int* __restrict__ tptr, const int* __restrict__ tlist,
+__global__ void __launch_bounds__(256, 3)
+    k_expand_few(const uint4* __restrict__ wx, const int* __restrict__ wxexp,
+                 const int* __restrict__ wxpe, TileGeom G, size_t ng, const int* __restrict__ tptr, const int* __restrict__ tlist,
                  const int* __restrict__ xoff, const double* __restrict__ H, long long hj,
                  long long hv, int m, int negate, double* __restrict__ out) {
   constexpr uint32_t XA_STEP = ExpandSizes<DIG>::XA_STEP;
+  constexpr int ND = ExpandSizes<DIG>::ND;
   const int T = blockIdx.x, v0 = blockIdx.y * 8;
   const int j0 = tptr[T], nJ = tptr[T + 1] - j0, x0 = xoff[T];
   if (nJ > XJ) return;  // uniform: the long-list kernel's
   const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3, p0 = 16 * (threadIdx.x >> 5);
   const long long o0 = tile_point(G, T, p0 + g), o1 = tile_point(G, T, p0 + g + 8);
-  float c[DIG][4];
+  int ep[2] = {0, 0};  // the points' exponents
+  if (DIG == 7 && nJ > 0)
+    for (int i = 0; i < 2; ++i) ep[i] = wxpe[(size_t)x0 * MBLK + p0 + g + 8 * i];
+  float c[ND][4];
 #pragma unroll
-  for (int k = 0; k < DIG; ++k) c[k][0] = c[k][1] = c[k][2] = c[k][3] = 0.f;
+  for (int k = 0; k < ND; ++k) c[k][0] = c[k][1] = c[k][2] = c[k][3] = 0.f;
   // entries j = 16 s + {2q, 2q + 1, 8 + 2q, 9 + 2q} of vector v0 + g
   double hval[2][4];
   int sh[2][4], em = 0;
@@ -1575,7 +1637,8 @@ __global__ void __launch_bounds__(256)
       auto word = [&](uint32_t off) { return __ldg(reinterpret_cast<const uint32_t*>(a + off)); };
       const uint32_t a0 = word(0), a1 = word(128), a2 = word(XA_LBO), a3 = word(XA_LBO + 128);
 #pragma unroll
-      for (int l = 0; k + l < DIG; ++l) mma_16816(c[k + l], a0, a1, a2, a3, pk[l][0], pk[l][1]);
+      for (int l = 0; l < DIG && k + l < ND; ++l)
+        mma_16816(c[k + l], a0, a1, a2, a3, pk[l][0], pk[l][1]);
     }
   }
   // c[d][i]: point p0 + g + 8 (i / 2), vector v0 + 2 q + (i & 1)
@@ -1584,12 +1647,14 @@ __global__ void __launch_bounds__(256)
     const int v = v0 + 2 * q + (i & 1);
     const long long o = i < 2 ? o0 : o1;
     const int ev = __shfl_sync(0xffffffffu, em, 8 * q + 4 * (i & 1));
-    uint32_t f[DIG];
+    uint32_t f[ND];
 #pragma unroll
-    for (int k = 0; k < DIG; ++k) f[k] = __float_as_uint(c[k][i]);
+    for (int k = 0; k < ND; ++k) f[k] = __float_as_uint(c[k][i]);
     double val;
     if constexpr (DIG == 7)
-      val = ev >= EV_NONFINITE ? quiet_nan() : scaled_i64_rn_cvt(combine7<6>(f), ev - 1022 - 63 + 6);
+      val = ev >= EV_NONFINITE
+                ? quiet_nan()
+                : scaled_i64_rn_cvt(combine7<6>(f), ev + ep[i >> 1] - 1022 - 63 + 6);
     else
       val = scaled_i64_rz_cvt(combine6(f), ev - 1022 - 55);
     if (nJ == 0) val = 0.0;
@@ -1661,37 +1726,44 @@ static bool make_a_map(const double* A, int m, const TileGeom& G, CUtensorMap* m
 static size_t xa_step(int digits) {
   return digits == 7 ? ExpandSizes<7>::XA_STEP : ExpandSizes<6>::XA_STEP;
 }
+// Images, the list entries' exponents and the points' (per K step, seven digits).
 size_t wx_digits_bytes(long long steps, long long slots, int digits) {
-  return (size_t)steps * xa_step(digits) + (size_t)std::max(slots, 1LL) * sizeof(int);
+  return (size_t)steps * xa_step(digits) +
+         ((size_t)std::max(slots, 1LL) + (digits == 7 ? (size_t)steps * MBLK : 0)) * sizeof(int);
+}
+static int* wx_exp(const void* wxbuf, long long steps, int digits) {
+  return (int*)((unsigned char*)wxbuf + (size_t)steps * xa_step(digits));
 }
 
 cudaError_t launch_wx_digits(cudaStream_t st, const double* W, const TileGeom& G, size_t ng,
                              int n_tiles, const int* tptr, const int* tlist, const int* tsub,
-                             const int* xoff, long long steps, void* wxbuf, int digits) {
+                             const int* xoff, long long steps, long long slots, void* wxbuf,
+                             int digits) {
   if (n_tiles <= 0) return cudaSuccess;
-  uint4* wx = (uint4*)wxbuf;
-  int* wxexp = (int*)((unsigned char*)wxbuf + (size_t)steps * xa_step(digits));
+  int* wxexp = wx_exp(wxbuf, steps, digits);
   (digits == 7 ? k_wx_digits<7> : k_wx_digits<6>)<<<n_tiles, MBLK, 0, st>>>(
-      W, G, ng, n_tiles, tptr, tlist, tsub, xoff, wx, wxexp);
+      W, G, ng, n_tiles, tptr, tlist, tsub, xoff, (uint4*)wxbuf, wxexp,
+      wxexp + std::max(slots, 1LL));
   return cudaGetLastError();
 }
 
 template <int DIG>
 static cudaError_t expand_tc(cudaStream_t st, int device, const void* wxbuf, const TileGeom& G,
                              size_t ng, int n_tiles, const int* tptr, const int* tlist,
-                             const int* xoff, long long steps, const double* H, long long hj,
-                             long long hv, int m, bool negate, double* out, int* evbuf, int* queue,
-                             unsigned* status) {
+                             const int* xoff, long long steps, long long slots, const double* H,
+                             long long hj, long long hv, int m, bool negate, double* out, int* evbuf,
+                             int* queue, unsigned* status) {
   constexpr size_t smem = ExpandSizes<DIG>::XE_SMEM;
   cudaError_t e =
       cudaFuncSetAttribute(k_expand_tc<DIG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   if (n_tiles <= 0 || m <= 0) return cudaSuccess;
   const uint4* wx = (const uint4*)wxbuf;
-  const int* wxexp = (const int*)((const unsigned char*)wxbuf + (size_t)steps * xa_step(DIG));
+  const int* wxexp = wx_exp(wxbuf, steps, DIG);
+  const int* wxpe = wxexp + std::max(slots, 1LL);
   if (m <= EXPAND_FEW) {
-    k_expand_few<DIG><<<dim3(n_tiles, (m + 7) / 8), 256, 0, st>>>(wx, wxexp, G, ng, tptr, tlist, xoff,
-                                                                  H, hj, hv, m, negate ? 1 : 0, out);
+    k_expand_few<DIG><<<dim3(n_tiles, (m + 7) / 8), 256, 0, st>>>(wx, wxexp, wxpe, G, ng, tptr, tlist,
+                                                                  xoff, H, hj, hv, m, negate ? 1 : 0, out);
     return cudaGetLastError();
   }
   int nsm = 0;
@@ -1701,18 +1773,18 @@ static cudaError_t expand_tc(cudaStream_t st, int device, const void* wxbuf, con
   k_expand_ev<DIG == 7><<<dim3(n_tiles, (m + 127) / 128), 128, 0, st>>>(tptr, tlist, wxexp, H, hj,
                                                                        hv, m, evbuf);
   k_expand_tc<DIG><<<std::min(nsm, n_tiles), XE_THREADS, smem, st>>>(
-      wx, wxexp, G, ng, n_tiles, tptr, tlist, xoff, H, hj, hv, m, negate ? 1 : 0, out, evbuf, queue,
-      status);
+      wx, wxexp, wxpe, G, ng, n_tiles, tptr, tlist, xoff, H, hj, hv, m, negate ? 1 : 0, out, evbuf,
+      queue, status);
   return cudaGetLastError();
 }
 
 cudaError_t launch_expand_tc(cudaStream_t st, int device, const void* wxbuf, const TileGeom& G,
                              size_t ng, int n_tiles, const int* tptr, const int* tlist,
-                             const int* xoff, long long steps, const double* H, long long hj,
-                             long long hv, int m, bool negate, double* out, int* evbuf, int* queue,
-                             unsigned* status, int digits) {
+                             const int* xoff, long long steps, long long slots, const double* H,
+                             long long hj, long long hv, int m, bool negate, double* out, int* evbuf,
+                             int* queue, unsigned* status, int digits) {
   return (digits == 7 ? expand_tc<7> : expand_tc<6>)(st, device, wxbuf, G, ng, n_tiles, tptr, tlist,
-                                                     xoff, steps, H, hj, hv, m, negate, out, evbuf,
+                                                     xoff, steps, slots, H, hj, hv, m, negate, out, evbuf,
                                                      queue, status);
 }
 

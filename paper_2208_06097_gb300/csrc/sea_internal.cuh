@@ -830,12 +830,13 @@ __host__ __device__ __forceinline__ int wx_tile_steps(int list) {
 size_t wx_digits_bytes(long long steps, long long slots, int digits);
 cudaError_t launch_wx_digits(cudaStream_t st, const double* W, const TileGeom& G, size_t ng,
                              int n_tiles, const int* tptr, const int* tlist, const int* tsub,
-                             const int* xoff, long long steps, void* wxbuf, int digits);
+                             const int* xoff, long long steps, long long slots, void* wxbuf,
+                             int digits);
 cudaError_t launch_expand_tc(cudaStream_t st, int device, const void* wxbuf, const TileGeom& G,
                              size_t ng, int n_tiles, const int* tptr, const int* tlist,
-                             const int* xoff, long long steps, const double* H, long long hj,
-                             long long hv, int m, bool negate, double* out, int* evbuf, int* queue,
-                             unsigned* status, int digits);
+                             const int* xoff, long long steps, long long slots, const double* H,
+                             long long hj, long long hv, int m, bool negate, double* out, int* evbuf,
+                             int* queue, unsigned* status, int digits);
 cudaError_t launch_gram_tc(cudaStream_t st, int device, const double* A, int m, const TileGeom& G,
                            size_t ng, int2 a, int2 b, const int* tptr, const void* wbuf,
                            double* partial, int* queue, unsigned* status, int digits);
