@@ -219,7 +219,7 @@ __global__ void __launch_bounds__(FAR_T, 4)
     const double* frow = fp + ((size_t)gz * ny + gy) * nx;
     double* orow = out + (size_t)(tz * e.wl[1] + ty) * e.wl[0];
     const bool cut = i >= nl.n_whole;
-    for (int tx = cut && x0 >= sp.b0[0] && x0 < sp.b1[0] ? sp.b1[0] : x0; tx < x1;) {
+    for (int tx = window_piece_first(sp, cut, x0); tx < x1; tx = window_piece_next(sp, cut, tx)) {
       int gx = gx0 + tx;
       gx -= gx >= nx ? nx : 0;
       const double f = frow[gx];
@@ -230,8 +230,6 @@ __global__ void __launch_bounds__(FAR_T, 4)
       } else {
         orow[tx] = __dmul_rn(v, f);
       }
-      ++tx;
-      if (cut && tx == sp.b0[0]) tx = sp.b1[0];
     }
   }
 }

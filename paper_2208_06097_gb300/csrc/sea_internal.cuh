@@ -705,6 +705,17 @@ __host__ __device__ __forceinline__ void window_outside_line(const WinSplit& s, 
   *ty = oy + ry;
 }
 
+// The points outside the box of a piece [x0, x1) of a line in the order above
+// (cut: a line that crosses the box): the first one is window_piece_first, the
+// one after tx window_piece_next, while they are below x1.
+__host__ __device__ __forceinline__ int window_piece_first(const WinSplit& s, bool cut, int x0) {
+  return cut && x0 >= s.b0[0] && x0 < s.b1[0] ? s.b1[0] : x0;
+}
+__host__ __device__ __forceinline__ int window_piece_next(const WinSplit& s, bool cut, int tx) {
+  ++tx;
+  return cut && tx == s.b0[0] ? s.b1[0] : tx;
+}
+
 // Window coordinates of point u (0 <= u < n_out, n_out < 2^24) of the window
 // points outside the pair box, line after line in the order above, on the
 // cut lines first all points left of the box, then all right of it.
