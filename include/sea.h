@@ -274,15 +274,20 @@ sea_status sea_get_stats(const sea_ctx* ctx, sea_stats* s);
  * values concatenated in order, each box [ez][ey][ex]; iters (host, may be
  * NULL) receives the iteration counts (negative: capped).  Allocates and
  * frees its own device scratch (3 vectors of the total length) on every
- * call and synchronizes the stream.  Returns SEA_ERR_CG_NOT_CONVERGED if a
- * box reached max_iter (x still written). */
+ * call and synchronizes the stream.  A call of few boxes lets several CTAs
+ * share one (their number follows from n_box and the largest boxes), which add
+ * their sums in another order: a call gives the same bits every time, but a box
+ * solved in another company of boxes, or on a GPU with another number of SMs,
+ * agrees to the tolerance and its iteration count to about one.  Returns
+ * SEA_ERR_CG_NOT_CONVERGED if a box reached max_iter (x still written). */
 sea_status sea_poisson_batch(const double h[3], int n_box, const int* ext, const double* rhs,
                              double* x, double tol, int tol_mode, int max_iter, int* iters,
                              void* cuda_stream);
 
-/* Same solve as sea_poisson_batch, for callers that cannot allocate device
- * memory: plugins whose host framework owns all device memory through its
- * own pool, and processes whose device footprint is fixed at start-up.  It
+/* Same solve as sea_poisson_batch (the same bits for the same boxes), for
+ * callers that cannot allocate device memory: plugins whose host framework
+ * owns all device memory through its own pool, and processes whose device
+ * footprint is fixed at start-up.  It
  * allocates nothing: its scratch is one fixed array of device memory inside
  * the library (about 25 MB, held on every GPU that loads the library until
  * the process exits).  The paper has no counterpart to this entry point.

@@ -1929,7 +1929,10 @@ cudaError_t launch_cg_batch(cudaStream_t st, const CgAux* aux, const void* descs
 // 4 and 8, us, boxes of 9 to 16 points an edge: 16 boxes 1019, 873, 770, 689; 48
 // boxes 1376, 1045, 933, 1055; 100 boxes 1335, 1337, 1136, 1721; 150 boxes 1450,
 // 1412, 1659, 2480; 450 boxes 1884, 2185, 3500, 6410 (there the teams' barriers
-// only delay SMs that have other boxes to work on).
+// only delay SMs that have other boxes to work on).  A box's sums, hence its last
+// bits, depend on its team, so on the other boxes of the call (sea.h says so); the
+// pairs of sea_apply_vxx stay on single CTAs, since batched and single calls give
+// the same bits.
 int cg_box_team(int n_box, const int* ext) {
   int dev = 0, nsm = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
