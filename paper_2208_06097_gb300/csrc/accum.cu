@@ -632,8 +632,7 @@ cudaError_t launch_accumulate_range(sea_ctx* c, double* out, int o_begin, int o_
       }
       slabs = (c->N[1] + rows - 1) / rows;
       const size_t smem = bytes(rows);
-      cudaError_t e = cudaFuncSetAttribute(k_accumulate, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)smem);
+      const cudaError_t e = sea_allow_smem((const void*)k_accumulate, smem);
       if (e != cudaSuccess) return e;
       // bulk plane copies: whole planes of 16-byte multiples into 16-byte
       // aligned outputs

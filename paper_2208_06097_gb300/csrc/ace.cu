@@ -1120,11 +1120,8 @@ cudaError_t launch_ace_build(sea_ctx* c) {
   {
     const size_t smem = (size_t)c->max_tile_list * EV * sizeof(double);
     if (smem > 48 * 1024) {
-      err = cudaFuncSetAttribute(k_tile_expand, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)smem);
-      if (err == cudaSuccess)
-        err = cudaFuncSetAttribute(k_tile_expand_x, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)smem);
+      err = sea_allow_smem((const void*)k_tile_expand, smem);
+      if (err == cudaSuccess) err = sea_allow_smem((const void*)k_tile_expand_x, smem);
       if (err != cudaSuccess) return err;
     }
   }

@@ -1638,8 +1638,7 @@ cudaError_t launch_pair_setup(sea_ctx* c) {
   auto moments = c->prm.precision == 1 ? k_pair_moments<true> : k_pair_moments<false>;
   const size_t msm = pair_moments_smem(c->N[1], c->N[2]);
   if (msm > 48 * 1024) {
-    const cudaError_t e = cudaFuncSetAttribute(moments, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)msm);
+    const cudaError_t e = sea_allow_smem((const void*)moments, msm);
     if (e != cudaSuccess) return e;
   }
   moments<<<c->P, 256, msm, c->stream>>>(

@@ -649,8 +649,7 @@ cudaError_t launch_row_col_sums(sea_ctx* c, const double* phi, int o0, int o1, d
   if (nx <= 192) return run(k_row_col_sums_reg<6, false>, k_row_col_sums_reg<6, true>);
   if (nx <= SEA_SUMS_REG_MAX) return run(k_row_col_sums_reg<8, false>, k_row_col_sums_reg<8, true>);
   const size_t rc_smem = rc_smem_bytes(nx);
-  const cudaError_t e = cudaFuncSetAttribute(
-      k_row_col_sums, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rc_smem);
+  const cudaError_t e = sea_allow_smem((const void*)k_row_col_sums, rc_smem);
   if (e != cudaSuccess) return e;
   k_row_col_sums<<<grid, 128, rc_smem, c->stream>>>(phi, nx, ny, nz, Rs, Cs);
   return cudaGetLastError();
@@ -668,8 +667,7 @@ cudaError_t launch_plan_boxes(sea_ctx* c) {
     const int mmin = std::max(1, std::min(nx, ny));
     const size_t mg_smem = (size_t)std::max(1, MG_THREADS / mmin) * Nmax * 2 * sizeof(unsigned long long);
     if (mg_smem > 48 * 1024) {
-      const cudaError_t e = cudaFuncSetAttribute(k_marginals, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)mg_smem);
+      const cudaError_t e = sea_allow_smem((const void*)k_marginals, mg_smem);
       if (e != cudaSuccess) return e;
     }
     k_marginals<<<n * 3, MG_THREADS, mg_smem, c->stream>>>(

@@ -561,7 +561,7 @@ static cudaError_t pivots_lazy(sea_ctx* c, const double* cn, const double* bv, i
   k_scdm_collect<<<(na + 7) / 8, 256, 0, st>>>((const double*)c->vxx_dev.p, n, N, list, na, cn, A, cA);
   const int smem = (2 * n + 1) * (int)sizeof(double);
   if (smem > 48 * 1024) {
-    e = cudaFuncSetAttribute(k_scdm_step, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    e = sea_allow_smem((const void*)k_scdm_step, smem);
     if (e != cudaSuccess) return e;
   }
   cudaMemcpyAsync(kept, &na, sizeof(int), cudaMemcpyHostToDevice, st);

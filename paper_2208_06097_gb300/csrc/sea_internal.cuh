@@ -8,7 +8,11 @@
 #include <nvtx3/nvToolsExt.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <cstddef>
+#include <map>
+#include <mutex>
+#include <utility>
 #include <vector>
 
 #include "../../include/sea.h"
@@ -597,6 +601,24 @@ inline cudaError_t run_graph(sea_ctx* c, LaunchGraph& gc, const std::vector<uint
 // access) or of the host goes through a copy by the runtime.
 inline bool sea_reads_in_place(const cudaPointerAttributes& a, int device) {
   return a.type == cudaMemoryTypeDevice && a.device == device;
+}
+
+// Lets `kernel` take `bytes` of dynamic shared memory on the current device.  The
+// attribute is the process's, and calls of other contexts and threads need other
+// sizes: it only ever grows, so that no launch finds it below its own size.
+inline cudaError_t sea_allow_smem(const void* kernel, size_t bytes) {
+  static std::mutex mutex;
+  static std::map<std::pair<int, const void*>, size_t> most;
+  int dev = 0;
+  const cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  std::lock_guard<std::mutex> lock(mutex);
+  size_t& m = most[{dev, kernel}];
+  const size_t want = std::max(m, bytes);
+  const cudaError_t e2 =
+      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)want);
+  if (e2 == cudaSuccess) m = want;
+  return e2;
 }
 
 // Host-side helpers implemented in api.cu.
