@@ -849,9 +849,6 @@ __device__ __forceinline__ double team_total(const CgTeam& T, const double* sums
   return s;
 }
 
-// Points of a team's CTA in registers: the largest of cg_fix_team's forms.
-#define SEA_CG_TEAM_NP 4
-
 // One pair's FP64-form solve (all CTAs of its team; teams solve bare boxes
 // only): the fixed-point stencil
 // where the padded planes fit the launch's shared memory (and a team's points
@@ -962,13 +959,6 @@ __device__ __forceinline__ int claim_item(int* queue, int P, unsigned long long 
     return P;
   }
   return atomicAdd(queue, 1);
-}
-
-__host__ __device__ constexpr int cg_threads(bool large) { return large ? 1024 : 512; }
-// Padded points of a box that fit shared memory, 8 bytes (plain form) or 4
-// (mixed form) each.
-__host__ __device__ constexpr int cg_pad_limit(bool mixed, bool large, bool team = false) {
-  return mixed ? (large ? 56000 : SEA_CG_SINGLE) : (large ? (team ? 27000 : 28000) : 13824);
 }
 
 // Each item's box is solved by the CTAs of a cluster (TEAM > 1) or one CTA.
@@ -1922,33 +1912,12 @@ cudaError_t launch_cg_batch(cudaStream_t st, const CgAux* aux, const void* descs
   });
 }
 
-// The rule: as many CTAs a box (8 at most, the portable cluster size) as fill two
-// places per SM, fewer where a box that one CTA solves in fixed point would not
-// fit the team's registers and shared memory.  Time of a call with teams of 1, 2,
-// 4 and 8, us, boxes of 9 to 16 points an edge: 16 boxes 1019, 873, 770, 689; 48
-// boxes 1376, 1045, 933, 1055; 100 boxes 1335, 1337, 1136, 1721; 150 boxes 1450,
-// 1412, 1659, 2480; 450 boxes 1884, 2185, 3500, 6410 (there the teams' barriers
-// only delay SMs that have other boxes to work on).  A box's sums, hence its last
-// bits, depend on its team, so on the other boxes of the call (sea.h says so); the
-// pairs of sea_apply_vxx stay on single CTAs, since batched and single calls give
-// the same bits.
 int cg_box_team(int n_box, const int* ext) {
   int dev = 0, nsm = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     return 1;
-  int team = SEA_CG_TEAM_MAX;
-  while (team > 1 && (long long)team * n_box > 2LL * nsm) team /= 2;
-  for (int b = 0; b < n_box && team > 1; ++b) {
-    const int* e = ext + 3 * b;
-    const int n = e[0] * e[1] * e[2];
-    const bool large = n > SEA_CG_SPLIT;
-    if (cg_pad_volume(e[0], e[1], e[2], 1) > cg_pad_limit(false, large)) continue;
-    while (team > 1 && (cg_share(n, team) > SEA_CG_TEAM_NP * cg_threads(large) ||
-                        cg_pad_volume(e[0], e[1], e[2], team) > cg_pad_limit(false, large, true)))
-      team /= 2;
-  }
-  return team;
+  return cg_team_rule(n_box, ext, nsm);
 }
 
 // Batched solve of -Lap_h x = rhs on independent boxes (no pair energies):

@@ -796,10 +796,60 @@ __host__ __device__ __forceinline__ bool cg_large(const int* ext, bool mixed) {
                : ext[0] * ext[1] * ext[2] > SEA_CG_SPLIT;
 }
 
+__host__ __device__ constexpr int cg_threads(bool large) { return large ? 1024 : 512; }
+// Padded points of a box that fit shared memory, 8 bytes (plain form) or 4
+// (mixed form) each.
+__host__ __device__ constexpr int cg_pad_limit(bool mixed, bool large, bool team = false) {
+  return mixed ? (large ? 56000 : SEA_CG_SINGLE) : (large ? (team ? 27000 : 28000) : 13824);
+}
+
+// Points of a team's CTA in registers: the largest of cg_fix_team's forms.
+#define SEA_CG_TEAM_NP 4
+
 // CTAs (a cluster, at most SEA_CG_TEAM_MAX) that share a box of a bare batch of
-// n_box boxes on the current device.
+// n_box boxes on a GPU of nsm SMs.
 #define SEA_CG_TEAM_MAX 8
-int cg_box_team(int n_box, const int* ext);
+// The rule: as many CTAs a box (8 at most, the portable cluster size) as fill two
+// places per SM, fewer where a box that one CTA solves in fixed point would not
+// fit the team's registers and shared memory.  Time of a call with teams of 1, 2,
+// 4 and 8, us, boxes of 9 to 16 points an edge: 16 boxes 1019, 873, 770, 689; 48
+// boxes 1376, 1045, 933, 1055; 100 boxes 1335, 1337, 1136, 1721; 150 boxes 1450,
+// 1412, 1659, 2480; 450 boxes 1884, 2185, 3500, 6410 (there the teams' barriers
+// only delay SMs that have other boxes to work on).  A box's sums, hence its last
+// bits, depend on its team, so on the other boxes of the call (sea.h says so); the
+// pairs of sea_apply_vxx stay on single CTAs, since batched and single calls give
+// the same bits.
+// A box that not even the team solves in fixed point (over the shared memory of
+// one CTA and the team's registers) is left to the team's first CTA: not more
+// teams' places than SMs then, since boxes of the large class take an SM a CTA
+// (152 boxes of 25^3 44.8 -> 22.6 ms, 64 of 40^3 262 -> 135 ms).
+inline int cg_team_rule(int n_box, const int* ext, int nsm) {
+  int team = SEA_CG_TEAM_MAX;
+  while (team > 1 && (long long)team * n_box > 2LL * nsm) team /= 2;
+  // fits(b): the team solves box b in fixed point
+  auto fits = [&](const int* e, bool large) {
+    return cg_share(e[0] * e[1] * e[2], team) <= SEA_CG_TEAM_NP * cg_threads(large) &&
+           cg_pad_volume(e[0], e[1], e[2], team) <= cg_pad_limit(false, large, true);
+  };
+  long long n_large = 0;
+  for (int b = 0; b < n_box; ++b) {
+    const int* e = ext + 3 * b;
+    const bool large = e[0] * e[1] * e[2] > SEA_CG_SPLIT;
+    n_large += large;
+    if (cg_pad_volume(e[0], e[1], e[2], 1) > cg_pad_limit(false, large)) continue;
+    while (team > 1 && !fits(e, large)) team /= 2;
+  }
+  auto one_left = [&] {
+    for (int b = 0; b < n_box; ++b) {
+      const int* e = ext + 3 * b;
+      if (e[0] * e[1] * e[2] > SEA_CG_SPLIT && !fits(e, true)) return true;
+    }
+    return false;
+  };
+  while (team > 1 && n_large * team > nsm && one_left()) team /= 2;
+  return team;
+}
+int cg_box_team(int n_box, const int* ext);  // on the current device
 
 // Launch wrappers (each file implements its own).
 // Rows that the plan's sums are formed of in registers.
