@@ -47,10 +47,9 @@ FORMS = {"plain": "plain FP64",
                   "double-float multipoles and Cholesky; ACE contractions on the tensor cores "
                   "from exact digit splits of FP64 values"}
 
-# Algorithmic FP64 flops per CG unknown and iteration: the symmetric 37-point
-# stencil as 18 pair sums, 18 multiply-adds and the centre product (55), plus
-# two dot products and three vector updates (10).
-CG_FLOPS_PER_UNKNOWN_ITER = 65
+# FP64 flops per CG unknown and iteration in the plain form: two dot products and
+# three vector updates (the 37-point stencil runs in exact fixed-point integers).
+CG_FLOPS_PER_UNKNOWN_ITER = 10
 # FP64 peak from the part's unit counts and clock: 152 SMs x 2 FP64 FMA/clk x
 # 2 flop x 2.07 GHz (the nominal 1.25 TFLOP/s FP64 figure).
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
@@ -287,48 +286,45 @@ def run_ours(args, ws, rank, local):
     # launch, peak, bound, note); work in the peak's unit (flop or FP32 op)
     cand = []
     gram_ms = (sm["gram_build"] + sm["gram_apply"]) / 2
-    if chosen == "plain":
-        note = ("FP64 ALU from unit counts: 152 SMs x 2 DFMA/clk x 2 flop x 2.07 GHz; "
-                "algorithmic flops: CG 65/unknown/iteration, ACE 2 x rows x nonzeros of W")
-        cand.append(("k_cg (persistent FP64 CG)", sm["cg"], 1,
+    hbm = float(_peaks().get("hbm_gbs", 6800.0))  # GB/s, measured copy
+    plain = chosen == "plain"
+    if plain:
+        cand.append(("k_cg (FP64-form CG, stencil in exact fixed-point integers)", sm["cg"], 1,
                      CG_FLOPS_PER_UNKNOWN_ITER * R["cg_unknown_iters"], FP64_PEAK_TFLOPS, "alu",
-                     note))
-        cand.append(("k_gram_partial (FP64 M = Phi^T W and W^T psi over W's tiles)", gram_ms, 2,
-                     2.0 * n * nnz_w, FP64_PEAK_TFLOPS, "alu", note))
-        cand.append(("k_tile_expand (FP64 W H over W's tiles)", sm["expand_apply"], 1,
-                     2.0 * N_TRIAL * nnz_w, FP64_PEAK_TFLOPS, "alu", note))
+                     "FP64 ALU from unit counts: 152 SMs x 2 DFMA/clk x 2 flop x 2.07 GHz; the "
+                     "five FP64 multiply-adds per unknown and iteration"))
     else:
-        hbm = float(_peaks().get("hbm_gbs", 6800.0))  # GB/s, measured copy
         note_cg = ("HBM of measured (copy, MEASURED_PEAKS.json); effective model bytes: 11 vector "
                    "passes x 4 B per unknown and FP32 inner iteration (the pair vectors stay "
                    "on chip, so DRAM traffic is lower)")
         cand.append(("k_cg_mixed (FP32 CG sweeps inside FP64 refinement)", sm["cg"], 1,
                      44.0 * R["cg_unknown_iters"], hbm, "hbm", note_cg))
-        # the CG's own roof: shared memory (37 four-byte stencil loads per
-        # unknown and inner iteration) against 152 SMs x 128 B/clk at the
-        # sampled SM clock
-        sm_mhz = (R["clocks"] or {}).get("sm_mhz") or 2070.0
-        smem_peak = 152 * 128 * sm_mhz * 1e6 / 1e9  # GB/s
-        cand.append(("k_cg_mixed [shared-memory roof]", sm["cg"], 1,
-                     37 * 4.0 * R["cg_unknown_iters"], smem_peak, "smem",
-                     "shared-memory bandwidth from unit counts: 152 SMs x 128 B/clk x the "
-                     "sampled SM clock; algorithmic bytes: the 37 stencil loads (4 B) per "
-                     "unknown and inner FP32 iteration"))
-        note_gt = ("HBM of measured (copy); algorithmic bytes: the A rows on the tiles where W is "
-                   "nonzero (8 B per point), W's FP16 digit planes (1536 B per tile slot and "
-                   "128-row block), the FP64 partials written")
-        slots = st["ace_support_points"] / 128  # total W list length over the tiles
-        gram_bytes = (n * 128 * 8.0 * tiles_w + 1536.0 * slots * ((n + 127) // 128) +
-                      8.0 * slots * n)
-        cand.append(("k_gram_tc (tensor-core M = Phi^T W and W^T psi, exact FP16 digits)",
-                     gram_ms, 2, gram_bytes, hbm, "hbm", note_gt))
-        note_x = ("HBM of measured (copy); algorithmic bytes: the FP64 output (8 B per grid "
-                  "point and vector) and W's per-tile BF16 digit image (24 KB per tile with "
-                  "support and K step of 16 W rows)")
-        ng = float(np.prod(s.grid))
-        expand_bytes = 8.0 * N_TRIAL * ng + 24576.0 * tiles_w
-        cand.append(("k_expand_tc (tensor-core W H, exact FP16 digits)", sm["expand_apply"], 1,
-                     expand_bytes, hbm, "hbm", note_x))
+    # the CG's own roof: shared memory (37 stencil loads per unknown and
+    # iteration) against 152 SMs x 128 B/clk at the sampled SM clock
+    sm_mhz = (R["clocks"] or {}).get("sm_mhz") or 2070.0
+    smem_peak = 152 * 128 * sm_mhz * 1e6 / 1e9  # GB/s
+    load = 8 if plain else 4
+    cand.append((("k_cg" if plain else "k_cg_mixed") + " [shared-memory roof]", sm["cg"], 1,
+                 37.0 * load * R["cg_unknown_iters"], smem_peak, "smem",
+                 "shared-memory bandwidth from unit counts: 152 SMs x 128 B/clk x the "
+                 f"sampled SM clock; algorithmic bytes: the 37 stencil loads ({load} B) per "
+                 "unknown and iteration"))
+    digits = 7 if plain else 6
+    slots = st["ace_support_points"] / 128  # total W list length over the tiles
+    gram_bytes = (n * 128 * 8.0 * tiles_w + 256.0 * digits * slots * ((n + 127) // 128) +
+                  8.0 * slots * n)
+    cand.append((f"k_gram_tc (tensor-core M = Phi^T W and W^T psi, exact FP16 digits x {digits})",
+                 gram_ms, 2, gram_bytes, hbm, "hbm",
+                 "HBM of measured (copy); algorithmic bytes: the A rows on the tiles where W is "
+                 f"nonzero (8 B per point), W's FP16 digit planes ({256 * digits} B per tile slot "
+                 "and 128-row block), the FP64 partials written"))
+    expand_bytes = 8.0 * N_TRIAL * float(np.prod(s.grid)) + 4096.0 * digits * tiles_w
+    cand.append((f"k_expand_tc (tensor-core W H, exact FP16 digits x {digits})",
+                 sm["expand_apply"], 1, expand_bytes, hbm, "hbm",
+                 "HBM of measured (copy); algorithmic bytes: the FP64 output (8 B per grid "
+                 f"point and vector) and W's per-tile FP16 digit image ({4 * digits} KB per tile "
+                 "with support and K step of 16 W rows)"))
+
     def _rate(c):  # work per launch / time: flop -> TFLOP/s, bytes -> GB/s
         return c[3] / (c[1] / 1e3) / (1e9 if c[5] in ("hbm", "smem") else 1e12) if c[1] > 0 else 0.0
 
@@ -404,7 +400,8 @@ def run_ours(args, ws, rank, local):
             "peak": peak,
             "unit": "GB/s" if bound == "hbm" else "TFLOP/s",
             "frac": achieved / peak,
-            "traffic": DRAM_BYTES_PER_LAUNCH.get(name.split(" ")[0]) if args.config == "h2o64_96" else None,
+            "traffic": DRAM_BYTES_PER_LAUNCH.get(name.split(" ")[0])
+            if args.config == "h2o64_96" and not plain else None,
             "traffic_unit": "bytes per launch (DRAM read + write, ncu)",
             "peak_note": peak_note,
             "other_kernels": others,
