@@ -139,9 +139,10 @@ typedef struct {
   int ace_dropped_eigenvalues;  /* eigenvalues treated as zero                  */
   int batch_graph;  /* last sea_apply_vxx_batch led by this context: 0 direct
                        launches, 1 graph captured, 2 graph replayed            */
-  int ace_max_tile_list; /* longest W list of a tile, last sea_build_ace (the
-                            mixed form expands lists up to 32 on the tensor
-                            cores, longer ones in FP32 error-free arithmetic) */
+  int ace_max_tile_list; /* longest W list of a tile, last sea_build_ace (lists
+                            up to 32 are expanded on the tensor cores, longer
+                            ones in FP64 or, in the mixed form, FP32 error-free
+                            arithmetic) */
   int batch_order;       /* last sea_apply_vxx_batch led by this context: the
                             autotuned order of the CG's work items (0 ranks
                             round-robin over configurations, 1 all pairs

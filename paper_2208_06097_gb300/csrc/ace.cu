@@ -8,8 +8,9 @@
 //   Mbar = (M + M^T)/2, -Mbar = L L^T (Cholesky, one CTA), L^-1
 //   Xi = W L^-T                              (materialized on request)
 //   V^ACE psi = -Xi Xi^T psi dV = -W L^-T L^-1 (W^T psi dV)
-// The contractions are FP64 FMA on the CUDA cores: on this part the measured
-// FP64 FMA rate is above the FP64 tensor (DMMA) rate.
+// The contractions with W run on the tensor cores by exact digit splitting
+// (gram_tc.cu); tiles with more than SEA_XJ rows of W, and all tiles where device
+// memory does not hold the digit images, take the expansion kernels here.
 #include <type_traits>
 
 #include "sea_internal.cuh"

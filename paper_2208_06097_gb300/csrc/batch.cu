@@ -153,7 +153,7 @@ extern "C" sea_status sea_apply_vxx_batch(sea_ctx* const* ctxs, int n, double* c
   // plans
   for (int k = 0; k < n; ++k) {
     ctxs[k]->have_vxx = ctxs[k]->have_ace = false;
-    ctxs[k]->far_side = false;  // the accumulation forms every contribution itself
+    ctxs[k]->far_side = false;  // until launch_contrib_far
   }
   SEA_BCK(each_on_its_stream(ctxs, n,
                              [](sea_ctx* c) {

@@ -203,8 +203,8 @@ __device__ __forceinline__ int small_float_int(uint32_t f) {
   return __float_as_int(__uint_as_float(f) + 12582912.0f) - 0x4B400000;
 }
 
-// v 2^e2 truncated toward zero to FP64, 0 below the normal range: the same
-// value as scaled_i64_rz, with the 64-bit truncating conversion done by the
+// v 2^e2 truncated toward zero to FP64, 0 below the normal range, with the
+// 64-bit truncating conversion done by the
 // conversion instruction (on the FP64 pipe, which the integer epilogues
 // otherwise leave idle) and the scaling by 2^e2 added to the exponent field.
 __device__ __forceinline__ double scaled_i64_rz_cvt(long long v, int e2) {

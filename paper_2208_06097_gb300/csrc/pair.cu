@@ -2,7 +2,7 @@
 //
 // k_pair_moments (one CTA per pair): rho_ij = phi_i phi_j on Omega_ij and
 //   its multipole moments about the box centre; b = 4 pi rho.
-// k_ghost_eval (one CTA per pair and axis), k_boundary_apply (one CTA per
+// k_ghost_eval (one CTA per pair and axis), k_boundary_apply (BND_CTAS CTAs per
 //   pair): the multipole potential at every point outside the box that the
 //   37-point stencil reaches (one coordinate outside, by 1..6), added to b
 //   with the stencil weights.
@@ -1234,10 +1234,11 @@ __device__ __forceinline__ int inner_cg_smem(const double* __restrict__ r, doubl
 // Inner solve by CG with two reductions per iteration and compensated dot
 // products, the search direction in shared memory in the same padded layout
 // (r, q and d in global memory): the boxes over SEA_CG_SINGLE padded points.  Its
-// iterates are those of the form on global vectors below, whatever the CTA
-// size; the single-reduction arrangement on 1024 threads stopped some of their
-// inner solves an iteration apart, which moved V_xx phi by up to 2.4e-9 of its
-// norm (19 waters on 91^3).  rf holds r / ||r||.  Returns the new total of inner
+// steps are those of the form on global vectors below, and the compensated sums
+// keep them to rounding whatever the CTA size: the inner solves stop at the same
+// iteration (V_xx phi of 19 waters on 91^3 within 6e-12 of its norm), where the
+// single-reduction arrangement on 1024 threads stopped some an iteration apart
+// (2.4e-9).  rf holds r / ||r||.  Returns the new total of inner
 // iterations.
 __device__ __forceinline__ int inner_cg2_smem(float* __restrict__ d, float* __restrict__ rf,
                                               float* __restrict__ qf, float* __restrict__ pS, int n,
@@ -1428,14 +1429,16 @@ __device__ __forceinline__ void cg_pair_mixed(const CgMixedArgs& A, const Stenci
     } else {
     const double inv = 1.0 / rnorm;
     DotF rr0;
+    const bool fits = pad <= A.cap[LARGE];
     for (int t = threadIdx.x; t < n; t += S) {
       const float v = dres ? fmaf(rd[t].x, (float)inv, rd[t].y * (float)inv) : (float)(r[t] * inv);
       rf[t] = v;
-      pf[t] = v;
-      d[t] = 0.f;
-      rr0.add(v, v);
+      if (!fits) {  // inner_cg2_smem sets its own
+        pf[t] = v;
+        d[t] = 0.f;
+        rr0.add(v, v);
+      }
     }
-    const bool fits = pad <= A.cap[LARGE];
     if (fits)
       inner_total = inner_cg2_smem(d, rf, qf, pS, n, ex, ey, ez, Wf, fs0, fs1, inner_total,
                                    A.max_iter);

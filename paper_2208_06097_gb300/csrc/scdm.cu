@@ -642,8 +642,9 @@ cudaError_t launch_scdm(sea_ctx* c, double* U_dev, long long* C_dev) {
     }
     c->launches += 3 * n;
   }
-  // B, then its polar factor: X^T X within 64 n units of rounding of the
-  // identity, or no longer approaching it, ends the iteration
+  // B, then its polar factor: X^T X within 1e-8 of the identity before a step
+  // (which squares the deviation, to rounding), or no longer approaching it, ends
+  // the iteration
   const unsigned gnn = (unsigned)((n * n + 255) / 256);
   const dim3 gp((n + 7) / 8, (n + 15) / 16);
   k_scdm_gather<<<gnn, 256, 0, st>>>(phi, n, N, C_dev, B);
