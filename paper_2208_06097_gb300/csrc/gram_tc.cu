@@ -29,10 +29,10 @@
 // errs by at most 2^-56 (|x| 2^Ew + |w| 2^Ex): an absolute bound per segment, not
 // one relative to the product as an FP64 multiply-add has it.  Values within a
 // factor of 8 (A) or 4 (W) of 2^E are kept whole; where large x meets small w
-// throughout a segment the sum keeps fewer digits than an FP64 chain (W falling
-// by 2^8 where A rises by as much: errors 2^5 times those of a chain, and at
-// 2^56 nothing is left), which matters only to sums that are as small against
-// the operands.  The expansion holds W against the largest value at each point
+// throughout a segment the sum keeps fewer digits than an FP64 chain (rms error
+// of a partial against one's: values of one size 0.25, W falling by 2^4 where A
+// rises by as much 1.1, 2^8 17, 2^14 900), which matters to sums that are as
+// small against the operands.  The expansion holds W against the largest value at each point
 // (k_wx_digits).  Errors of V^ACE psi against extended precision, relative to its
 // norm, 16 to 256 orbitals, 27^3 to 101^3: 3.3 to 6.0e-16, with FP64 multiply-adds
 // 3.9 to 6.3e-16 (with the seven diagonals, W truncated and the tile's scale in
@@ -939,10 +939,10 @@ __global__ void __launch_bounds__(GT2_THREADS, 1)
 // the image.  Digits, diagonals and the final combination are those of
 // k_gram_tc, every D_d the same exact integer, so the partials are the same
 // bits.  Bound by the latency of its loads and conversions; 8 rows of 75^3
-// against 128 orbitals 320 -> 46 us.  Three CTAs an SM (168 registers, 80 in
-// k_expand_few) where the registers left alone allow two: apply of 8 vectors on
-// 75^3 141 -> 122 us mixed, 208 -> 170 us plain (164 with seven diagonals; four
-// CTAs 175).
+// against 128 orbitals 320 -> 35 us.  Three CTAs an SM (168 registers, 80 in
+// k_expand_few; four spill, the registers left alone allow two) and the digits of
+// one z-plane at a time: apply of 8 vectors on 75^3 141 -> 118 us mixed, 208 -> 162
+// us plain.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void mma_16816(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2,
                                           uint32_t a3, uint32_t b0, uint32_t b1) {
@@ -970,9 +970,10 @@ __device__ __forceinline__ double join6(long long a0, int e0, long long a1, int 
 
 constexpr int FEW_WARPS = 4;
 // Rows (GRAM_FEW) and vectors (EXPAND_FEW) up to which the warp-wide kernels are
-// the faster ones.  Measured (128 orbitals on 76^3, six digits): contraction of
-// 8, 24, 32 rows 51, 98, 125 us against 169 to 171 (256 orbitals on 96^3: 32
-// rows 302 against 316); expansion of 8 and 16 vectors 49 and 88 us against 83.
+// the faster ones.  Measured with six digits (seven): contraction of 8 and 32 rows
+// of 75^3 against 128 orbitals 35 and 90 us (45, 129), of 33 rows of 76^3 on the
+// other 177 (217); of 32 and 33 rows of 96^3 against 256 orbitals 211 and 323 (260,
+// 397); expansion of 8 vectors 43 us (66), of 9 to 16 as much again, against 84 (91).
 constexpr int GRAM_FEW = 32, EXPAND_FEW = 8;
 template <int DIG>
 __global__ void __launch_bounds__(32 * FEW_WARPS, 3)
@@ -994,7 +995,6 @@ __global__ void __launch_bounds__(32 * FEW_WARPS, 3)
 #pragma unroll 1
     for (int h = 0; h < 2; ++h) {
       // row a0 + g: x-runs y = q of the planes 2h, 2h + 1
-      uint4 d[2][DIG];
       double v[2][8];
       uint32_t emf = 0;
 #pragma unroll
@@ -1012,8 +1012,6 @@ __global__ void __launch_bounds__(32 * FEW_WARPS, 3)
       emf = max(emf, __shfl_xor_sync(0xffffffffu, emf, 2));
       const int em = (int)(emf >> 20);
       const uint32_t em_sh = DIG == 6 ? (em < 64 ? 0xF0000000u : emf + (5u << 20)) : emf;
-      digits8_u<DIG>(v[0], em_sh, d[0]);
-      digits8_u<DIG>(v[1], em_sh, d[1]);
       float c[ND][4];
 #pragma unroll
       for (int k = 0; k < ND; ++k) c[k][0] = c[k][1] = c[k][2] = c[k][3] = 0.f;
@@ -1023,15 +1021,17 @@ __global__ void __launch_bounds__(32 * FEW_WARPS, 3)
       const uint4* w0 = ws + (in0 ? g : 0) * 2 * DIG * 8;
       const uint4* w1 = ws + (in1 ? g + 8 : 0) * 2 * DIG * 8;
 #pragma unroll
-      for (int l = 0; l < DIG; ++l) {
+      for (int qq = 0; qq < 2; ++qq) {  // the planes in turn: one's digits in registers
+        uint4 d[DIG];
+        digits8_u<DIG>(v[qq], em_sh, d);
         const uint4 z4 = make_uint4(0, 0, 0, 0);
 #pragma unroll
-        for (int qq = 0; qq < 2; ++qq) {
+        for (int l = 0; l < DIG; ++l) {
           const uint4 u0 = in0 ? w0[l * 8 + 4 * qq] : z4, u1 = in1 ? w1[l * 8 + 4 * qq] : z4;
 #pragma unroll
           for (int k = 0; k < DIG && k + l < ND; ++k) {
-            mma_16816(c[k + l], u0.x, u1.x, u0.y, u1.y, d[qq][k].x, d[qq][k].y);
-            mma_16816(c[k + l], u0.z, u1.z, u0.w, u1.w, d[qq][k].z, d[qq][k].w);
+            mma_16816(c[k + l], u0.x, u1.x, u0.y, u1.y, d[k].x, d[k].y);
+            mma_16816(c[k + l], u0.z, u1.z, u0.w, u1.w, d[k].z, d[k].w);
           }
         }
       }
