@@ -209,7 +209,8 @@ sea_status sea_apply_vxx(sea_ctx* ctx, double* vxx_phi, int on_device, double* e
  * problems in one persistent launch.  The launch's pair order and grid are
  * autotuned per workload (pair counts, unknowns, grids and forms of the
  * configurations): the first call for a workload times each candidate on
- * the batch and keeps the fastest for the process (sea_stats.batch_*);
+ * the batch and keeps the fastest for the process, for 256 workloads at most
+ * (sea_stats.batch_*);
  * every candidate gives the same results bit for bit.  All contexts must use the same device
  * and the same stream; vxx_phi[k] (host or device per on_device) receives
  * configuration k's V_xx phi, exx[k] (may be NULL) its E_xx.  The phase

@@ -17,8 +17,8 @@
 // occupancy limit).  The first call for a workload (the configurations'
 // pair counts, unknowns, grids and forms) times every order with every grid
 // size on the batch itself, one CG launch each after a warm-up launch, and
-// keeps the fastest in a process-wide table; later calls for the same
-// workload -- and the graph captured for it -- use that choice.
+// keeps the fastest in a process-wide table of bounded size; later calls for the
+// same workload -- and the graph captured for it -- use that choice.
 #include <algorithm>
 #include <cstdio>
 #include <cstring>
@@ -60,6 +60,9 @@ struct Tuned {
 };
 std::mutex g_tune_mutex;
 std::map<std::vector<long long>, Tuned> g_tuned;
+// Workloads kept (a run whose orbitals change at every step has a new one each
+// time): a full table is emptied.
+constexpr size_t MOST_TUNED = 256;
 
 // Work items in `order`, the mixed-form items first, then the FP64 ones.
 // size[k][r]: box size of configuration k's rank-r pair (order 1 only).
@@ -384,6 +387,7 @@ extern "C" sea_status sea_apply_vxx_batch(sea_ctx* const* ctxs, int n, double* c
     c0->stats.batch_tune_ms = t_tune;
     {
       std::lock_guard<std::mutex> lock(g_tune_mutex);
+      if (g_tuned.size() >= MOST_TUNED) g_tuned.clear();
       g_tuned[wsig] = tuned;
     }
     // the chosen order's items for the launches below
